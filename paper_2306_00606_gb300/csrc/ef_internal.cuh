@@ -375,8 +375,18 @@ struct F2Sum {
 };
 __device__ __forceinline__ double f2_value(float2 t) { return (double)t.x + (double)t.y; }
 
-// d * log2(d) for integral d >= 1 held in a float (MUFU lg2).
-__device__ __forceinline__ float dlog2d(float d) { return d * __log2f(d); }
+// log2(d) for d >= 1: the MUFU instruction alone.  (__log2f, without -ftz,
+// adds a test and two scaling instructions for subnormal arguments; on normal
+// ones the two agree bit for bit.  FP32C class passes on the power-law graph
+// 0.64 -> 0.55 ms, small wedges 0.286 -> 0.257 ms.)
+__device__ __forceinline__ float lg2(float d) {
+    float r;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return r;
+}
+
+// d * log2(d) for integral d >= 1 held in a float.
+__device__ __forceinline__ float dlog2d(float d) { return d * lg2(d); }
 
 // Two floats rounded to BF16 (nearest, ties to even), lo in the low half.
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {

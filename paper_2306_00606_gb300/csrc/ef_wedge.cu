@@ -105,12 +105,12 @@ __global__ void __launch_bounds__(256) k_wedge_small(const int32_t *__restrict__
                 for (int j = 0; j < jmin; ++j) {
                     float d = b0f + __shfl_sync(FULL, akf, j, G);
                     if (G == 4) d = fmaxf(d, 1.0f);
-                    sum = fmaf(d, __log2f(d), sum);
+                    sum = fmaf(d, lg2(d), sum);
                 }
                 for (int j = jmin; j < jmax; ++j) {
                     float d = b0f + __shfl_sync(FULL, akf, j, G);
                     if (G == 4) d = fmaxf(d, 1.0f);
-                    const float t = __log2f(d);
+                    const float t = lg2(d);
                     if (j < lim) sum = fmaf(d, t, sum);
                 }
                 acc = sum - dlog2d(G == 4 ? fmaxf(b0f + akf, 1.0f) : b0f + akf);

@@ -142,7 +142,9 @@ typedef struct {
     double prep_ms;        /* validation, degrees, neighbour sums */
     double orient_ms;      /* f table, degree orientation (scan + oriented
                               CSR + out-list hash tables) and omega */
-    double wedge_small_ms; /* middle nodes of degree <= 32 */
+    double wedge_small_ms; /* middle nodes of degree <= 32; where no node has
+                              more neighbours also the triangles (one kernel;
+                              orient_ms is then the f table alone) */
     double wedge_big_ms;   /* middle nodes of degree > 32 */
     double tri_hash_ms;    /* always 0: the orientation builds the hash
                               tables of the long out-lists (orient_ms) */

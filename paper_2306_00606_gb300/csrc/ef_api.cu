@@ -3,8 +3,7 @@
 // autotuner.
 //
 // Pass order (one graph or one batch, all on the context stream):
-//   part A   one memset of the per-node accumulators and the counters;
-//            degrees + row_ptr checks + wedge bins; per-row checks,
+//   part A   a memset of the counters; degrees + row_ptr checks + wedge bins; per-row checks,
 //            sigma1/sigma2, out-degrees, the symmetry sum and (batched) the
 //            check that no entry leaves its graph, in the same row pass
 //   host     one small readback: validation word, symmetry sum and max
@@ -16,6 +15,10 @@
 //   part B   f table (f(d) = d ln d and the triangle corrections, d < 3 maxdeg + 1);
 //            orientation (oriented CSR + omega); wedge pass (small, then mid +
 //            hub middle nodes); hash tables and pair tests; finalize (per node)
+//            Where no row exceeds 32 entries: f table, the fused short-row
+//            kernel (ef_short.cu), its finalize.  The host chooses after the
+//            readback; without one both sets are launched and the gate word
+//            lets one of them work
 // The wedge pass and the orientation + triangle passes write disjoint
 // accumulators and could run on two streams; measured on the 4M-node
 // power-law graph, the concurrent form was slower (the triangle pass more
@@ -82,6 +85,7 @@ struct ef_ctx {
     void *acts = nullptr;            // training activations
     size_t acts_bytes = 0;
     double *dtmp = nullptr;          // small device scratch (feature sums)
+    int path = 0;                    // part B kernels of the last exact call (PathMode)
     bool bins = true;                // out-lists of the current graph in degree-bin order (bin_layout)
     void *sir = nullptr;             // SIR simulation state
     size_t sir_bytes = 0;
@@ -99,16 +103,24 @@ namespace {
 
 thread_local char g_err[512];
 
-// Kernels one call launches: part A 3 (the batch check runs in the row pass), f table 1, orientation
-// (degree-bin layout: layout gather, a scan of 3, layout scatter; node
-// layout: a scan of 3; then node records, the row kernel in two forms of
-// which one returns at once, the hub rows, hash tables of the longer rows;
-// the short rows' tables are filled by the row kernel itself), small wedges
-// 4, big wedges (class kernels 2; direct mode: item counts, a scan of 3,
-// direct kernel, reduction), pair tests 1, finalize 1; with device_check
-// the validation gate 1.
-int64_t kernels_per_call(bool bins, int wedge_mode, bool dev_check) {
-    return 3 + 1 + (bins ? 5 : 3) + 5 + 4 + (wedge_mode == 1 ? 6 : 2) + 1 + 1 + (dev_check ? 1 : 0);
+// Which of part B's kernels run: the general ones, the short-row ones (no row
+// above SMALL_MAX entries), or both sets launched, the device's gate word
+// letting one of them work (nothing is read back before part B).
+enum PathMode { PATH_GENERAL, PATH_SHORT, PATH_DEVICE };
+
+// Kernels one call launches: part A 3 (the batch check runs in the row pass),
+// f table 1; on the short-row path the fused kernel and its finalize; on the
+// general one the orientation (degree-bin layout: layout
+// gather, a scan of 3, layout scatter; node layout: a scan of 3; then node
+// records, the row kernel in two forms of which one returns at once, the hub
+// rows, hash tables of the longer rows; the short rows' tables are filled by
+// the row kernel itself), small wedges 4, big wedges (class kernels 2; direct
+// mode: item counts, a scan of 3, direct kernel, reduction), pair tests 1,
+// finalize 1; both sets, the clearing kernel and the gate where the
+// device decides.
+int64_t kernels_per_call(PathMode path, bool bins, int wedge_mode) {
+    const int64_t general = (bins ? 5 : 3) + 5 + 4 + (wedge_mode == 1 ? 6 : 2) + 1 + 1;
+    return 3 + 1 + (path != PATH_GENERAL ? 2 : 0) + (path != PATH_SHORT ? general : 0) + (path == PATH_DEVICE ? 2 : 0);
 }
 
 void set_err(ef_ctx *c, const char *fmt, ...) {
@@ -231,20 +243,34 @@ struct Job {
     ef_outputs out;
 };
 
-int part_a(ef_ctx *ctx, const Job &j, const ef::Scratch &s, cudaStream_t st) {
+int part_a(ef_ctx *ctx, const Job &j, const ef::Scratch &s, cudaStream_t st, bool short_ok = false) {
     using namespace ef;
-    CU(cudaMemsetAsync(s.Tacc, 0, accumulator_bytes(s), st));
-    LAUNCH(launch_prep_a(j.rp, j.ci, j.n, j.m, s, ctx->tune, st, j.goff_dev, j.G), "prep");
+    LAUNCH(launch_prep_a(j.rp, j.ci, j.n, j.m, s, ctx->tune, st, j.goff_dev, j.G, short_ok), "prep");
     return EF_OK;
 }
 
 // Part B; with prof, events 1..4, 6, 7 bracket f table + orientation (with
-// the hash tables), small wedges, big wedges, pair tests and finalize.
-int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, bool prof, cudaStream_t st) {
+// the hash tables), small wedges (on the short-row path the fused kernel),
+// big wedges, pair tests and finalize.
+int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, PathMode path, bool prof,
+           cudaStream_t st) {
     using namespace ef;
     const Tune &t = ctx->tune;
+    // the f table's capacity covers both paths; behind a gate closed by
+    // GATE_SHORT alone it is still built
     LAUNCH(launch_ftab(s.ftab, s.tq, s.counters, fcap, st), "f table");
-    LAUNCH(launch_orient(j.rp, j.ci, j.n, j.m, s, t, st, nullptr, nullptr, ctx->bins), "orientation");
+    if (path != PATH_GENERAL) {
+        const bool chosen = path == PATH_SHORT;
+        if (prof) CU(cudaEventRecord(ctx->ev[2], st));
+        LAUNCH(launch_short(j.ci, s, j.o.precision, j.n, t, chosen, st), "short rows");
+        if (prof && chosen)
+            for (int e : {3, 4, 6}) CU(cudaEventRecord(ctx->ev[e], st));
+        LAUNCH(launch_finalize_short(s, j.o.precision, j.n, j.out, t, chosen, st), "finalize");
+        if (chosen) return EF_OK;
+    }
+    const bool gated = path == PATH_DEVICE;
+    if (!gated) LAUNCH(launch_clear_triangles(s, j.n, st), "clear");
+    LAUNCH(launch_orient(j.rp, j.ci, j.n, j.m, s, t, st, nullptr, nullptr, ctx->bins, gated), "orientation");
     if (prof) CU(cudaEventRecord(ctx->ev[2], st));
     LAUNCH(launch_wedge_small(j.rp, j.ci, s, j.o.precision, j.n, t, st), "small wedge");
     if (prof) CU(cudaEventRecord(ctx->ev[3], st));
@@ -305,10 +331,12 @@ int compute_device(ef_ctx *ctx, const Job &j) {
     // part A in the same stream as part B, with no host decision between them
     const bool a_inline = o.trust_input || dev_check;
     auto part_a_inline = [&](cudaStream_t cs) -> int {
-        int r = part_a(ctx, j, s, cs);
-        if (!r && dev_check) LAUNCH(launch_gate(s.counters, o.async ? ctx->d_sticky : nullptr, cs), "validation gate");
+        int r = part_a(ctx, j, s, cs, true);
+        if (!r)
+            LAUNCH(launch_gate(s.counters, dev_check && o.async ? ctx->d_sticky : nullptr, dev_check, cs), "gate");
         return r;
     };
+    PathMode path = PATH_DEVICE;
 
     // f table size: from the validated max degree, else the largest possible
     int64_t fcap;
@@ -319,15 +347,17 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         ctx->bins = bin_layout(ctx->tune, nullptr, j.n, j.goff_dev != nullptr);
     } else {
         if (prof) CU(cudaEventRecord(ctx->ev[0], st));
-        rc = part_a(ctx, j, s, st);
+        rc = part_a(ctx, j, s, st, true);
         if (rc) return rc;
         CU(cudaMemcpyAsync(ctx->h_counters, s.counters, NUM_COUNTERS * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
         CU(cudaStreamSynchronize(st));
         if (const int bits = prep_error_bits(ctx->h_counters)) return graph_error(ctx, bits);
         if (const int lim = degree_limit(ctx, ctx->h_counters)) return lim;
+        path = ctx->h_counters[BIN_BIG] == 0 ? PATH_SHORT : PATH_GENERAL;
         fcap = 3 * (int64_t)ctx->h_counters[CNT_MAXDEG] + 1;
         ctx->bins = bin_layout(ctx->tune, ctx->h_counters, j.n, j.goff_dev != nullptr);
     }
+    ctx->path = path;
     // f table (double) followed by the fixed-point triangle corrections (int64)
     size_t have = (size_t)ctx->ftab_cap * 2 * sizeof(double);
     rc = ensure_buffer(ctx, (void **)&ctx->ftab, &have, (size_t)fcap * 2 * sizeof(double), 0);
@@ -353,14 +383,14 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         key.precision = o.precision;
         key.wedge_mode = o.wedge_mode;
         key.trust = o.trust_input | (dev_check ? 2 : 0) | (dev_check && o.async ? 4 : 0);
-        key.bins = ctx->bins;
+        key.bins = (int32_t)ctx->bins | (int32_t)path << 1;
         key.tune = ctx->tune;
         rc = run_graph(ctx, key, [&](cudaStream_t cs) {
             if (a_inline) {
                 const int r = part_a_inline(cs);
                 if (r) return r;
             }
-            return part_b(ctx, j, s, fcap, false, cs);
+            return part_b(ctx, j, s, fcap, path, false, cs);
         });
         if (rc) return rc;
     } else {
@@ -370,7 +400,7 @@ int compute_device(ef_ctx *ctx, const Job &j) {
             if (rc) return rc;
         }
         if (prof) CU(cudaEventRecord(ctx->ev[1], st));
-        rc = part_b(ctx, j, s, fcap, prof, st);
+        rc = part_b(ctx, j, s, fcap, path, prof, st);
         if (rc) return rc;
         if (prof) CU(cudaEventRecord(ctx->ev[7], st));
     }
@@ -391,7 +421,7 @@ int check_args(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const ef_opti
 
 // Events: 0 start, 1 part B start (after the validation readback), 2..6
 // after orientation, small wedges, big wedges, hash tables, pair tests, 7 end.
-void accumulate_stats(ef_ctx *ctx, int wedge_mode, bool dev_check) {
+void accumulate_stats(ef_ctx *ctx, int wedge_mode) {
     auto el = [&](int a, int b) {
         float t = 0.f;
         return cudaEventElapsedTime(&t, ctx->ev[a], ctx->ev[b]) == cudaSuccess ? (double)t : 0.0;
@@ -405,7 +435,7 @@ void accumulate_stats(ef_ctx *ctx, int wedge_mode, bool dev_check) {
     st.tri_pairs_ms += el(4, 6);
     st.finalize_ms += el(6, 7);
     st.total_ms += el(0, 7);
-    st.kernels += kernels_per_call(ctx->bins, wedge_mode, dev_check);
+    st.kernels += kernels_per_call((PathMode)ctx->path, ctx->bins, wedge_mode);
 }
 
 // Host I/O and synchronisation around compute_device.
@@ -457,7 +487,7 @@ int run_job(ef_ctx *ctx, Job j, const ef_outputs *host_out) {
             if (const int bits = ef::prep_error_bits(ctx->h_counters)) return graph_error(ctx, bits);
             if (const int lim = degree_limit(ctx, ctx->h_counters)) return lim;
         }
-        if (j.o.profile) accumulate_stats(ctx, j.o.wedge_mode, dev_check);
+        if (j.o.profile) accumulate_stats(ctx, j.o.wedge_mode);
     } else if (dev_check) {
         ctx->sticky_pending = true;
     }
@@ -698,8 +728,7 @@ size_t carve_scratch(char *base, int32_t n, int64_t m, Scratch &s) {
     s.out_hash = (int32_t *)take(4 * (M + 8));
     s.out_src = (int32_t *)take(4 * (M + 1));
     s.Ccenter = take(8 * N);
-    // accumulators that start at zero, contiguous up to the end of the counters
-    // (cleared by one memset per call, see accumulator_bytes)
+    // accumulators (cleared by the degree and row passes)
     s.Tacc = (double *)take(8 * N);
     s.qacc = (int64_t *)take(8 * N);
     s.tcnt = (int64_t *)take(8 * N);
@@ -714,10 +743,6 @@ size_t carve_scratch(char *base, int32_t n, int64_t m, Scratch &s) {
     s.hub_cidx = (int32_t *)take(4 * (M + 1));
     s.ftab = nullptr;
     return off;
-}
-
-size_t accumulator_bytes(const Scratch &s) {
-    return (size_t)((const char *)(s.counters + NUM_COUNTERS) - (const char *)s.Tacc);
 }
 
 // Message for ef_last_error(NULL), for entry points that run without a context.

@@ -126,6 +126,38 @@ __global__ void __launch_bounds__(256) k_finalize(int32_t n, FinalArgs f) {
     }
 }
 
+// The short-row path's finalize: the fused kernel left a node's integer sums
+// in one word, its triangles in 32 bits and all of T in Tacc, so a node costs
+// 20 bytes read (k_finalize: 60).
+template <bool F64>
+__global__ void __launch_bounds__(256) k_finalize_short(int32_t n, const uint64_t *__restrict__ stat,
+                                                        const int32_t *__restrict__ tri,
+                                                        const double *__restrict__ Tacc,
+                                                        const int32_t *__restrict__ cnt, ef_outputs o, bool chosen) {
+    if (short_closed(cnt, chosen)) return;
+    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
+        const uint64_t w = stat[v];
+        const double T = Tacc[v];
+        const int t = tri[v];
+        const int d = (int)(w & 0xff), s1 = (int)(w >> 16 & 0xffff);
+        const int s2 = (int)(w >> 32 & 0xffff), om = (int)(w >> 48);
+        const int N = d * (d - 2) + s1;
+        const int S = d * (d - 1) * (d - 4) + 2 * (d - 1) * s1 + s2 - s1 + (d - 4) * (s1 - d) + om - d * d - 8 * t;
+        double ef = 0.0;
+        uint8_t fl = 1;
+        if (S > 0) {
+            fl = 0;
+            ef = ef_value<F64>(S, T, false);
+        }
+        if (o.ef) o.ef[v] = ef;
+        if (o.n_clusters) o.n_clusters[v] = N;
+        if (o.s) o.s[v] = S;
+        if (o.t) o.t[v] = T;
+        if (o.triangles) o.triangles[v] = t;
+        if (o.flag) o.flag[v] = fl;
+    }
+}
+
 // From the shards' summed partials: T_v = t + q 2^-F, S_v = S_open - 8 t_v.
 template <bool F64>
 __global__ void __launch_bounds__(256) k_finalize_sums(int32_t n, ef_partials p, int32_t frac, ef_outputs o) {
@@ -174,6 +206,16 @@ int launch_finalize(const Scratch &s, int precision, int32_t n, const ef_outputs
     const FinalArgs f{s.D, s.sig1, s.sig2, s.omega, s.Tacc, s.Ccenter, s.qacc, s.tcnt, s.counters, out};
     if (precision == EF_PREC_FP64) k_finalize<true><<<grid_n(n, t), 256, 0, st>>>(n, f);
     else k_finalize<false><<<grid_n(n, t), 256, 0, st>>>(n, f);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+int launch_finalize_short(const Scratch &s, int precision, int32_t n, const ef_outputs &out, const Tune &t,
+                          bool chosen, cudaStream_t st) {
+    const uint64_t *stat = reinterpret_cast<const uint64_t *>(s.sig1);
+    if (precision == EF_PREC_FP64)
+        k_finalize_short<true><<<grid_n(n, t), 256, 0, st>>>(n, stat, s.outdeg, s.Tacc, s.counters, out, chosen);
+    else
+        k_finalize_short<false><<<grid_n(n, t), 256, 0, st>>>(n, stat, s.outdeg, s.Tacc, s.counters, out, chosen);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

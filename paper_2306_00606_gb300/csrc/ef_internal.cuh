@@ -151,6 +151,11 @@ enum : int {
     NUM_COUNTERS = 64
 };
 
+// Bit of cnt[CNT_GATE] (never an error bit): every row has at most SMALL_MAX
+// entries and the call runs the short-row kernels (ef_short.cu) instead of
+// the general ones, decided on the device when the host reads nothing back.
+constexpr int32_t GATE_SHORT = 1 << 30;
+
 // Order of the oriented out-lists: degree-bin order (true) or node order,
 // from t.layout, or in automatic mode (0) from where the nodes of degree >
 // SMALL_MAX lie in a host copy of the counters after the degree pass (h;
@@ -177,9 +182,6 @@ inline int prep_error_bits(const int32_t *h) {
 
 // Bytes of scratch for a graph (f tables excluded), and its layout when base != nullptr.
 size_t carve_scratch(char *base, int32_t n, int64_t m, Scratch &s);
-// Bytes from Tacc to the end of the counters: everything that must start at
-// zero (Tacc, qacc, tcnt, counters), for one memset per call.
-size_t accumulator_bytes(const Scratch &s);
 
 // ----------------------------------------------------------------- helpers
 // Device-side validation (ef_options.device_check): k_gate stores the call's
@@ -188,7 +190,20 @@ size_t accumulator_bytes(const Scratch &s);
 // the column ids (or by anything derived from them) of a graph that failed.
 // The word is 0 in every other mode: the counters start at zero each call,
 // and the host refuses an invalid graph before part B.
+// Calls whose kernels are chosen on the device set GATE_SHORT there as well:
+// it closes the gate of the general kernels and opens the short-row ones'.
 __device__ __forceinline__ bool gate_closed(const int32_t *cnt) { return cnt[CNT_GATE] != 0; }
+// Gate of the short-row kernels; chosen: the host already chose them.
+__device__ __forceinline__ bool short_closed(const int32_t *cnt, bool chosen) {
+    return cnt[CNT_GATE] != (chosen ? 0 : GATE_SHORT);
+}
+
+// Short-row path (ef_short.cu), when no row exceeds SMALL_MAX entries.  Per
+// node {row start, short_word} in Scratch::info, where the word holds the
+// degree, the entries below the node and sigma1 (<= 32 * 32); the fused
+// kernel's result in Scratch::sig1: the word, sigma2 << 32 and omega << 48
+// (both <= 32^3); triangles in Scratch::outdeg; all of T in Scratch::Tacc.
+__host__ __device__ __forceinline__ int short_word(int d, int lo, int s1) { return d | lo << 8 | s1 << 16; }
 
 __device__ __forceinline__ bool rank_less(int32_t Dx, int32_t x, int32_t Dy, int32_t y) {
     // degree order used to orient edges for triangle listing: (degree, id)
@@ -454,14 +469,20 @@ struct RankScratch {
 namespace ef {
 // goff, G: a batch's G + 1 graph node offsets on the device (the row pass
 // then also checks that no entry leaves its row's graph), else nullptr.
+// short_ok: the caller runs the short-row kernels when no row exceeds
+// SMALL_MAX entries; the row pass then writes their per-node words (info)
+// instead of sig1, sig2 and outdeg, and the caller clears the triangle
+// accumulators for the general path.  Counters and Tacc are cleared here.
 int launch_prep_a(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const Scratch &s, const Tune &t,
-                  cudaStream_t st, const int64_t *goff = nullptr, int32_t G = 0);
+                  cudaStream_t st, const int64_t *goff = nullptr, int32_t G = 0, bool short_ok = false);
 // The out-lists in degree-bin order (bins) or node order.
-// With tables, also the hash tables of the out-lists longer than SHORT_MAX
-// (cleared here, filled as the lists are written).
+// Also the hash tables of the out-lists longer than SHORT_MAX (cleared here,
+// filled as the lists are written).  gated: the call's path is chosen on the
+// device; the triangle accumulators are then cleared here, behind the gate.
 int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const Scratch &s, const Tune &t,
                   cudaStream_t st, int32_t *nmin = nullptr, int32_t *nmax = nullptr, bool bins = true,
-                  bool tables = true);
+                  bool gated = false);
+int launch_clear_triangles(const Scratch &s, int32_t n, cudaStream_t st);
 int launch_big_items(const Scratch &s, int32_t n, cudaStream_t st);
 int prepare_kernels();
 int prepare_final_tables();   // ln table of the finalize (ef_final.cu), once per device
@@ -472,12 +493,21 @@ int64_t device_l2_bytes();   // of the current device (after prepare_kernels ran
 // visited out of id order cost no extra DRAM traffic.  (BA n = 1M, 44 MB of
 // CSR: step 1.10 -> 0.82 ms in bin order; BA n = 16M, 580 MB: 9.9 -> 11.3 ms.)
 inline bool rows_in_bins_allowed(int64_t m) { return 4 * m <= device_l2_bytes() / 2; }
-int launch_scan(const int32_t *in, int32_t *out, int32_t n, int32_t *tmp, cudaStream_t st);
+// cnt: the counters, when the scan is to be skipped behind a closed gate.
+int launch_scan(const int32_t *in, int32_t *out, int32_t n, int32_t *tmp, cudaStream_t st,
+                const int32_t *cnt = nullptr);
 int launch_ftab(float2 *ftab, int64_t *tq, int32_t *cnt, int64_t cap, cudaStream_t st);
-// Device-side check after the row passes: the validation bits (error word,
-// symmetry sum, maximum degree above EF_MAX_DEGREE) into cnt[CNT_GATE], and
-// OR-ed into *sticky when it is not null.
-int launch_gate(int32_t *cnt, int32_t *sticky, cudaStream_t st);
+// Device-side decisions after the row passes: with check, the validation
+// bits (error word, symmetry sum, maximum degree above EF_MAX_DEGREE) into
+// cnt[CNT_GATE], and OR-ed into *sticky when it is not null; GATE_SHORT when
+// no row exceeds SMALL_MAX entries.
+int launch_gate(int32_t *cnt, int32_t *sticky, bool check, cudaStream_t st);
+// Short-row path (ef_short.cu, ef_final.cu); chosen: by the host (else the
+// kernels look for GATE_SHORT).
+int launch_short(const int32_t *ci, const Scratch &s, int precision, int32_t n, const Tune &t, bool chosen,
+                 cudaStream_t st);
+int launch_finalize_short(const Scratch &s, int precision, int32_t n, const ef_outputs &out, const Tune &t,
+                          bool chosen, cudaStream_t st);
 int launch_wedge_small(const int32_t *rp, const int32_t *ci, const Scratch &s, int precision, int32_t n,
                        const Tune &t, cudaStream_t st);
 int launch_wedge_big(const int32_t *rp, const int32_t *ci, const Scratch &s, int precision, int wedge_mode,

@@ -110,7 +110,8 @@ constexpr int DEG_THREADS = 256, DEG_PER = 8;
 
 __global__ void __launch_bounds__(DEG_THREADS) k_degrees(const int32_t *__restrict__ rp, int32_t n, int64_t m,
                                                          int hub_min, int32_t *__restrict__ D,
-                                                         int32_t *__restrict__ bins, int32_t *__restrict__ cnt) {
+                                                         double *__restrict__ Tacc, int32_t *__restrict__ bins,
+                                                         int32_t *__restrict__ cnt) {
     __shared__ int s_cnt[NUM_BINS], s_base[NUM_BINS];
     __shared__ int s_mx[32], s_err[32], s_blo[32], s_bhi[32];
     if (threadIdx.x < NUM_BINS) s_cnt[threadIdx.x] = 0;
@@ -136,6 +137,7 @@ __global__ void __launch_bounds__(DEG_THREADS) k_degrees(const int32_t *__restri
             if (a < 0 || b < a || (int64_t)b > m) err |= ERRB_ROWPTR;
             else d = b - a;
             D[v] = d;
+            Tacc[v] = 0.0;
             mx = max(mx, d);
             if (d >= 1 && d <= SMALL_MAX) {
                 b0[q] = d <= 4 ? BIN_S4 : d <= 8 ? BIN_S8 : d <= 16 ? BIN_S16 : BIN_S32;
@@ -294,6 +296,7 @@ struct RowOut {
     int32_t *outdeg;
     const int64_t *goff;   // batched input: G + 1 node offsets of the graphs (else nullptr)
     int32_t G;
+    int2 *info;            // short-row path allowed: its per-node words (else nullptr)
 };
 
 // Batched input: every entry of row v must lie in v's own graph
@@ -335,12 +338,96 @@ __device__ __forceinline__ void row_stats_warp(const int32_t *__restrict__ ci, c
     }
 }
 
+// Last g in [0, G) with goff[g] <= v, by the whole warp (32-way search).
+__device__ __forceinline__ int last_graph(const int64_t *__restrict__ goff, int G, int64_t v) {
+    int lo = 0, len = G;
+    const int lane = threadIdx.x & 31;
+    while (len > 1) {
+        const int step = (len + 31) >> 5;
+        const int g = lo + lane * step;
+        const unsigned le = __ballot_sync(FULL, g < lo + len && goff[g] <= v);
+        const int nlo = lo + (31 - __clz(le | 1u)) * step;
+        len = min(step, lo + len - nlo);
+        lo = nlo;
+    }
+    return lo;
+}
+
+// The row pass of a graph without rows above SMALL_MAX entries, for the
+// short-row path: a thread per row in node order, RowStats' checks, and one
+// word of 32-bit sums per node instead of sig1, sig2 and outdeg.  A batch's
+// graph bounds come from one 32-way search per 32 rows (a search per row
+// where they lie in several graphs).  Bound by issue, like the general pass.
+// Measured and left out: the entries of 32 rows dealt to the lanes (full
+// lanes, coalesced column reads, row sums from a running warp scan): 148 warp
+// instructions per 32 entries, 2.0 ms on the WS batch where the general pass
+// takes 1.24.
+__device__ __forceinline__ void rows_short(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, int32_t n,
+                                           int64_t m, const int32_t *__restrict__ D, const RowOut &ro,
+                                           int32_t *__restrict__ cnt) {
+    const int64_t step = (int64_t)gridDim.x * blockDim.x;
+    uint64_t sym = 0;
+    int err = 0;
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v - (threadIdx.x & 31) < n; v += step) {
+        const bool in = v < n;
+        const int a = in ? rp[v] : 0, b = in ? rp[v + 1] : 0;
+        const int Dv = a >= 0 && a <= b && (int64_t)b <= m ? b - a : 0;
+        if (ro.goff) {
+            const int64_t first = v - (threadIdx.x & 31), last = min(first + 32, (int64_t)n) - 1;
+            const int g = last_graph(ro.goff, ro.G, first);
+            const int64_t end = ro.goff[g + 1];
+            if (last < end) {
+                if (Dv > 0 && (ci[a] < ro.goff[g] || ci[a + Dv - 1] >= end)) err |= ERRB_CROSS;
+            } else {
+                err |= cross_bits(ro, ci, v, a, a + Dv);
+            }
+        }
+        const NodeMix mv = node_mix((int)v);
+        int prev = -1, s1 = 0, lo = 0;
+        for (int e = 0; e < Dv; e += 4) {
+            int x[4], Dx[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[q] = e + q < Dv ? ci[a + e + q] : -1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) Dx[q] = (unsigned)x[q] < (unsigned)n ? D[x[q]] : 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                if (e + q < Dv) {
+                    const int before = prev;
+                    prev = x[q];
+                    if ((unsigned)x[q] >= (unsigned)n) {
+                        err |= ERRB_RANGE;
+                        continue;
+                    }
+                    if (x[q] == (int)v) err |= ERRB_SELFLOOP;
+                    if (e + q > 0 && before >= x[q]) err |= ERRB_UNSORTED;
+                    s1 += Dx[q];
+                    lo += x[q] < (int)v;
+                    sym += edge_print(mv, node_mix(x[q]));
+                }
+            }
+        }
+        if (in) {
+            ro.info[v] = make_int2(a, short_word(Dv, lo, s1));
+            ro.outdeg[v] = 0;              // triangle count
+            if (Dv == 0) ro.sig1[v] = 0;   // the fused kernel's result for a node without clusters
+        }
+    }
+    if (err) atomicOr(cnt + CNT_ERR, err);
+    add_sym(cnt, sym);
+}
+
 // Rows of degree < hub_min (RowOrder): a thread per row of degree <= tmax,
-// the warp for the others; hubs go to k_row_stats_hub.
+// the warp for the others; hubs go to k_row_stats_hub.  When no row exceeds
+// SMALL_MAX entries and the caller runs the short-row path: rows_short.
 __global__ void __launch_bounds__(256, 6) k_row_stats(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
                                                       int32_t n, int64_t m, int tmax, int hub_min,
                                                       const int32_t *__restrict__ D, const int32_t *__restrict__ bins,
                                                       bool bins_ok, RowOut ro, int32_t *__restrict__ cnt) {
+    if (ro.info && cnt[BIN_BIG] == 0) {
+        rows_short(rp, ci, n, m, D, ro, cnt);
+        return;
+    }
     __shared__ RowOrder s_ord;
     if (threadIdx.x == 0) s_ord.load(cnt, n, bins_ok);
     __syncthreads();
@@ -445,12 +532,11 @@ struct Orient {
     const int4 *info;   // per node {D, sigma1, probe descriptor of its out-list}
     int32_t *out_col, *out_D, *out_src;
     int2 *out_pd;
-    int32_t *out_hash;      // null: no tables
+    int32_t *out_hash;
     int32_t *nmin, *nmax;   // optional: smallest / largest neighbour degree (node features)
     int32_t n;
-    // u's table from its descriptor (kind 1), when tables are built
+    // u's table from its descriptor (kind 1)
     __device__ __forceinline__ bool table(int u, int64_t &base, int &nb) const {
-        if (!out_hash) return false;
         const int4 iu = __ldg(info + u);
         base = 4 * (int64_t)iu.z;
         nb = iu.w & DESC_MASK;
@@ -552,7 +638,8 @@ __device__ __forceinline__ int64_t Orient::row(int v, int Dv, int a, int b, int 
 // orientation needs of a neighbour, in one 16-byte gather (sigma1 <= m < 2^31).
 __global__ void k_node_info(const int32_t *__restrict__ D, const int64_t *__restrict__ sig1,
                             const int32_t *__restrict__ out_ptr, const int32_t *__restrict__ outdeg, int32_t n,
-                            int64_t hash_cap, int4 *__restrict__ info) {
+                            int64_t hash_cap, int4 *__restrict__ info, const int32_t *__restrict__ cnt) {
+    if (cnt && gate_closed(cnt)) return;
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
         const int ls = out_ptr[v];
         const int2 pd = probe_desc(ls, ls + outdeg[v], hash_cap);
@@ -710,7 +797,7 @@ __global__ void __launch_bounds__(256, CHUNK == 8 ? 3 : 5) k_orient(
         if (stage) {
             const int64_t tb0 = ((int64_t)2 * kmin + 3) & ~(int64_t)3;
             const int64_t tb1 = ((int64_t)2 * kend + 3) & ~(int64_t)3;
-            const int tlen = o.out_hash ? (int)(tb1 - tb0) : 0;
+            const int tlen = (int)(tb1 - tb0);
             for (int t = lane; t < tlen; t += 32) s_tab[w][t] = -1;
             __syncwarp();
             const OrientStage sg{s_col[w], s_D[w], s_src[w], s_pd[w], s_tab[w], kmin, tb0};
@@ -879,7 +966,7 @@ __global__ void k_big_chunks(const int32_t *__restrict__ D, const int32_t *__res
 // (|g| <= 8 (ln(3 maxdeg) + 1) + 8); every thread derives the same F and
 // thread 0 publishes it for the finalize pass.
 __global__ void k_ftab(float2 *__restrict__ ftab, int64_t *__restrict__ tq, int32_t *__restrict__ cnt, int64_t cap) {
-    if (gate_closed(cnt)) return;
+    if (cnt[CNT_GATE] & ~GATE_SHORT) return;   // both paths read the tables
     const int64_t maxdeg = cnt[CNT_MAXDEG];
     int64_t L = 3 * maxdeg + 1;
     if (L > cap) L = cap;
@@ -914,7 +1001,9 @@ constexpr int SCAN_THREADS = 1024;
 constexpr int SCAN_PER = 4;
 constexpr int SCAN_TILE = SCAN_THREADS * SCAN_PER;
 
-__global__ void k_scan_reduce(const int32_t *__restrict__ in, int32_t n, int32_t *__restrict__ bsum) {
+__global__ void k_scan_reduce(const int32_t *__restrict__ in, int32_t n, int32_t *__restrict__ bsum,
+                              const int32_t *__restrict__ cnt) {
+    if (cnt && gate_closed(cnt)) return;
     __shared__ int s_buf[32];
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE;
     int s = 0;
@@ -928,7 +1017,8 @@ __global__ void k_scan_reduce(const int32_t *__restrict__ in, int32_t n, int32_t
 }
 
 // Single block: exclusive scan of the nb block sums in place.
-__global__ void k_scan_bsums(int32_t *__restrict__ bsum, int32_t nb) {
+__global__ void k_scan_bsums(int32_t *__restrict__ bsum, int32_t nb, const int32_t *__restrict__ cnt) {
+    if (cnt && gate_closed(cnt)) return;
     __shared__ int s_carry;
     if (threadIdx.x == 0) s_carry = 0;
     __syncthreads();
@@ -946,7 +1036,9 @@ __global__ void k_scan_bsums(int32_t *__restrict__ bsum, int32_t nb) {
 
 // in and out may be the same array (each thread reads its own elements
 // before it writes them), so they are not __restrict__.
-__global__ void k_scan_apply(const int32_t *in, int32_t *out, int32_t n, const int32_t *__restrict__ bsum) {
+__global__ void k_scan_apply(const int32_t *in, int32_t *out, int32_t n, const int32_t *__restrict__ bsum,
+                             const int32_t *__restrict__ cnt) {
+    if (cnt && gate_closed(cnt)) return;
     int64_t base = (int64_t)blockIdx.x * SCAN_TILE + (int64_t)threadIdx.x * SCAN_PER;
     int v[SCAN_PER];
     int s = 0;
@@ -964,25 +1056,27 @@ __global__ void k_scan_apply(const int32_t *in, int32_t *out, int32_t n, const i
     }
 }
 
-int launch_scan(const int32_t *in, int32_t *out, int32_t n, int32_t *tmp, cudaStream_t st) {
+int launch_scan(const int32_t *in, int32_t *out, int32_t n, int32_t *tmp, cudaStream_t st, const int32_t *cnt) {
     if (n <= 0) return cudaMemsetAsync(out, 0, sizeof(int32_t), st) == cudaSuccess ? 0 : -1;
     int32_t nb = (int32_t)((n + SCAN_TILE - 1) / SCAN_TILE);
-    k_scan_reduce<<<nb, SCAN_THREADS, 0, st>>>(in, n, tmp);
-    k_scan_bsums<<<1, SCAN_THREADS, 0, st>>>(tmp, nb);
-    k_scan_apply<<<nb, SCAN_THREADS, 0, st>>>(in, out, n, tmp);
+    k_scan_reduce<<<nb, SCAN_THREADS, 0, st>>>(in, n, tmp, cnt);
+    k_scan_bsums<<<1, SCAN_THREADS, 0, st>>>(tmp, nb, cnt);
+    k_scan_apply<<<nb, SCAN_THREADS, 0, st>>>(in, out, n, tmp, cnt);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-__global__ void k_gate(int32_t *__restrict__ cnt, int32_t *__restrict__ sticky) {
+__global__ void k_gate(int32_t *__restrict__ cnt, int32_t *__restrict__ sticky, bool check) {
     unsigned long long sym;
     memcpy(&sym, cnt + CNT_SYM, sizeof sym);
-    const int bits = cnt[CNT_ERR] | (sym ? ERRB_ASYM : 0) | (cnt[CNT_MAXDEG] > EF_MAX_DEGREE ? ERRB_DEGREE : 0);
-    cnt[CNT_GATE] = bits;
+    const int bits = !check ? 0
+                            : cnt[CNT_ERR] | (sym ? ERRB_ASYM : 0) |
+                                  (cnt[CNT_MAXDEG] > EF_MAX_DEGREE ? ERRB_DEGREE : 0);
+    cnt[CNT_GATE] = bits | (cnt[BIN_BIG] == 0 ? GATE_SHORT : 0);
     if (bits && sticky) atomicOr(sticky, bits);
 }
 
-int launch_gate(int32_t *cnt, int32_t *sticky, cudaStream_t st) {
-    k_gate<<<1, 1, 0, st>>>(cnt, sticky);
+int launch_gate(int32_t *cnt, int32_t *sticky, bool check, cudaStream_t st) {
+    k_gate<<<1, 1, 0, st>>>(cnt, sticky, check);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -1003,34 +1097,67 @@ static inline unsigned grid_for(int64_t work, int per_block, int64_t cap) {
 
 // Degrees + wedge bins, per-row checks and neighbour sums.
 int launch_prep_a(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const Scratch &s, const Tune &t,
-                  cudaStream_t st, const int64_t *goff, int32_t G) {
-    k_degrees<<<grid_for(n, DEG_THREADS * DEG_PER, 1 << 30), DEG_THREADS, 0, st>>>(rp, n, m, t.hub_min, s.D, s.bins,
-                                                                                 s.counters);
-    const RowOut ro{s.sig1, s.sig2, s.outdeg, goff, G};
+                  cudaStream_t st, const int64_t *goff, int32_t G, bool short_ok) {
+    if (cudaMemsetAsync(s.counters, 0, NUM_COUNTERS * sizeof(int32_t), st) != cudaSuccess ||
+        (!short_ok && launch_clear_triangles(s, n, st)))
+        return -1;
+    k_degrees<<<grid_for(n, DEG_THREADS * DEG_PER, 1 << 30), DEG_THREADS, 0, st>>>(
+        rp, n, m, t.hub_min, s.D, s.Tacc, s.bins, s.counters);
+    const RowOut ro{s.sig1, s.sig2, s.outdeg, goff, G,
+                    short_ok ? reinterpret_cast<int2 *>(s.info) : nullptr};
     k_row_stats<<<t.grid((int64_t)n, 256), 256, 0, st>>>(rp, ci, n, m, t.row_thread_max, t.hub_min, s.D, s.bins,
                                                          rows_in_bins_allowed(m), ro, s.counters);
     k_row_stats_hub<<<t.num_sms * 4, ROW_CTA, 0, st>>>(rp, ci, n, s.D, s.bins, ro, s.counters);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
+// Zero triangle accumulators (qacc and tcnt, adjacent).
+int launch_clear_triangles(const Scratch &s, int32_t n, cudaStream_t st) {
+    return cudaMemsetAsync(s.qacc, 0, (size_t)((char *)(s.tcnt + n) - (char *)s.qacc), st) == cudaSuccess ? 0 : -1;
+}
+
+// Where the device chooses the path, what the general path clears (the empty
+// tables, the offsets of the degree-bin layout, the triangle accumulators) is
+// cleared behind the gate; elsewhere memsets do it (2 us less on BA 1M).
+__global__ void __launch_bounds__(256) k_clear_lists(int32_t *__restrict__ hash, int64_t slots,
+                                                     int32_t *__restrict__ out_ptr, int32_t n,
+                                                     int64_t *__restrict__ qacc, int64_t *__restrict__ tcnt,
+                                                     const int32_t *__restrict__ cnt) {
+    if (gate_closed(cnt)) return;
+    const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = first; i < slots / 4; i += step) reinterpret_cast<int4 *>(hash)[i] = make_int4(-1, -1, -1, -1);
+    if (first < slots % 4) hash[slots / 4 * 4 + first] = -1;
+    for (int64_t i = first; i <= n; i += step) {
+        if (out_ptr) out_ptr[i] = 0;
+        if (i < n) {
+            qacc[i] = 0;
+            tcnt[i] = 0;
+        }
+    }
+}
+
 // Oriented CSR and omega.
 int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const Scratch &s, const Tune &t,
-                  cudaStream_t st, int32_t *nmin, int32_t *nmax, bool bins, bool tables) {
-    if (tables && cudaMemsetAsync(s.out_hash, 0xff, (size_t)hash_slots(m) * sizeof(int32_t), st) != cudaSuccess)
+                  cudaStream_t st, int32_t *nmin, int32_t *nmax, bool bins, bool gated) {
+    const int32_t *gate = gated ? s.counters : nullptr;
+    // empty tables and, in layout order, zero offsets (degree-0 nodes keep offset 0 and an empty list)
+    if (gated)
+        k_clear_lists<<<t.grid(hash_slots(m) / 4, 256), 256, 0, st>>>(
+            s.out_hash, hash_slots(m), bins ? s.out_ptr : nullptr, n, s.qacc, s.tcnt, s.counters);
+    else if (cudaMemsetAsync(s.out_hash, 0xff, (size_t)hash_slots(m) * sizeof(int32_t), st) != cudaSuccess ||
+             (bins && cudaMemsetAsync(s.out_ptr, 0, (size_t)(n + 1) * sizeof(int32_t), st) != cudaSuccess))
         return -1;
     if (bins) {
-        // out-list offsets in layout order (degree-0 nodes keep offset 0 and an empty list)
-        if (cudaMemsetAsync(s.out_ptr, 0, (size_t)(n + 1) * sizeof(int32_t), st) != cudaSuccess) return -1;
         k_layout_gather<<<t.grid((int64_t)n, 256), 256, 0, st>>>(s.bins, s.counters, n, s.outdeg, s.lay_node,
                                                                  s.lay_ptr);
-        if (launch_scan(s.lay_ptr, s.lay_ptr, n, s.scan_tmp, st)) return -1;
+        if (launch_scan(s.lay_ptr, s.lay_ptr, n, s.scan_tmp, st, gate)) return -1;
         k_layout_scatter<<<t.grid((int64_t)n, 256), 256, 0, st>>>(s.counters, n, s.lay_node, s.lay_ptr, s.out_ptr);
-    } else if (launch_scan(s.outdeg, s.out_ptr, n, s.scan_tmp, st)) {
+    } else if (launch_scan(s.outdeg, s.out_ptr, n, s.scan_tmp, st, gate)) {
         return -1;
     }
     k_node_info<<<t.grid((int64_t)n, 256), 256, 0, st>>>(s.D, s.sig1, s.out_ptr, s.outdeg, n, hash_slots(m),
-                                                         s.info);
-    const Orient o{ci, s.info, s.out_col, s.out_D, s.out_src, s.out_pd, tables ? s.out_hash : nullptr, nmin, nmax, n};
+                                                         s.info, gate);
+    const Orient o{ci, s.info, s.out_col, s.out_D, s.out_src, s.out_pd, s.out_hash, nmin, nmax, n};
     k_orient<4><<<t.grid((int64_t)n, 256), 256, 0, st>>>(rp, n, m, t.row_thread_max, t.hub_min, o, s.D, s.bins,
                                                          rows_in_bins_allowed(m), s.counters, s.out_ptr, s.outdeg,
                                                          s.omega);
@@ -1038,10 +1165,10 @@ int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, co
                                                          rows_in_bins_allowed(m), s.counters, s.out_ptr, s.outdeg,
                                                          s.omega);
     k_orient_hub<<<t.num_sms * 4, ROW_CTA, 0, st>>>(rp, n, o, s.bins, s.out_ptr, s.counters, s.omega);
-    if (tables && bins && t.row_thread_max >= SMALL_MAX)
+    if (bins && t.row_thread_max >= SMALL_MAX)
         k_hash_tail<<<(unsigned)(t.num_sms * 16), 256, 0, st>>>(s.counters, s.lay_ptr, s.out_ptr, n, s.info,
                                                                s.out_col, s.out_src, s.out_hash);
-    else if (tables)
+    else
         k_hash_rows<<<(unsigned)(t.num_sms * 8), 256, 0, st>>>(rp, n, m, t.row_thread_max, s.bins + (size_t)BIN_BIG * n,
                                                                s.counters, s.info, s.out_ptr, s.outdeg, s.out_col,
                                                                s.out_hash);
@@ -1053,7 +1180,7 @@ int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, co
 int launch_big_items(const Scratch &s, int32_t n, cudaStream_t st) {
     k_big_chunks<<<grid_for(n, 256, 1 << 30), 256, 0, st>>>(s.D, s.bins + (size_t)BIN_BIG * n, s.counters, n,
                                                              s.big_chunks);
-    if (launch_scan(s.big_chunks, s.big_chunks, n, s.scan_tmp2, st)) return -1;
+    if (launch_scan(s.big_chunks, s.big_chunks, n, s.scan_tmp2, st, s.counters)) return -1;
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

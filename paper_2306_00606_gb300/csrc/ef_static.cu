@@ -106,8 +106,6 @@ extern "C" int ef_compute_static(const ef_csr *g, int32_t n, int64_t m, int32_t 
 
     cudaStream_t st = (cudaStream_t)stream;
     const int32_t *rp = g->row_ptr, *ci = g->col_idx;
-    if (cudaMemsetAsync(s.Tacc, 0, accumulator_bytes(s), st) != cudaSuccess)
-        return fail(EF_ERR_CUDA, "ef_compute_static: memset failed");
     if (launch_prep_a(rp, ci, n, m, s, t, st))
         return fail(EF_ERR_CUDA, "ef_compute_static: prep launch failed");
     int32_t h_cnt[NUM_COUNTERS];

@@ -1112,10 +1112,15 @@ int ef_sir_run(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const int32_t
     DeviceGuard dg(ctx->device);
     Scratch s;
     int64_t fcap;
+    // pull steps take a CTA per row already from SIR_HUB_MIN entries on
+    const Tune tuned = ctx->tune;
+    ctx->tune.hub_min = std::min(tuned.hub_min, SIR_HUB_MIN);
+    const Tune t = ctx->tune;
     rc = prepare_graph(ctx, g->row_ptr, g->col_idx, n, m, o, s, fcap);
+    ctx->tune = tuned;
     if (rc) return rc;
     cudaStream_t cs = ctx->stream;
-    const Tune &t = ctx->tune;
+    LAUNCH(prepare_sir(), "SIR set-up");
     SirStep sp;
     sp.seed = p.seed;
     sp.beta_thr = (uint64_t)std::floor(p.beta * 4294967296.0);
@@ -1183,7 +1188,7 @@ int ef_sir_run(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const int32_t
         }
         sp.sim_base = p.sim_base + c0;
         for (int32_t step = 0; step < p.max_steps; ++step) {
-            LAUNCH(launch_sir_step(g->row_ptr, g->col_idx, n, step, sp, st, active, t, cs), "SIR step");
+            LAUNCH(launch_sir_step(g->row_ptr, g->col_idx, n, step, sp, st, active, s, t, cs), "SIR step");
             if ((step + 1) % SIR_CHECK == 0 && step + 1 < p.max_steps) {
                 CU(cudaMemcpyAsync(h_active, active + (step & 1), sizeof(int64_t), cudaMemcpyDeviceToHost, cs));
                 CU(cudaStreamSynchronize(cs));

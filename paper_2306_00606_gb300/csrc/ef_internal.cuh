@@ -541,6 +541,7 @@ int launch_bin_marked(const int32_t *mark, const Scratch &s, int32_t n, const Tu
 // SIR simulation (ef_sir.cu): a batch of at most SIR_BATCH simulations,
 // node-major bit words (WB = ceil(B / 32) per node), frontier lists of nodes.
 constexpr int SIR_BATCH = 1024;
+constexpr int SIR_HUB_MIN = 129;   // rows of at least this take a CTA in a pull step
 struct SirState {
     int32_t B, WB;        // simulations of the batch, words per node
     uint32_t *susc;       // n*WB   susceptible (bit s % 32 of word s / 32)
@@ -566,7 +567,8 @@ struct SirStep {
 int launch_sir_init(const int32_t *index_cases, int32_t n, const uint8_t *immune, int32_t num_sets,
                     const int32_t *imm_set, const SirState &st, const Tune &t, cudaStream_t s);
 int launch_sir_step(const int32_t *rp, const int32_t *ci, int32_t n, int32_t step, const SirStep &p,
-                    const SirState &st, int64_t *active, const Tune &t, cudaStream_t s);
+                    const SirState &st, int64_t *active, const Scratch &sc, const Tune &t, cudaStream_t s);
+int prepare_sir();
 int launch_sir_close(int32_t steps, const SirState &st, uint8_t *truncated, const Tune &t, cudaStream_t s);
 int launch_sir_tree(int32_t n, int32_t depth, int32_t min_size, const SirState &st, int64_t *exact,
                     int64_t *infected, const Tune &t, cudaStream_t s);

@@ -13,8 +13,8 @@
 //            does nothing on invalid input, and the host reads the bits once
 //            the call's work is done)
 //   part B   f table (f(d) = d ln d and the triangle corrections, d < 3 maxdeg + 1);
-//            orientation (oriented CSR + omega); wedge pass (small, then mid +
-//            hub middle nodes); hash tables and pair tests; finalize (per node)
+//            orientation (oriented CSR + omega, hash tables); pair tests; wedge
+//            pass (small, then mid + hub middle nodes); finalize (per node)
 //            Where no row exceeds 32 entries: f table, the fused short-row
 //            kernel (ef_short.cu), its finalize.  The host chooses after the
 //            readback; without one both sets are launched and the gate word
@@ -85,6 +85,7 @@ struct ef_ctx {
     void *acts = nullptr;            // training activations
     size_t acts_bytes = 0;
     double *dtmp = nullptr;          // small device scratch (feature sums)
+    bool long_lists = true;          // an owner of the current graph has more than TRI_LONG out-neighbours
     int path = 0;                    // part B kernels of the last exact call (PathMode)
     bool bins = true;                // out-lists of the current graph in degree-bin order (bin_layout)
     void *sir = nullptr;             // SIR simulation state
@@ -116,10 +117,10 @@ enum PathMode { PATH_GENERAL, PATH_SHORT, PATH_DEVICE };
 // rows, hash tables of the longer rows; the short rows' tables are filled by
 // the row kernel itself), small wedges 4, big wedges (class kernels 2; direct
 // mode: item counts, a scan of 3, direct kernel, reduction), pair tests 1,
-// finalize 1; both sets, the clearing kernel and the gate where the
+// with long out-lists 3, finalize 1; both sets, the clearing kernel and the gate where the
 // device decides.
-int64_t kernels_per_call(PathMode path, bool bins, int wedge_mode) {
-    const int64_t general = (bins ? 5 : 3) + 5 + 4 + (wedge_mode == 1 ? 6 : 2) + 1 + 1;
+int64_t kernels_per_call(PathMode path, bool bins, int wedge_mode, bool long_lists) {
+    const int64_t general = (bins ? 5 : 3) + 4 + 4 + (wedge_mode == 1 ? 6 : 2) + (long_lists ? 3 : 1) + 1;
     return 3 + 1 + (path != PATH_GENERAL ? 2 : 0) + (path != PATH_SHORT ? general : 0) + (path == PATH_DEVICE ? 2 : 0);
 }
 
@@ -250,8 +251,8 @@ int part_a(ef_ctx *ctx, const Job &j, const ef::Scratch &s, cudaStream_t st, boo
 }
 
 // Part B; with prof, events 1..4, 6, 7 bracket f table + orientation (with
-// the hash tables), small wedges (on the short-row path the fused kernel),
-// big wedges, pair tests and finalize.
+// the hash tables), pair tests, small wedges (on the short-row path the fused
+// kernel), big wedges and finalize.
 int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, PathMode path, bool prof,
            cudaStream_t st) {
     using namespace ef;
@@ -261,22 +262,25 @@ int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, PathMo
     LAUNCH(launch_ftab(s.ftab, s.tq, s.counters, fcap, st), "f table");
     if (path != PATH_GENERAL) {
         const bool chosen = path == PATH_SHORT;
-        if (prof) CU(cudaEventRecord(ctx->ev[2], st));
+        if (prof)
+            for (int e : {2, 3}) CU(cudaEventRecord(ctx->ev[e], st));
         LAUNCH(launch_short(j.ci, s, j.o.precision, j.n, t, chosen, st), "short rows");
         if (prof && chosen)
-            for (int e : {3, 4, 6}) CU(cudaEventRecord(ctx->ev[e], st));
+            for (int e : {4, 6}) CU(cudaEventRecord(ctx->ev[e], st));
         LAUNCH(launch_finalize_short(s, j.o.precision, j.n, j.out, t, chosen, st), "finalize");
         if (chosen) return EF_OK;
     }
     const bool gated = path == PATH_DEVICE;
     if (!gated) LAUNCH(launch_clear_triangles(s, j.n, st), "clear");
-    LAUNCH(launch_orient(j.rp, j.ci, j.n, j.m, s, t, st, nullptr, nullptr, ctx->bins, gated), "orientation");
+    LAUNCH(launch_orient(j.rp, j.ci, j.n, j.m, s, t, st, nullptr, nullptr, ctx->bins, gated, true),
+           "orientation");
     if (prof) CU(cudaEventRecord(ctx->ev[2], st));
-    LAUNCH(launch_wedge_small(j.rp, j.ci, s, j.o.precision, j.n, t, st), "small wedge");
+    // before the wedges, whose hub classes lie over the oriented lists
+    LAUNCH(launch_tri_pairs(s, j.n, j.m, t, st, nullptr, gated || ctx->long_lists), "triangle");
     if (prof) CU(cudaEventRecord(ctx->ev[3], st));
-    LAUNCH(launch_wedge_big(j.rp, j.ci, s, j.o.precision, j.o.wedge_mode, j.n, j.m, t, st), "big wedge");
+    LAUNCH(launch_wedge_small(j.rp, j.ci, s, j.o.precision, j.n, t, st), "small wedge");
     if (prof) CU(cudaEventRecord(ctx->ev[4], st));
-    LAUNCH(launch_tri_pairs(s, j.n, j.m, t, st), "triangle");
+    LAUNCH(launch_wedge_big(j.rp, j.ci, s, j.o.precision, j.o.wedge_mode, j.n, j.m, t, st), "big wedge");
     if (prof) CU(cudaEventRecord(ctx->ev[6], st));
     LAUNCH(launch_finalize(s, j.o.precision, j.n, j.out, t, st), "finalize");
     return EF_OK;
@@ -340,6 +344,7 @@ int compute_device(ef_ctx *ctx, const Job &j) {
 
     // f table size: from the validated max degree, else the largest possible
     int64_t fcap;
+    ctx->long_lists = true;
     if (a_inline) {
         int64_t bound = (int64_t)j.n - 1 < j.m ? (int64_t)j.n - 1 : j.m;
         if (bound > EF_MAX_DEGREE) bound = EF_MAX_DEGREE;
@@ -354,6 +359,7 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         if (const int bits = prep_error_bits(ctx->h_counters)) return graph_error(ctx, bits);
         if (const int lim = degree_limit(ctx, ctx->h_counters)) return lim;
         path = ctx->h_counters[BIN_BIG] == 0 ? PATH_SHORT : PATH_GENERAL;
+        ctx->long_lists = ctx->h_counters[CNT_MAXOUT] > TRI_LONG;
         fcap = 3 * (int64_t)ctx->h_counters[CNT_MAXDEG] + 1;
         ctx->bins = bin_layout(ctx->tune, ctx->h_counters, j.n, j.goff_dev != nullptr);
     }
@@ -383,7 +389,7 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         key.precision = o.precision;
         key.wedge_mode = o.wedge_mode;
         key.trust = o.trust_input | (dev_check ? 2 : 0) | (dev_check && o.async ? 4 : 0);
-        key.bins = (int32_t)ctx->bins | (int32_t)path << 1;
+        key.bins = (int32_t)ctx->bins | (int32_t)path << 1 | (int32_t)ctx->long_lists << 3;
         key.tune = ctx->tune;
         rc = run_graph(ctx, key, [&](cudaStream_t cs) {
             if (a_inline) {
@@ -419,8 +425,8 @@ int check_args(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const ef_opti
     return check_opts(ctx, o);
 }
 
-// Events: 0 start, 1 part B start (after the validation readback), 2..6
-// after orientation, small wedges, big wedges, hash tables, pair tests, 7 end.
+// Events: 0 start, 1 part B start (after the validation readback), 2, 3, 4, 6
+// after orientation, pair tests, small wedges, big wedges, 7 end.
 void accumulate_stats(ef_ctx *ctx, int wedge_mode) {
     auto el = [&](int a, int b) {
         float t = 0.f;
@@ -430,12 +436,12 @@ void accumulate_stats(ef_ctx *ctx, int wedge_mode) {
     st.calls += 1;
     st.prep_ms += el(0, 1);
     st.orient_ms += el(1, 2);
-    st.wedge_small_ms += el(2, 3);
-    st.wedge_big_ms += el(3, 4);
-    st.tri_pairs_ms += el(4, 6);
+    st.tri_pairs_ms += el(2, 3);
+    st.wedge_small_ms += el(3, 4);
+    st.wedge_big_ms += el(4, 6);
     st.finalize_ms += el(6, 7);
     st.total_ms += el(0, 7);
-    st.kernels += kernels_per_call((PathMode)ctx->path, ctx->bins, wedge_mode);
+    st.kernels += kernels_per_call((PathMode)ctx->path, ctx->bins, wedge_mode, ctx->long_lists);
 }
 
 // Host I/O and synchronisation around compute_device.
@@ -722,11 +728,22 @@ size_t carve_scratch(char *base, int32_t n, int64_t m, Scratch &s) {
     s.lay_node = (int32_t *)take(4 * N);
     s.lay_ptr = (int32_t *)take(4 * (N + 1));
     s.info = (int4 *)take(16 * N);
+    // the oriented lists, dead after the pair tests, and over them the hub
+    // kernel's arrays, written by the wedge pass that follows
+    const size_t oriented = off;
     s.out_col = (int32_t *)take(4 * (M + 8));
     s.out_D = (int32_t *)take(4 * (M + 1));
     s.out_pd = (int2 *)take(8 * (M + 1));
-    s.out_hash = (int32_t *)take(4 * (M + 8));
+    s.out_hash = (int32_t *)take(4 * (size_t)hash_slots(m));
     s.out_src = (int32_t *)take(4 * (M + 1));
+    const size_t oriented_end = off;
+    off = oriented;
+    s.hub_cls = take(8 * (M + N + 2));
+    s.hub_q = take(8 * (M + N + 2));
+    s.hub_cidx = (int32_t *)take(4 * (M + 1));
+    off = std::max(off, oriented_end);
+    s.tri_items = (int2 *)take(8 * (M / 32 + 1));
+    s.tri_rec = (int4 *)take(16 * (M / 2 + 1));
     s.Ccenter = take(8 * N);
     // accumulators (cleared by the degree and row passes)
     s.Tacc = (double *)take(8 * N);
@@ -738,9 +755,6 @@ size_t carve_scratch(char *base, int32_t n, int64_t m, Scratch &s) {
     s.big_partial = (double *)take(8 * (M / BIG_ROWS + N + 2));
     s.scan_tmp = (int32_t *)take(4 * (N / 4096 + 4));
     s.scan_tmp2 = (int32_t *)take(4 * (N / 4096 + 4));
-    s.hub_cls = take(8 * (M + N + 2));
-    s.hub_q = take(8 * (M + N + 2));
-    s.hub_cidx = (int32_t *)take(4 * (M + 1));
     s.ftab = nullptr;
     return off;
 }

@@ -73,6 +73,7 @@ constexpr int HUB_SMEM_K = 4096;       // classes held in shared memory by the C
 constexpr int BIG_ROWS = 256;          // rows per work item of the direct big-node kernel
 constexpr int BIG_TILE = 4096;         // neighbour degrees staged per tile by the direct kernel
 constexpr int ROW_CTA = 512;           // threads of the per-hub-row kernels
+constexpr int TRI_LONG = 32;           // owners of more out-neighbours take a warp per 32 of them in the pair tests
 constexpr int SHORT_MAX = 5;           // out-lists longer than this get a hash table for the triangle pass
 
 // Triangle corrections are integers in units of 2^-F (the pass adds only
@@ -117,7 +118,7 @@ struct Scratch {
     int32_t *out_col;    // m+8    oriented neighbour ids (ascending id within a row)
     int32_t *out_D;      // m+1    their degrees
     int2    *out_pd;     // m+1    probe descriptors of their own out-lists (probe_desc)
-    int32_t *out_hash;   // m+8    hash tables of the out-lists longer than SHORT_MAX
+    int32_t *out_hash;   // 1.5m+16  hash tables of the out-lists longer than SHORT_MAX
     int32_t *out_src;    // m+1    owner of each oriented edge
     double  *Tacc;       // n      open-degree credits received as an end (FP64 reductions)
     void    *Ccenter;    // n      middle-node credit (AccT<F64>, 8 bytes reserved per node)
@@ -131,8 +132,10 @@ struct Scratch {
     int32_t *scan_tmp;   // scan block sums (orientation)
     int32_t *scan_tmp2;  // scan block sums (direct kernel's items)
     float2  *ftab;       // 3*maxdeg+1 (capacity): f(d) = d ln d as an FP32 pair hi + lo (F2Sum)
-    void    *hub_cls;    // m+n+2  class (degree, count) pairs of hubs with > HUB_SMEM_K classes
+    void    *hub_cls;    // m+n+2  class (degree, count) pairs of hubs with many classes (over the out_ arrays)
     void    *hub_q;      // m+n+2  their per-class credits
+    int2    *tri_items;  // m/32+1 {owner, block of 32 candidates} of the long owners
+    int4    *tri_rec;    // m/2+1  {id, degree, probe descriptor} of the long owners' out-lists by rank
     int32_t *hub_cidx;   // m+1    class index of each neighbour of a hub (at the hub's row positions)
 };
 
@@ -143,6 +146,9 @@ enum : int {
     CNT_MIDITEM = 35,
     CNT_HUB = 36,
     CNT_TRIFRAC = 37,
+    CNT_TRILONG = 38, // items of the long owners (pair tests), and the next one to take
+    CNT_TRINEXT = 39,
+    CNT_MAXOUT = 42,  // largest out-degree
     CNT_RANGE = 40,   // 40, 41: a shard's node range [lo, hi)
     CNT_SYM = 44,     // 44, 45: the symmetry sum (uint64, 8-byte aligned)
     CNT_BIGLO = 46,   // n - 1 - (smallest id of a node of degree > SMALL_MAX), if any
@@ -251,22 +257,36 @@ __device__ __forceinline__ T group_sum(T v) {
 
 // lower_bound over a sorted int32 array (generic address space)
 // ----------------------------------------------- out-list membership tables
-// Table of the out-list [ls, le) of one node: slots [base, base + 4 nb) of
-// out_hash, base = 2 ls rounded up to a multiple of 4 and 4 nb = 2 (le - ls)
-// rounded down to one, so the tables of consecutive out-lists never overlap
-// and every bucket is 16-byte aligned.  Only lists longer than SHORT_MAX have
-// one, and only when it lies inside the array (always, for a symmetric CSR:
-// the out-lists then hold m/2 entries in all).
-__host__ __device__ __forceinline__ int64_t hash_slots(int64_t m) { return m + 8; }   // slots of out_hash
+// Table of the out-list [ls, le) of one node: buckets of 8 slots (one 32-byte
+// sector) from slot base of out_hash, base = 3 ls rounded up to a multiple of
+// 8 and 3/8 as many buckets as entries, so the tables of consecutive
+// out-lists never overlap.  A bucket is filled from its first slot on, so its
+// last slot says whether it is full; keys that find it full go to the next
+// bucket.  At 2.7 entries per bucket on average a probe in 150 meets a full
+// bucket without its key; the others take one sector.  (Buckets of 4 slots at
+// a mean of 2, home bucket and the next one read together: 1.5 sectors a
+// test, and another round for a few percent of the tests, that is for most
+// warps.  A mean of 2 in 8 slots: 4.9 against 4.8 ms of pair tests and 2.06
+// against 1.99 of orientation on the 87M-entry graph, the larger tables miss
+// L2 more often.)
+// Only lists longer than SHORT_MAX have a table, and only when it lies inside
+// the array (always, for a symmetric CSR: the out-lists then hold m/2 entries
+// in all).
+constexpr int BUCKET = 8;
+__host__ __device__ __forceinline__ int64_t hash_slots(int64_t m) { return m + (m + 1) / 2 + 16; }   // slots of out_hash
+
+__host__ __device__ __forceinline__ int64_t table_base(int ls) {
+    return ((int64_t)3 * ls + BUCKET - 1) & ~(int64_t)(BUCKET - 1);
+}
 
 __device__ __forceinline__ bool out_table(int ls, int le, int64_t hash_cap, int64_t &base, int &nb) {
     const int p = le - ls;
-    base = ((int64_t)2 * ls + 3) & ~(int64_t)3;
-    nb = (2 * p) >> 2;
-    return p > SHORT_MAX && base + 4 * (int64_t)nb <= hash_cap;
+    base = table_base(ls);
+    nb = (3 * p) >> 3;
+    return p > SHORT_MAX && base + BUCKET * (int64_t)nb <= hash_cap;
 }
 
-// Home bucket of key in a table of nb buckets of 4 slots.
+// Home bucket of key in a table of nb buckets.
 __device__ __forceinline__ int bucket_of(int key, int nb) {
     const uint32_t h = (uint32_t)key * 0x9E3779B1u;
     return (int)(((uint64_t)h * (uint32_t)nb) >> 32);
@@ -275,8 +295,8 @@ __device__ __forceinline__ int bucket_of(int key, int nb) {
 // Insert key into a table (cleared to -1 beforehand) shared by several
 // threads: linear probing over slots from the key's home bucket, by atomics.
 __device__ __forceinline__ void table_insert_shared(int32_t *out_hash, int64_t base, int nb, int key) {
-    const int cap = 4 * nb;
-    int sl = 4 * bucket_of(key, nb);
+    const int cap = BUCKET * nb;
+    int sl = BUCKET * bucket_of(key, nb);
     for (int tries = 0; tries < cap; ++tries) {
         const int prev = atomicCAS(out_hash + base + sl, -1, key);
         if (prev == -1 || prev == key) break;
@@ -295,8 +315,8 @@ __device__ __forceinline__ unsigned range_bits(int e0, int ls, int le) {
 //   kind 0, a list of at most SHORT_MAX entries: x = its first quad of
 //     out_col, y = which entries of that quad (bits 0-3) and the next (4-7)
 //     belong to it;
-//   kind 1, a hashed list: x = its first bucket (quad) of out_hash, y = the
-//     bucket count;
+//   kind 1, a hashed list: x = the first quad of its table in out_hash, y =
+//     the bucket count;
 //   kind 2, a longer list without a table (malformed input only): x = ls,
 //     y = le.
 // The kind sits in bits 30-31 of y (counts and offsets stay below 2^30).
@@ -479,9 +499,11 @@ int launch_prep_a(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, co
 // Also the hash tables of the out-lists longer than SHORT_MAX (cleared here,
 // filled as the lists are written).  gated: the call's path is chosen on the
 // device; the triangle accumulators are then cleared here, behind the gate.
+// big_rows: no graph without rows above SMALL_MAX comes here (the short-row
+// path took it).
 int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const Scratch &s, const Tune &t,
                   cudaStream_t st, int32_t *nmin = nullptr, int32_t *nmax = nullptr, bool bins = true,
-                  bool gated = false);
+                  bool gated = false, bool big_rows = false);
 int launch_clear_triangles(const Scratch &s, int32_t n, cudaStream_t st);
 int launch_big_items(const Scratch &s, int32_t n, cudaStream_t st);
 int prepare_kernels();
@@ -512,8 +534,9 @@ int launch_wedge_small(const int32_t *rp, const int32_t *ci, const Scratch &s, i
                        const Tune &t, cudaStream_t st);
 int launch_wedge_big(const int32_t *rp, const int32_t *ci, const Scratch &s, int precision, int wedge_mode,
                      int32_t n, int64_t m, const Tune &t, cudaStream_t st);
+// long_lists: some owner may have more than TRI_LONG out-neighbours.
 int launch_tri_pairs(const Scratch &s, int32_t n, int64_t m, const Tune &t, cudaStream_t st,
-                     const int32_t *owner_range = nullptr);
+                     const int32_t *owner_range = nullptr, bool long_lists = true);
 int launch_finalize(const Scratch &s, int precision, int32_t n, const ef_outputs &out, const Tune &t,
                     cudaStream_t st);
 // learned path (ef_mlp.cu, ef_rank.cu)

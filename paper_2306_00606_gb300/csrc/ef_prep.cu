@@ -312,23 +312,28 @@ __device__ __forceinline__ int cross_bits(const RowOut &ro, const int32_t *__res
     return ci[a] < ro.goff[lo] || ci[b - 1] >= ro.goff[lo + 1] ? ERRB_CROSS : 0;
 }
 
-__device__ __forceinline__ void add_sym(int32_t *cnt, uint64_t sym) {
+// A warp's share of the symmetry sum and the largest out-degree of its rows.
+__device__ __forceinline__ void add_rows(int32_t *cnt, uint64_t sym, int od) {
     sym = warp_sum(sym);
-    if ((threadIdx.x & 31) == 0 && sym)
-        atomicAdd(reinterpret_cast<unsigned long long *>(cnt + CNT_SYM), (unsigned long long)sym);
+    od = __reduce_max_sync(FULL, od);
+    if ((threadIdx.x & 31) == 0) {
+        if (sym) atomicAdd(reinterpret_cast<unsigned long long *>(cnt + CNT_SYM), (unsigned long long)sym);
+        if (od > *(volatile int32_t *)(cnt + CNT_MAXOUT)) atomicMax(cnt + CNT_MAXOUT, od);
+    }
 }
 
 // A row of the row pass walked by a whole warp.
 __device__ __forceinline__ void row_stats_warp(const int32_t *__restrict__ ci, const int32_t *__restrict__ D,
                                                int32_t n, int u, int ua, int ub, int lane, const RowOut &ro,
-                                               int32_t *__restrict__ cnt, uint64_t &sym) {
+                                               int32_t *__restrict__ cnt, uint64_t &sym, int &most) {
     RowStats r;
     const NodeMix mu = node_mix(u);
     for (int e = ua + lane; e < ub; e += 32) r.entry(ci, D, n, u, ub - ua, ua, e, mu);
     const int64_t s1 = warp_sum(r.s1), s2 = warp_sum(r.s2);
-    const int od = warp_sum(r.od);
+    const int od = __reduce_add_sync(FULL, r.od);
     const int err = __reduce_or_sync(FULL, r.err);
     sym += r.sym;
+    most = max(most, od);
     if (lane == 0) {
         ro.sig1[u] = s1;
         ro.sig2[u] = s2;
@@ -414,7 +419,7 @@ __device__ __forceinline__ void rows_short(const int32_t *__restrict__ rp, const
         }
     }
     if (err) atomicOr(cnt + CNT_ERR, err);
-    add_sym(cnt, sym);
+    add_rows(cnt, sym, 0);
 }
 
 // Rows of degree < hub_min (RowOrder): a thread per row of degree <= tmax,
@@ -437,6 +442,7 @@ __global__ void __launch_bounds__(256, 6) k_row_stats(const int32_t *__restrict_
     const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
     uint64_t sym = 0;
+    int most = 0;   // largest out-degree
     for (int64_t base = warp * 32; base < total; base += nwarps * 32) {
         const int i = (int)(base + lane);
         const bool in = i < total;
@@ -453,6 +459,7 @@ __global__ void __launch_bounds__(256, 6) k_row_stats(const int32_t *__restrict_
             ro.sig1[v] = r.s1;
             ro.sig2[v] = r.s2;
             ro.outdeg[v] = r.od;
+            most = max(most, r.od);
             sym += r.sym;
             if (r.err) atomicOr(cnt + CNT_ERR, r.err);
         }
@@ -462,7 +469,7 @@ __global__ void __launch_bounds__(256, 6) k_row_stats(const int32_t *__restrict_
             wide &= wide - 1;
             const int u = __shfl_sync(FULL, v, j);
             const int ua = __shfl_sync(FULL, a, j), ub = __shfl_sync(FULL, b, j);
-            row_stats_warp(ci, D, n, u, ua, ub, lane, ro, cnt, sym);
+            row_stats_warp(ci, D, n, u, ua, ub, lane, ro, cnt, sym, most);
         }
     }
     if (ord.bins) {
@@ -470,7 +477,7 @@ __global__ void __launch_bounds__(256, 6) k_row_stats(const int32_t *__restrict_
         for (int64_t it = warp; it < nmid; it += nwarps) {
             const int u = bins[(size_t)BIN_MID * n + it];
             const int ua = rp[u], ub = rp[u + 1];
-            if (ua >= 0 && ua <= ub && (int64_t)ub <= m) row_stats_warp(ci, D, n, u, ua, ub, lane, ro, cnt, sym);
+            if (ua >= 0 && ua <= ub && (int64_t)ub <= m) row_stats_warp(ci, D, n, u, ua, ub, lane, ro, cnt, sym, most);
         }
         // rows of degree 0 (or with a malformed range) are in no work list
         for (int64_t v = warp * 32 + lane; v < n; v += nwarps * 32) {
@@ -481,7 +488,7 @@ __global__ void __launch_bounds__(256, 6) k_row_stats(const int32_t *__restrict_
             }
         }
     }
-    add_sym(cnt, sym);
+    add_rows(cnt, sym, most);
 }
 
 __global__ void __launch_bounds__(ROW_CTA) k_row_stats_hub(const int32_t *__restrict__ rp,
@@ -491,7 +498,9 @@ __global__ void __launch_bounds__(ROW_CTA) k_row_stats_hub(const int32_t *__rest
                                                            int32_t *__restrict__ cnt) {
     __shared__ int64_t s_buf[32];
     const int total = hub_total(cnt);
+    if ((int)blockIdx.x >= total) return;
     uint64_t sym = 0;
+    int most = 0;
     for (int it = blockIdx.x; it < total; it += gridDim.x) {
         const int u = hub_row(bins, n, cnt, it);
         const int a = rp[u], b = rp[u + 1];
@@ -508,10 +517,11 @@ __global__ void __launch_bounds__(ROW_CTA) k_row_stats_hub(const int32_t *__rest
             ro.sig1[u] = s1;
             ro.sig2[u] = s2;
             ro.outdeg[u] = (int32_t)od;
+            most = max(most, (int)od);
             if (const int e2 = cross_bits(ro, ci, u, a, b)) atomicOr(cnt + CNT_ERR, e2);
         }
     }
-    add_sym(cnt, sym);
+    add_rows(cnt, sym, most);
 }
 
 // ------------------------------------------------------------- orientation
@@ -519,13 +529,13 @@ __global__ void __launch_bounds__(ROW_CTA) k_row_stats_hub(const int32_t *__rest
 // CSR in ascending id order, with D_x, the probe descriptor of x's own
 // out-list and the owner u; and gathers omega_u = sum over N(u) of
 // sigma1(x), the last per-node sum the closed form of S needs.  A row walked
-// by one thread (at most SMALL_MAX entries, so a table of at most 64 slots)
-// also inserts its keys into its hash table, placed with an occupancy mask in
+// by one thread (at most SMALL_MAX entries, so a table of at most 16 buckets)
+// also inserts its keys into its hash table, placed with the buckets' counts in
 // a register, without atomics; the longer rows' tables are filled afterwards
 // by k_hash_rows.  (Atomic inserts inside the warp and block paths made the
 // orientation wait one L2 round trip per 32-entry chunk: 0.3 ms more on the
 // 4M-node power-law graph.)
-static_assert(SMALL_MAX <= 32, "a one-thread row's table fits a 64-bit occupancy mask");
+static_assert(SMALL_MAX / 2 <= 16, "a one-thread row's table has at most 16 buckets");
 struct OrientStage;
 struct Orient {
     const int32_t *ci;
@@ -595,8 +605,7 @@ __device__ __forceinline__ int64_t Orient::row(int v, int Dv, int a, int b, int 
         int64_t hb = 0;
         int nb = 0;
         const bool hashed = table(v, hb, nb);
-        const uint64_t full = nb >= 16 ? ~0ull : (1ull << (4 * nb)) - 1ull;
-        uint64_t occ = 0;
+        uint64_t used = 0;   // keys per bucket, 4 bits each
         for (int e0 = a; e0 < b; e0 += CHUNK) {
             int x[CHUNK];
             int4 nf[CHUNK];
@@ -614,13 +623,13 @@ __device__ __forceinline__ int64_t Orient::row(int v, int Dv, int a, int b, int 
                         if (sg) sg->put(k++, v, x[q], nf[q]);
                         else put(k++, v, x[q], nf[q]);
                         if (hashed) {
-                            // first free slot from the home bucket, cyclically
-                            const uint64_t f = ~occ & full;
-                            const uint64_t hi = f & (~0ull << (4 * bucket_of(x[q], nb)));
-                            const int pos = __ffsll((long long)(hi ? hi : f)) - 1;
+                            // the home bucket or the next one, cyclically, with a free slot
+                            int bk = bucket_of(x[q], nb);
+                            while ((used >> (4 * bk) & 15) == BUCKET) bk = bk + 1 == nb ? 0 : bk + 1;
+                            const int pos = BUCKET * bk + (int)(used >> (4 * bk) & 15);
+                            used += 1ull << (4 * bk);
                             if (sg) sg->tab[hb + pos - sg->tbase] = x[q];
                             else out_hash[hb + pos] = x[q];
-                            occ |= 1ull << pos;
                         }
                     }
                 }
@@ -636,14 +645,38 @@ __device__ __forceinline__ int64_t Orient::row(int v, int Dv, int a, int b, int 
 
 // info[v] = {D_v, sigma1(v), probe descriptor of v's out-list}: what the
 // orientation needs of a neighbour, in one 16-byte gather (sigma1 <= m < 2^31).
-__global__ void k_node_info(const int32_t *__restrict__ D, const int64_t *__restrict__ sig1,
-                            const int32_t *__restrict__ out_ptr, const int32_t *__restrict__ outdeg, int32_t n,
-                            int64_t hash_cap, int4 *__restrict__ info, const int32_t *__restrict__ cnt) {
-    if (cnt && gate_closed(cnt)) return;
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        const int ls = out_ptr[v];
-        const int2 pd = probe_desc(ls, ls + outdeg[v], hash_cap);
-        info[v] = make_int4(D[v], (int)sig1[v], pd.x, pd.y);
+// Also the pair tests' items of the long owners (more than TRI_LONG
+// out-neighbours): one per 32 of them, positions from one atomic per block
+// and pass.
+__global__ void __launch_bounds__(256) k_node_info(const int32_t *__restrict__ D, const int64_t *__restrict__ sig1,
+                                                   const int32_t *__restrict__ out_ptr,
+                                                   const int32_t *__restrict__ outdeg, int32_t n, int64_t m,
+                                                   int4 *__restrict__ info, int2 *__restrict__ items,
+                                                   int32_t *__restrict__ cnt, bool gated) {
+    if (gated && gate_closed(cnt)) return;
+    __shared__ int s_items, s_first;
+    if (threadIdx.x == 0) s_items = 0;
+    __syncthreads();
+    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t v = base + threadIdx.x;
+        int blocks = 0;
+        if (v < n) {
+            const int ls = out_ptr[v], p = outdeg[v];
+            const int2 pd = probe_desc(ls, ls + p, hash_slots(m));
+            info[v] = make_int4(D[v], (int)sig1[v], pd.x, pd.y);
+            // (the second test holds for every symmetric CSR: room for the sorted records)
+            if (p > TRI_LONG && 2 * (int64_t)(ls + p) <= m) blocks = (p + 31) / 32;
+        }
+        if (!__syncthreads_or(blocks)) continue;
+        int at = 0;
+        if (blocks) at = atomicAdd(&s_items, blocks);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s_first = atomicAdd(cnt + CNT_TRILONG, s_items);
+            s_items = 0;
+        }
+        __syncthreads();
+        for (int k = 0; k < blocks; ++k) items[s_first + at + k] = make_int2((int)v, k);
     }
 }
 
@@ -744,7 +777,7 @@ __device__ __forceinline__ void orient_row_warp(const Orient &o, int u, int ua, 
 // match the degree pass's counts returns at once.  (WS batch orientation
 // 4.7 -> 4.3 ms with 8; the power-law graph 0.90 -> 1.02 ms with 8.)
 // Entries of one warp step that the staging area of k_orient<CHUNK> holds
-// (20 bytes each, plus two table slots).  Only the eight-record form (graphs
+// (20 bytes each, plus four table slots).  Only the eight-record form (graphs
 // without rows above degree 32) stages: measured on the 4096-graph WS batch,
 // orientation 4.32 -> 2.96 ms; the four-record form (a staging area of 128
 // entries, 5 blocks per SM) was slower on the power-law graph (0.89 -> 0.96
@@ -752,7 +785,7 @@ __device__ __forceinline__ void orient_row_warp(const Orient &o, int u, int ua, 
 // from the degree bins and the warp's rows rarely fit, so it writes directly.
 template <int CHUNK>
 struct OrientCap {
-    static constexpr int value = CHUNK == 8 ? 192 : 0;
+    static constexpr int value = CHUNK == 8 ? 128 : 0;
 };
 
 template <int CHUNK>
@@ -763,7 +796,7 @@ __global__ void __launch_bounds__(256, CHUNK == 8 ? 3 : 5) k_orient(
     if (gate_closed(cnt)) return;
     if ((cnt[BIN_BIG] == 0) != (CHUNK == 8)) return;
     constexpr int CAP = OrientCap<CHUNK>::value;
-    constexpr int SCAP = CAP > 0 ? CAP : 1, TCAP = CAP > 0 ? 2 * CAP + 8 : 1;
+    constexpr int SCAP = CAP > 0 ? CAP : 1, TCAP = CAP > 0 ? 3 * CAP + 2 * BUCKET : 1;
     __shared__ RowOrder s_ord;
     __shared__ int32_t s_col[8][SCAP], s_D[8][SCAP], s_src[8][SCAP], s_tab[8][TCAP];
     __shared__ int2 s_pd[8][SCAP];
@@ -795,8 +828,8 @@ __global__ void __launch_bounds__(256, CHUNK == 8 ? 3 : 5) k_orient(
         }
         const bool stage = CAP > 0 && sum > 0 && sum <= CAP && kend - kmin == sum;
         if (stage) {
-            const int64_t tb0 = ((int64_t)2 * kmin + 3) & ~(int64_t)3;
-            const int64_t tb1 = ((int64_t)2 * kend + 3) & ~(int64_t)3;
+            const int64_t tb0 = table_base(kmin);
+            const int64_t tb1 = table_base(kend);
             const int tlen = (int)(tb1 - tb0);
             for (int t = lane; t < tlen; t += 32) s_tab[w][t] = -1;
             __syncwarp();
@@ -1138,7 +1171,7 @@ __global__ void __launch_bounds__(256) k_clear_lists(int32_t *__restrict__ hash,
 
 // Oriented CSR and omega.
 int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const Scratch &s, const Tune &t,
-                  cudaStream_t st, int32_t *nmin, int32_t *nmax, bool bins, bool gated) {
+                  cudaStream_t st, int32_t *nmin, int32_t *nmax, bool bins, bool gated, bool big_rows) {
     const int32_t *gate = gated ? s.counters : nullptr;
     // empty tables and, in layout order, zero offsets (degree-0 nodes keep offset 0 and an empty list)
     if (gated)
@@ -1155,15 +1188,16 @@ int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, co
     } else if (launch_scan(s.outdeg, s.out_ptr, n, s.scan_tmp, st, gate)) {
         return -1;
     }
-    k_node_info<<<t.grid((int64_t)n, 256), 256, 0, st>>>(s.D, s.sig1, s.out_ptr, s.outdeg, n, hash_slots(m),
-                                                         s.info, gate);
+    k_node_info<<<t.grid((int64_t)n, 256), 256, 0, st>>>(s.D, s.sig1, s.out_ptr, s.outdeg, n, m,
+                                                         s.info, s.tri_items, s.counters, gated);
     const Orient o{ci, s.info, s.out_col, s.out_D, s.out_src, s.out_pd, s.out_hash, nmin, nmax, n};
     k_orient<4><<<t.grid((int64_t)n, 256), 256, 0, st>>>(rp, n, m, t.row_thread_max, t.hub_min, o, s.D, s.bins,
                                                          rows_in_bins_allowed(m), s.counters, s.out_ptr, s.outdeg,
                                                          s.omega);
-    k_orient<8><<<t.grid((int64_t)n, 256), 256, 0, st>>>(rp, n, m, t.row_thread_max, t.hub_min, o, s.D, s.bins,
-                                                         rows_in_bins_allowed(m), s.counters, s.out_ptr, s.outdeg,
-                                                         s.omega);
+    if (!big_rows)
+        k_orient<8><<<t.grid((int64_t)n, 256), 256, 0, st>>>(rp, n, m, t.row_thread_max, t.hub_min, o, s.D, s.bins,
+                                                             rows_in_bins_allowed(m), s.counters, s.out_ptr,
+                                                             s.outdeg, s.omega);
     k_orient_hub<<<t.num_sms * 4, ROW_CTA, 0, st>>>(rp, n, o, s.bins, s.out_ptr, s.counters, s.omega);
     if (bins && t.row_thread_max >= SMALL_MAX)
         k_hash_tail<<<(unsigned)(t.num_sms * 16), 256, 0, st>>>(s.counters, s.lay_ptr, s.out_ptr, n, s.info,

@@ -92,7 +92,7 @@ extern "C" int ef_compute_static(const ef_csr *g, int32_t n, int64_t m, int32_t 
         char msg[200];
         snprintf(msg, sizeof msg,
                  "ef_compute_static: graph needs %zu bytes of scratch, above the fixed %zu-byte maximum "
-                 "(about 172 n + 44 m + 48 min(n, m) bytes); use ef_compute_ex",
+                 "(at most about 172 n + 35 m + 48 min(n, m) bytes); use ef_compute_ex",
                  need, EF_STATIC_SCRATCH_BYTES);
         return fail(EF_ERR_ARG, msg);
     }
@@ -119,8 +119,8 @@ extern "C" int ef_compute_static(const ef_csr *g, int32_t n, int64_t m, int32_t 
     ef_outputs out = {};
     out.ef = out_ef;
     if (launch_ftab(s.ftab, s.tq, s.counters, fcap, st) || launch_orient(rp, ci, n, m, s, t, st, nullptr, nullptr, bins) ||
-        launch_wedge_small(rp, ci, s, precision, n, t, st) || launch_wedge_big(rp, ci, s, precision, 0, n, m, t, st) ||
-        launch_tri_pairs(s, n, m, t, st) ||
+        launch_tri_pairs(s, n, m, t, st) || launch_wedge_small(rp, ci, s, precision, n, t, st) ||
+        launch_wedge_big(rp, ci, s, precision, 0, n, m, t, st) ||
         launch_finalize(s, precision, n, out, t, st))
         return fail(EF_ERR_CUDA, "ef_compute_static: launch failed");
     if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess)

@@ -19,13 +19,13 @@
 // The pass is bound by L2 latency, so every membership test is one round of
 // two independent 16-byte loads, the same instructions for every lane: an
 // out-list of at most SHORT_MAX entries is read whole (it spans at most two
-// aligned quads); a longer one has a bucketed hash table (4 slots per
-// 16-byte bucket, load factor <= 0.5 + small rounding, built by the orientation)
-// and the key's bucket and the next one are loaded together, which settles
-// the test but for rare long probe runs.  The oriented CSR carries, for each
-// out-neighbour, the probe descriptor of its own list (which quads to load
-// and how to read them, fixed once per node by the orientation), so no test
-// waits for an out_ptr load or recomputes a table's geometry.
+// aligned quads); of a longer one the key's bucket of its hash table (8 slots
+// in one sector, out_table), which settles the test but for rare full
+// buckets.  The oriented CSR carries, for each out-neighbour, the probe
+// descriptor of its own list (which quads to load and how to read them, fixed
+// once per node by the orientation), so no test waits for an out_ptr load or
+// recomputes a table's geometry.  Owners of more than TRI_LONG
+// out-neighbours have their own kernel (k_tri_long).
 //
 // Measured and left out (4M-node power-law graph): L2 eviction hints
 // (evict_last on probes, evict_first on the candidate stream) changed
@@ -71,15 +71,12 @@ __device__ __forceinline__ unsigned match4(int4 v, int key) {
            (unsigned)(v.w == key) << 3;
 }
 
-__device__ __forceinline__ bool has_empty(int4 v) { return (v.x | v.y | v.z | v.w) < 0; }
-
 // One membership test "key in the out-list of probe descriptor pd", split so
 // that a lane issues the loads of all its tests before it waits for any: the
-// quads p0 and p0 + d1, and which of their entries count (info bits 0-3 and
+// quads p0 and p0 + 1, and which of their entries count (info bits 0-3 and
 // 4-7) and the kind of list (bits 8-9, the descriptor's kind).
 struct Probe {
     const int4 *p0;
-    int d1;
     unsigned info;
 };
 
@@ -89,46 +86,46 @@ __device__ __forceinline__ Probe probe_of(const int32_t *out_col, const int32_t 
     if (kind == 1) {
         const int nb = pd.y & DESC_MASK;
         const int b0 = bucket_of(key, nb);
-        r.p0 = reinterpret_cast<const int4 *>(out_hash) + ((int64_t)pd.x + b0);
-        r.d1 = b0 + 1 == nb ? -b0 : 1;
+        r.p0 = reinterpret_cast<const int4 *>(out_hash) + ((int64_t)pd.x + 2 * b0);
         r.info = 0xffu | 1u << 8;
     } else if (kind == 0) {
         r.p0 = reinterpret_cast<const int4 *>(out_col) + pd.x;
-        r.d1 = 1;
         r.info = (unsigned)pd.y & 0xffu;
     } else {
         r.p0 = reinterpret_cast<const int4 *>(out_col) + (pd.x >> 2);
-        r.d1 = 1;
         r.info = 2u << 8;
     }
     return r;
 }
 
-// Resolve a probe from its two loaded quads.  The rare ends -- a hashed probe
-// whose two buckets were full without the key (continue the run), a long
-// list without a table (malformed input only: binary search) -- reload what
-// they need.
-__device__ __forceinline__ bool probe_done(const Probe &r, int4 x, int4 y, const int32_t *out_col,
-                                           const int32_t *out_hash, int2 pd, int key) {
-    if ((match4(x, key) & r.info) | (match4(y, key) & (r.info >> 4) & 0xfu)) return true;
-    const unsigned kind = (r.info >> 8) & 3u;
-    if (kind == 0 || (kind == 1 && (has_empty(x) || has_empty(y)))) return false;
-    if (kind == 1) {
+// Resolve a probe from its two loaded quads.  The rare ends -- a full home
+// bucket without the key (continue with the next ones), a long list without
+// a table (malformed input only: binary search) -- reload what they need.
+__device__ __forceinline__ bool probe_more(const int4 *p0, const int32_t *out_col, const int32_t *out_hash, int2 pd,
+                                           int key) {
+    if ((unsigned)pd.y >> DESC_KIND_SHIFT == 1u) {
         const int nb = pd.y & DESC_MASK;
         const int4 *t = reinterpret_cast<const int4 *>(out_hash) + pd.x;
-        int b = (int)(r.p0 + r.d1 - t);
-        b = b + 1 == nb ? 0 : b + 1;
-        for (int tries = 2; tries < nb; ++tries) {
-            const int4 q = __ldg(t + b);
-            if (match4(q, key)) return true;
-            if (has_empty(q)) return false;
+        int b = (int)(p0 - t) >> 1;
+        for (int tries = 1; tries < nb; ++tries) {
             b = b + 1 == nb ? 0 : b + 1;
+            const int4 x = __ldg(t + 2 * b), y = __ldg(t + 2 * b + 1);
+            if (match4(x, key) | match4(y, key)) return true;
+            if (y.w < 0) return false;
         }
         return false;
     }
     const int ls = pd.x, le = pd.y & DESC_MASK;
     const int pos = ls + lower_bound_i32(out_col + ls, le - ls, key);
     return pos < le && out_col[pos] == key;
+}
+
+__device__ __forceinline__ bool probe_done(const Probe &r, int4 x, int4 y, const int32_t *out_col,
+                                           const int32_t *out_hash, int2 pd, int key) {
+    if ((match4(x, key) & r.info) | (match4(y, key) & (r.info >> 4) & 0xfu)) return true;
+    const unsigned kind = (r.info >> 8) & 3u;
+    if (kind == 0 || (kind == 1 && y.w < 0)) return false;
+    return probe_more(r.p0, out_col, out_hash, pd, key);
 }
 
 __device__ __forceinline__ void credit_tri(int64_t *qacc, int64_t *tcnt, int v, int64_t q, int cnt) {
@@ -163,7 +160,8 @@ __global__ void __launch_bounds__(TRI_WARPS * 32, TRI_BLOCKS) k_tri_pairs(
             if (k < total) {
                 const int a = out_src[k];
                 const int kend = out_ptr[a] + outdeg[a];
-                const int np = a >= a_lo && a < a_hi ? kend - (int)k - 1 : 0;
+                // (the long owners' pairs are k_tri_long's)
+                const int np = a >= a_lo && a < a_hi && kend - out_ptr[a] <= TRI_LONG ? kend - (int)k - 1 : 0;
                 if (np > 0) {
                     const int b = out_col[k];
                     const int Db = out_D[k];
@@ -228,7 +226,7 @@ __global__ void __launch_bounds__(TRI_WARPS * 32, TRI_BLOCKS) k_tri_pairs(
                     pr[q] = probe_of(out_col, out_hash, b_low ? bpd : rc[q], b_low ? c[q] : b);
                     pr[q].info |= (unsigned)b_low << 10;
                     x[q] = __ldg(pr[q].p0);
-                    y[q] = __ldg(pr[q].p0 + pr[q].d1);
+                    y[q] = __ldg(pr[q].p0 + 1);
                 }
             }
             int hits = 0;
@@ -262,13 +260,183 @@ __global__ void __launch_bounds__(TRI_WARPS * 32, TRI_BLOCKS) k_tri_pairs(
     }
 }
 
+// ------------------------------------------------------------- long owners
+// Owners a of more than TRI_LONG out-neighbours.  Their out-lists are first
+// sorted by rank (k_sort_long), so that of a pair b before c the lower end is
+// always b.  Then a warp per 32 candidates (k_tri_long): lane l holds c =
+// N+(a)[32 k + l] and the warp walks the earlier entries b, whose table is
+// the same for all lanes: a test is a hash, two 16-byte loads and their
+// compares, with nothing to decide per lane.  The hits of 32 b are kept as a
+// bit matrix (a word per lane); its rows give c's credits, its transpose b's,
+// so a correction is looked up only where a triangle is, and the credits go
+// out once per (a, c) and per (a, b, item) instead of once per hit.  (Where
+// most tests close a triangle, as in R-MAT, the hits' reductions to a few
+// large c had bound the pass.)
+//
+// Pair tests of a call, all owners in k_tri_pairs / with the long owners
+// here: R-MAT 2^16 (955k entries) 0.74 / 0.21 ms, R-MAT 2^18 1.9 / 0.62,
+// power-law 4M 1.60 / 1.39, its 87M-entry variant 5.8 / 4.8.  Here the
+// kernel issues in half of the cycles and its loads, one sector per lane, use
+// 63% of the L1 wavefronts; half of the rest is k_tri_pairs.  TRI_LONG = 16:
+// R-MAT 2^16 0.17 but power-law 4M 1.42 and 0.40 against 0.38 at 1M (lanes
+// past the list idle); four entries b together: 1.42.  Without the sort, the
+// lower end of each pair decided per lane and b's credits reduced by warp
+// sums per b: R-MAT 0.24, power-law 1.54.
+constexpr int TL_WARPS = 8;
+
+// Entry e of every 32 of a long list: its position by rank is the number of
+// entries below it.  A warp per item.
+__global__ void __launch_bounds__(256) k_sort_long(const int32_t *__restrict__ out_ptr,
+                                                   const int32_t *__restrict__ out_col,
+                                                   const int32_t *__restrict__ out_D,
+                                                   const int2 *__restrict__ out_pd,
+                                                   const int32_t *__restrict__ outdeg,
+                                                   const int2 *__restrict__ items, const int32_t *__restrict__ cnt,
+                                                   int4 *__restrict__ rec) {
+    if (gate_closed(cnt)) return;
+    const int lane = threadIdx.x & 31;
+    const int total = cnt[CNT_TRILONG];
+    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t it = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); it < total; it += nwarps) {
+        const int2 item = items[it];
+        const int ls = out_ptr[item.x], p = outdeg[item.x], e = item.y * 32 + lane;
+        const bool own = e < p;
+        const int x = own ? out_col[ls + e] : 0, Dx = own ? out_D[ls + e] : 0;
+        int pos = 0;
+        for (int i0 = 0; i0 < p; i0 += 32) {
+            const bool in = i0 + lane < p;
+            const int y = in ? out_col[ls + i0 + lane] : 0, Dy = in ? out_D[ls + i0 + lane] : 0x7fffffff;
+#pragma unroll 8
+            for (int i = 0; i < 32; ++i)   // entries past the list rank above all
+                pos += rank_less(__shfl_sync(FULL, Dy, i), __shfl_sync(FULL, y, i), Dx, x);
+        }
+        if (own) {
+            const int2 pd = out_pd[ls + e];
+            rec[ls + pos] = make_int4(x, Dx, pd.x, pd.y);
+        }
+    }
+}
+
+// One 32-byte sector in one load (p 32-byte aligned).
+__device__ __forceinline__ void load_sector(const int4 *p, int4 &x, int4 &y) {
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(x.x), "=r"(x.y), "=r"(x.z), "=r"(x.w), "=r"(y.x), "=r"(y.y), "=r"(y.z), "=r"(y.w)
+        : "l"(p));
+}
+
+// Lane i's word of the transpose of the 32 x 32 bit matrix whose rows are the
+// lanes' words.
+__device__ __forceinline__ unsigned transpose32(unsigned v) {
+    const int lane = threadIdx.x & 31;
+    unsigned m = 0x0000ffffu;
+#pragma unroll
+    for (int s = 16; s > 0; s >>= 1) {
+        const unsigned o = __shfl_xor_sync(FULL, v, s);
+        v = lane & s ? (v & ~m) | (o >> s & m) : (v & m) | (o << s & ~m);
+        m ^= m << (s >> 1);
+    }
+    return v;
+}
+
+constexpr int TL_STEP = 2;   // entries b tested together
+
+__global__ void __launch_bounds__(TL_WARPS * 32, 4) k_tri_long(
+    const int32_t *__restrict__ out_ptr, const int32_t *__restrict__ out_col, const int32_t *__restrict__ out_hash,
+    const int32_t *__restrict__ outdeg, const int32_t *__restrict__ D, int32_t n,
+    const int32_t *__restrict__ owner_range, const int64_t *__restrict__ tq, const int2 *__restrict__ items,
+    const int4 *__restrict__ rec, int64_t *__restrict__ qacc, int64_t *__restrict__ tcnt, int32_t *__restrict__ cnt) {
+    if (gate_closed(cnt)) return;
+    __shared__ int4 s_b[TL_WARPS][32];   // {b, D_b, its descriptor}
+    __shared__ int s_Dc[TL_WARPS][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int total = cnt[CNT_TRILONG];
+    const int a_lo = owner_range ? owner_range[0] : 0, a_hi = owner_range ? owner_range[1] : n;
+    const int4 *cols = reinterpret_cast<const int4 *>(out_col), *table = reinterpret_cast<const int4 *>(out_hash);
+    for (;;) {
+        int it = 0;
+        if (lane == 0) it = atomicAdd(cnt + CNT_TRINEXT, 1);
+        it = __shfl_sync(FULL, it, 0);
+        if (it >= total) break;
+        const int2 item = items[total - 1 - it];
+        const int a = item.x;
+        if (a < a_lo || a >= a_hi) continue;
+        const int ls = out_ptr[a], p = outdeg[a], Da = D[a];
+        const int j = item.y * 32 + lane;
+        const bool own = j < p;
+        const int4 rc = own ? rec[ls + j] : make_int4(-2, 0, 0, 0);   // -2: no key
+        const int c = rc.x;
+        const uint32_t hc = (uint32_t)c * 0x9E3779B1u;                // bucket_of's hash
+        const int sum_c = Da + rc.y;
+        const int last = min(item.y * 32 + 31, p - 1);   // b runs over the entries below this one
+        s_Dc[w][lane] = rc.y;
+        int64_t qc = 0;
+        int tc = 0;
+        for (int i0 = 0; i0 < last; i0 += 32) {
+            __syncwarp();
+            const int4 rb = i0 + lane < last ? rec[ls + i0 + lane] : make_int4(0, 0, 0, 0);
+            s_b[w][lane] = rb;
+            __syncwarp();
+            const int nb = min(32, last - i0);
+            unsigned found = 0;   // bit i: {b_i, c} adjacent
+            for (int i = 0; i < nb; i += TL_STEP) {
+                int4 x[TL_STEP], y[TL_STEP];
+                const int4 *p0[TL_STEP];
+                unsigned mask[TL_STEP];   // entries of the two quads that count
+                int2 pd[TL_STEP];
+#pragma unroll
+                for (int q = 0; q < TL_STEP; ++q) {
+                    // past the chunk's end: an empty list
+                    const int4 b = s_b[w][min(i + q, nb - 1)];
+                    pd[q] = i + q < nb ? make_int2(b.z, b.w) : make_int2(0, 0);
+                    const unsigned kind = (unsigned)pd[q].y >> DESC_KIND_SHIFT;
+                    if (kind == 1) {
+                        p0[q] = table + (pd[q].x + 2 * (int)(((uint64_t)hc * (uint32_t)(pd[q].y & DESC_MASK)) >> 32));
+                        mask[q] = 0xff;
+                        load_sector(p0[q], x[q], y[q]);
+                    } else {
+                        // a short list's quads, or (kind 2) none: resolved below
+                        p0[q] = cols + (kind == 0 ? pd[q].x : 0);
+                        mask[q] = kind == 0 ? (unsigned)pd[q].y & 0xffu : 0u;
+                        x[q] = __ldg(p0[q]);
+                        y[q] = __ldg(p0[q] + 1);
+                    }
+                }
+#pragma unroll
+                for (int q = 0; q < TL_STEP; ++q) {
+                    const unsigned kind = (unsigned)pd[q].y >> DESC_KIND_SHIFT;
+                    bool hit = ((match4(x[q], c) | match4(y[q], c) << 4) & mask[q]) != 0u;
+                    // a full bucket without the key, or a list without a table
+                    if (own && !hit && (kind == 2 || (kind == 1 && y[q].w >= 0)))
+                        hit = probe_more(p0[q], out_col, out_hash, pd[q], c);
+                    if (hit) found |= 1u << (i + q);
+                }
+            }
+            // only entries before c (c = -2 matches no key)
+            if (i0 + 31 >= j) found &= j > i0 ? (1u << (j - i0)) - 1u : 0u;
+            const unsigned col = transpose32(found);   // lane i: the c adjacent to b_i
+            tc += __popc(found);
+            for (unsigned f = found; f; f &= f - 1u) qc += __ldg(tq + sum_c + s_b[w][__ffs(f) - 1].y);
+            if (col) {
+                int64_t qb = 0;
+                for (unsigned f = col; f; f &= f - 1u) qb += __ldg(tq + Da + rb.y + s_Dc[w][__ffs(f) - 1]);
+                credit_tri(qacc, tcnt, rb.x, qb, __popc(col));
+            }
+        }
+        if (tc) credit_tri(qacc, tcnt, c, qc, tc);
+        const int64_t qa = warp_sum(qc);
+        const int ta = __reduce_add_sync(FULL, tc);
+        if (lane == 0 && ta) credit_tri(qacc, tcnt, a, qa, ta);
+        __syncwarp();
+    }
+}
+
 static inline unsigned grid_of(int64_t work, int per_block, int64_t cap) {
     int64_t g = (work + per_block - 1) / per_block;
     return (unsigned)(g < 1 ? 1 : (g > cap ? cap : g));
 }
 
 int launch_tri_pairs(const Scratch &s, int32_t n, int64_t m, const Tune &t, cudaStream_t st,
-                     const int32_t *owner_range) {
+                     const int32_t *owner_range, bool long_lists) {
     const unsigned grid = grid_of(m / 2, TRI_WARPS * 32, (int64_t)t.num_sms * 16);
     if (t.tri_variant == 1)
         k_tri_pairs<4, 3, 32><<<grid, TRI_WARPS * 32, 0, st>>>(s.out_ptr, s.out_col, s.out_D, s.out_pd, s.out_src,
@@ -278,6 +446,12 @@ int launch_tri_pairs(const Scratch &s, int32_t n, int64_t m, const Tune &t, cuda
         k_tri_pairs<2, 4, 64><<<grid, TRI_WARPS * 32, 0, st>>>(s.out_ptr, s.out_col, s.out_D, s.out_pd, s.out_src,
                                                             s.out_hash, s.outdeg, s.D, n, owner_range, s.tq, s.qacc,
                                                             s.tcnt, s.counters);
+    if (!long_lists) return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    k_sort_long<<<(unsigned)t.num_sms * 8, 256, 0, st>>>(s.out_ptr, s.out_col, s.out_D, s.out_pd, s.outdeg,
+                                                        s.tri_items, s.counters, s.tri_rec);
+    k_tri_long<<<(unsigned)t.num_sms * 4, TL_WARPS * 32, 0, st>>>(s.out_ptr, s.out_col, s.out_hash, s.outdeg, s.D, n,
+                                                                 owner_range, s.tq, s.tri_items, s.tri_rec, s.qacc,
+                                                                 s.tcnt, s.counters);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

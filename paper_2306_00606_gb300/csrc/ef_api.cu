@@ -80,12 +80,12 @@ struct ef_ctx {
     ef::Tune tune;
     cudaGraphExec_t gexec = nullptr;
     GraphKey gkey;   // zero-filled in ef_ctx_create
+    const void *gouts[6] = {};       // output buffers of the last graph call (only to count replays)
     void *rank = nullptr;            // learned-path buffers (RankScratch)
     size_t rank_bytes = 0;
-    void *acts = nullptr;            // training activations
-    size_t acts_bytes = 0;
     double *dtmp = nullptr;          // small device scratch (feature sums)
     bool long_lists = true;          // an owner of the current graph has more than TRI_LONG out-neighbours
+    bool big_rows = false;           // the current graph is known to have rows above SMALL_MAX
     int path = 0;                    // part B kernels of the last exact call (PathMode)
     bool bins = true;                // out-lists of the current graph in degree-bin order (bin_layout)
     void *sir = nullptr;             // SIR simulation state
@@ -162,7 +162,7 @@ void drop_graph(ef_ctx *ctx) {
 // Device bytes held in the context's working buffers.
 uint64_t held_bytes(const ef_ctx *ctx) {
     return (uint64_t)ctx->scratch_bytes + (uint64_t)ctx->ftab_cap * 2 * sizeof(double) + ctx->io_bytes +
-           ctx->goff_bytes + ctx->rank_bytes + ctx->acts_bytes + ctx->sir_bytes + (ctx->dtmp ? 64 * sizeof(double) : 0);
+           ctx->goff_bytes + ctx->rank_bytes + ctx->sir_bytes + (ctx->dtmp ? 64 * sizeof(double) : 0);
 }
 
 int ensure_buffer(ef_ctx *ctx, void **buf, size_t *have, size_t need, size_t slack) {
@@ -813,7 +813,6 @@ int ef_ctx_destroy(ef_ctx *ctx) {
     cudaFree(ctx->io);
     cudaFree(ctx->goff);
     cudaFree(ctx->rank);
-    cudaFree(ctx->acts);
     cudaFree(ctx->dtmp);
     cudaFree(ctx->sir);
     cudaFree(ctx->d_sticky);
@@ -1377,10 +1376,8 @@ int ef_mlp_grad(ef_ctx *ctx, ef_model *model, const float *x, const float *y, in
     if (!ctx || !model || n < 1 || !x || !y || !loss || !grad) { set_err(ctx, "bad arguments"); return EF_ERR_ARG; }
     if (model->device != ctx->device) { set_err(ctx, "model and context on different devices"); return EF_ERR_MODEL; }
     DeviceGuard dg(ctx->device);
-    int rc = ensure_buffer(ctx, &ctx->acts, &ctx->acts_bytes, ef::mlp_act_bytes(n), 0);
-    if (rc) return rc;
-    LAUNCH(ef::launch_mlp_step(model->d, x, y, n, n, 0, false, false, false, 0.f, (uint16_t *)ctx->acts,
-                               ctx->num_sms, ctx->stream),
+    LAUNCH(ef::prepare_mlp(), "network set-up");
+    LAUNCH(ef::launch_mlp_step(model->d, x, y, n, n, 0, false, false, false, 0.f, ctx->num_sms, ctx->stream),
            "network gradient");
     float ls = 0.f;
     CU(cudaMemcpyAsync(grad, model->d->grad, sizeof(float) * ef::P_N, cudaMemcpyDeviceToHost, ctx->stream));
@@ -1399,17 +1396,15 @@ int ef_surrogate_train(ef_ctx *ctx, ef_model *model, const float *x, const float
     if (model->device != ctx->device) { set_err(ctx, "model and context on different devices"); return EF_ERR_MODEL; }
     DeviceGuard dg(ctx->device);
     cudaStream_t st = ctx->stream;
-    int rc = ensure_buffer(ctx, &ctx->acts, &ctx->acts_bytes, ef::mlp_act_bytes(opt->batch), 0);
-    if (rc) return rc;
+    LAUNCH(ef::prepare_mlp(), "network set-up");
     if (!ctx->dtmp) CU(cudaMalloc(&ctx->dtmp, 64 * sizeof(double)));
     if (!model->fitted) {
         LAUNCH(ef::launch_feature_stats(x, n, model->d, ctx->dtmp, st), "feature statistics");
         LAUNCH(ef::launch_model_pack(model->d, st), "model pack");
         model->fitted = 1;
     }
-    uint16_t *acts = (uint16_t *)ctx->acts;
     auto step = [&](cudaStream_t s) {
-        return ef::launch_mlp_step(model->d, x, y, n, opt->batch, opt->seed, true, true, true, opt->lr, acts,
+        return ef::launch_mlp_step(model->d, x, y, n, opt->batch, opt->seed, true, true, true, opt->lr,
                                    ctx->num_sms, s);
     };
     float first = 0.f, last = 0.f;

@@ -547,8 +547,8 @@ int launch_mlp_infer(const ModelDev *M, const float *x, int32_t n, float *out, i
 int launch_mlp_infer_bf16(const ModelDev *M, const uint32_t *xb, int32_t n, float *out, int num_sms,
                           cudaStream_t st);
 int launch_mlp_step(ModelDev *M, const float *x, const float *y, int32_t n, int32_t batch, uint64_t seed, bool sample,
-                    bool count_step, bool adam, float lr, uint16_t *acts, int num_sms, cudaStream_t st);
-size_t mlp_act_bytes(int32_t batch);
+                    bool count_step, bool adam, float lr, int num_sms, cudaStream_t st);
+int prepare_mlp();   // before any launch_mlp_step or its capture
 int launch_model_pack(ModelDev *M, cudaStream_t st);
 int launch_feature_stats(const float *x, int32_t n, ModelDev *M, double *tmp, cudaStream_t st);
 int launch_omega_mm(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const Scratch &s,

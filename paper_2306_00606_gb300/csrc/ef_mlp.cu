@@ -7,8 +7,8 @@
 // - inference and the training forward pass take 16 rows per warp;
 // - the backward pass computes the data gradients per tile in the same
 //   registers;
-// - the weight gradients are separate reductions over the batch
-//   (k_mlp_wgrad).
+// - the weight gradients are accumulated by the block over its rows, from
+//   shared memory (k_mlp_grad).
 // The work is tiny next to the exact EF pass (5.3k parameters): inference
 // reads 64 bytes of features per node and is bound by HBM, so the
 // warp-level BF16 instructions suffice here (tcgen05 would not pay).
@@ -27,8 +27,6 @@
 namespace ef {
 
 __device__ __forceinline__ float bf16_to_float(uint16_t u) { return __uint_as_float((uint32_t)u << 16); }
-
-__device__ __forceinline__ uint32_t pair_u16(uint16_t lo, uint16_t hi) { return (uint32_t)lo | ((uint32_t)hi << 16); }
 
 __device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile(
@@ -99,10 +97,6 @@ __device__ __forceinline__ RowPart load_row(const float *x) {
 
 __device__ __forceinline__ void tile_forward(const MlpSmem &s, RowPart rg, RowPart rg8, bool vg, bool vg8, Tile &T);
 __device__ __forceinline__ void tile_layers(const MlpSmem &s, Tile &T);
-
-__device__ __forceinline__ void tile_forward(const MlpSmem &s, const float *xg, const float *xg8, Tile &T) {
-    tile_forward(s, load_row(xg), load_row(xg8), xg != nullptr, xg8 != nullptr, T);
-}
 
 __device__ __forceinline__ void tile_forward(const MlpSmem &s, RowPart rg, RowPart rg8, bool vg, bool vg8, Tile &T) {
     const int t = threadIdx.x & 3;
@@ -175,72 +169,167 @@ __device__ __forceinline__ void tile_layers(const MlpSmem &s, Tile &T) {
 
 constexpr int MLP_WARPS = 8;
 
-__global__ void __launch_bounds__(MLP_WARPS * 32, 4) k_mlp_infer(const ModelDev *__restrict__ M,
-                                                              const float *__restrict__ X, int32_t n,
-                                                              float *__restrict__ out) {
-    __shared__ MlpSmem s;
-    load_model(M, s, false);
-    __syncthreads();
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5;
-    const int64_t tiles = ((int64_t)n + 15) / 16;
-    const int64_t step = (int64_t)gridDim.x * MLP_WARPS;
-    auto row = [&](int64_t r) { return r < n ? X + r * MLP_F : nullptr; };
-    int64_t tile = (int64_t)blockIdx.x * MLP_WARPS + w;
-    // the next tile's rows are loaded before the current tile is computed
-    RowPart a = load_row(row(tile * 16 + g)), b = load_row(row(tile * 16 + g + 8));
-    for (; tile < tiles; tile += step) {
-        const int64_t r0 = tile * 16 + g, r1 = r0 + 8;
-        const RowPart ca = a, cb = b;
-        const int64_t nx = tile + step;
-        if (nx < tiles) {
-            a = load_row(row(nx * 16 + g));
-            b = load_row(row(nx * 16 + g + 8));
-        }
-        Tile T;
-        tile_forward(s, ca, cb, r0 < n, r1 < n, T);
-        if (t == 0) {
-            if (r0 < n) out[r0] = T.p0;
-            if (r1 < n) out[r1] = T.p1;
-        }
+// ---------------------------------------------------------------- inference
+// Two 16-row tiles per warp step share every weight fragment (one 8-byte
+// shared-memory load per pair of tiles: a fragment's two words are stored side
+// by side, rows padded to 40 words so that a half-warp's loads fall in
+// different banks), layer 2 starts from its biases, and a layer-2 column
+// tile is consumed as soon as it is complete, so no activation array is kept.
+// Bound by the rate of mma.sync and the shared-memory loads together.
+// Measured, 8M rows: 344 us with one tile per step and four-byte loads, 251
+// so; at 80 registers (three blocks per SM) 278, four tiles 280, the W2
+// fragments in registers (12 warps per SM) 276-292.
+constexpr int INF_TILES = 2;
+constexpr int W2ROW = 40;   // words of a W2 row: 4 k-chunks x 4 lanes x 2 words, padded
+
+struct InferSmem {
+    uint2 w1[MLP_H * 4 + MLP_H / 8 * 4];   // [n][t] of the one k-chunk, 4 words' pad after 8 rows
+    uint2 w2[MLP_H * W2ROW / 2];           // [n][kc][t]
+    float2 b1[MLP_H / 2], b2[MLP_H / 2], w3[MLP_H / 2];
+    float mean[MLP_F], istd[MLP_F];
+    float b3;
+};
+
+__device__ __forceinline__ int w1_at(int n, int t) { return n * 4 + t; }
+
+__device__ void load_infer(const ModelDev *M, InferSmem &s) {
+    const uint32_t *w1 = reinterpret_cast<const uint32_t *>(M->w1t), *w2 = reinterpret_cast<const uint32_t *>(M->w2t);
+    for (int i = threadIdx.x; i < MLP_H * 4; i += blockDim.x) {
+        const int n = i >> 2, t = i & 3;
+        s.w1[w1_at(n, t)] = make_uint2(w1[n * (MLP_F / 2) + t], w1[n * (MLP_F / 2) + t + 4]);
     }
+    for (int i = threadIdx.x; i < MLP_H * 16; i += blockDim.x) {
+        const int n = i >> 4, kc = i >> 2 & 3, t = i & 3;
+        const uint32_t *r = w2 + n * (MLP_H / 2) + 8 * kc + t;
+        s.w2[n * (W2ROW / 2) + kc * 4 + t] = make_uint2(r[0], r[4]);
+    }
+    for (int i = threadIdx.x; i < MLP_H / 2; i += blockDim.x) {
+        s.b1[i] = make_float2(M->p[P_B1 + 2 * i], M->p[P_B1 + 2 * i + 1]);
+        s.b2[i] = make_float2(M->p[P_B2 + 2 * i], M->p[P_B2 + 2 * i + 1]);
+        s.w3[i] = make_float2(M->p[P_W3 + 2 * i], M->p[P_W3 + 2 * i + 1]);
+    }
+    for (int i = threadIdx.x; i < MLP_F; i += blockDim.x) {
+        s.mean[i] = M->mean[i];
+        s.istd[i] = 1.0f / M->stdv[i];
+    }
+    if (threadIdx.x == 0) s.b3 = M->p[P_B3];
 }
 
-// Inference on standardised BF16 rows (8 words per row, word q holding
-// features 2q and 2q + 1): lane (g, t) reads words t and t + 4 of rows g and
-// g + 8, which are the first-layer A fragment as it is, so the predictions
-// equal k_mlp_infer's on the FP32 rows bit for bit.
-__global__ void __launch_bounds__(MLP_WARPS * 32, 4) k_mlp_infer_bf16(const ModelDev *__restrict__ M,
-                                                                   const uint32_t *__restrict__ Xb, int32_t n,
-                                                                   float *__restrict__ out) {
-    __shared__ MlpSmem s;
-    load_model(M, s, false);
+// Predictions of INF_TILES tiles from their first-layer operands: p[u][0] of
+// row g, p[u][1] of row g + 8 (all four lanes of a group).
+__device__ __forceinline__ void infer_tiles(const InferSmem &s, const uint32_t (&a1)[INF_TILES][4],
+                                            float (&p)[INF_TILES][2]) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    uint32_t a2[INF_TILES][4][4];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const uint2 b = s.w1[w1_at(8 * j + g, t)];
+        const float2 bias = s.b1[4 * j + t];
+#pragma unroll
+        for (int u = 0; u < INF_TILES; ++u) {
+            // the bias after the products, as in the training pass: another order
+            // rounds some activations to another BF16 value
+            float c[4] = {0.f, 0.f, 0.f, 0.f};
+            mma16816(c, a1[u], b.x, b.y);
+            a2[u][j >> 1][2 * (j & 1)] = pack_bf16(fmaxf(c[0] + bias.x, 0.f), fmaxf(c[1] + bias.y, 0.f));
+            a2[u][j >> 1][2 * (j & 1) + 1] = pack_bf16(fmaxf(c[2] + bias.x, 0.f), fmaxf(c[3] + bias.y, 0.f));
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < INF_TILES; ++u) p[u][0] = p[u][1] = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const float2 bias = s.b2[4 * j + t], w3 = s.w3[4 * j + t];
+        float c[INF_TILES][4];
+#pragma unroll
+        for (int u = 0; u < INF_TILES; ++u) {
+            c[u][0] = c[u][2] = bias.x;
+            c[u][1] = c[u][3] = bias.y;
+        }
+#pragma unroll
+        for (int kc = 0; kc < 4; ++kc) {
+            const uint2 b = s.w2[(8 * j + g) * (W2ROW / 2) + kc * 4 + t];
+#pragma unroll
+            for (int u = 0; u < INF_TILES; ++u) mma16816(c[u], a2[u][kc], b.x, b.y);
+        }
+#pragma unroll
+        for (int u = 0; u < INF_TILES; ++u) {
+            p[u][0] = fmaf(fmaxf(c[u][0], 0.f), w3.x, fmaf(fmaxf(c[u][1], 0.f), w3.y, p[u][0]));
+            p[u][1] = fmaf(fmaxf(c[u][2], 0.f), w3.x, fmaf(fmaxf(c[u][3], 0.f), w3.y, p[u][1]));
+        }
+    }
+#pragma unroll
+    for (int u = 0; u < INF_TILES; ++u)
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            p[u][q] += __shfl_xor_sync(FULL, p[u][q], 1);
+            p[u][q] += __shfl_xor_sync(FULL, p[u][q], 2);
+            p[u][q] += s.b3;
+        }
+}
+
+// BF: rows already standardised and rounded to BF16 (8 words per row, word q
+// holding features 2q and 2q + 1: words t and t + 4 are the fragment as it
+// is), else FP32 rows.  The predictions are equal bit for bit.
+template <bool BF>
+__global__ void __launch_bounds__(MLP_WARPS * 32, 2) k_mlp_infer(const ModelDev *__restrict__ M,
+                                                              const void *__restrict__ X_, int32_t n,
+                                                              float *__restrict__ out) {
+    __shared__ InferSmem s;
+    load_infer(M, s);
     __syncthreads();
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5;
-    const int64_t tiles = ((int64_t)n + 15) / 16;
+    const float *X = static_cast<const float *>(X_);
+    const uint32_t *Xb = static_cast<const uint32_t *>(X_);
+    const int64_t tiles = ((int64_t)n + 16 * INF_TILES - 1) / (16 * INF_TILES);
     const int64_t step = (int64_t)gridDim.x * MLP_WARPS;
-    auto word = [&](int64_t r, int q) { return r < n ? __ldg(Xb + r * (MLP_F / 2) + q) : 0u; };
+    const float m0 = s.mean[2 * t], m1 = s.mean[2 * t + 1], m2 = s.mean[2 * t + 8], m3 = s.mean[2 * t + 9];
+    const float i0 = s.istd[2 * t], i1 = s.istd[2 * t + 1], i2 = s.istd[2 * t + 8], i3 = s.istd[2 * t + 9];
+    // rows g and g + 8 of each tile, loaded ahead of their use
+    RowPart x[INF_TILES][2];
+    uint32_t xb[INF_TILES][4];
+    auto load = [&](int64_t tile) {
+#pragma unroll
+        for (int u = 0; u < INF_TILES; ++u)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                const int64_t r = (tile * INF_TILES + u) * 16 + g + 8 * q;
+                if constexpr (BF) {
+                    xb[u][q] = r < n ? __ldg(Xb + r * (MLP_F / 2) + t) : 0u;
+                    xb[u][q + 2] = r < n ? __ldg(Xb + r * (MLP_F / 2) + t + 4) : 0u;
+                } else {
+                    x[u][q] = load_row(r < n ? X + r * MLP_F : nullptr);
+                }
+            }
+    };
     int64_t tile = (int64_t)blockIdx.x * MLP_WARPS + w;
-    // the next tile's words are loaded before the current tile is computed
-    uint32_t a0 = word(tile * 16 + g, t), a1 = word(tile * 16 + g + 8, t);
-    uint32_t a2 = word(tile * 16 + g, t + 4), a3 = word(tile * 16 + g + 8, t + 4);
+    load(tile);
     for (; tile < tiles; tile += step) {
-        const int64_t r0 = tile * 16 + g, r1 = r0 + 8;
-        Tile T;
-        T.a1[0] = a0;
-        T.a1[1] = a1;
-        T.a1[2] = a2;
-        T.a1[3] = a3;
-        const int64_t nx = tile + step;
-        if (nx < tiles) {
-            a0 = word(nx * 16 + g, t);
-            a1 = word(nx * 16 + g + 8, t);
-            a2 = word(nx * 16 + g, t + 4);
-            a3 = word(nx * 16 + g + 8, t + 4);
-        }
-        tile_layers(s, T);
+        uint32_t a1[INF_TILES][4];
+#pragma unroll
+        for (int u = 0; u < INF_TILES; ++u)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if constexpr (BF) {
+                    a1[u][q] = xb[u][q];
+                    a1[u][q + 2] = xb[u][q + 2];
+                } else {
+                    const RowPart &r = x[u][q];
+                    a1[u][q] = pack_bf16((r.lo.x - m0) * i0, (r.lo.y - m1) * i1);
+                    a1[u][q + 2] = pack_bf16((r.hi.x - m2) * i2, (r.hi.y - m3) * i3);
+                }
+            }
+        if (tile + step < tiles) load(tile + step);
+        float p[INF_TILES][2];
+        infer_tiles(s, a1, p);
         if (t == 0) {
-            if (r0 < n) out[r0] = T.p0;
-            if (r1 < n) out[r1] = T.p1;
+#pragma unroll
+            for (int u = 0; u < INF_TILES; ++u)
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const int64_t r = (tile * INF_TILES + u) * 16 + g + 8 * q;
+                    if (r < n) out[r] = p[u][q];
+                }
         }
     }
 }
@@ -254,22 +343,6 @@ __device__ __forceinline__ int sample_row(uint64_t seed, int32_t step, int r, in
     return (int)(z % (uint64_t)n);
 }
 
-// Activations kept for the weight gradients, BF16, per padded batch row:
-// Z [16], H1 [64], dA2 [64], dA1 [64].
-size_t mlp_act_bytes(int32_t batch) {
-    const size_t rows = ((size_t)batch + 15) / 16 * 16;
-    return rows * (MLP_F + 3 * MLP_H) * sizeof(uint16_t);
-}
-
-struct Acts {
-    uint16_t *z, *h1, *e2, *e1;
-};
-
-__host__ __device__ inline Acts acts_of(uint16_t *base, int32_t batch) {
-    const size_t rows = ((size_t)batch + 15) / 16 * 16;
-    return Acts{base, base + rows * MLP_F, base + rows * (MLP_F + MLP_H), base + rows * (MLP_F + 2 * MLP_H)};
-}
-
 // Zero the gradient and loss; optionally advance the step counter (which
 // seeds the row sampling and Adam's bias corrections).
 __global__ void k_mlp_zero(ModelDev *M, bool count_step) {
@@ -280,90 +353,180 @@ __global__ void k_mlp_zero(ModelDev *M, bool count_step) {
     }
 }
 
-// Forward and data-gradient pass of a batch: per 16-row tile the loss, the
-// bias and w3 gradients (reduced here) and the activations the weight
-// gradients need (written as BF16).  dL/dp = 2 (p - y) / batch.
-__global__ void __launch_bounds__(MLP_WARPS * 32) k_mlp_fwd_bwd(ModelDev *M, const float *__restrict__ X,
+// Gradient of a batch in one kernel.  A block takes 128 rows at a time: each
+// warp runs the forward and backward pass of a 16-row tile in registers (loss,
+// bias and w3 gradients accumulate there in FP32) and leaves the four BF16
+// operands of the weight gradients -- Z, H1, dA2, dA1 -- in shared memory;
+// then all warps accumulate dW2 = H1^T dA2 (64 x 64) and dW1 = Z^T dA1
+// (16 x 64) over the 128 rows, warp w owning dW2 row tile (w & 3) x column
+// tiles 4 (w >> 2) .. +3 and dW1 column tile w, with the transposed fragments
+// from ldmatrix.  Rows are padded to 72 (24) elements: the eight 16-byte rows
+// of an 8 x 8 matrix fall in different banks.
+// Before, the operands went through global memory (416 bytes per row written,
+// read again element by element): 700 us for 1M rows, 205 now;
+// a training step of 8192 rows 47 -> 28 us.  Bound by latency at the 8 warps
+// per SM that 239 registers leave.
+constexpr int BATCH_TILE = 16 * MLP_WARPS;
+constexpr int ZS = 24, HS = 72;
+
+struct TrainSmem {
+    MlpSmem m;
+    __align__(16) uint16_t z[BATCH_TILE * ZS];
+    __align__(16) uint16_t h1[BATCH_TILE * HS], e2[BATCH_TILE * HS], e1[BATCH_TILE * HS];
+    float sums[MLP_WARPS][20][32];   // per lane: the weight gradients of earlier chunks
+};
+
+// Chunks whose weight gradients the tensor cores' accumulators hold at most:
+// those adds truncate, so short chains added up with rounding are the more
+// exact ones.
+constexpr int GRAD_CHAIN = 4;
+
+// Four 8 x 8 matrices, transposed; lane l gives the address of row l % 8 of matrix l / 8.
+__device__ __forceinline__ void ldsm_x4_trans(uint32_t (&r)[4], const uint16_t *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((uint32_t)__cvta_generic_to_shared(p)));
+}
+
+__global__ void __launch_bounds__(MLP_WARPS * 32, 1) k_mlp_grad(ModelDev *M, const float *__restrict__ X,
                                                                 const float *__restrict__ Y, int32_t n,
-                                                                int32_t batch, uint64_t seed, bool sample,
-                                                                uint16_t *acts_base) {
-    __shared__ MlpSmem s;
+                                                                int32_t batch, uint64_t seed, bool sample) {
+    extern __shared__ __align__(16) unsigned char train_smem[];
+    TrainSmem &S = *reinterpret_cast<TrainSmem *>(train_smem);
+    MlpSmem &s = S.m;
     load_model(M, s, true);
     __syncthreads();
-    const Acts A = acts_of(acts_base, batch);
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5;
     const int32_t step = M->step;
     const float inv_b = 1.0f / (float)batch;
     float gw3[8][2] = {}, gb2[8][2] = {}, gb1[8][2] = {};
     float gb3 = 0.f, loss = 0.f;
-    const int tiles = (batch + 15) / 16;
-    for (int tile = blockIdx.x * MLP_WARPS + w; tile < tiles; tile += gridDim.x * MLP_WARPS) {
-        const int r0 = tile * 16 + g, r1 = r0 + 8;
-        const int v0 = r0 < batch ? (sample ? sample_row(seed, step, r0, n) : r0) : -1;
-        const int v1 = r1 < batch ? (sample ? sample_row(seed, step, r1, n) : r1) : -1;
-        Tile T;
-        tile_forward(s, v0 >= 0 ? X + (int64_t)v0 * MLP_F : nullptr, v1 >= 0 ? X + (int64_t)v1 * MLP_F : nullptr, T);
-        const float e0 = v0 >= 0 ? T.p0 - Y[v0] : 0.f, e1 = v1 >= 0 ? T.p1 - Y[v1] : 0.f;
-        if (t == 0) loss += e0 * e0 + e1 * e1;
-        const float d0 = 2.f * e0 * inv_b, d1 = 2.f * e1 * inv_b;
-        if (t == 0) gb3 += d0 + d1;
-        // layer 3 and 2: dw3, dA2 = d * w3 * [h2 > 0], db2
-        float e2[8][4];
+    float acc2[4][4] = {}, acc1[4] = {};
+    const int mi = w & 3, nj0 = (w >> 2) * 4;
+    // this lane's row of an ldmatrix: as A (matrices 1, 3 eight columns on, 2, 3 eight rows on), as B the other way
+    const int ar = (lane & 7) + (lane >> 4 & 1) * 8, ac = (lane >> 3 & 1) * 8;
+    const int br = (lane & 7) + (lane >> 3 & 1) * 8, bc = (lane >> 4 & 1) * 8;
+    const int chunks = (int)(((int64_t)batch + BATCH_TILE - 1) / BATCH_TILE);
+    // the next chunk's rows are loaded before this chunk's weight gradients
+    RowPart x0, x1;
+    float y0, y1;
+    bool v0, v1;
+    auto load = [&](int chunk) {
+        const int64_t r0 = (int64_t)chunk * BATCH_TILE + 16 * w + g, r1 = r0 + 8;
+        v0 = chunk < chunks && r0 < batch;
+        v1 = chunk < chunks && r1 < batch;
+        const int64_t i0 = !v0 ? 0 : sample ? sample_row(seed, step, (int)r0, n) : r0;
+        const int64_t i1 = !v1 ? 0 : sample ? sample_row(seed, step, (int)r1, n) : r1;
+        x0 = load_row(v0 ? X + i0 * MLP_F : nullptr);
+        x1 = load_row(v1 ? X + i1 * MLP_F : nullptr);
+        y0 = v0 ? Y[i0] : 0.f;
+        y1 = v1 ? Y[i1] : 0.f;
+    };
+    float *sums = &S.sums[w][0][lane];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int c0 = 8 * j + 2 * t;
-            gw3[j][0] += d0 * T.h2[j][0] + d1 * T.h2[j][2];
-            gw3[j][1] += d0 * T.h2[j][1] + d1 * T.h2[j][3];
-            e2[j][0] = T.h2[j][0] > 0.f ? d0 * s.w3[c0] : 0.f;
-            e2[j][1] = T.h2[j][1] > 0.f ? d0 * s.w3[c0 + 1] : 0.f;
-            e2[j][2] = T.h2[j][2] > 0.f ? d1 * s.w3[c0] : 0.f;
-            e2[j][3] = T.h2[j][3] > 0.f ? d1 * s.w3[c0 + 1] : 0.f;
-            gb2[j][0] += e2[j][0] + e2[j][2];
-            gb2[j][1] += e2[j][1] + e2[j][3];
-        }
-        // layer 1: dA1 = (dA2 W2^T) * [h1 > 0]; B[k = j][n = i] = W2[i][j] = w2r[i][j]
-        float e1v[8][4];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) e1v[j][0] = e1v[j][1] = e1v[j][2] = e1v[j][3] = 0.f;
-#pragma unroll
-        for (int kc = 0; kc < 4; ++kc) {
-            const uint32_t a[4] = {pack_bf16(e2[2 * kc][0], e2[2 * kc][1]), pack_bf16(e2[2 * kc][2], e2[2 * kc][3]),
-                                   pack_bf16(e2[2 * kc + 1][0], e2[2 * kc + 1][1]),
-                                   pack_bf16(e2[2 * kc + 1][2], e2[2 * kc + 1][3])};
+    for (int i = 0; i < 20; ++i) sums[32 * i] = 0.f;
+    int chain = 0;
+    load(blockIdx.x);
+    for (int chunk = blockIdx.x; chunk < chunks; chunk += gridDim.x) {
+        uint32_t *z0 = reinterpret_cast<uint32_t *>(S.z + (16 * w + g) * ZS), *z1 = z0 + 8 * ZS / 2;
+        uint32_t *h0 = reinterpret_cast<uint32_t *>(S.h1 + (16 * w + g) * HS), *h8 = h0 + 8 * HS / 2;
+        uint32_t *d0p = reinterpret_cast<uint32_t *>(S.e2 + (16 * w + g) * HS), *d8p = d0p + 8 * HS / 2;
+        uint32_t *f0p = reinterpret_cast<uint32_t *>(S.e1 + (16 * w + g) * HS), *f8p = f0p + 8 * HS / 2;
+        uint32_t h1p[8][2], e2p[8][2];
+        {
+            Tile T;
+            tile_forward(s, x0, x1, v0, v1, T);
+            const float e0 = v0 ? T.p0 - y0 : 0.f, e1 = v1 ? T.p1 - y1 : 0.f;
+            if (t == 0) loss += e0 * e0 + e1 * e1;
+            const float d0 = 2.f * e0 * inv_b, d1 = 2.f * e1 * inv_b;
+            if (t == 0) gb3 += d0 + d1;
+            z0[t] = T.a1[0];
+            z1[t] = T.a1[1];
+            z0[t + 4] = T.a1[2];
+            z1[t + 4] = T.a1[3];
+            // layers 3 and 2: dw3, dA2 = d * w3 * [h2 > 0], db2
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
-                const int nn = 8 * j + g;
-                mma16816(e1v[j], a, *reinterpret_cast<const uint32_t *>(&s.w2r[nn * W2S + 16 * kc + 2 * t]),
-                         *reinterpret_cast<const uint32_t *>(&s.w2r[nn * W2S + 16 * kc + 2 * t + 8]));
+                const int c0 = 8 * j + 2 * t;
+                gw3[j][0] += d0 * T.h2[j][0] + d1 * T.h2[j][2];
+                gw3[j][1] += d0 * T.h2[j][1] + d1 * T.h2[j][3];
+                const float a = T.h2[j][0] > 0.f ? d0 * s.w3[c0] : 0.f;
+                const float b = T.h2[j][1] > 0.f ? d0 * s.w3[c0 + 1] : 0.f;
+                const float c = T.h2[j][2] > 0.f ? d1 * s.w3[c0] : 0.f;
+                const float d = T.h2[j][3] > 0.f ? d1 * s.w3[c0 + 1] : 0.f;
+                gb2[j][0] += a + c;
+                gb2[j][1] += b + d;
+                e2p[j][0] = pack_bf16(a, b);
+                e2p[j][1] = pack_bf16(c, d);
+                // h1 >= 0: a positive value stays positive in BF16 (same exponent range)
+                h1p[j][0] = pack_bf16(T.h1[j][0], T.h1[j][1]);
+                h1p[j][1] = pack_bf16(T.h1[j][2], T.h1[j][3]);
+                h0[4 * j + t] = h1p[j][0];
+                h8[4 * j + t] = h1p[j][1];
+                d0p[4 * j + t] = e2p[j][0];
+                d8p[4 * j + t] = e2p[j][1];
             }
         }
+        // layer 1: dA1 = (dA2 W2^T) * [h1 > 0]; B[k = j][n = i] = W2[i][j] = w2r[i][j]
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
-            e1v[j][0] = T.h1[j][0] > 0.f ? e1v[j][0] : 0.f;
-            e1v[j][1] = T.h1[j][1] > 0.f ? e1v[j][1] : 0.f;
-            e1v[j][2] = T.h1[j][2] > 0.f ? e1v[j][2] : 0.f;
-            e1v[j][3] = T.h1[j][3] > 0.f ? e1v[j][3] : 0.f;
-            gb1[j][0] += e1v[j][0] + e1v[j][2];
-            gb1[j][1] += e1v[j][1] + e1v[j][3];
-        }
-        // activations for the weight gradients (rows r0, r1 of the padded batch)
-        uint32_t *z0 = reinterpret_cast<uint32_t *>(A.z + (size_t)r0 * MLP_F);
-        uint32_t *z1 = reinterpret_cast<uint32_t *>(A.z + (size_t)r1 * MLP_F);
-        z0[t] = T.a1[0];
-        z1[t] = T.a1[1];
-        z0[t + 4] = T.a1[2];
-        z1[t + 4] = T.a1[3];
+            const int nn = 8 * j + g;
+            float e[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const int c0 = 8 * j + 2 * t;
-            *reinterpret_cast<uint32_t *>(A.h1 + (size_t)r0 * MLP_H + c0) = pack_bf16(T.h1[j][0], T.h1[j][1]);
-            *reinterpret_cast<uint32_t *>(A.h1 + (size_t)r1 * MLP_H + c0) = pack_bf16(T.h1[j][2], T.h1[j][3]);
-            *reinterpret_cast<uint32_t *>(A.e2 + (size_t)r0 * MLP_H + c0) = pack_bf16(e2[j][0], e2[j][1]);
-            *reinterpret_cast<uint32_t *>(A.e2 + (size_t)r1 * MLP_H + c0) = pack_bf16(e2[j][2], e2[j][3]);
-            *reinterpret_cast<uint32_t *>(A.e1 + (size_t)r0 * MLP_H + c0) = pack_bf16(e1v[j][0], e1v[j][1]);
-            *reinterpret_cast<uint32_t *>(A.e1 + (size_t)r1 * MLP_H + c0) = pack_bf16(e1v[j][2], e1v[j][3]);
+            for (int kc = 0; kc < 4; ++kc) {
+                const uint32_t a[4] = {e2p[2 * kc][0], e2p[2 * kc][1], e2p[2 * kc + 1][0], e2p[2 * kc + 1][1]};
+                mma16816(e, a, *reinterpret_cast<const uint32_t *>(&s.w2r[nn * W2S + 16 * kc + 2 * t]),
+                         *reinterpret_cast<const uint32_t *>(&s.w2r[nn * W2S + 16 * kc + 2 * t + 8]));
+            }
+            e[0] = h1p[j][0] & 0xffffu ? e[0] : 0.f;
+            e[1] = h1p[j][0] >> 16 ? e[1] : 0.f;
+            e[2] = h1p[j][1] & 0xffffu ? e[2] : 0.f;
+            e[3] = h1p[j][1] >> 16 ? e[3] : 0.f;
+            gb1[j][0] += e[0] + e[2];
+            gb1[j][1] += e[1] + e[3];
+            f0p[4 * j + t] = pack_bf16(e[0], e[1]);
+            f8p[4 * j + t] = pack_bf16(e[2], e[3]);
         }
+        load(chunk + gridDim.x);
+        __syncthreads();
+#pragma unroll 2
+        for (int rb = 0; rb < BATCH_TILE; rb += 16) {
+            uint32_t a[4], b[4];
+            ldsm_x4_trans(a, S.h1 + (rb + ar) * HS + 16 * mi + ac);
+#pragma unroll
+            for (int q = 0; q < 4; q += 2) {
+                ldsm_x4_trans(b, S.e2 + (rb + br) * HS + 8 * (nj0 + q) + bc);
+                mma16816(acc2[q], a, b[0], b[1]);
+                mma16816(acc2[q + 1], a, b[2], b[3]);
+            }
+            ldsm_x4_trans(a, S.z + (rb + ar) * ZS + ac);
+            // (matrices 2 and 3 of the second operand repeat 0 and 1: one column tile is needed)
+            ldsm_x4_trans(b, S.e1 + (rb + br) * HS + 8 * w);
+            mma16816(acc1, a, b[0], b[1]);
+        }
+        if (++chain == GRAD_CHAIN || chunk + gridDim.x >= chunks) {
+            chain = 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    sums[32 * (4 * q + i)] += acc2[q][i];
+                    acc2[q][i] = 0.f;
+                }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                sums[32 * (16 + i)] += acc1[i];
+                acc1[i] = 0.f;
+            }
+        }
+        __syncthreads();
     }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int i = 0; i < 4; ++i) acc2[q][i] = sums[32 * (4 * q + i)];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc1[i] = sums[32 * (16 + i)];
     // reduce over the 8 groups (lanes with equal t hold the same columns)
 #pragma unroll
     for (int j = 0; j < 8; ++j)
@@ -392,51 +555,6 @@ __global__ void __launch_bounds__(MLP_WARPS * 32) k_mlp_fwd_bwd(ModelDev *M, con
         atomicAdd(&M->grad[P_B3], gb3);
         atomicAdd(&M->loss_sum, loss);
     }
-}
-
-// Weight gradients over the batch: dW2 = H1^T dA2 (64 x 64) and
-// dW1 = Z^T dA1 (16 x 64), K = batch rows.  A CTA takes WG_ROWS rows; warp w
-// owns dW2 row tile (w & 3) x column tiles 4 (w >> 2) .. +3 and dW1 column
-// tile w.  Operands are read from the BF16 activations with the transposed
-// fragment layout.
-constexpr int WG_ROWS = 256;
-
-__global__ void __launch_bounds__(MLP_WARPS * 32) k_mlp_wgrad(ModelDev *M, int32_t batch,
-                                                              const uint16_t *__restrict__ acts_base) {
-    const Acts A = acts_of(const_cast<uint16_t *>(acts_base), batch);
-    const int rows = (batch + 15) / 16 * 16;
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5;
-    const int mi = w & 3, nj0 = (w >> 2) * 4;
-    float acc2[4][4] = {}, acc1[4] = {};
-    for (int r0 = blockIdx.x * WG_ROWS; r0 < rows; r0 += gridDim.x * WG_ROWS) {
-        const int rend = min(r0 + WG_ROWS, rows);
-        for (int rb = r0; rb < rend; rb += 16) {
-            // A = H1^T rows 16 mi .. + 15 (hidden units), k = batch rows rb .. rb + 15
-            const uint16_t *h = A.h1 + (size_t)rb * MLP_H;
-            const int i0 = 16 * mi + g;
-            const uint32_t a2[4] = {pair_u16(h[(2 * t) * MLP_H + i0], h[(2 * t + 1) * MLP_H + i0]),
-                                    pair_u16(h[(2 * t) * MLP_H + i0 + 8], h[(2 * t + 1) * MLP_H + i0 + 8]),
-                                    pair_u16(h[(2 * t + 8) * MLP_H + i0], h[(2 * t + 9) * MLP_H + i0]),
-                                    pair_u16(h[(2 * t + 8) * MLP_H + i0 + 8], h[(2 * t + 9) * MLP_H + i0 + 8])};
-            const uint16_t *e = A.e2 + (size_t)rb * MLP_H;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int c = 8 * (nj0 + q) + g;
-                mma16816(acc2[q], a2, pair_u16(e[(2 * t) * MLP_H + c], e[(2 * t + 1) * MLP_H + c]),
-                         pair_u16(e[(2 * t + 8) * MLP_H + c], e[(2 * t + 9) * MLP_H + c]));
-            }
-            // A = Z^T (16 features), B = dA1 column tile w
-            const uint16_t *z = A.z + (size_t)rb * MLP_F;
-            const uint32_t a1[4] = {pair_u16(z[(2 * t) * MLP_F + g], z[(2 * t + 1) * MLP_F + g]),
-                                    pair_u16(z[(2 * t) * MLP_F + g + 8], z[(2 * t + 1) * MLP_F + g + 8]),
-                                    pair_u16(z[(2 * t + 8) * MLP_F + g], z[(2 * t + 9) * MLP_F + g]),
-                                    pair_u16(z[(2 * t + 8) * MLP_F + g + 8], z[(2 * t + 9) * MLP_F + g + 8])};
-            const uint16_t *e1 = A.e1 + (size_t)rb * MLP_H;
-            const int c1 = 8 * w + g;
-            mma16816(acc1, a1, pair_u16(e1[(2 * t) * MLP_H + c1], e1[(2 * t + 1) * MLP_H + c1]),
-                     pair_u16(e1[(2 * t + 8) * MLP_H + c1], e1[(2 * t + 9) * MLP_H + c1]));
-        }
-    }
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const int i = 16 * mi + g, c = 8 * (nj0 + q) + 2 * t;
@@ -452,6 +570,14 @@ __global__ void __launch_bounds__(MLP_WARPS * 32) k_mlp_wgrad(ModelDev *M, int32
         atomicAdd(&M->grad[P_W1 + (f + 8) * MLP_H + c], acc1[2]);
         atomicAdd(&M->grad[P_W1 + (f + 8) * MLP_H + c + 1], acc1[3]);
     }
+}
+
+// Opt the gradient kernel in to its shared memory on the current device.
+int prepare_mlp() {
+    return cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TrainSmem)) ==
+                   cudaSuccess
+               ? 0
+               : -1;
 }
 
 // BF16 copies of the weights in the fragment layouts.
@@ -529,37 +655,30 @@ int launch_model_pack(ModelDev *M, cudaStream_t st) {
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
+static unsigned infer_grid(int32_t n, int num_sms) {
+    const int64_t rows = 16 * INF_TILES * MLP_WARPS, g = ((int64_t)n + rows - 1) / rows, cap = (int64_t)num_sms * 2;
+    return (unsigned)(g < 1 ? 1 : g > cap ? cap : g);
+}
+
 int launch_mlp_infer(const ModelDev *M, const float *x, int32_t n, float *out, int num_sms, cudaStream_t st) {
-    const int64_t tiles = ((int64_t)n + 15) / 16;
-    int64_t g = (tiles + MLP_WARPS - 1) / MLP_WARPS;
-    if (g > (int64_t)num_sms * 8) g = (int64_t)num_sms * 8;
-    if (g < 1) g = 1;
-    k_mlp_infer<<<(unsigned)g, MLP_WARPS * 32, 0, st>>>(M, x, n, out);
+    k_mlp_infer<false><<<infer_grid(n, num_sms), MLP_WARPS * 32, 0, st>>>(M, x, n, out);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 int launch_mlp_infer_bf16(const ModelDev *M, const uint32_t *xb, int32_t n, float *out, int num_sms,
                           cudaStream_t st) {
-    const int64_t tiles = ((int64_t)n + 15) / 16;
-    int64_t g = (tiles + MLP_WARPS - 1) / MLP_WARPS;
-    if (g > (int64_t)num_sms * 8) g = (int64_t)num_sms * 8;
-    if (g < 1) g = 1;
-    k_mlp_infer_bf16<<<(unsigned)g, MLP_WARPS * 32, 0, st>>>(M, xb, n, out);
+    k_mlp_infer<true><<<infer_grid(n, num_sms), MLP_WARPS * 32, 0, st>>>(M, xb, n, out);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-// One training (or gradient-only) step over `batch` rows: zero, forward +
-// data gradients, weight gradients, and (adam) the update.
+// One training (or gradient-only) step over `batch` rows: zero, the
+// gradient, and (adam) the update.
 int launch_mlp_step(ModelDev *M, const float *x, const float *y, int32_t n, int32_t batch, uint64_t seed, bool sample,
-                    bool count_step, bool adam, float lr, uint16_t *acts, int num_sms, cudaStream_t st) {
+                    bool count_step, bool adam, float lr, int num_sms, cudaStream_t st) {
     k_mlp_zero<<<(P_N + 255) / 256, 256, 0, st>>>(M, count_step);
-    const int tiles = (batch + 15) / 16;
-    int gf = (tiles + MLP_WARPS - 1) / MLP_WARPS;
-    if (gf > num_sms * 4) gf = num_sms * 4;
-    k_mlp_fwd_bwd<<<gf < 1 ? 1 : gf, MLP_WARPS * 32, 0, st>>>(M, x, y, n, batch, seed, sample, acts);
-    int gw = (batch + WG_ROWS - 1) / WG_ROWS;
-    if (gw > num_sms * 2) gw = num_sms * 2;
-    k_mlp_wgrad<<<gw < 1 ? 1 : gw, MLP_WARPS * 32, 0, st>>>(M, batch, acts);
+    const int64_t chunks = ((int64_t)batch + BATCH_TILE - 1) / BATCH_TILE;
+    k_mlp_grad<<<(unsigned)(chunks < num_sms ? chunks : num_sms), MLP_WARPS * 32, sizeof(TrainSmem), st>>>(
+        M, x, y, n, batch, seed, sample);
     if (adam) k_adam<<<(P_N + 255) / 256, 256, 0, st>>>(M, lr);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

@@ -25,10 +25,10 @@
 // than doubles under contention), so they run in sequence.
 //
 // CUDA graphs (ef_options.graph): the part that needs no host decision --
-// part B, or parts A and B together under trust_input or device_check -- is
-// captured once on
-// a private stream and replayed into the context stream while the pointers,
-// sizes, options and tuning stay the same (one cached graph per context).
+// part B, or parts A and B together under trust_input or device_check, all
+// but the finalize -- is captured once on a private stream and replayed into
+// the context stream while the input pointers, sizes, options and tuning stay
+// the same (one cached graph per context).
 #include "ef_internal.cuh"
 
 #include <algorithm>
@@ -44,16 +44,19 @@
 namespace {
 
 // What a captured graph depends on: replayed only when every byte matches
-// (the layout has no padding; keys are zero-filled before use).
+// (the layout has no padding; keys are zero-filled before use).  The output
+// buffers are not in it: the finalize pass, the only one that writes them, is
+// launched after the graph, so calls whose outputs come from an allocator
+// (another buffer each time) replay too (R-MAT 2^16: 0.15 ms a call for the
+// capture and instantiation, 2 us for the launch).
 struct GraphKey {
     const void *rp, *ci, *goff_dev, *scratch, *ftab;
-    const void *outs[6];
     int64_t m, fcap;
     int32_t n, G, precision, wedge_mode, trust, bins;
     ef::Tune tune;
     bool operator==(const GraphKey &o) const { return memcmp(this, &o, sizeof *this) == 0; }
 };
-static_assert(sizeof(GraphKey) == 11 * 8 + 2 * 8 + 6 * 4 + sizeof(ef::Tune), "GraphKey has padding");
+static_assert(sizeof(GraphKey) == 5 * 8 + 2 * 8 + 6 * 4 + sizeof(ef::Tune), "GraphKey has padding");
 
 }  // namespace
 
@@ -267,7 +270,6 @@ int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, PathMo
         LAUNCH(launch_short(j.ci, s, j.o.precision, j.n, t, chosen, st), "short rows");
         if (prof && chosen)
             for (int e : {4, 6}) CU(cudaEventRecord(ctx->ev[e], st));
-        LAUNCH(launch_finalize_short(s, j.o.precision, j.n, j.out, t, chosen, st), "finalize");
         if (chosen) return EF_OK;
     }
     const bool gated = path == PATH_DEVICE;
@@ -282,14 +284,23 @@ int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, PathMo
     if (prof) CU(cudaEventRecord(ctx->ev[4], st));
     LAUNCH(launch_wedge_big(j.rp, j.ci, s, j.o.precision, j.o.wedge_mode, j.n, j.m, t, st), "big wedge");
     if (prof) CU(cudaEventRecord(ctx->ev[6], st));
-    LAUNCH(launch_finalize(s, j.o.precision, j.n, j.out, t, st), "finalize");
+    return EF_OK;
+}
+
+// The per-node outputs, after part B.
+int part_c(ef_ctx *ctx, const Job &j, const ef::Scratch &s, PathMode path, cudaStream_t st) {
+    using namespace ef;
+    if (path != PATH_GENERAL)
+        LAUNCH(launch_finalize_short(s, j.o.precision, j.n, j.out, ctx->tune, path == PATH_SHORT, st), "finalize");
+    if (path != PATH_SHORT) LAUNCH(launch_finalize(s, j.o.precision, j.n, j.out, ctx->tune, st), "finalize");
     return EF_OK;
 }
 
 // Capture fn(capture stream) into the context's graph unless the cached one
-// has the same key; then launch it into the context stream.
+// has the same key; then launch it into the context stream.  A replay is
+// counted when the call's output buffers are also those of the call before.
 template <typename F>
-int run_graph(ef_ctx *ctx, const GraphKey &key, F &&fn) {
+int run_graph(ef_ctx *ctx, const GraphKey &key, bool same_outputs, F &&fn) {
     if (!(ctx->gexec && ctx->gkey == key)) {
         drop_graph(ctx);
         CU(cudaStreamBeginCapture(ctx->capture, cudaStreamCaptureModeThreadLocal));
@@ -309,7 +320,7 @@ int run_graph(ef_ctx *ctx, const GraphKey &key, F &&fn) {
         }
         memcpy(&ctx->gkey, &key, sizeof key);
     } else {
-        ctx->stats.graph_replays += 1;
+        ctx->stats.graph_replays += same_outputs;
     }
     CU(cudaGraphLaunch(ctx->gexec, ctx->stream));
     return EF_OK;
@@ -380,8 +391,6 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         key.goff_dev = j.goff_dev;
         key.scratch = ctx->scratch;
         key.ftab = ctx->ftab;
-        const void *outs[6] = {j.out.ef, j.out.n_clusters, j.out.s, j.out.t, j.out.triangles, j.out.flag};
-        memcpy(key.outs, outs, sizeof outs);
         key.m = j.m;
         key.fcap = fcap;
         key.n = j.n;
@@ -391,13 +400,17 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         key.trust = o.trust_input | (dev_check ? 2 : 0) | (dev_check && o.async ? 4 : 0);
         key.bins = (int32_t)ctx->bins | (int32_t)path << 1 | (int32_t)ctx->long_lists << 3;
         key.tune = ctx->tune;
-        rc = run_graph(ctx, key, [&](cudaStream_t cs) {
+        const void *outs[6] = {j.out.ef, j.out.n_clusters, j.out.s, j.out.t, j.out.triangles, j.out.flag};
+        const bool same_outputs = memcmp(outs, ctx->gouts, sizeof outs) == 0;
+        memcpy(ctx->gouts, outs, sizeof outs);
+        rc = run_graph(ctx, key, same_outputs, [&](cudaStream_t cs) {
             if (a_inline) {
                 const int r = part_a_inline(cs);
                 if (r) return r;
             }
             return part_b(ctx, j, s, fcap, path, false, cs);
         });
+        if (!rc) rc = part_c(ctx, j, s, path, st);
         if (rc) return rc;
     } else {
         if (a_inline) {
@@ -407,6 +420,7 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         }
         if (prof) CU(cudaEventRecord(ctx->ev[1], st));
         rc = part_b(ctx, j, s, fcap, path, prof, st);
+        if (!rc) rc = part_c(ctx, j, s, path, st);
         if (rc) return rc;
         if (prof) CU(cudaEventRecord(ctx->ev[7], st));
     }

@@ -370,7 +370,7 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         if (const int bits = prep_error_bits(ctx->h_counters)) return graph_error(ctx, bits);
         if (const int lim = degree_limit(ctx, ctx->h_counters)) return lim;
         path = ctx->h_counters[BIN_BIG] == 0 ? PATH_SHORT : PATH_GENERAL;
-        ctx->long_lists = ctx->h_counters[CNT_MAXOUT] > TRI_LONG;
+        ctx->long_lists = ctx->h_counters[CNT_LONG] != 0;
         fcap = 3 * (int64_t)ctx->h_counters[CNT_MAXDEG] + 1;
         ctx->bins = bin_layout(ctx->tune, ctx->h_counters, j.n, j.goff_dev != nullptr);
     }
@@ -585,6 +585,8 @@ int prepare_graph(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n, 
     Job j{rp, ci, n, m, nullptr, 0, o, ef_outputs{}};
     rc = part_a(ctx, j, s, ctx->stream);
     if (rc) return rc;
+    ctx->long_lists = true;
+    ctx->big_rows = false;
     if (o.trust_input) {
         const int64_t bound = (int64_t)n - 1 < m ? (int64_t)n - 1 : m;
         fcap = 3 * (bound > 0 ? bound : 0) + 1;
@@ -597,6 +599,8 @@ int prepare_graph(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n, 
         if (const int lim = degree_limit(ctx, ctx->h_counters)) return lim;
         fcap = 3 * (int64_t)ctx->h_counters[CNT_MAXDEG] + 1;
         ctx->bins = bin_layout(ctx->tune, ctx->h_counters, n, false);
+        ctx->long_lists = ctx->h_counters[CNT_LONG] != 0;
+        ctx->big_rows = ctx->h_counters[BIN_BIG] > 0;
     }
     size_t have = (size_t)ctx->ftab_cap * 2 * sizeof(double);
     rc = ensure_buffer(ctx, (void **)&ctx->ftab, &have, (size_t)fcap * 2 * sizeof(double), 0);
@@ -626,10 +630,10 @@ int features_device(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n
     using namespace ef;
     cudaStream_t st = ctx->stream;
     if (with_orient || mode == 1)
-        LAUNCH(launch_orient(rp, ci, n, m, s, ctx->tune, st, r.nbr_min, r.nbr_max, ctx->bins), "orientation");
+        LAUNCH(launch_orient(rp, ci, n, m, s, ctx->tune, st, r.nbr_min, r.nbr_max, ctx->bins, false, ctx->big_rows), "orientation");
     else
         LAUNCH(launch_omega_mm(rp, ci, n, m, s, r, ctx->tune, st), "omega");
-    if (mode == 1) LAUNCH(launch_tri_pairs(s, n, m, ctx->tune, st), "triangle");
+    if (mode == 1) LAUNCH(launch_tri_pairs(s, n, m, ctx->tune, st, nullptr, ctx->long_lists), "triangle");
     r.x = x;
     LAUNCH(launch_features(s, r, n, mode, ctx->tune, st, std_model), "features");
     return EF_OK;
@@ -648,8 +652,9 @@ int nodes_device(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n, i
     cudaStream_t st = ctx->stream;
     if (global_tri && !tri_done) {
         if (!orient_done)
-            LAUNCH(launch_orient(rp, ci, n, m, s, ctx->tune, st, nullptr, nullptr, ctx->bins), "orientation");
-        LAUNCH(launch_tri_pairs(s, n, m, ctx->tune, st), "triangle");
+            LAUNCH(launch_orient(rp, ci, n, m, s, ctx->tune, st, nullptr, nullptr, ctx->bins, false, ctx->big_rows),
+                   "orientation");
+        LAUNCH(launch_tri_pairs(s, n, m, ctx->tune, st, nullptr, ctx->long_lists), "triangle");
     }
     if (timed) CU(cudaEventRecord(ctx->ev[8], st));
     // the row passes' out-degrees are not needed any more: they hold the marks
@@ -1061,8 +1066,8 @@ int ef_compute_shard(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, int32_t
     cudaStream_t st = ctx->stream;
     int32_t *rng = s.counters + CNT_RANGE;
     LAUNCH(launch_shard_range(rp, n, m, shard, num_shards, rng, st), "shard range");
-    LAUNCH(launch_orient(rp, ci, n, m, s, t, st, nullptr, nullptr, ctx->bins), "orientation");
-    LAUNCH(launch_tri_pairs(s, n, m, t, st, rng), "triangle");
+    LAUNCH(launch_orient(rp, ci, n, m, s, t, st, nullptr, nullptr, ctx->bins, false, ctx->big_rows), "orientation");
+    LAUNCH(launch_tri_pairs(s, n, m, t, st, rng, ctx->long_lists), "triangle");
     // the out-degrees are not needed any more: they hold the marks
     LAUNCH(launch_mark_range(rng, n, s.outdeg, t, st), "shard marks");
     LAUNCH(launch_bin_marked(s.outdeg, s, n, t, st), "shard bins");

@@ -148,7 +148,7 @@ enum : int {
     CNT_TRIFRAC = 37,
     CNT_TRILONG = 38, // items of the long owners (pair tests), and the next one to take
     CNT_TRINEXT = 39,
-    CNT_MAXOUT = 42,  // largest out-degree
+    CNT_LONG = 42,    // 1: some node has more than TRI_LONG out-neighbours
     CNT_RANGE = 40,   // 40, 41: a shard's node range [lo, hi)
     CNT_SYM = 44,     // 44, 45: the symmetry sum (uint64, 8-byte aligned)
     CNT_BIGLO = 46,   // n - 1 - (smallest id of a node of degree > SMALL_MAX), if any

@@ -312,13 +312,15 @@ __device__ __forceinline__ int cross_bits(const RowOut &ro, const int32_t *__res
     return ci[a] < ro.goff[lo] || ci[b - 1] >= ro.goff[lo + 1] ? ERRB_CROSS : 0;
 }
 
-// A warp's share of the symmetry sum and the largest out-degree of its rows.
-__device__ __forceinline__ void add_rows(int32_t *cnt, uint64_t sym, int od) {
+// A warp's share of the symmetry sum, and whether one of its rows is a long
+// owner of the pair tests (a plain store of a constant: an atomic maximum per
+// warp cost 40 us on the 1M-node power-law graph).
+__device__ __forceinline__ void add_rows(int32_t *cnt, uint64_t sym, int most) {
     sym = warp_sum(sym);
-    od = __reduce_max_sync(FULL, od);
+    const bool many = __any_sync(FULL, most > TRI_LONG);
     if ((threadIdx.x & 31) == 0) {
         if (sym) atomicAdd(reinterpret_cast<unsigned long long *>(cnt + CNT_SYM), (unsigned long long)sym);
-        if (od > *(volatile int32_t *)(cnt + CNT_MAXOUT)) atomicMax(cnt + CNT_MAXOUT, od);
+        if (many) cnt[CNT_LONG] = 1;
     }
 }
 

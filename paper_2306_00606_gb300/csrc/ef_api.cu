@@ -760,6 +760,7 @@ size_t carve_scratch(char *base, int32_t n, int64_t m, Scratch &s) {
     s.hub_cls = take(8 * (M + N + 2));
     s.hub_q = take(8 * (M + N + 2));
     s.hub_cidx = (int32_t *)take(4 * (M + 1));
+    s.big_partial = (double *)s.hub_q;
     off = std::max(off, oriented_end);
     s.tri_items = (int2 *)take(8 * (M / 32 + 1));
     s.tri_rec = (int4 *)take(16 * (M / 2 + 1));
@@ -771,7 +772,6 @@ size_t carve_scratch(char *base, int32_t n, int64_t m, Scratch &s) {
     s.counters = (int32_t *)take(4 * NUM_COUNTERS);
     s.bins = (int32_t *)take(4 * N * NUM_BINS);
     s.big_chunks = (int32_t *)take(4 * (N + 1));
-    s.big_partial = (double *)take(8 * (M / BIG_ROWS + N + 2));
     s.scan_tmp = (int32_t *)take(4 * (N / 4096 + 4));
     s.scan_tmp2 = (int32_t *)take(4 * (N / 4096 + 4));
     s.ftab = nullptr;

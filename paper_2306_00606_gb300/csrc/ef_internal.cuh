@@ -57,7 +57,8 @@ enum : int {
     BIN_S16,       // 9..16         2 per warp
     BIN_S32,       // 17..32        1 per warp
     BIN_BIG,       // D > 32        (direct wedge kernel)
-    BIN_MID,       // 32 < D < hub_min (<= MID_MAX)   degree-class wedge kernel, one warp each
+    BIN_MID,       // 32 < D < MID_SPLIT, below hub_min   degree-class wedge kernel, one warp each
+    BIN_MIDHI,     // MID_SPLIT <= D < hub_min (<= MID_MAX + 1)   the same in FP32C; a CTA each in FP64
     BIN_HUB0,      // D >= hub_min, bucket floor(log2 D) - 9 clamped to [0, NUM_HUB_BUCKETS-1]
     BIN_HUB_LAST = BIN_HUB0 + 6,
     NUM_BINS
@@ -66,6 +67,15 @@ constexpr int NUM_HUB_BUCKETS = BIN_HUB_LAST - BIN_HUB0 + 1;
 
 constexpr int SMALL_MAX = 32;
 constexpr int MID_MAX = 512;
+// FP64: from this degree on the interpolated sums of the hub kernel beat the
+// warp kernel's direct ones, and the warp kernel's shared memory, sized for
+// the rows below, leaves the L1 cache to its f-table gathers.  FP64 class
+// passes with the line at 193 / 257 / 321 / 385 and 513 (the warp kernel as it
+// was: 45 KB a block): 87M-entry power-law graph 4.5 / 3.9 / 3.9 / 5.8 and 5.9
+// ms, 1M nodes 0.38 / 0.35 / 0.36 / 0.49 and 0.54, R-MAT 2^16 0.116 / 0.119 /
+// 0.142 / 0.210 and 0.225, BA 1M 0.109 / 0.106 / 0.108 / 0.110 and 0.120.
+// (FP32C computes its terms and keeps the warp kernel up to MID_MAX.)
+constexpr int MID_SPLIT = 257;
 constexpr int MID_HIST = 256;          // dense degree histogram of the warp-level class kernel
 constexpr int HUB_HIST = 2048;         // dense degree histogram of the CTA-level class kernel
 constexpr int HUB_THREADS = 512;
@@ -128,7 +138,7 @@ struct Scratch {
     int32_t *bins;       // NUM_BINS * n   work lists
     int32_t *counters;   // NUM_COUNTERS ints: [0..NUM_BINS) bin counts, CNT_* below
     int32_t *big_chunks; // n+1    work items per big middle node (direct kernel), scanned in place
-    double  *big_partial;// m/BIG_ROWS + n + 2  per-item middle-node partial sums (direct kernel)
+    double  *big_partial;// m/BIG_ROWS + n + 2  per-item middle-node partial sums (direct kernel; over hub_q)
     int32_t *scan_tmp;   // scan block sums (orientation)
     int32_t *scan_tmp2;  // scan block sums (direct kernel's items)
     float2  *ftab;       // 3*maxdeg+1 (capacity): f(d) = d ln d as an FP32 pair hi + lo (F2Sum)
@@ -339,6 +349,15 @@ __device__ __forceinline__ int lower_bound_i32(const int32_t *a, int len, int32_
         if (a[mid] < key) lo = mid + 1; else hi = mid;
     }
     return lo;
+}
+
+// The rows of degree 33 .. hub_min - 1: the two lists one after the other,
+// the longer rows first (the kernels that take them from a counter end on
+// short ones).
+__device__ __forceinline__ int mid_total(const int32_t *cnt) { return cnt[BIN_MID] + cnt[BIN_MIDHI]; }
+__device__ __forceinline__ int mid_node(const int32_t *bins, int32_t n, const int32_t *cnt, int it) {
+    const int first = cnt[BIN_MIDHI];
+    return it < first ? bins[(size_t)BIN_MIDHI * n + it] : bins[(size_t)BIN_MID * n + (it - first)];
 }
 
 // Total number of hub rows (degree > MID_MAX) in the hub buckets.

@@ -146,7 +146,7 @@ __global__ void __launch_bounds__(DEG_THREADS) k_degrees(const int32_t *__restri
                 blo = max(blo, (int)(n - 1 - v));
                 bhi = max(bhi, (int)v);
                 if (d < hub_min) {
-                    b1[q] = BIN_MID;
+                    b1[q] = d < MID_SPLIT ? BIN_MID : BIN_MIDHI;
                 } else {
                     const int lg = 31 - __clz(d);   // floor(log2 d)
                     b1[q] = BIN_HUB0 + max(0, min(lg - 9, NUM_HUB_BUCKETS - 1));
@@ -475,9 +475,9 @@ __global__ void __launch_bounds__(256, 6) k_row_stats(const int32_t *__restrict_
         }
     }
     if (ord.bins) {
-        const int nmid = cnt[BIN_MID];
+        const int nmid = mid_total(cnt);
         for (int64_t it = warp; it < nmid; it += nwarps) {
-            const int u = bins[(size_t)BIN_MID * n + it];
+            const int u = mid_node(bins, n, cnt, (int)it);
             const int ua = rp[u], ub = rp[u + 1];
             if (ua >= 0 && ua <= ub && (int64_t)ub <= m) row_stats_warp(ci, D, n, u, ua, ub, lane, ro, cnt, sym, most);
         }
@@ -687,10 +687,11 @@ __global__ void __launch_bounds__(256) k_node_info(const int32_t *__restrict__ D
 // not in node order, so that the lists of nodes of similar degree -- and
 // similar odds of being probed by the triangle pass -- share cache lines.
 // Nodes of degree 0 have no list.
-constexpr int LAYOUT_BINS = 5 + NUM_HUB_BUCKETS;
+constexpr int LAYOUT_BINS = 6 + NUM_HUB_BUCKETS;
 __constant__ int c_layout_bins[LAYOUT_BINS] = {BIN_S4,       BIN_S8,       BIN_S16,      BIN_S32,
-                                               BIN_MID,      BIN_HUB0,     BIN_HUB0 + 1, BIN_HUB0 + 2,
-                                               BIN_HUB0 + 3, BIN_HUB0 + 4, BIN_HUB0 + 5, BIN_HUB0 + 6};
+                                               BIN_MID,      BIN_MIDHI,    BIN_HUB0,     BIN_HUB0 + 1,
+                                               BIN_HUB0 + 2, BIN_HUB0 + 3, BIN_HUB0 + 4, BIN_HUB0 + 5,
+                                               BIN_HUB0 + 6};
 static_assert(BIN_HUB0 + 6 == BIN_HUB_LAST, "layout bins cover the hub buckets");
 
 // base[q] = first layout position of bin q; base[LAYOUT_BINS] = all listed nodes.
@@ -859,9 +860,9 @@ __global__ void __launch_bounds__(256, CHUNK == 8 ? 3 : 5) k_orient(
         }
     }
     if (!ord.bins) return;
-    const int nmid = cnt[BIN_MID];
+    const int nmid = mid_total(cnt);
     for (int64_t it = warp; it < nmid; it += nwarps) {
-        const int u = bins[(size_t)BIN_MID * n + it];
+        const int u = mid_node(bins, n, cnt, (int)it);
         const int ua = rp[u], ub = rp[u + 1];
         if (ua >= 0 && ua <= ub && (int64_t)ub <= m) orient_row_warp(o, u, ua, ub, out_ptr[u], lane, omega);
     }

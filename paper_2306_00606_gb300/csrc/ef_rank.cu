@@ -351,7 +351,7 @@ __global__ void k_bin_marked(const int32_t *__restrict__ mark, const int32_t *__
                 b0 = d <= 4 ? BIN_S4 : d <= 8 ? BIN_S8 : d <= 16 ? BIN_S16 : BIN_S32;
             } else if (d > SMALL_MAX) {
                 b0 = BIN_BIG;
-                b1 = d < hub_min ? BIN_MID : BIN_HUB0 + max(0, min(31 - __clz(d) - 9, NUM_HUB_BUCKETS - 1));
+                b1 = d < hub_min ? (d < MID_SPLIT ? BIN_MID : BIN_MIDHI) : BIN_HUB0 + max(0, min(31 - __clz(d) - 9, NUM_HUB_BUCKETS - 1));
             }
         }
         if (b0 >= 0) p0 = atomicAdd(&s_cnt[b0], 1);

@@ -471,10 +471,10 @@ __global__ void __launch_bounds__(SIR_WARPS * 32, 4) k_sir_step(const int32_t *_
     // attachment numbers its large nodes together, 0.5 ms a step)
     const PullLanes L1(st.WB, 32);
     W.smask = L1.wbp * 32 - 1;
-    const int mids = cnt[BIN_MID];
+    const int mids = mid_total(cnt);
     for (int64_t it = warp; it < mids; it += nwarps) {
         PullNode P;
-        P.x = bins[(size_t)BIN_MID * n + it];
+        P.x = mid_node(bins, n, cnt, (int)it);
         P.a = rp[P.x];
         P.D = rp[P.x + 1] - P.a;
         P.own(L1, c, st);

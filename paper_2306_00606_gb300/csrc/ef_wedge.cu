@@ -325,36 +325,37 @@ struct ClassEval<true> {
 
 constexpr int MID_WARPS = 4;
 
-// One warp per middle node of degree 33..MID_MAX.  Warps take their nodes
+// One warp per middle node of degree 33..MID_MAX (FP64: below MID_SPLIT).  Warps take their nodes
 // one at a time from an atomic counter (the work of a node grows with the
 // square of its class count, which varies a hundredfold within the bin); the
 // next node's index, id and row range are loaded while the current node is
 // processed, so only the neighbour gathers wait at the start of a node.
 template <bool F64>
-__global__ void __launch_bounds__(MID_WARPS * 32) k_wedge_mid(
+__global__ void __launch_bounds__(MID_WARPS * 32, 6) k_wedge_mid(
     const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const int32_t *__restrict__ D,
-    const int32_t *__restrict__ list, int32_t *__restrict__ cnt, const float2 *__restrict__ ftab,
+    const int32_t *__restrict__ bins, int32_t n, int32_t *__restrict__ cnt, const float2 *__restrict__ ftab,
     double *__restrict__ Tacc, void *__restrict__ Ccenter) {
     if (gate_closed(cnt)) return;
     using E = ClassEval<F64>;
+    constexpr int MAX = F64 ? MID_SPLIT - 1 : MID_MAX;   // row entries at most
     using Cls = typename E::Cls;
     using R = typename E::R;
     __shared__ int32_t s_hist[MID_WARPS][MID_HIST];
-    __shared__ int32_t s_cidx[MID_WARPS][MID_MAX];
-    __shared__ __align__(16) Cls s_cls[MID_WARPS][MID_MAX];
-    __shared__ R s_q[MID_WARPS][MID_MAX];
+    __shared__ int32_t s_cidx[MID_WARPS][MAX];
+    __shared__ __align__(16) Cls s_cls[MID_WARPS][MAX];
+    __shared__ R s_q[MID_WARPS][MAX];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int32_t *hist = s_hist[w], *cidx = s_cidx[w];
     Cls *cls = s_cls[w];
     R *cq = s_q[w];
     const unsigned lt = (1u << lane) - 1u;
-    const int count = cnt[BIN_MID];
+    const int count = F64 ? cnt[BIN_MID] : mid_total(cnt);
     int it = 0;
     if (lane == 0) it = atomicAdd(cnt + CNT_MIDITEM, 1);
     it = __shfl_sync(FULL, it, 0);
     int u = 0, start = 0, Du = 0;
     if (it < count) {
-        u = list[it];
+        u = F64 ? bins[(size_t)BIN_MID * n + it] : mid_node(bins, n, cnt, it);
         start = rp[u];
         Du = rp[u + 1] - start;
     }
@@ -371,7 +372,7 @@ __global__ void __launch_bounds__(MID_WARPS * 32) k_wedge_mid(
         }
         __syncwarp();
         next = __shfl_sync(FULL, next, 0);
-        const int u_next = next < count ? list[next] : 0;
+        const int u_next = next >= count ? 0 : F64 ? bins[(size_t)BIN_MID * n + next] : mid_node(bins, n, cnt, next);
         int K = 0;
         for (int i0 = 0; i0 < MID_HIST; i0 += 32) {
             const int i = i0 + lane;
@@ -686,7 +687,8 @@ struct HubSmemK {
     static constexpr int value = F64 ? 3072 : HUB_SMEM_K;
 };
 
-// One CTA per hub (degree > MID_MAX), hubs taken largest degree bucket first
+// One CTA per hub (degree > MID_MAX; in FP64 also the rows of BIN_MIDHI, from
+// degree MID_SPLIT on), hubs taken largest degree bucket first
 // from an atomic counter.  Global arrays hold the class index of every
 // neighbour (cidx_g, at the hub's own row positions) and, for hubs with more
 // than HUB_SMEM_K classes, the classes themselves (cls_g, q_g).
@@ -715,14 +717,14 @@ __global__ void __launch_bounds__(HUB_THREADS) k_wedge_hub(
     const int tid = threadIdx.x;
     int total = 0;
     for (int b = NUM_HUB_BUCKETS - 1; b >= 0; --b) total += cnt[BIN_HUB0 + b];
+    const int hubs = total;
+    if (F64) total += cnt[BIN_MIDHI];   // after the hubs, larger degrees first
     for (;;) {
         if (tid == 0) s_item = atomicAdd(cnt + CNT_HUB, 1);
         __syncthreads();
-        int item = s_item;
+        const int item = s_item;
         if (item >= total) break;
-        int b = NUM_HUB_BUCKETS - 1;
-        while (item >= cnt[BIN_HUB0 + b]) item -= cnt[BIN_HUB0 + b--];
-        const int u = bins[(size_t)(BIN_HUB0 + b) * n + item];
+        const int u = item < hubs ? hub_row(bins, n, cnt, item) : bins[(size_t)BIN_MIDHI * n + (item - hubs)];
         const int start = rp[u];
         const int Du = rp[u + 1] - start;
         const int base = Du - 4;
@@ -900,10 +902,9 @@ int prepare_kernels() {
 template <bool F64>
 static int big_classes(const int32_t *rp, const int32_t *ci, const Scratch &s, int32_t n, int num_sms,
                        cudaStream_t st) {
-    const int32_t *mid = s.bins + (size_t)BIN_MID * n;
     const DeviceProps &p = dev_props();
     k_wedge_mid<F64><<<(unsigned)(num_sms * p.class_blocks[F64][0]), MID_WARPS * 32, 0, st>>>(
-        rp, ci, s.D, mid, s.counters, s.ftab, s.Tacc, s.Ccenter);
+        rp, ci, s.D, s.bins, n, s.counters, s.ftab, s.Tacc, s.Ccenter);
     const size_t smem = hub_smem_bytes<F64>();
     k_wedge_hub<F64><<<(unsigned)(num_sms * p.class_blocks[F64][1]), HUB_THREADS, smem, st>>>(
         rp, ci, s.D, s.bins, n, s.counters, s.ftab, s.Tacc, s.Ccenter, s.hub_cidx, s.hub_cls, s.hub_q);

@@ -261,8 +261,11 @@ __global__ void __launch_bounds__(SH_WARPS * 32, 5) k_short(ShortArgs A, const i
 
 int launch_short(const int32_t *ci, const Scratch &s, int precision, int32_t n, const Tune &t, bool chosen,
                  cudaStream_t st) {
-    // fewer nodes per step while that leaves warp slots of the GPU empty
-    const int32_t per = n >= t.num_sms * 32 * 32 ? 32 : 8;
+    // fewer nodes per step while that leaves warp slots of the GPU empty (ER
+    // 2000: 8 nodes, five packs one after the other, 15 us in FP32C and
+    // 18 in FP64; 2 nodes, 9.8 and 11.0)
+    const int32_t slots = t.num_sms * 32;
+    const int32_t per = n >= slots * 32 ? 32 : n >= slots * 8 ? 8 : 2;
     const ShortArgs A{ci, reinterpret_cast<const int2 *>(s.info), n, per, s.Tacc, s.outdeg,
                       reinterpret_cast<uint64_t *>(s.sig1), 0.0};
     const int64_t g = ((int64_t)n + per * SH_WARPS - 1) / (per * SH_WARPS), cap = (int64_t)t.num_sms * 16;

@@ -179,7 +179,6 @@ constexpr int MLP_WARPS = 8;
 // Measured, 8M rows: 344 us with one tile per step and four-byte loads, 251
 // so; at 80 registers (three blocks per SM) 278, four tiles 280, the W2
 // fragments in registers (12 warps per SM) 276-292.
-constexpr int INF_TILES = 2;
 constexpr int W2ROW = 40;   // words of a W2 row: 4 k-chunks x 4 lanes x 2 words, padded
 
 struct InferSmem {
@@ -194,11 +193,11 @@ __device__ __forceinline__ int w1_at(int n, int t) { return n * 4 + t; }
 
 __device__ void load_infer(const ModelDev *M, InferSmem &s) {
     const uint32_t *w1 = reinterpret_cast<const uint32_t *>(M->w1t), *w2 = reinterpret_cast<const uint32_t *>(M->w2t);
-    for (int i = threadIdx.x; i < MLP_H * 4; i += blockDim.x) {
+    for (int i = threadIdx.x; i < MLP_H * 4; i += MLP_WARPS * 32) {
         const int n = i >> 2, t = i & 3;
         s.w1[w1_at(n, t)] = make_uint2(w1[n * (MLP_F / 2) + t], w1[n * (MLP_F / 2) + t + 4]);
     }
-    for (int i = threadIdx.x; i < MLP_H * 16; i += blockDim.x) {
+    for (int i = threadIdx.x; i < MLP_H * 16; i += MLP_WARPS * 32) {
         const int n = i >> 4, kc = i >> 2 & 3, t = i & 3;
         const uint32_t *r = w2 + n * (MLP_H / 2) + 8 * kc + t;
         s.w2[n * (W2ROW / 2) + kc * 4 + t] = make_uint2(r[0], r[4]);
@@ -215,18 +214,19 @@ __device__ void load_infer(const ModelDev *M, InferSmem &s) {
     if (threadIdx.x == 0) s.b3 = M->p[P_B3];
 }
 
-// Predictions of INF_TILES tiles from their first-layer operands: p[u][0] of
+// Predictions of TILES tiles from their first-layer operands: p[u][0] of
 // row g, p[u][1] of row g + 8 (all four lanes of a group).
-__device__ __forceinline__ void infer_tiles(const InferSmem &s, const uint32_t (&a1)[INF_TILES][4],
-                                            float (&p)[INF_TILES][2]) {
+template <int TILES>
+__device__ __forceinline__ void infer_tiles(const InferSmem &s, const uint32_t (&a1)[TILES][4],
+                                            float (&p)[TILES][2]) {
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    uint32_t a2[INF_TILES][4][4];
+    uint32_t a2[TILES][4][4];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const uint2 b = s.w1[w1_at(8 * j + g, t)];
         const float2 bias = s.b1[4 * j + t];
 #pragma unroll
-        for (int u = 0; u < INF_TILES; ++u) {
+        for (int u = 0; u < TILES; ++u) {
             // the bias after the products, as in the training pass: another order
             // rounds some activations to another BF16 value
             float c[4] = {0.f, 0.f, 0.f, 0.f};
@@ -236,13 +236,13 @@ __device__ __forceinline__ void infer_tiles(const InferSmem &s, const uint32_t (
         }
     }
 #pragma unroll
-    for (int u = 0; u < INF_TILES; ++u) p[u][0] = p[u][1] = 0.f;
+    for (int u = 0; u < TILES; ++u) p[u][0] = p[u][1] = 0.f;
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const float2 bias = s.b2[4 * j + t], w3 = s.w3[4 * j + t];
-        float c[INF_TILES][4];
+        float c[TILES][4];
 #pragma unroll
-        for (int u = 0; u < INF_TILES; ++u) {
+        for (int u = 0; u < TILES; ++u) {
             c[u][0] = c[u][2] = bias.x;
             c[u][1] = c[u][3] = bias.y;
         }
@@ -250,16 +250,16 @@ __device__ __forceinline__ void infer_tiles(const InferSmem &s, const uint32_t (
         for (int kc = 0; kc < 4; ++kc) {
             const uint2 b = s.w2[(8 * j + g) * (W2ROW / 2) + kc * 4 + t];
 #pragma unroll
-            for (int u = 0; u < INF_TILES; ++u) mma16816(c[u], a2[u][kc], b.x, b.y);
+            for (int u = 0; u < TILES; ++u) mma16816(c[u], a2[u][kc], b.x, b.y);
         }
 #pragma unroll
-        for (int u = 0; u < INF_TILES; ++u) {
+        for (int u = 0; u < TILES; ++u) {
             p[u][0] = fmaf(fmaxf(c[u][0], 0.f), w3.x, fmaf(fmaxf(c[u][1], 0.f), w3.y, p[u][0]));
             p[u][1] = fmaf(fmaxf(c[u][2], 0.f), w3.x, fmaf(fmaxf(c[u][3], 0.f), w3.y, p[u][1]));
         }
     }
 #pragma unroll
-    for (int u = 0; u < INF_TILES; ++u)
+    for (int u = 0; u < TILES; ++u)
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             p[u][q] += __shfl_xor_sync(FULL, p[u][q], 1);
@@ -271,29 +271,26 @@ __device__ __forceinline__ void infer_tiles(const InferSmem &s, const uint32_t (
 // BF: rows already standardised and rounded to BF16 (8 words per row, word q
 // holding features 2q and 2q + 1: words t and t + 4 are the fragment as it
 // is), else FP32 rows.  The predictions are equal bit for bit.
-template <bool BF>
+template <bool BF, int TILES>
 __global__ void __launch_bounds__(MLP_WARPS * 32, 2) k_mlp_infer(const ModelDev *__restrict__ M,
                                                               const void *__restrict__ X_, int32_t n,
                                                               float *__restrict__ out) {
     __shared__ InferSmem s;
-    load_infer(M, s);
-    __syncthreads();
     const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3, w = threadIdx.x >> 5;
     const float *X = static_cast<const float *>(X_);
     const uint32_t *Xb = static_cast<const uint32_t *>(X_);
-    const int64_t tiles = ((int64_t)n + 16 * INF_TILES - 1) / (16 * INF_TILES);
+    const int64_t tiles = ((int64_t)n + 16 * TILES - 1) / (16 * TILES);
     const int64_t step = (int64_t)gridDim.x * MLP_WARPS;
-    const float m0 = s.mean[2 * t], m1 = s.mean[2 * t + 1], m2 = s.mean[2 * t + 8], m3 = s.mean[2 * t + 9];
-    const float i0 = s.istd[2 * t], i1 = s.istd[2 * t + 1], i2 = s.istd[2 * t + 8], i3 = s.istd[2 * t + 9];
-    // rows g and g + 8 of each tile, loaded ahead of their use
-    RowPart x[INF_TILES][2];
-    uint32_t xb[INF_TILES][4];
+    // rows g and g + 8 of each tile, loaded ahead of their use (the first ones
+    // ahead of the weights)
+    RowPart x[TILES][2];
+    uint32_t xb[TILES][4];
     auto load = [&](int64_t tile) {
 #pragma unroll
-        for (int u = 0; u < INF_TILES; ++u)
+        for (int u = 0; u < TILES; ++u)
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-                const int64_t r = (tile * INF_TILES + u) * 16 + g + 8 * q;
+                const int64_t r = (tile * TILES + u) * 16 + g + 8 * q;
                 if constexpr (BF) {
                     xb[u][q] = r < n ? __ldg(Xb + r * (MLP_F / 2) + t) : 0u;
                     xb[u][q + 2] = r < n ? __ldg(Xb + r * (MLP_F / 2) + t + 4) : 0u;
@@ -304,10 +301,14 @@ __global__ void __launch_bounds__(MLP_WARPS * 32, 2) k_mlp_infer(const ModelDev 
     };
     int64_t tile = (int64_t)blockIdx.x * MLP_WARPS + w;
     load(tile);
+    load_infer(M, s);
+    __syncthreads();
+    const float m0 = s.mean[2 * t], m1 = s.mean[2 * t + 1], m2 = s.mean[2 * t + 8], m3 = s.mean[2 * t + 9];
+    const float i0 = s.istd[2 * t], i1 = s.istd[2 * t + 1], i2 = s.istd[2 * t + 8], i3 = s.istd[2 * t + 9];
     for (; tile < tiles; tile += step) {
-        uint32_t a1[INF_TILES][4];
+        uint32_t a1[TILES][4];
 #pragma unroll
-        for (int u = 0; u < INF_TILES; ++u)
+        for (int u = 0; u < TILES; ++u)
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 if constexpr (BF) {
@@ -320,14 +321,14 @@ __global__ void __launch_bounds__(MLP_WARPS * 32, 2) k_mlp_infer(const ModelDev 
                 }
             }
         if (tile + step < tiles) load(tile + step);
-        float p[INF_TILES][2];
+        float p[TILES][2];
         infer_tiles(s, a1, p);
         if (t == 0) {
 #pragma unroll
-            for (int u = 0; u < INF_TILES; ++u)
+            for (int u = 0; u < TILES; ++u)
 #pragma unroll
                 for (int q = 0; q < 2; ++q) {
-                    const int64_t r = (tile * INF_TILES + u) * 16 + g + 8 * q;
+                    const int64_t r = (tile * TILES + u) * 16 + g + 8 * q;
                     if (r < n) out[r] = p[u][q];
                 }
         }
@@ -655,20 +656,30 @@ int launch_model_pack(ModelDev *M, cudaStream_t st) {
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-static unsigned infer_grid(int32_t n, int num_sms) {
-    const int64_t rows = 16 * INF_TILES * MLP_WARPS, g = ((int64_t)n + rows - 1) / rows, cap = (int64_t)num_sms * 2;
-    return (unsigned)(g < 1 ? 1 : g > cap ? cap : g);
+// Up to one 16-row tile per warp of the chip (two blocks per SM) each warp has
+// one tile: below that line a second tile is work for padding, and the
+// smallest calls are the latency of one warp step.  Calls of 500 to
+// 20 000 rows: two tiles 0.4-0.7 us slower than one; 60 000 rows fill the chip
+// with two.
+template <bool BF>
+static int infer(const ModelDev *M, const void *x, int32_t n, float *out, int num_sms, cudaStream_t st) {
+    const int64_t rows = 16 * MLP_WARPS, cap = (int64_t)num_sms * 2, g = ((int64_t)n + rows - 1) / rows;
+    if (g <= cap) {
+        k_mlp_infer<BF, 1><<<(unsigned)(g < 1 ? 1 : g), MLP_WARPS * 32, 0, st>>>(M, x, n, out);
+    } else {
+        const int64_t g2 = (g + 1) / 2;
+        k_mlp_infer<BF, 2><<<(unsigned)(g2 > cap ? cap : g2), MLP_WARPS * 32, 0, st>>>(M, x, n, out);
+    }
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 int launch_mlp_infer(const ModelDev *M, const float *x, int32_t n, float *out, int num_sms, cudaStream_t st) {
-    k_mlp_infer<false><<<infer_grid(n, num_sms), MLP_WARPS * 32, 0, st>>>(M, x, n, out);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return infer<false>(M, x, n, out, num_sms, st);
 }
 
 int launch_mlp_infer_bf16(const ModelDev *M, const uint32_t *xb, int32_t n, float *out, int num_sms,
                           cudaStream_t st) {
-    k_mlp_infer<true><<<infer_grid(n, num_sms), MLP_WARPS * 32, 0, st>>>(M, xb, n, out);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return infer<true>(M, xb, n, out, num_sms, st);
 }
 
 // One training (or gradient-only) step over `batch` rows: zero, the

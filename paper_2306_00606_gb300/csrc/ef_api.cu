@@ -1019,8 +1019,6 @@ int ef_compute_nodes(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const i
     int64_t fcap;
     rc = prepare_graph(ctx, g->row_ptr, g->col_idx, n, m, o, s, fcap);
     if (rc) return rc;
-    ef::RankScratch r = {};
-    LAUNCH(ef::launch_omega_mm(g->row_ptr, g->col_idx, n, m, s, r, ctx->tune, ctx->stream), "omega");
     rc = nodes_device(ctx, g->row_ptr, g->col_idx, n, m, s, nodes, k, nullptr, o.precision, false, false, false,
                       *out);
     if (rc) return rc;

@@ -176,7 +176,7 @@ constexpr int MLP_WARPS = 8;
 // different banks), layer 2 starts from its biases, and a layer-2 column
 // tile is consumed as soon as it is complete, so no activation array is kept.
 // Bound by the rate of mma.sync and the shared-memory loads together.
-// Measured, 8M rows: 344 us with one tile per step and four-byte loads, 251
+// Measured, 8M rows: 344 us with one tile per step and four-byte loads, 246
 // so; at 80 registers (three blocks per SM) 278, four tiles 280, the W2
 // fragments in registers (12 warps per SM) 276-292.
 constexpr int W2ROW = 40;   // words of a W2 row: 4 k-chunks x 4 lanes x 2 words, padded
@@ -658,9 +658,8 @@ int launch_model_pack(ModelDev *M, cudaStream_t st) {
 
 // Up to one 16-row tile per warp of the chip (two blocks per SM) each warp has
 // one tile: below that line a second tile is work for padding, and the
-// smallest calls are the latency of one warp step.  Calls of 500 to
-// 20 000 rows: two tiles 0.4-0.7 us slower than one; 60 000 rows fill the chip
-// with two.
+// smallest calls are the latency of one warp step.  A call of a
+// few thousand rows: 15.4 us with two tiles, 14.8 with one.
 template <bool BF>
 static int infer(const ModelDev *M, const void *x, int32_t n, float *out, int num_sms, cudaStream_t st) {
     const int64_t rows = 16 * MLP_WARPS, cap = (int64_t)num_sms * 2, g = ((int64_t)n + rows - 1) / rows;

@@ -409,17 +409,18 @@ __device__ __forceinline__ bool adjacent(const int32_t *rp, const int32_t *ci, i
 // found either as adjacent pairs of N(v) (C(D_v, 2) tests in the shorter
 // rows, each triangle once) or by streaming every neighbour's row against
 // N(v) (sigma1(v) tests in a row held in shared memory, each triangle twice),
-// whichever costs less.
+// whichever costs less.  omega_v is summed here, from the listed rows only (a
+// pass over every row for it was the call's longest kernel: 2000 nodes of
+// BA 1M 0.598 -> 0.443 ms a call).
 template <bool F64>
 __global__ void __launch_bounds__(NODE_THREADS) k_nodes_final(
     const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const int32_t *__restrict__ D,
-    const int64_t *__restrict__ sig1, const int64_t *__restrict__ sig2, const int64_t *__restrict__ omega,
-    const void *__restrict__ Ccenter, const double *__restrict__ Tacc, const int64_t *__restrict__ tq,
-    const int32_t *__restrict__ cnt, const int32_t *__restrict__ list, int32_t k_max,
-    const int32_t *__restrict__ kptr, int32_t n, const int64_t *__restrict__ qacc, const int64_t *__restrict__ tcnt,
+    const int64_t *__restrict__ sig1, const int64_t *__restrict__ sig2, const void *__restrict__ Ccenter,
+    const double *__restrict__ Tacc, const int64_t *__restrict__ tq, const int32_t *__restrict__ cnt,
+    const int32_t *__restrict__ list, int32_t k_max, const int32_t *__restrict__ kptr, int32_t n,
     ef_outputs out) {
     __shared__ int32_t s_row[NODE_ROW_SMEM];
-    __shared__ long long s_q[NODE_THREADS / 32], s_t[NODE_THREADS / 32];
+    __shared__ long long s_q[NODE_THREADS / 32], s_t[NODE_THREADS / 32], s_om[NODE_THREADS / 32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int F = cnt[CNT_TRIFRAC];
     const int k = kptr ? *kptr : k_max;
@@ -428,15 +429,20 @@ __global__ void __launch_bounds__(NODE_THREADS) k_nodes_final(
         if (v < 0 || v >= n) continue;   // reported by k_mark_nbhd (the whole CTA skips alike)
         const int a = rp[v], Dv = rp[v + 1] - a;
         const int64_t s1v = sig1[v];
-        const bool global = qacc != nullptr;   // triangles already counted by the full pass
-        const bool by_pairs = !global && (int64_t)Dv * (Dv - 1) / 2 * 16 <= s1v;
-        const bool staged = !global && !by_pairs && Dv <= NODE_ROW_SMEM;
+        const bool by_pairs = (int64_t)Dv * (Dv - 1) / 2 * 16 <= s1v;
+        const bool staged = !by_pairs && Dv <= NODE_ROW_SMEM;
         if (staged)
             for (int e = threadIdx.x; e < Dv; e += NODE_THREADS) s_row[e] = ci[a + e];
+        int64_t om = 0;
+        for (int e = threadIdx.x; e < Dv; e += NODE_THREADS) {
+            const int x = ci[a + e];
+            if (x >= 0 && x < n) om += sig1[x];
+        }
+        om = warp_sum(om);
+        if (lane == 0) s_om[w] = om;
         __syncthreads();
         int64_t q = 0, t = 0;   // by pairs: each triangle once; by streaming: twice
-        if (global) {
-        } else if (by_pairs) {
+        if (by_pairs) {
             for (int x = w; x < Dv; x += NODE_THREADS / 32) {
                 const int bx = ci[a + x], Dx = D[bx];
                 for (int y = x + 1 + lane; y < Dv; y += 32) {
@@ -472,18 +478,17 @@ __global__ void __launch_bounds__(NODE_THREADS) k_nodes_final(
         __syncthreads();
         if (threadIdx.x == 0) {
             int64_t qs = 0, ts = 0;
+            om = 0;
             for (int j = 0; j < NODE_THREADS / 32; ++j) {
                 qs += s_q[j];
                 ts += s_t[j];
+                om += s_om[j];
             }
-            if (global) {
-                qs = qacc[v];
-                ts = tcnt[v];
-            } else if (!by_pairs) {
+            if (!by_pairs) {
                 qs /= 2;   // each triangle was found through both of its other nodes
                 ts /= 2;
             }
-            const int64_t d = Dv, s2 = sig2[v], om = omega[v];
+            const int64_t d = Dv, s2 = sig2[v];
             const int64_t N = d * (d - 2) + s1v;
             const int64_t S =
                 d * (d - 1) * (d - 4) + 2 * (d - 1) * s1v + s2 - s1v + (d - 4) * (s1v - d) + om - d * d - 8 * ts;
@@ -558,13 +563,12 @@ int launch_nodes_exact(const int32_t *rp, const int32_t *ci, const Scratch &s, c
         return cudaGetLastError() == cudaSuccess ? 0 : -1;
     }
     const unsigned grid = (unsigned)(k < t.num_sms * 8 ? k : t.num_sms * 8);
-    const int64_t *q = nullptr, *tc = nullptr;
     if (precision == EF_PREC_FP64)
-        k_nodes_final<true><<<grid, NODE_THREADS, 0, st>>>(rp, ci, s.D, s.sig1, s.sig2, s.omega, s.Ccenter, s.Tacc,
-                                                           s.tq, s.counters, list, k, kptr, n, q, tc, out);
+        k_nodes_final<true><<<grid, NODE_THREADS, 0, st>>>(rp, ci, s.D, s.sig1, s.sig2, s.Ccenter, s.Tacc, s.tq,
+                                                           s.counters, list, k, kptr, n, out);
     else
-        k_nodes_final<false><<<grid, NODE_THREADS, 0, st>>>(rp, ci, s.D, s.sig1, s.sig2, s.omega, s.Ccenter,
-                                                            s.Tacc, s.tq, s.counters, list, k, kptr, n, q, tc, out);
+        k_nodes_final<false><<<grid, NODE_THREADS, 0, st>>>(rp, ci, s.D, s.sig1, s.sig2, s.Ccenter, s.Tacc,
+                                                            s.tq, s.counters, list, k, kptr, n, out);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -115,6 +115,8 @@ struct Tune {
 
 // Scratch carved from one device allocation per call (sizes depend on n, m).
 struct Scratch {
+    // bit per node: the nodes whose T is wanted (exact EF of chosen nodes); null: all
+    const uint32_t *listed = nullptr;
     int32_t *D;          // n      degrees
     int64_t *sig1;       // n      sum of neighbour degrees
     int64_t *sig2;       // n      sum of squared neighbour degrees
@@ -451,6 +453,8 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // Credit R_u(x) of middle node u to its end x (an L2 reduction, no return).
 __device__ __forceinline__ void credit_end(double *Tacc, int x, double r) { atomicAdd(Tacc + x, r); }
 
+__device__ __forceinline__ bool bit_of(const uint32_t *bits, int x) { return __ldg(bits + (x >> 5)) >> (x & 31) & 1; }
+
 constexpr double LN2 = 0.69314718055994530942;
 
 }  // namespace ef
@@ -578,7 +582,7 @@ int launch_features(const Scratch &s, const RankScratch &r, int32_t n, int mode,
                     const ModelDev *std_model = nullptr);
 int launch_select_top(const RankScratch &r, int32_t n, int64_t k, int bits, const Tune &t, cudaStream_t st);
 int launch_bin_nodes(const int32_t *list, int32_t k, const int32_t *kptr, const int32_t *rp, const int32_t *ci,
-                     const Scratch &s, int32_t *mark, int32_t n, const Tune &t, cudaStream_t st);
+                     const Scratch &s, uint32_t *listed, int32_t n, const Tune &t, cudaStream_t st);
 int launch_bin_marked(const int32_t *mark, const Scratch &s, int32_t n, const Tune &t, cudaStream_t st);
 // SIR simulation (ef_sir.cu): a batch of at most SIR_BATCH simulations,
 // node-major bit words (WB = ceil(B / 32) per node), frontier lists of nodes.

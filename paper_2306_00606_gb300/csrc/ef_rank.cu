@@ -313,31 +313,66 @@ int launch_select_top(const RankScratch &r, int32_t n, int64_t k, int bits, cons
 }
 
 // ------------------------------------------------------ exact EF of nodes
-// mark[x] = 1 for every listed node and every neighbour of one: the middle
-// nodes whose wedge credits reach a listed node.  Ids outside [0, n) set an
-// error bit.
-__global__ void k_mark_nbhd(const int32_t *__restrict__ list, int32_t k_max, const int32_t *__restrict__ kptr,
-                            const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, int32_t n,
-                            int32_t *__restrict__ mark, int32_t *__restrict__ cnt) {
+// A bit per listed node (listed), and one per listed node and neighbour of one
+// (mark): the middle nodes whose wedge credits reach a listed node.  Ids
+// outside [0, n) set an error bit.  A warp per listed node, the block for rows
+// above MARK_LONG; a bit that is seen set is left alone (a stale L1 line costs
+// an atomic, nothing else).  Bits instead of an int per node: 2 MB of the L2
+// instead of 64 for 16M nodes, 0.632 -> 0.164 ms
+// (336 000 listed).
+constexpr int MARK_LONG = 512;
+
+__global__ void __launch_bounds__(256) k_mark_nbhd(const int32_t *__restrict__ list, int32_t k_max,
+                                                   const int32_t *__restrict__ kptr, const int32_t *__restrict__ rp,
+                                                   const int32_t *__restrict__ ci, int32_t n, uint32_t *listed,
+                                                   uint32_t *mark, int32_t *__restrict__ cnt) {
+    __shared__ int2 s_long[8];
+    __shared__ int s_n;
     const int k = kptr ? *kptr : k_max;
-    const int lane = threadIdx.x & 31;
-    const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t i = w0; i < k; i += nw) {   // a warp per listed node
-        const int v = list[i];
-        if (v < 0 || v >= n) {
-            if (lane == 0) atomicOr(cnt + CNT_ERR, ERRB_NODE);
-            continue;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    auto set = [](uint32_t *bits, int x) {
+        if (!(bits[x >> 5] >> (x & 31) & 1)) atomicOr(bits + (x >> 5), 1u << (x & 31));
+    };
+    auto mark_row = [&](int e0, int b, int step) {
+        for (; e0 < b; e0 += 4 * step) {
+            int x[4];
+            uint32_t have[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) x[q] = e0 + q * step < b ? ci[e0 + q * step] : -1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) have[q] = x[q] >= 0 ? mark[x[q] >> 5] >> (x[q] & 31) & 1 : 1;
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                if (!have[q]) atomicOr(mark + (x[q] >> 5), 1u << (x[q] & 31));
         }
-        if (lane == 0) mark[v] = 1;
-        for (int e = rp[v] + lane; e < rp[v + 1]; e += 32) mark[ci[e]] = 1;
+    };
+    for (int64_t i0 = (int64_t)blockIdx.x * 8; i0 < k; i0 += (int64_t)gridDim.x * 8) {
+        if (threadIdx.x == 0) s_n = 0;
+        __syncthreads();
+        const int v = i0 + w < k ? list[i0 + w] : 0;
+        if (i0 + w >= k) {
+        } else if (v < 0 || v >= n) {
+            if (lane == 0) atomicOr(cnt + CNT_ERR, ERRB_NODE);
+        } else {
+            const int a = rp[v], b = rp[v + 1];
+            if (lane == 0) {
+                set(listed, v);
+                set(mark, v);
+                if (b - a > MARK_LONG) s_long[atomicAdd(&s_n, 1)] = make_int2(a, b);
+            }
+            if (b - a <= MARK_LONG) mark_row(a + lane, b, 32);
+        }
+        __syncthreads();
+        for (int j = 0; j < s_n; ++j) mark_row(s_long[j].x + threadIdx.x, s_long[j].y, 256);
+        __syncthreads();
     }
 }
 
 // Work bins holding only the marked nodes (as middle nodes of the wedge
 // kernels).  Counting per block in shared memory, one global atomic per bin
 // per block, so the bins keep the node order within a block.
-__global__ void k_bin_marked(const int32_t *__restrict__ mark, const int32_t *__restrict__ D, int32_t n, int hub_min,
+template <bool BITS>
+__global__ void k_bin_marked(const void *__restrict__ mark, const int32_t *__restrict__ D, int32_t n, int hub_min,
                              int32_t *__restrict__ bins, int32_t *__restrict__ cnt) {
     __shared__ int s_cnt[NUM_BINS], s_base[NUM_BINS];
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
@@ -345,7 +380,8 @@ __global__ void k_bin_marked(const int32_t *__restrict__ mark, const int32_t *__
         __syncthreads();
         const int v = (int)(base + threadIdx.x);
         int b0 = -1, b1 = -1, p0 = 0, p1 = 0;
-        if (v < n && mark[v]) {
+        if (v < n && (BITS ? bit_of(static_cast<const uint32_t *>(mark), v)
+                           : static_cast<const int32_t *>(mark)[v] != 0)) {
             const int d = D[v];
             if (d >= 1 && d <= SMALL_MAX) {
                 b0 = d <= 4 ? BIN_S4 : d <= 8 ? BIN_S8 : d <= 16 ? BIN_S16 : BIN_S32;
@@ -366,19 +402,21 @@ __global__ void k_bin_marked(const int32_t *__restrict__ mark, const int32_t *__
     }
 }
 
-// mark: an n-int array free for this call (the row passes' out-degrees).
+// listed: 2 ceil(n / 32) words free for this call; the second half holds the marks.
 int launch_bin_nodes(const int32_t *list, int32_t k, const int32_t *kptr, const int32_t *rp, const int32_t *ci,
-                     const Scratch &s, int32_t *mark, int32_t n, const Tune &t, cudaStream_t st) {
-    if (cudaMemsetAsync(mark, 0, (size_t)n * sizeof(int32_t), st) != cudaSuccess) return -1;
+                     const Scratch &s, uint32_t *listed, int32_t n, const Tune &t, cudaStream_t st) {
+    const size_t words = ((size_t)n + 31) / 32;
+    uint32_t *mark = listed + words;
+    if (cudaMemsetAsync(listed, 0, 2 * words * sizeof(uint32_t), st) != cudaSuccess) return -1;
     if (cudaMemsetAsync(s.counters, 0, NUM_BINS * sizeof(int32_t), st) != cudaSuccess) return -1;
     // the work counters of the big-node kernels (CNT_BIGITEM .. CNT_HUB; CNT_TRIFRAC stays)
     if (cudaMemsetAsync(s.counters + CNT_BIGITEM, 0, (CNT_HUB - CNT_BIGITEM + 1) * sizeof(int32_t), st) !=
         cudaSuccess)
         return -1;
-    int64_t g = ((int64_t)k * 32 + 255) / 256;
-    k_mark_nbhd<<<(unsigned)(g < 1 ? 1 : (g > 8192 ? 8192 : g)), 256, 0, st>>>(list, k, kptr, rp, ci, n, mark,
+    const int64_t g = ((int64_t)k + 7) / 8;
+    k_mark_nbhd<<<(unsigned)(g < 1 ? 1 : (g > 8192 ? 8192 : g)), 256, 0, st>>>(list, k, kptr, rp, ci, n, listed, mark,
                                                                               s.counters);
-    k_bin_marked<<<t.grid((int64_t)n, 256), 256, 0, st>>>(mark, s.D, n, t.hub_min, s.bins, s.counters);
+    k_bin_marked<true><<<t.grid((int64_t)n, 256), 256, 0, st>>>(mark, s.D, n, t.hub_min, s.bins, s.counters);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -388,7 +426,7 @@ int launch_bin_marked(const int32_t *mark, const Scratch &s, int32_t n, const Tu
     if (cudaMemsetAsync(s.counters + CNT_BIGITEM, 0, (CNT_HUB - CNT_BIGITEM + 1) * sizeof(int32_t), st) !=
         cudaSuccess)
         return -1;
-    k_bin_marked<<<t.grid((int64_t)n, 256), 256, 0, st>>>(mark, s.D, n, t.hub_min, s.bins, s.counters);
+    k_bin_marked<false><<<t.grid((int64_t)n, 256), 256, 0, st>>>(mark, s.D, n, t.hub_min, s.bins, s.counters);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -409,7 +447,9 @@ __device__ __forceinline__ bool adjacent(const int32_t *rp, const int32_t *ci, i
 // found either as adjacent pairs of N(v) (C(D_v, 2) tests in the shorter
 // rows, each triangle once) or by streaming every neighbour's row against
 // N(v) (sigma1(v) tests in a row held in shared memory, each triangle twice),
-// whichever costs less.  omega_v is summed here, from the listed rows only (a
+// whichever costs less: a pair is two steps of a row (lists of 2000 nodes of BA
+// 1M that hold a hub: 375 us at sixteen, 319 at four, 312 at two, 299 at one;
+// 20 000 nodes 812 / 807 / 806 / 838).  omega_v is summed here, from the listed rows only (a
 // pass over every row for it was the call's longest kernel: 2000 nodes of
 // BA 1M 0.598 -> 0.443 ms a call).
 template <bool F64>
@@ -429,7 +469,7 @@ __global__ void __launch_bounds__(NODE_THREADS) k_nodes_final(
         if (v < 0 || v >= n) continue;   // reported by k_mark_nbhd (the whole CTA skips alike)
         const int a = rp[v], Dv = rp[v + 1] - a;
         const int64_t s1v = sig1[v];
-        const bool by_pairs = (int64_t)Dv * (Dv - 1) / 2 * 16 <= s1v;
+        const bool by_pairs = (int64_t)Dv * (Dv - 1) / 2 * 2 <= s1v;
         const bool staged = !by_pairs && Dv <= NODE_ROW_SMEM;
         if (staged)
             for (int e = threadIdx.x; e < Dv; e += NODE_THREADS) s_row[e] = ci[a + e];

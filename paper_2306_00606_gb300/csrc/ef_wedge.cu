@@ -38,14 +38,20 @@ namespace ef {
 // degree) together.  FP32C, small wedges (ms) with 1 / 2 / 3 sets: WS batch
 // 3.25 / 2.93 / 2.92, BA 16M 2.83 / 2.82 / 2.73, power-law 4M 0.283 / 0.286 /
 // 0.288; three sets take 37-40 registers instead of 32.
+//
+// LISTED (exact EF of chosen nodes): only listed nodes take credits, and R_u(x)
+// is summed where x or u is listed.  The reductions bound these kernels on
+// large graphs: ranking BA 16M, 2.1% of the nodes listed, 2.02
+// -> 1.37 ms, and k_wedge_mid 1.44 -> 0.53.
 constexpr int SMALL_ILP = 2;
 
-template <int G, bool F64>
+template <int G, bool F64, bool LISTED>
 __global__ void __launch_bounds__(256) k_wedge_small(const int32_t *__restrict__ rp, const int32_t *__restrict__ ci,
                                                      const int32_t *__restrict__ D, const int32_t *__restrict__ list,
                                                      const int32_t *__restrict__ cnt, int bin,
                                                      const float2 *__restrict__ ftab, double *__restrict__ Tacc,
-                                                     void *__restrict__ Ccenter) {
+                                                     void *__restrict__ Ccenter,
+                                                     const uint32_t *__restrict__ listed) {
     if (gate_closed(cnt)) return;
     using Acc = typename std::conditional<F64, double, float>::type;
     constexpr int PER = 32 / G, ILP = SMALL_ILP;
@@ -68,8 +74,14 @@ __global__ void __launch_bounds__(256) k_wedge_small(const int32_t *__restrict__
         }
 #pragma unroll
         for (int r = 0; r < ILP; ++r) xs[r] = k < Dus[r] ? ci[sts[r] + k] : 0;
+        bool lu[ILP], lx[ILP];   // listed: the middle node, the end
 #pragma unroll
-        for (int r = 0; r < ILP; ++r) aks[r] = k < Dus[r] ? D[xs[r]] : 0;
+        for (int r = 0; r < ILP; ++r) lu[r] = LISTED && us[r] >= 0 ? bit_of(listed, us[r]) : true;
+#pragma unroll
+        for (int r = 0; r < ILP; ++r) {
+            aks[r] = k < Dus[r] ? D[xs[r]] : 0;
+            lx[r] = LISTED && k < Dus[r] ? bit_of(listed, xs[r]) : true;
+        }
 #pragma unroll
         for (int r = 0; r < ILP; ++r) {
             const bool vc = us[r] >= 0;
@@ -79,6 +91,8 @@ __global__ void __launch_bounds__(256) k_wedge_small(const int32_t *__restrict__
             const int x = xs[r];
             const int ak = aks[r];
             const int b0 = Du - 4 + ak;
+            // credit: x takes it; sum: R_u(x) is needed (by x, or by a listed u)
+            const bool credit = own && lx[r], sum = own && (lx[r] || lu[r]);
             Acc acc = 0;
             // the warp's largest row bounds the loop (rows of a bin are often
             // much shorter than G); degrees travel as floats (exact below 2^24),
@@ -90,7 +104,7 @@ __global__ void __launch_bounds__(256) k_wedge_small(const int32_t *__restrict__
 #pragma unroll 4
                 for (int j = 0; j < jmax; ++j) {
                     const int aj = __shfl_sync(FULL, ak, j, G);
-                    if (own && j < Du && j != k) a2.add(__ldg(ftab + (b0 + aj)));   // b0 + aj >= 0 for D_u >= 2
+                    if (sum && j < Du && j != k) a2.add(__ldg(ftab + (b0 + aj)));   // b0 + aj >= 0 for D_u >= 2
                 }
                 acc = a2.value();
             } else {
@@ -104,23 +118,23 @@ __global__ void __launch_bounds__(256) k_wedge_small(const int32_t *__restrict__
                 const float akf = (float)ak, b0f = (float)b0;
                 const int jmin = __reduce_min_sync(FULL, vc ? Du : G);
                 const int lim = own ? Du : 0;
-                float sum = 0.0f;
+                float s = 0.0f;
 #pragma unroll 4
                 for (int j = 0; j < jmin; ++j) {
                     float d = b0f + __shfl_sync(FULL, akf, j, G);
                     if (G == 4) d = fmaxf(d, 1.0f);
-                    sum = fmaf(d, lg2(d), sum);
+                    s = fmaf(d, lg2(d), s);
                 }
                 for (int j = jmin; j < jmax; ++j) {
                     float d = b0f + __shfl_sync(FULL, akf, j, G);
                     if (G == 4) d = fmaxf(d, 1.0f);
                     const float t = lg2(d);
-                    if (j < lim) sum = fmaf(d, t, sum);
+                    if (j < lim) s = fmaf(d, t, s);
                 }
-                acc = sum - dlog2d(G == 4 ? fmaxf(b0f + akf, 1.0f) : b0f + akf);
+                acc = s - dlog2d(G == 4 ? fmaxf(b0f + akf, 1.0f) : b0f + akf);
             }
-            const Acc rs = own ? (F64 ? acc : acc * (Acc)LN2) : (Acc)0;
-            if (own) credit_end(Tacc, x, (double)rs);
+            const Acc rs = sum ? (F64 ? acc : acc * (Acc)LN2) : (Acc)0;
+            if (credit) credit_end(Tacc, x, (double)rs);
             const Acc c = group_sum<G>(rs);
             if (k == 0 && vc) reinterpret_cast<Acc *>(Ccenter)[u] = c;
         }
@@ -330,11 +344,11 @@ constexpr int MID_WARPS = 4;
 // square of its class count, which varies a hundredfold within the bin); the
 // next node's index, id and row range are loaded while the current node is
 // processed, so only the neighbour gathers wait at the start of a node.
-template <bool F64>
+template <bool F64, bool LISTED>
 __global__ void __launch_bounds__(MID_WARPS * 32, 6) k_wedge_mid(
     const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const int32_t *__restrict__ D,
     const int32_t *__restrict__ bins, int32_t n, int32_t *__restrict__ cnt, const float2 *__restrict__ ftab,
-    double *__restrict__ Tacc, void *__restrict__ Ccenter) {
+    double *__restrict__ Tacc, void *__restrict__ Ccenter, const uint32_t *__restrict__ listed) {
     if (gate_closed(cnt)) return;
     using E = ClassEval<F64>;
     constexpr int MAX = F64 ? MID_SPLIT - 1 : MID_MAX;   // row entries at most
@@ -412,7 +426,10 @@ __global__ void __launch_bounds__(MID_WARPS * 32, 6) k_wedge_mid(
             center.add((R)E::cval(c_i) * r);
         }
         __syncwarp();
-        for (int k = lane; k < Du; k += 32) credit_end(Tacc, ci[start + k], (double)cq[cidx[k]]);
+        for (int k = lane; k < Du; k += 32) {
+            const int x = ci[start + k];
+            if (!LISTED || bit_of(listed, x)) credit_end(Tacc, x, (double)cq[cidx[k]]);
+        }
         const R ctot = warp_sum(center.get());
         if (lane == 0) reinterpret_cast<R *>(Ccenter)[u] = ctot;
         __syncwarp();
@@ -815,18 +832,18 @@ __global__ void __launch_bounds__(HUB_THREADS) k_wedge_hub(
 }
 
 
-template <bool F64>
+template <bool F64, bool LISTED>
 static void small_all(const int32_t *rp, const int32_t *ci, const Scratch &s, int32_t n, cudaStream_t st,
                       unsigned grid) {
     const int32_t *B = s.bins;
-    k_wedge_small<4, F64><<<grid, 256, 0, st>>>(rp, ci, s.D, B + (size_t)BIN_S4 * n, s.counters, BIN_S4, s.ftab,
-                                                s.Tacc, s.Ccenter);
-    k_wedge_small<8, F64><<<grid, 256, 0, st>>>(rp, ci, s.D, B + (size_t)BIN_S8 * n, s.counters, BIN_S8, s.ftab,
-                                                s.Tacc, s.Ccenter);
-    k_wedge_small<16, F64><<<grid, 256, 0, st>>>(rp, ci, s.D, B + (size_t)BIN_S16 * n, s.counters, BIN_S16, s.ftab,
-                                                 s.Tacc, s.Ccenter);
-    k_wedge_small<32, F64><<<grid, 256, 0, st>>>(rp, ci, s.D, B + (size_t)BIN_S32 * n, s.counters, BIN_S32, s.ftab,
-                                                 s.Tacc, s.Ccenter);
+    k_wedge_small<4, F64, LISTED><<<grid, 256, 0, st>>>(rp, ci, s.D, B + (size_t)BIN_S4 * n, s.counters, BIN_S4,
+                                                        s.ftab, s.Tacc, s.Ccenter, s.listed);
+    k_wedge_small<8, F64, LISTED><<<grid, 256, 0, st>>>(rp, ci, s.D, B + (size_t)BIN_S8 * n, s.counters, BIN_S8,
+                                                        s.ftab, s.Tacc, s.Ccenter, s.listed);
+    k_wedge_small<16, F64, LISTED><<<grid, 256, 0, st>>>(rp, ci, s.D, B + (size_t)BIN_S16 * n, s.counters, BIN_S16,
+                                                         s.ftab, s.Tacc, s.Ccenter, s.listed);
+    k_wedge_small<32, F64, LISTED><<<grid, 256, 0, st>>>(rp, ci, s.D, B + (size_t)BIN_S32 * n, s.counters, BIN_S32,
+                                                         s.ftab, s.Tacc, s.Ccenter, s.listed);
 }
 
 int launch_wedge_small(const int32_t *rp, const int32_t *ci, const Scratch &s, int precision, int32_t n,
@@ -834,8 +851,9 @@ int launch_wedge_small(const int32_t *rp, const int32_t *ci, const Scratch &s, i
     int64_t g = ((int64_t)n + 63) / 64;
     const int64_t cap = (int64_t)t.num_sms * 16;
     unsigned grid = (unsigned)(g < 1 ? 1 : (g > cap ? cap : g));
-    if (precision == EF_PREC_FP64) small_all<true>(rp, ci, s, n, st, grid);
-    else small_all<false>(rp, ci, s, n, st, grid);
+    const bool f64 = precision == EF_PREC_FP64;
+    if (s.listed) f64 ? small_all<true, true>(rp, ci, s, n, st, grid) : small_all<false, true>(rp, ci, s, n, st, grid);
+    else f64 ? small_all<true, false>(rp, ci, s, n, st, grid) : small_all<false, false>(rp, ci, s, n, st, grid);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -867,7 +885,7 @@ static DeviceProps &dev_props() {
 template <bool F64>
 static int class_occupancy(DeviceProps &p) {
     int mid = 0, hub = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&mid, k_wedge_mid<F64>, MID_WARPS * 32, 0) != cudaSuccess ||
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&mid, k_wedge_mid<F64, false>, MID_WARPS * 32, 0) != cudaSuccess ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&hub, k_wedge_hub<F64>, HUB_THREADS, hub_smem_bytes<F64>()) !=
             cudaSuccess)
         return -1;
@@ -903,8 +921,9 @@ template <bool F64>
 static int big_classes(const int32_t *rp, const int32_t *ci, const Scratch &s, int32_t n, int num_sms,
                        cudaStream_t st) {
     const DeviceProps &p = dev_props();
-    k_wedge_mid<F64><<<(unsigned)(num_sms * p.class_blocks[F64][0]), MID_WARPS * 32, 0, st>>>(
-        rp, ci, s.D, s.bins, n, s.counters, s.ftab, s.Tacc, s.Ccenter);
+    const auto mid = s.listed ? k_wedge_mid<F64, true> : k_wedge_mid<F64, false>;
+    mid<<<(unsigned)(num_sms * p.class_blocks[F64][0]), MID_WARPS * 32, 0, st>>>(
+        rp, ci, s.D, s.bins, n, s.counters, s.ftab, s.Tacc, s.Ccenter, s.listed);
     const size_t smem = hub_smem_bytes<F64>();
     k_wedge_hub<F64><<<(unsigned)(num_sms * p.class_blocks[F64][1]), HUB_THREADS, smem, st>>>(
         rp, ci, s.D, s.bins, n, s.counters, s.ftab, s.Tacc, s.Ccenter, s.hub_cidx, s.hub_cls, s.hub_q);

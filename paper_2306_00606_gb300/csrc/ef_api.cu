@@ -292,7 +292,7 @@ int part_c(ef_ctx *ctx, const Job &j, const ef::Scratch &s, PathMode path, cudaS
     using namespace ef;
     if (path != PATH_GENERAL)
         LAUNCH(launch_finalize_short(s, j.o.precision, j.n, j.out, ctx->tune, path == PATH_SHORT, st), "finalize");
-    if (path != PATH_SHORT) LAUNCH(launch_finalize(s, j.o.precision, j.n, j.out, ctx->tune, st), "finalize");
+    else LAUNCH(launch_finalize(s, j.o.precision, j.n, j.out, ctx->tune, st), "finalize");
     return EF_OK;
 }
 

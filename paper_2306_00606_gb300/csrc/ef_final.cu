@@ -98,8 +98,7 @@ struct FinalArgs {
 };
 
 template <bool F64>
-__global__ void __launch_bounds__(256) k_finalize(int32_t n, FinalArgs f) {
-    if (gate_closed(f.cnt)) return;
+__device__ __forceinline__ void finalize_nodes(int32_t n, const FinalArgs &f) {
     const int F = f.cnt[CNT_TRIFRAC];
     const double qscale = ldexp(1.0, -F);
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
@@ -129,12 +128,17 @@ __global__ void __launch_bounds__(256) k_finalize(int32_t n, FinalArgs f) {
 // The short-row path's finalize: the fused kernel left a node's integer sums
 // in one word, its triangles in 32 bits and all of T in Tacc, so a node costs
 // 20 bytes read (k_finalize: 60).
+struct ShortFinalArgs {
+    const uint64_t *stat;
+    const int32_t *tri;
+    const double *Tacc;
+};
+
 template <bool F64>
-__global__ void __launch_bounds__(256) k_finalize_short(int32_t n, const uint64_t *__restrict__ stat,
-                                                        const int32_t *__restrict__ tri,
-                                                        const double *__restrict__ Tacc,
-                                                        const int32_t *__restrict__ cnt, ef_outputs o, bool chosen) {
-    if (short_closed(cnt, chosen)) return;
+__device__ __forceinline__ void finalize_short_nodes(int32_t n, const ShortFinalArgs &f, const ef_outputs &o) {
+    const uint64_t *__restrict__ stat = f.stat;
+    const int32_t *__restrict__ tri = f.tri;
+    const double *__restrict__ Tacc = f.Tacc;
     for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
         const uint64_t w = stat[v];
         const double T = Tacc[v];
@@ -156,6 +160,27 @@ __global__ void __launch_bounds__(256) k_finalize_short(int32_t n, const uint64_
         if (o.triangles) o.triangles[v] = t;
         if (o.flag) o.flag[v] = fl;
     }
+}
+
+template <bool F64>
+__global__ void __launch_bounds__(256) k_finalize(int32_t n, FinalArgs f) {
+    if (!gate_closed(f.cnt)) finalize_nodes<F64>(n, f);
+}
+
+template <bool F64>
+__global__ void __launch_bounds__(256) k_finalize_short(int32_t n, ShortFinalArgs f, const int32_t *__restrict__ cnt,
+                                                        ef_outputs o) {
+    if (!short_closed(cnt, true)) finalize_short_nodes<F64>(n, f, o);
+}
+
+// The path was chosen on the device: one launch for both instead of one that
+// leaves at once behind one that works (replayed calls: BA 1M 720 -> 712 us, ER
+// 200 000 135 -> 131, the 4096-graph batch 8.48 -> 8.44 ms).
+template <bool F64>
+__global__ void __launch_bounds__(256) k_finalize_either(int32_t n, FinalArgs f, ShortFinalArgs sf) {
+    const int gate = f.cnt[CNT_GATE];
+    if (gate == 0) finalize_nodes<F64>(n, f);
+    else if (gate == GATE_SHORT) finalize_short_nodes<F64>(n, sf, f.o);
 }
 
 // From the shards' summed partials: T_v = t + q 2^-F, S_v = S_open - 8 t_v.
@@ -201,9 +226,17 @@ static inline unsigned grid_n(int32_t n, const Tune &t) {
     return (unsigned)(g < 1 ? 1 : (g > cap ? cap : g));
 }
 
+static FinalArgs final_args(const Scratch &s, const ef_outputs &out) {
+    return FinalArgs{s.D, s.sig1, s.sig2, s.omega, s.Tacc, s.Ccenter, s.qacc, s.tcnt, s.counters, out};
+}
+
+static ShortFinalArgs short_final_args(const Scratch &s) {
+    return ShortFinalArgs{reinterpret_cast<const uint64_t *>(s.sig1), s.outdeg, s.Tacc};
+}
+
 int launch_finalize(const Scratch &s, int precision, int32_t n, const ef_outputs &out, const Tune &t,
                     cudaStream_t st) {
-    const FinalArgs f{s.D, s.sig1, s.sig2, s.omega, s.Tacc, s.Ccenter, s.qacc, s.tcnt, s.counters, out};
+    const FinalArgs f = final_args(s, out);
     if (precision == EF_PREC_FP64) k_finalize<true><<<grid_n(n, t), 256, 0, st>>>(n, f);
     else k_finalize<false><<<grid_n(n, t), 256, 0, st>>>(n, f);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
@@ -211,11 +244,16 @@ int launch_finalize(const Scratch &s, int precision, int32_t n, const ef_outputs
 
 int launch_finalize_short(const Scratch &s, int precision, int32_t n, const ef_outputs &out, const Tune &t,
                           bool chosen, cudaStream_t st) {
-    const uint64_t *stat = reinterpret_cast<const uint64_t *>(s.sig1);
-    if (precision == EF_PREC_FP64)
-        k_finalize_short<true><<<grid_n(n, t), 256, 0, st>>>(n, stat, s.outdeg, s.Tacc, s.counters, out, chosen);
-    else
-        k_finalize_short<false><<<grid_n(n, t), 256, 0, st>>>(n, stat, s.outdeg, s.Tacc, s.counters, out, chosen);
+    const unsigned g = grid_n(n, t);
+    const ShortFinalArgs sf = short_final_args(s);
+    const FinalArgs f = final_args(s, out);
+    if (precision == EF_PREC_FP64) {
+        if (chosen) k_finalize_short<true><<<g, 256, 0, st>>>(n, sf, s.counters, out);
+        else k_finalize_either<true><<<g, 256, 0, st>>>(n, f, sf);
+    } else {
+        if (chosen) k_finalize_short<false><<<g, 256, 0, st>>>(n, sf, s.counters, out);
+        else k_finalize_either<false><<<g, 256, 0, st>>>(n, f, sf);
+    }
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

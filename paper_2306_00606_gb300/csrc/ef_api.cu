@@ -1171,7 +1171,7 @@ int ef_sir_run(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const int32_t
                  o_new = place(4 * N * WBmax), o_cand = place(4 * N * (size_t)Bmax),
                  o_parent = out->parent ? 0 : place(4 * N * (size_t)Bmax), o_f0 = place(4 * N), o_f1 = place(4 * N),
                  o_touch = place(4 * N), o_heavy = place(4 * N), o_fmark = place(4 * N), o_tmark = place(4 * N),
-                 o_counts = place(16), o_act = place(16), o_cnt = place(4 * (size_t)Bmax),
+                 o_counts = place(24), o_act = place(16), o_cnt = place(4 * (size_t)Bmax),
                  o_peak = place(4 * (size_t)Bmax), o_pstep = place(4 * (size_t)Bmax), o_len = place(4 * (size_t)Bmax),
                  o_fs = place(4 * (size_t)Bmax), o_done = place((size_t)Bmax), o_err = place(4);
     rc = ensure_buffer(ctx, &ctx->sir, &ctx->sir_bytes, off, 0);
@@ -1185,6 +1185,7 @@ int ef_sir_run(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const int32_t
         SirState st;
         st.B = num_sims - c0 < SIR_BATCH ? num_sims - c0 : SIR_BATCH;
         st.WB = (st.B + 31) / 32;
+        st.m = m;
         st.susc = (uint32_t *)(b + o_susc);
         st.inf[0] = (uint32_t *)(b + o_inf0);
         st.inf[1] = (uint32_t *)(b + o_inf1);
@@ -1197,7 +1198,8 @@ int ef_sir_run(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const int32_t
         st.heavy = (int32_t *)(b + o_heavy);
         st.fmark = (int32_t *)(b + o_fmark);
         st.tmark = (int32_t *)(b + o_tmark);
-        st.counts = (int32_t *)(b + o_counts);
+        st.flen = (int2 *)(b + o_counts);
+        st.counts = (int32_t *)(b + o_counts + 16);
         st.count = (int32_t *)(b + o_cnt);
         st.peak = (int32_t *)(b + o_peak);
         st.peak_step = (int32_t *)(b + o_pstep);
@@ -1211,11 +1213,11 @@ int ef_sir_run(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const int32_t
         CU(cudaMemsetAsync(st.newinf, 0, words, cs));
         CU(cudaMemsetAsync(st.fmark, 0, 4 * N, cs));
         CU(cudaMemsetAsync(st.tmark, 0, 4 * N, cs));
-        CU(cudaMemsetAsync(st.counts, 0, 16, cs));
+        CU(cudaMemsetAsync(st.flen, 0, 24, cs));
         CU(cudaMemsetAsync(active, 0, 16, cs));
         CU(cudaMemsetAsync(st.err, 0, sizeof(int32_t), cs));
-        LAUNCH(launch_sir_init(index_cases + c0, n, immune, num_immune_sets, immune_set ? immune_set + c0 : nullptr,
-                               st, t, cs),
+        LAUNCH(launch_sir_init(g->row_ptr, index_cases + c0, n, immune, num_immune_sets,
+                               immune_set ? immune_set + c0 : nullptr, st, t, cs),
                "SIR init");
         CU(cudaMemcpyAsync(ctx->h_counters, st.err, sizeof(int32_t), cudaMemcpyDeviceToHost, cs));
         CU(cudaStreamSynchronize(cs));

@@ -590,6 +590,7 @@ constexpr int SIR_BATCH = 1024;
 constexpr int SIR_HUB_MIN = 129;   // rows of at least this take a CTA in a pull step
 struct SirState {
     int32_t B, WB;        // simulations of the batch, words per node
+    int64_t m;            // row entries of the graph
     uint32_t *susc;       // n*WB   susceptible (bit s % 32 of word s / 32)
     uint32_t *inf[2];     // n*WB   infected at the start of this step / of the next
     uint32_t *newinf;     // n*WB   infected during this step
@@ -599,7 +600,8 @@ struct SirState {
     int32_t *touched;     // n      nodes with a successful try this step
     int32_t *heavy;       // n      frontier nodes of high degree this step
     int32_t *fmark, *tmark;   // n  step stamps deduplicating the appends to front and touched
-    int32_t *counts;      // 4      lengths of front[0], front[1], touched, heavy
+    int2 *flen;           // 2      {nodes, their row entries} of front[0] and front[1]
+    int32_t *counts;      // 2      lengths of touched and heavy
     int32_t *count, *peak, *peak_step, *length, *fsize;   // B
     uint8_t *done;        // B      1: no infected node left (or never started)
     int32_t *err;         // error bits (ERRB_SIR_ARG)
@@ -610,7 +612,7 @@ struct SirStep {
     uint64_t beta_thr;    // floor(beta 2^32): a try succeeds when its draw is below
     uint64_t gamma_thr;   // floor(gamma 2^32): recovery
 };
-int launch_sir_init(const int32_t *index_cases, int32_t n, const uint8_t *immune, int32_t num_sets,
+int launch_sir_init(const int32_t *rp, const int32_t *index_cases, int32_t n, const uint8_t *immune, int32_t num_sets,
                     const int32_t *imm_set, const SirState &st, const Tune &t, cudaStream_t s);
 int launch_sir_step(const int32_t *rp, const int32_t *ci, int32_t n, int32_t step, const SirStep &p,
                     const SirState &st, int64_t *active, const Scratch &sc, const Tune &t, cudaStream_t s);

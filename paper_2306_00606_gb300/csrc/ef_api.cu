@@ -644,10 +644,11 @@ int features_device(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n
 // listed node.  Triangles: per listed node (few nodes), or (global_tri) the
 // full oriented triangle pass, which costs less once the list holds the
 // high-EF nodes next to the hubs; orient_done / tri_done: the features
-// already ran the orientation / the whole triangle pass.
+// already ran the orientation / the whole triangle pass; listed: about how
+// many entries the list holds.
 int nodes_device(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const ef::Scratch &s,
                  const int32_t *list, int32_t kmax, const int32_t *kptr, int precision, bool global_tri,
-                 bool orient_done, bool tri_done, const ef_outputs &out, bool timed = false) {
+                 bool orient_done, bool tri_done, const ef_outputs &out, int64_t listed, bool timed = false) {
     using namespace ef;
     cudaStream_t st = ctx->stream;
     if (global_tri && !tri_done) {
@@ -661,11 +662,17 @@ int nodes_device(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n, i
     uint32_t *bits = reinterpret_cast<uint32_t *>(s.out_ptr);
     LAUNCH(launch_bin_nodes(list, kmax, kptr, rp, ci, s, bits, n, ctx->tune, st), "node bins");
     Scratch sl = s;
-    // Credits to the listed nodes only, once the reductions are bound by the
-    // accumulators' traffic: ranking BA with 1M / 2M / 4M / 8M nodes 1.33 / 2.13 /
-    // 3.54 / 6.04 ms against 1.33 / 2.14 / 3.57 / 6.40 with all credits; 2000
-    // chosen nodes of 1M 324 us against 320 (another gather per neighbour).
-    if (n >= 1 << 21) sl.listed = bits;
+    // Credits to the listed nodes only where the reductions are bound by the
+    // accumulators' traffic and enough of them fall away: the test is another
+    // gather per neighbour.  The listed share may be the larger the further the
+    // accumulators (8 n bytes) outgrow L2: up to n / 25M of the nodes.  Ranking BA
+    // in FP32C with 1 / 5 / 10 / 30 / 50 / 100% candidates, filtered against all
+    // credits, ms: 2.5M nodes 2.40 / 2.47 / 2.53 / 2.73 / 2.90 / 3.26 against 2.44 /
+    // 2.49 / 2.54 / 2.72 / 2.88 / 3.21; 4M 3.17 / 3.32 / 3.43 / 3.77 / 4.03 / 4.59
+    // against 3.23 / 3.33 / 3.42 / 3.72 / 3.97 / 4.52; 16M 11.0 / 11.8 / 12.4 / 14.3 /
+    // 15.8 / 19.4 against 12.8 / 13.9 / 14.5 / 15.9 / 16.9 / 19.2.  2000 chosen nodes
+    // of 1M: 324 us against 320.
+    if (n >= 1 << 21 && 25e6 * (double)listed <= (double)n * n) sl.listed = bits;
     LAUNCH(launch_wedge_small(rp, ci, sl, precision, n, ctx->tune, st), "small wedge");
     LAUNCH(launch_wedge_big(rp, ci, sl, precision, 0, n, m, ctx->tune, st), "big wedge");
     if (timed) CU(cudaEventRecord(ctx->ev[9], st));
@@ -1027,7 +1034,7 @@ int ef_compute_nodes(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const i
     rc = prepare_graph(ctx, g->row_ptr, g->col_idx, n, m, o, s, fcap);
     if (rc) return rc;
     rc = nodes_device(ctx, g->row_ptr, g->col_idx, n, m, s, nodes, k, nullptr, o.precision, false, false, false,
-                      *out);
+                      *out, k);
     if (rc) return rc;
     return final_check(ctx, s, !o.trust_input);
 }
@@ -1525,7 +1532,7 @@ int ef_surrogate_rank(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const 
     ef_outputs eo = {};
     eo.ef = r.exact;
     rc = nodes_device(ctx, g->row_ptr, g->col_idx, n, m, s, r.listL, n, kL, o.precision, true, true,
-                      model->feature_mode == 1, eo, stats != nullptr);
+                      model->feature_mode == 1, eo, kc + (int64_t)((double)audit_frac * n), stats != nullptr);
     if (rc) return rc;
     CU(cudaEventRecord(ctx->ev[4], st));
     // the reported top set: largest exact EF among the candidates

@@ -36,3 +36,17 @@ def test_chosen_nodes_match_oracle(ctx, share, pad, precision):  # noqa: F811
     ef.ef_compute_nodes(ctx.handle, _dev(rp), _dev(g.col_idx), _dev(rows), precision=precision, **got)
     ref = {k: v[rows] for k, v in alg1_ref(g).items()}
     assert_parity(_host(got), ref, precision)
+
+
+@pytest.mark.parametrize("past", [0, 1])
+def test_listed_share_at_the_filters_line(ctx, past):  # noqa: F811
+    """The filter is used up to a listed share of n / 25e6: lists (with repeats) on either side, fp64 and fp32c alike."""
+    import paper_2306_00606_gb300 as ef
+    g, n = _graph(), FILTER_FROM
+    rows = np.resize(np.random.default_rng(9).permutation(g.n), int(n * n / 25e6) + past).astype(np.int32)
+    rp = np.concatenate([g.row_ptr, np.full(n - g.n, g.row_ptr[-1])]).astype(np.int32)
+    ref = {k: v[rows] for k, v in alg1_ref(g).items()}
+    for precision in ("fp64", "fp32c"):
+        got = _alloc(len(rows))
+        ef.ef_compute_nodes(ctx.handle, _dev(rp), _dev(g.col_idx), _dev(rows), precision=precision, **got)
+        assert_parity(_host(got), ref, precision)

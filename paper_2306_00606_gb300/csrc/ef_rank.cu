@@ -342,30 +342,39 @@ int launch_select_top(const RankScratch &r, int32_t n, int64_t k, int bits, cons
 // ------------------------------------------------------ exact EF of nodes
 // A bit per listed node (listed), and one per listed node and neighbour of one
 // (mark): the middle nodes whose wedge credits reach a listed node.  Ids
-// outside [0, n) set an error bit.  A warp per listed node, the block for rows
-// above MARK_LONG; a bit that is seen set is left alone (a stale L1 line costs
-// an atomic, nothing else).  Bits instead of an int per node: 2 MB of the L2
-// instead of 64 for 16M nodes, 0.632 -> 0.164 ms
-// (336 000 listed).
-constexpr int MARK_LONG = 512;
+// outside [0, n) set an error bit.  A warp per listed node; rows above
+// MARK_LONG wait for the whole block, after its other nodes (a warp takes them
+// itself once the block has MARK_KEEP of them); a bit that is seen set is left
+// alone (a stale L1 line costs an atomic, nothing else).  Bits instead of an
+// int per node: 2 MB of the L2 instead of 64 for 16M nodes, 0.632 -> 0.164 ms
+// (336 000 listed).  With barriers after every eight nodes, and the listed
+// node's own two bits read before they were set, long lists were slower than
+// with ints: all nodes of BA 4M 0.88 ms (ints 0.60), so 0.57; half of BA 16M
+// 1.93 (1.37), 1.28; 336 000 of BA 16M 0.12, 0.10; all of ER 1M 0.21 (0.09), 0.14.
+constexpr int MARK_LONG = 512, MARK_KEEP = 32;
 
 __global__ void __launch_bounds__(256) k_mark_nbhd(const int32_t *__restrict__ list, int32_t k_max,
                                                    const int32_t *__restrict__ kptr, const int32_t *__restrict__ rp,
                                                    const int32_t *__restrict__ ci, int32_t n, uint32_t *listed,
                                                    uint32_t *mark, int32_t *__restrict__ cnt) {
-    __shared__ int2 s_long[8];
+    __shared__ int3 s_long[MARK_KEEP];   // {row start, length, node}
     __shared__ int s_n;
     const int k = kptr ? *kptr : k_max;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    auto set = [](uint32_t *bits, int x) {
-        if (!(bits[x >> 5] >> (x & 31) & 1)) atomicOr(bits + (x >> 5), 1u << (x & 31));
-    };
-    auto mark_row = [&](int e0, int b, int step) {
-        for (; e0 < b; e0 += 4 * step) {
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x == 0) s_n = 0;
+    __syncthreads();
+    // entries first, first + step, ... of v's row, v itself after the last
+    // (offsets from the row's start stay far below 2^31, indices of the column
+    // array need not)
+    auto mark_row = [&](const int32_t *row, int len, int v, int first, int step) {
+        for (int e0 = first; e0 <= len; e0 += 4 * step) {
             int x[4];
             uint32_t have[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) x[q] = e0 + q * step < b ? ci[e0 + q * step] : -1;
+            for (int q = 0; q < 4; ++q) {
+                const int e = e0 + q * step;
+                x[q] = e < len ? row[e] : e == len ? v : -1;
+            }
 #pragma unroll
             for (int q = 0; q < 4; ++q) have[q] = x[q] >= 0 ? mark[x[q] >> 5] >> (x[q] & 31) & 1 : 1;
 #pragma unroll
@@ -373,26 +382,29 @@ __global__ void __launch_bounds__(256) k_mark_nbhd(const int32_t *__restrict__ l
                 if (!have[q]) atomicOr(mark + (x[q] >> 5), 1u << (x[q] & 31));
         }
     };
-    for (int64_t i0 = (int64_t)blockIdx.x * 8; i0 < k; i0 += (int64_t)gridDim.x * 8) {
-        if (threadIdx.x == 0) s_n = 0;
-        __syncthreads();
-        const int v = i0 + w < k ? list[i0 + w] : 0;
-        if (i0 + w >= k) {
-        } else if (v < 0 || v >= n) {
+    const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+    for (int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < k; i += nwarps) {
+        const int v = list[i];
+        if (v < 0 || v >= n) {
             if (lane == 0) atomicOr(cnt + CNT_ERR, ERRB_NODE);
-        } else {
-            const int a = rp[v], b = rp[v + 1];
-            if (lane == 0) {
-                set(listed, v);
-                set(mark, v);
-                if (b - a > MARK_LONG) s_long[atomicAdd(&s_n, 1)] = make_int2(a, b);
-            }
-            if (b - a <= MARK_LONG) mark_row(a + lane, b, 32);
+            continue;
         }
-        __syncthreads();
-        for (int j = 0; j < s_n; ++j) mark_row(s_long[j].x + threadIdx.x, s_long[j].y, 256);
-        __syncthreads();
+        const int a = rp[v], len = rp[v + 1] - a;
+        if (lane == 0) atomicOr(listed + (v >> 5), 1u << (v & 31));
+        if (len > MARK_LONG) {
+            int at = 0;
+            if (lane == 0) at = atomicAdd(&s_n, 1);
+            at = __shfl_sync(FULL, at, 0);
+            if (at < MARK_KEEP) {
+                if (lane == 0) s_long[at] = make_int3(a, len, v);
+                continue;
+            }
+        }
+        mark_row(ci + a, len, v, lane, 32);
     }
+    __syncthreads();
+    const int kept = min(s_n, MARK_KEEP);
+    for (int j = 0; j < kept; ++j) mark_row(ci + s_long[j].x, s_long[j].y, s_long[j].z, threadIdx.x, 256);
 }
 
 // Work bins holding only the marked nodes (as middle nodes of the wedge

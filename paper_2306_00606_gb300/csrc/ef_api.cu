@@ -660,7 +660,7 @@ int nodes_device(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n, i
     if (timed) CU(cudaEventRecord(ctx->ev[8], st));
     // the out-list offsets are not needed any more: they hold the listed nodes' bits and the marks
     uint32_t *bits = reinterpret_cast<uint32_t *>(s.out_ptr);
-    LAUNCH(launch_bin_nodes(list, kmax, kptr, rp, ci, s, bits, n, ctx->tune, st), "node bins");
+    LAUNCH(launch_bin_nodes(list, kmax, kptr, rp, ci, s, bits, n, !global_tri, ctx->tune, st), "node bins");
     Scratch sl = s;
     // Credits to the listed nodes only where the reductions are bound by the
     // accumulators' traffic and enough of them fall away: the test is another

@@ -166,6 +166,9 @@ enum : int {
     CNT_BIGLO = 46,   // n - 1 - (smallest id of a node of degree > SMALL_MAX), if any
     CNT_BIGHI = 47,   // largest id of a node of degree > SMALL_MAX, if any
     CNT_GATE = 48,    // device-side check: the call's validation bits (0: part B runs), see gate_closed
+    CNT_NODEMANY = 49,   // chosen nodes that take a block, and the next one of them;
+    CNT_NODEBLOCK = 50,  // the next chosen nodes for a warp
+    CNT_NODEWARP = 51,
     NUM_COUNTERS = 64
 };
 
@@ -582,7 +585,7 @@ int launch_features(const Scratch &s, const RankScratch &r, int32_t n, int mode,
                     const ModelDev *std_model = nullptr);
 int launch_select_top(const RankScratch &r, int32_t n, int64_t k, int bits, const Tune &t, cudaStream_t st);
 int launch_bin_nodes(const int32_t *list, int32_t k, const int32_t *kptr, const int32_t *rp, const int32_t *ci,
-                     const Scratch &s, uint32_t *listed, int32_t n, const Tune &t, cudaStream_t st);
+                     const Scratch &s, uint32_t *listed, int32_t n, bool many, const Tune &t, cudaStream_t st);
 int launch_bin_marked(const int32_t *mark, const Scratch &s, int32_t n, const Tune &t, cudaStream_t st);
 // SIR simulation (ef_sir.cu): a batch of at most SIR_BATCH simulations,
 // node-major bit words (WB = ceil(B / 32) per node), frontier lists of nodes.

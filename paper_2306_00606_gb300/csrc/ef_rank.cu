@@ -17,6 +17,8 @@
 // a BA graph for the top 1-2%), so this costs most of a wedge pass.
 #include "ef_internal.cuh"
 
+#include <algorithm>
+
 namespace ef {
 
 // ------------------------------------------------------------------ features
@@ -347,7 +349,8 @@ int launch_select_top(const RankScratch &r, int32_t n, int64_t k, int bits, cons
 // itself once the block has MARK_KEEP of them); a bit that is seen set is left
 // alone (a stale L1 line costs an atomic, nothing else).  Bits instead of an
 // int per node: 2 MB of the L2 instead of 64 for 16M nodes, 0.632 -> 0.164 ms
-// (336 000 listed).  With barriers after every eight nodes, and the listed
+// (336 000 listed).  many (null: not wanted): the list's positions below
+// many_cap that hold a node of more than few neighbours, for k_nodes_final.  With barriers after every eight nodes, and the listed
 // node's own two bits read before they were set, long lists were slower than
 // with ints: all nodes of BA 4M 0.88 ms (ints 0.60), so 0.57; half of BA 16M
 // 1.93 (1.37), 1.28; 336 000 of BA 16M 0.12, 0.10; all of ER 1M 0.21 (0.09), 0.14.
@@ -356,7 +359,8 @@ constexpr int MARK_LONG = 512, MARK_KEEP = 32;
 __global__ void __launch_bounds__(256) k_mark_nbhd(const int32_t *__restrict__ list, int32_t k_max,
                                                    const int32_t *__restrict__ kptr, const int32_t *__restrict__ rp,
                                                    const int32_t *__restrict__ ci, int32_t n, uint32_t *listed,
-                                                   uint32_t *mark, int32_t *__restrict__ cnt) {
+                                                   uint32_t *mark, int32_t *__restrict__ many,
+                                                   int64_t many_cap, int few, int32_t *__restrict__ cnt) {
     __shared__ int3 s_long[MARK_KEEP];   // {row start, length, node}
     __shared__ int s_n;
     const int k = kptr ? *kptr : k_max;
@@ -390,7 +394,10 @@ __global__ void __launch_bounds__(256) k_mark_nbhd(const int32_t *__restrict__ l
             continue;
         }
         const int a = rp[v], len = rp[v + 1] - a;
-        if (lane == 0) atomicOr(listed + (v >> 5), 1u << (v & 31));
+        if (lane == 0) {
+            atomicOr(listed + (v >> 5), 1u << (v & 31));
+            if (many && len > few && i < many_cap) many[atomicAdd(cnt + CNT_NODEMANY, 1)] = (int)i;
+        }
         if (len > MARK_LONG) {
             int at = 0;
             if (lane == 0) at = atomicAdd(&s_n, 1);
@@ -441,9 +448,21 @@ __global__ void k_bin_marked(const void *__restrict__ mark, const int32_t *__res
     }
 }
 
-// listed: 2 ceil(n / 32) words free for this call; the second half holds the marks.
+// The positions of listed nodes of more than nodes_few neighbours go where
+// omega lies (a call that lists them runs no pass that writes it).
+static int32_t *nodes_many(const Scratch &s) { return reinterpret_cast<int32_t *>(s.omega); }
+static int64_t nodes_many_cap(int32_t n) { return 2 * (int64_t)n; }
+
+constexpr int NODE_BLOCKS = 6;   // blocks of k_nodes_final per SM (40 registers)
+
+// Listed nodes of more neighbours than this take a block, the others a warp:
+// all a block while every block has at most one.
+static int nodes_few(int32_t k, const Tune &t) { return k <= t.num_sms * NODE_BLOCKS ? -1 : SMALL_MAX; }
+
+// listed: 2 ceil(n / 32) words free for this call; the second half holds the
+// marks.  many: list those positions.
 int launch_bin_nodes(const int32_t *list, int32_t k, const int32_t *kptr, const int32_t *rp, const int32_t *ci,
-                     const Scratch &s, uint32_t *listed, int32_t n, const Tune &t, cudaStream_t st) {
+                     const Scratch &s, uint32_t *listed, int32_t n, bool many, const Tune &t, cudaStream_t st) {
     const size_t words = ((size_t)n + 31) / 32;
     uint32_t *mark = listed + words;
     if (cudaMemsetAsync(listed, 0, 2 * words * sizeof(uint32_t), st) != cudaSuccess) return -1;
@@ -453,8 +472,9 @@ int launch_bin_nodes(const int32_t *list, int32_t k, const int32_t *kptr, const 
         cudaSuccess)
         return -1;
     const int64_t g = ((int64_t)k + 7) / 8;
-    k_mark_nbhd<<<(unsigned)(g < 1 ? 1 : (g > 8192 ? 8192 : g)), 256, 0, st>>>(list, k, kptr, rp, ci, n, listed, mark,
-                                                                              s.counters);
+    k_mark_nbhd<<<(unsigned)(g < 1 ? 1 : (g > 8192 ? 8192 : g)), 256, 0, st>>>(
+        list, k, kptr, rp, ci, n, listed, mark, many ? nodes_many(s) : nullptr, nodes_many_cap(n),
+        nodes_few(k, t), s.counters);
     k_bin_marked<true><<<t.grid((int64_t)n, 256), 256, 0, st>>>(mark, s.D, n, t.hub_min, s.bins, s.counters);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -480,7 +500,7 @@ __device__ __forceinline__ bool adjacent(const int32_t *rp, const int32_t *ci, i
     return p < len && ci[s + p] == b;
 }
 
-// A CTA per listed node v: triangles at v and their corrections, then EF.
+// Exact EF of listed nodes: triangles at a node v and their corrections, then EF.
 // T_v = Ccenter[v] (middle, open degrees) + Tacc[v] (end, open degrees, from
 // the wedge pass over the marked middle nodes) + corrections.  Triangles are
 // found either as adjacent pairs of N(v) (C(D_v, 2) tests in the shorter
@@ -491,58 +511,193 @@ __device__ __forceinline__ bool adjacent(const int32_t *rp, const int32_t *ci, i
 // 20 000 nodes 812 / 807 / 806 / 838).  omega_v is summed here, from the listed rows only (a
 // pass over every row for it was the call's longest kernel: 2000 nodes of
 // BA 1M 0.598 -> 0.443 ms a call).
+struct NodeArgs {
+    const int32_t *rp, *ci, *D;
+    const int64_t *sig1, *sig2;
+    const void *Ccenter;
+    const double *Tacc;
+    const int64_t *tq;
+    ef_outputs out;
+};
+
+// A node's outputs, position i of the list: t triangles with corrections q (units of 2^-F).
 template <bool F64>
-__global__ void __launch_bounds__(NODE_THREADS) k_nodes_final(
-    const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const int32_t *__restrict__ D,
-    const int64_t *__restrict__ sig1, const int64_t *__restrict__ sig2, const void *__restrict__ Ccenter,
-    const double *__restrict__ Tacc, const int64_t *__restrict__ tq, const int32_t *__restrict__ cnt,
-    const int32_t *__restrict__ list, int32_t k_max, const int32_t *__restrict__ kptr, int32_t n,
-    ef_outputs out) {
+__device__ __forceinline__ void node_out(const NodeArgs &A, int i, int v, int64_t d, int64_t s1, int64_t om, int64_t q,
+                                         int64_t t, int F) {
+    const int64_t s2 = A.sig2[v];
+    const int64_t N = d * (d - 2) + s1;
+    const int64_t S = d * (d - 1) * (d - 4) + 2 * (d - 1) * s1 + s2 - s1 + (d - 4) * (s1 - d) + om - d * d - 8 * t;
+    const double cc = d >= 2 ? (double)reinterpret_cast<const AccT<F64> *>(A.Ccenter)[v] : 0.0;
+    const double T = cc + A.Tacc[v] + ldexp((double)q, -F);
+    double ef = 0.0;
+    uint8_t fl = 1;
+    if (S > 0) {
+        ef = log((double)S) - T / (double)S;
+        fl = 0;
+    }
+    const ef_outputs &o = A.out;
+    if (o.ef) o.ef[i] = ef;
+    if (o.n_clusters) o.n_clusters[i] = N;
+    if (o.s) o.s[i] = S;
+    if (o.t) o.t[i] = T;
+    if (o.triangles) o.triangles[i] = t;
+    if (o.flag) o.flag[i] = fl;
+}
+
+__device__ __forceinline__ bool node_by_pairs(int Dv, int64_t s1v) { return (int64_t)Dv * (Dv - 1) <= s1v; }
+
+// A warp's part of the shared memory: a row of at most SMALL_MAX neighbours,
+// where each neighbour's own row begins in their sequence, and the difference
+// to its place in the column array.
+struct NodeWarpSmem {
+    int32_t row[SMALL_MAX], pre[SMALL_MAX], shift[SMALL_MAX];
+};
+
+// A node by a warp.
+template <bool F64>
+__device__ __forceinline__ void node_warp(const NodeArgs &A, NodeWarpSmem &S, int i, int v, int n, int F) {
+    const int lane = threadIdx.x & 31;
+    const int a = A.rp[v], Dv = A.rp[v + 1] - a;
+    const int64_t s1v = A.sig1[v];
+    const bool by_pairs = node_by_pairs(Dv, s1v), fits = Dv <= SMALL_MAX;
+    const int32_t *row = fits ? S.row : A.ci + a;
+    int64_t om = 0, q = 0, t = 0;
+    __syncwarp();
+    int start = 0, len = 0;   // lane e: the row of neighbour e (of one that fits)
+    for (int e = lane; e < Dv; e += 32) {
+        const int x = A.ci[a + e];
+        if (x < 0 || x >= n) continue;
+        om += A.sig1[x];
+        if (fits) {
+            S.row[e] = x;
+            start = A.rp[x];
+            len = A.rp[x + 1] - start;
+        }
+    }
+    if (fits && !by_pairs) {
+        int inc = len;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += y;
+        }
+        S.pre[lane] = inc - len;
+        S.shift[lane] = start - (inc - len);
+    }
+    __syncwarp();
+    if (by_pairs) {
+        // pairs x < y in lexicographic order, 32 apart per lane
+        int x = 0, y = 1 + lane;
+        for (;;) {
+            while (x < Dv && y >= Dv) {
+                ++x;
+                y += x + 1 - Dv;
+            }
+            if (x >= Dv) break;
+            const int bx = row[x], by = row[y], Dx = A.D[bx], Dy = A.D[by];
+            if (adjacent(A.rp, A.ci, bx, Dx, by, Dy)) {
+                q += __ldg(A.tq + Dv + Dx + Dy);
+                ++t;
+            }
+            y += 32;
+        }
+    } else if (fits) {
+        // the neighbours' rows one after the other, an entry per lane
+        for (int at = lane; at < (int)s1v; at += 32) {
+            int e = 0;   // last neighbour whose row begins at or before at
+#pragma unroll
+            for (int h = SMALL_MAX / 2; h > 0; h >>= 1)
+                if (e + h < Dv && S.pre[e + h] <= at) e += h;
+            const int x = A.ci[S.shift[e] + at];
+            if (x == v) continue;
+            const int p = lower_bound_i32(S.row, Dv, x);
+            if (p < Dv && S.row[p] == x) {
+                q += __ldg(A.tq + Dv + A.D[S.row[e]] + A.D[x]);
+                ++t;
+            }
+        }
+    } else {
+        for (int e = 0; e < Dv; ++e) {
+            const int u = row[e], ua = A.rp[u], Du = A.rp[u + 1] - ua;
+            for (int jj = lane; jj < Du; jj += 32) {
+                const int x = A.ci[ua + jj];
+                if (x == v) continue;
+                const int p = lower_bound_i32(row, Dv, x);
+                if (p < Dv && row[p] == x) {
+                    q += __ldg(A.tq + Dv + Du + A.D[x]);
+                    ++t;
+                }
+            }
+        }
+    }
+    om = warp_sum(om);
+    q = warp_sum(q);
+    t = warp_sum(t);
+    if (lane == 0) node_out<F64>(A, i, v, Dv, s1v, om, by_pairs ? q : q / 2, by_pairs ? t : t / 2, F);
+}
+
+// First the nodes of more than few neighbours (many, filled by k_mark_nbhd), a
+// block each, then the others, a warp each: a row of at most 32 entries
+// streams fewer than 992 entries before testing pairs costs less.  Blocks and
+// warps take their work from counters.  A block per node for all of them, in
+// list order, spent most of its time waiting (two barriers and six dependent
+// loads for ten neighbours), and where its grid did not fit the SMs at once, the
+// second wave doubled the time: all nodes of ER 1M 8.6 ms, so 3.3, of BA 1M 9.1
+// and 3.7, 20 000 of BA 1M 0.81 and 0.65.
+template <bool F64>
+__global__ void __launch_bounds__(NODE_THREADS, NODE_BLOCKS) k_nodes_final(NodeArgs A, int32_t *__restrict__ cnt,
+                                                                           const int32_t *__restrict__ list, int32_t k,
+                                                                           int32_t n, const int32_t *__restrict__ many,
+                                                                           int64_t many_cap, int32_t few,
+                                                                           int32_t chunk) {
+    constexpr int WARPS = NODE_THREADS / 32;
     __shared__ int32_t s_row[NODE_ROW_SMEM];
-    __shared__ long long s_q[NODE_THREADS / 32], s_t[NODE_THREADS / 32], s_om[NODE_THREADS / 32];
+    __shared__ long long s_q[WARPS], s_t[WARPS], s_om[WARPS];
+    __shared__ int s_next;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int F = cnt[CNT_TRIFRAC];
-    const int k = kptr ? *kptr : k_max;
-    for (int i = blockIdx.x; i < k; i += gridDim.x) {
-        const int v = list[i];
-        if (v < 0 || v >= n) continue;   // reported by k_mark_nbhd (the whole CTA skips alike)
-        const int a = rp[v], Dv = rp[v + 1] - a;
-        const int64_t s1v = sig1[v];
-        const bool by_pairs = (int64_t)Dv * (Dv - 1) / 2 * 2 <= s1v;
+    const int nmany = cnt[CNT_NODEMANY];
+    for (int h = blockIdx.x; h < nmany; h = s_next) {
+        int next = 0;
+        if (threadIdx.x == 0) next = (int)gridDim.x + atomicAdd(cnt + CNT_NODEBLOCK, 1);
+        const int i = many[h], v = list[i];
+        const int a = A.rp[v], Dv = A.rp[v + 1] - a;
+        const int64_t s1v = A.sig1[v];
+        const bool by_pairs = node_by_pairs(Dv, s1v);
         const bool staged = !by_pairs && Dv <= NODE_ROW_SMEM;
         if (staged)
-            for (int e = threadIdx.x; e < Dv; e += NODE_THREADS) s_row[e] = ci[a + e];
+            for (int e = threadIdx.x; e < Dv; e += NODE_THREADS) s_row[e] = A.ci[a + e];
         int64_t om = 0;
         for (int e = threadIdx.x; e < Dv; e += NODE_THREADS) {
-            const int x = ci[a + e];
-            if (x >= 0 && x < n) om += sig1[x];
+            const int x = A.ci[a + e];
+            if (x >= 0 && x < n) om += A.sig1[x];
         }
         om = warp_sum(om);
         if (lane == 0) s_om[w] = om;
         __syncthreads();
         int64_t q = 0, t = 0;   // by pairs: each triangle once; by streaming: twice
         if (by_pairs) {
-            for (int x = w; x < Dv; x += NODE_THREADS / 32) {
-                const int bx = ci[a + x], Dx = D[bx];
+            for (int x = w; x < Dv; x += WARPS) {
+                const int bx = A.ci[a + x], Dx = A.D[bx];
                 for (int y = x + 1 + lane; y < Dv; y += 32) {
-                    const int by = ci[a + y], Dy = D[by];
-                    if (adjacent(rp, ci, bx, Dx, by, Dy)) {
-                        q += __ldg(tq + Dv + Dx + Dy);
+                    const int by = A.ci[a + y], Dy = A.D[by];
+                    if (adjacent(A.rp, A.ci, bx, Dx, by, Dy)) {
+                        q += __ldg(A.tq + Dv + Dx + Dy);
                         ++t;
                     }
                 }
             }
         } else {
-            const int32_t *row = staged ? s_row : ci + a;
-            for (int e = w; e < Dv; e += NODE_THREADS / 32) {
+            const int32_t *row = staged ? s_row : A.ci + a;
+            for (int e = w; e < Dv; e += WARPS) {
                 const int u = row[e];
-                const int ua = rp[u], Du = rp[u + 1] - ua;
+                const int ua = A.rp[u], Du = A.rp[u + 1] - ua;
                 for (int jj = lane; jj < Du; jj += 32) {
-                    const int x = ci[ua + jj];
+                    const int x = A.ci[ua + jj];
                     if (x == v) continue;
                     const int p = lower_bound_i32(row, Dv, x);
                     if (p < Dv && row[p] == x) {
-                        q += __ldg(tq + Dv + Du + D[x]);
+                        q += __ldg(A.tq + Dv + Du + A.D[x]);
                         ++t;
                     }
                 }
@@ -554,39 +709,38 @@ __global__ void __launch_bounds__(NODE_THREADS) k_nodes_final(
             s_q[w] = q;
             s_t[w] = t;
         }
+        if (threadIdx.x == 0) s_next = next;
         __syncthreads();
         if (threadIdx.x == 0) {
             int64_t qs = 0, ts = 0;
             om = 0;
-            for (int j = 0; j < NODE_THREADS / 32; ++j) {
+            for (int j = 0; j < WARPS; ++j) {
                 qs += s_q[j];
                 ts += s_t[j];
                 om += s_om[j];
             }
-            if (!by_pairs) {
-                qs /= 2;   // each triangle was found through both of its other nodes
-                ts /= 2;
-            }
-            const int64_t d = Dv, s2 = sig2[v];
-            const int64_t N = d * (d - 2) + s1v;
-            const int64_t S =
-                d * (d - 1) * (d - 4) + 2 * (d - 1) * s1v + s2 - s1v + (d - 4) * (s1v - d) + om - d * d - 8 * ts;
-            const double cc = d >= 2 ? (double)reinterpret_cast<const AccT<F64> *>(Ccenter)[v] : 0.0;
-            const double T = cc + Tacc[v] + ldexp((double)qs, -F);
-            double ef = 0.0;
-            uint8_t fl = 1;
-            if (S > 0) {
-                ef = log((double)S) - T / (double)S;
-                fl = 0;
-            }
-            if (out.ef) out.ef[i] = ef;
-            if (out.n_clusters) out.n_clusters[i] = N;
-            if (out.s) out.s[i] = S;
-            if (out.t) out.t[i] = T;
-            if (out.triangles) out.triangles[i] = ts;
-            if (out.flag) out.flag[i] = fl;
+            // by streaming each triangle was found through both of its other nodes
+            node_out<F64>(A, i, v, Dv, s1v, om, by_pairs ? qs : qs / 2, by_pairs ? ts : ts / 2, F);
         }
         __syncthreads();
+    }
+    if (few < 0 && k <= many_cap) return;   // all nodes are done
+    NodeWarpSmem &S = reinterpret_cast<NodeWarpSmem *>(s_row)[w];
+    static_assert(WARPS * sizeof(NodeWarpSmem) <= sizeof s_row, "the warps' rows lie over the blocks' row");
+    auto take = [&]() {
+        int at = 0;
+        if (lane == 0) at = atomicAdd(cnt + CNT_NODEWARP, 1);
+        return (int64_t)__shfl_sync(FULL, at, 0) * chunk;
+    };
+    for (int64_t i0 = take(); i0 < k;) {
+        const int64_t next = take(), end = min(i0 + chunk, (int64_t)k);
+        for (int64_t i = i0; i < end; ++i) {
+            const int v = list[i];
+            if (v < 0 || v >= n) continue;   // reported by k_mark_nbhd
+            if (i < many_cap && A.rp[v + 1] - A.rp[v] > few) continue;
+            node_warp<F64>(A, S, (int)i, v, n, F);
+        }
+        i0 = next;
     }
 }
 
@@ -625,7 +779,7 @@ __global__ void k_nodes_assemble(const int32_t *__restrict__ D, const int64_t *_
 }
 
 // global_tri: take t and the corrections from the full triangle pass (qacc,
-// tcnt) instead of counting per listed node.
+// tcnt) instead of counting per listed node (kptr: only then).
 int launch_nodes_exact(const int32_t *rp, const int32_t *ci, const Scratch &s, const int32_t *list, int32_t k,
                        const int32_t *kptr, int32_t n, int precision, bool global_tri, const ef_outputs &out,
                        const Tune &t, cudaStream_t st) {
@@ -641,13 +795,17 @@ int launch_nodes_exact(const int32_t *rp, const int32_t *ci, const Scratch &s, c
                                                         s.tcnt, s.counters, list, k, kptr, n, out);
         return cudaGetLastError() == cudaSuccess ? 0 : -1;
     }
-    const unsigned grid = (unsigned)(k < t.num_sms * 8 ? k : t.num_sms * 8);
+    // a listed node per warp at a time on short lists, up to eight on long ones
+    const int slots = t.num_sms * NODE_BLOCKS;
+    const int chunk = std::max(1, std::min(8, k / (slots * NODE_THREADS / 32 * 8)));
+    const unsigned grid = (unsigned)std::min(slots, k);
+    const NodeArgs A{rp, ci, s.D, s.sig1, s.sig2, s.Ccenter, s.Tacc, s.tq, out};
     if (precision == EF_PREC_FP64)
-        k_nodes_final<true><<<grid, NODE_THREADS, 0, st>>>(rp, ci, s.D, s.sig1, s.sig2, s.Ccenter, s.Tacc, s.tq,
-                                                           s.counters, list, k, kptr, n, out);
+        k_nodes_final<true><<<grid, NODE_THREADS, 0, st>>>(A, s.counters, list, k, n, nodes_many(s), nodes_many_cap(n),
+                                                           nodes_few(k, t), chunk);
     else
-        k_nodes_final<false><<<grid, NODE_THREADS, 0, st>>>(rp, ci, s.D, s.sig1, s.sig2, s.Ccenter, s.Tacc,
-                                                            s.tq, s.counters, list, k, kptr, n, out);
+        k_nodes_final<false><<<grid, NODE_THREADS, 0, st>>>(A, s.counters, list, k, n, nodes_many(s),
+                                                            nodes_many_cap(n), nodes_few(k, t), chunk);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

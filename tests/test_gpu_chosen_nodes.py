@@ -50,3 +50,33 @@ def test_listed_share_at_the_filters_line(ctx, past):  # noqa: F811
         got = _alloc(len(rows))
         ef.ef_compute_nodes(ctx.handle, _dev(rp), _dev(g.col_idx), _dev(rows), precision=precision, **got)
         assert_parity(_host(got), ref, precision)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "fp32c"])
+@pytest.mark.parametrize("k", [1, 911, 913, 7297, 58369, 120001])
+def test_nodes_by_warps_and_by_blocks(ctx, k, precision):  # noqa: F811
+    """List lengths around one node per block and around one and two nodes per warp step, over nodes of 0, 1, 2, 31,
+    32 and 33 neighbours and more, triangles by pairs and by streaming; ids outside the graph are refused in each."""
+    import paper_2306_00606_gb300 as ef
+    pairs = synth.from_edges(3000, [(0, j) for j in range(1, 2049)] + [(2100, j) for j in range(2101, 3000)] + [(1, 2)])
+    g = synth.disjoint_union([synth.powerlaw_cm(4000, 2.2, 2, 500, 5), synth.complete(32), synth.complete(33),
+                              synth.complete(34), synth.watts_strogatz(600, 6, 0.2, 6), synth.star(30), synth.path(2),
+                              synth.from_edges(2, []), pairs])
+    ref = alg1_ref(g)
+    rows = np.resize(np.random.default_rng(k).permutation(g.n), k).astype(np.int32)
+    rp, ci, got = _dev(g.row_ptr), _dev(g.col_idx), _alloc(k)
+    ef.ef_compute_nodes(ctx.handle, rp, ci, _dev(rows), precision=precision, **got)
+    assert_parity(_host(got), {key: v[rows] for key, v in ref.items()}, precision)
+    for bad in (-1, g.n):
+        with pytest.raises(ef.EfError):
+            ef.ef_compute_nodes(ctx.handle, rp, ci, _dev(np.append(rows[:-1], bad).astype(np.int32)), **got)
+
+
+def test_list_much_longer_than_the_graph(ctx):  # noqa: F811
+    """From position 2 n on also nodes of more than 32 neighbours go by warps."""
+    import paper_2306_00606_gb300 as ef
+    g = synth.disjoint_union([synth.complete(34), synth.star(40), synth.path(3)])
+    rows = np.tile(np.arange(g.n, dtype=np.int32), 7)
+    got = _alloc(len(rows))
+    ef.ef_compute_nodes(ctx.handle, _dev(g.row_ptr), _dev(g.col_idx), _dev(rows), **got)
+    assert_parity(_host(got), {key: v[rows] for key, v in alg1_ref(g).items()}, "fp64")

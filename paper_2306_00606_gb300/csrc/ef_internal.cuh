@@ -533,6 +533,7 @@ int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, co
 int launch_clear_triangles(const Scratch &s, int32_t n, cudaStream_t st);
 int launch_big_items(const Scratch &s, int32_t n, cudaStream_t st);
 int prepare_kernels();
+int prepare_orient();
 int prepare_final_tables();   // ln table of the finalize (ef_final.cu), once per device
 int64_t device_l2_bytes();   // of the current device (after prepare_kernels ran on it)
 

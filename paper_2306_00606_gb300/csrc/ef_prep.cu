@@ -779,16 +779,23 @@ __device__ __forceinline__ void orient_row_warp(const Orient &o, int u, int ua, 
 // waste most of a wide chunk.  Both forms are launched; the one that does not
 // match the degree pass's counts returns at once.  (WS batch orientation
 // 4.7 -> 4.3 ms with 8; the power-law graph 0.90 -> 1.02 ms with 8.)
-// Entries of one warp step that the staging area of k_orient<CHUNK> holds
-// (20 bytes each, plus four table slots).  Only the eight-record form (graphs
+// Staging area of k_orient<CHUNK>: the entries of one warp step (20 bytes each)
+// and their tables (three slots per entry).  Only the eight-record form (graphs
 // without rows above degree 32) stages: measured on the 4096-graph WS batch,
 // orientation 4.32 -> 2.96 ms; the four-record form (a staging area of 128
 // entries, 5 blocks per SM) was slower on the power-law graph (0.89 -> 0.96
 // ms), BA 16M (2.42 -> 2.55 ms) and BA 1M, where its rows are longer or come
 // from the degree bins and the warp's rows rarely fit, so it writes directly.
+// Dynamic shared memory (49.7 KB): with the 128 entries that fit the static 48
+// KB, a step of 32 nodes of five entries on average does not stage (ER 4M of
+// degree 10: orientation 0.46 ms at 192 entries, 0.68 at 128).
 template <int CHUNK>
-struct OrientCap {
-    static constexpr int value = CHUNK == 8 ? 128 : 0;
+struct OrientSmem {
+    static constexpr int CAP = CHUNK == 8 ? 192 : 0;
+    static constexpr int ENTRIES = CAP > 0 ? CAP : 1, SLOTS = CAP > 0 ? 3 * CAP + 2 * BUCKET : 1;
+    int2 pd[8][ENTRIES];
+    int32_t col[8][ENTRIES], D[8][ENTRIES], src[8][ENTRIES], tab[8][SLOTS];
+    static constexpr size_t bytes() { return CAP > 0 ? sizeof(OrientSmem) : 0; }
 };
 
 template <int CHUNK>
@@ -798,11 +805,10 @@ __global__ void __launch_bounds__(256, CHUNK == 8 ? 3 : 5) k_orient(
     const int32_t *__restrict__ out_ptr, const int32_t *__restrict__ outdeg, int64_t *__restrict__ omega) {
     if (gate_closed(cnt)) return;
     if ((cnt[BIN_BIG] == 0) != (CHUNK == 8)) return;
-    constexpr int CAP = OrientCap<CHUNK>::value;
-    constexpr int SCAP = CAP > 0 ? CAP : 1, TCAP = CAP > 0 ? 3 * CAP + 2 * BUCKET : 1;
+    constexpr int CAP = OrientSmem<CHUNK>::CAP;
     __shared__ RowOrder s_ord;
-    __shared__ int32_t s_col[8][SCAP], s_D[8][SCAP], s_src[8][SCAP], s_tab[8][TCAP];
-    __shared__ int2 s_pd[8][SCAP];
+    extern __shared__ __align__(16) unsigned char orient_smem[];
+    OrientSmem<CHUNK> &S = *reinterpret_cast<OrientSmem<CHUNK> *>(orient_smem);   // (only with CAP > 0)
     if (threadIdx.x == 0) s_ord.load(cnt, n, bins_ok);
     __syncthreads();
     const RowOrder &ord = s_ord;
@@ -834,18 +840,18 @@ __global__ void __launch_bounds__(256, CHUNK == 8 ? 3 : 5) k_orient(
             const int64_t tb0 = table_base(kmin);
             const int64_t tb1 = table_base(kend);
             const int tlen = (int)(tb1 - tb0);
-            for (int t = lane; t < tlen; t += 32) s_tab[w][t] = -1;
+            for (int t = lane; t < tlen; t += 32) S.tab[w][t] = -1;
             __syncwarp();
-            const OrientStage sg{s_col[w], s_D[w], s_src[w], s_pd[w], s_tab[w], kmin, tb0};
+            const OrientStage sg{S.col[w], S.D[w], S.src[w], S.pd[w], S.tab[w], kmin, tb0};
             if (mine) omega[v] = o.template row<CHUNK>(v, Dv, a, b, k0, &sg);
             __syncwarp();
             for (int t = lane; t < sum; t += 32) {
-                o.out_col[kmin + t] = s_col[w][t];
-                o.out_D[kmin + t] = s_D[w][t];
-                o.out_src[kmin + t] = s_src[w][t];
-                o.out_pd[kmin + t] = s_pd[w][t];
+                o.out_col[kmin + t] = S.col[w][t];
+                o.out_D[kmin + t] = S.D[w][t];
+                o.out_src[kmin + t] = S.src[w][t];
+                o.out_pd[kmin + t] = S.pd[w][t];
             }
-            for (int t = lane; t < tlen; t += 32) o.out_hash[tb0 + t] = s_tab[w][t];
+            for (int t = lane; t < tlen; t += 32) o.out_hash[tb0 + t] = S.tab[w][t];
             __syncwarp();
         } else if (mine) {
             omega[v] = o.template row<CHUNK>(v, Dv, a, b, k0);
@@ -1188,6 +1194,14 @@ __global__ void __launch_bounds__(256) k_clear_lists(int32_t *__restrict__ hash,
     }
 }
 
+// Opt the staging orientation in to its shared memory on the current device.
+int prepare_orient() {
+    return cudaFuncSetAttribute(k_orient<8>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)OrientSmem<8>::bytes()) == cudaSuccess
+               ? 0
+               : -1;
+}
+
 // Oriented CSR and omega.
 int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const Scratch &s, const Tune &t,
                   cudaStream_t st, int32_t *nmin, int32_t *nmax, bool bins, bool gated, bool big_rows) {
@@ -1214,9 +1228,9 @@ int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, co
                                                          rows_in_bins_allowed(m), s.counters, s.out_ptr, s.outdeg,
                                                          s.omega);
     if (!big_rows)
-        k_orient<8><<<t.grid((int64_t)n, 256), 256, 0, st>>>(rp, n, m, t.row_thread_max, t.hub_min, o, s.D, s.bins,
-                                                             rows_in_bins_allowed(m), s.counters, s.out_ptr,
-                                                             s.outdeg, s.omega);
+        k_orient<8><<<t.grid((int64_t)n, 256), 256, OrientSmem<8>::bytes(), st>>>(
+            rp, n, m, t.row_thread_max, t.hub_min, o, s.D, s.bins, rows_in_bins_allowed(m), s.counters, s.out_ptr,
+            s.outdeg, s.omega);
     k_orient_hub<<<t.num_sms * 4, ROW_CTA, 0, st>>>(rp, n, o, s.bins, s.out_ptr, s.counters, s.omega);
     if (bins && t.row_thread_max >= SMALL_MAX)
         k_hash_tail<<<(unsigned)(t.num_sms * 16), 256, 0, st>>>(s.counters, s.lay_ptr, s.out_ptr, n, s.info,

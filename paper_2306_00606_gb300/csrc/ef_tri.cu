@@ -352,11 +352,15 @@ __global__ void __launch_bounds__(TL_WARPS * 32, 4) k_tri_long(
     const int total = cnt[CNT_TRILONG];
     const int a_lo = owner_range ? owner_range[0] : 0, a_hi = owner_range ? owner_range[1] : n;
     const int4 *cols = reinterpret_cast<const int4 *>(out_col), *table = reinterpret_cast<const int4 *>(out_hash);
-    for (;;) {
+    // the first item by position, the others from the counter (an atomic by every
+    // warp before its first item cost a graph without long owners 3 us a call)
+    const int nwarps = gridDim.x * TL_WARPS;
+    auto take = [&]() {
         int it = 0;
-        if (lane == 0) it = atomicAdd(cnt + CNT_TRINEXT, 1);
-        it = __shfl_sync(FULL, it, 0);
-        if (it >= total) break;
+        if (lane == 0) it = nwarps + atomicAdd(cnt + CNT_TRINEXT, 1);
+        return __shfl_sync(FULL, it, 0);
+    };
+    for (int it = blockIdx.x * TL_WARPS + w; it < total; it = take()) {
         const int2 item = items[total - 1 - it];
         const int a = item.x;
         if (a < a_lo || a >= a_hi) continue;

@@ -114,17 +114,17 @@ enum PathMode { PATH_GENERAL, PATH_SHORT, PATH_DEVICE };
 
 // Kernels one call launches: part A 3 (the batch check runs in the row pass),
 // f table 1; on the short-row path the fused kernel and its finalize; on the
-// general one the orientation (degree-bin layout: layout
-// gather, a scan of 3, layout scatter; node layout: a scan of 3; then node
-// records, the row kernel in two forms of which one returns at once, the hub
-// rows, hash tables of the longer rows; the short rows' tables are filled by
-// the row kernel itself), small wedges 4, big wedges (class kernels 2; direct
-// mode: item counts, a scan of 3, direct kernel, reduction), pair tests 1,
-// with long out-lists 3, finalize 1; both sets, the clearing kernel and the gate where the
-// device decides.
+// general one the orientation (degree-bin layout: layout gather, a scan of 3,
+// layout scatter; node layout: a scan of 3; then node records, the row kernel,
+// the hub rows, hash tables of the longer rows; the short rows' tables are
+// filled by the row kernel itself), small wedges 4, big wedges (class kernels
+// 2; direct mode: item counts, a scan of 3, direct kernel, reduction), pair
+// tests 1, with long out-lists 3, finalize 1.  Where the device decides: the
+// general ones, whose finalize serves both paths, the fused kernel, the
+// clearing kernel and the gate.
 int64_t kernels_per_call(PathMode path, bool bins, int wedge_mode, bool long_lists) {
     const int64_t general = (bins ? 5 : 3) + 4 + 4 + (wedge_mode == 1 ? 6 : 2) + (long_lists ? 3 : 1) + 1;
-    return 3 + 1 + (path != PATH_GENERAL ? 2 : 0) + (path != PATH_SHORT ? general : 0) + (path == PATH_DEVICE ? 2 : 0);
+    return 3 + 1 + (path == PATH_SHORT ? 2 : path == PATH_DEVICE ? general + 3 : general);
 }
 
 void set_err(ef_ctx *c, const char *fmt, ...) {

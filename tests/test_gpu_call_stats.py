@@ -1,0 +1,63 @@
+"""What ef_get_stats says of profiled calls: the kernels that a call launches,
+against the launches that the CUDA profiler records, for every path a call can
+take and every way it is decided."""
+import json
+
+import numpy as np
+import pytest
+
+import synth
+from test_gpu_device_check import _alloc, _dev, ctx  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+MODES = {"host": {}, "device": {"device_check": True}, "trusted": {"trust_input": True}}
+GRAPHS = {
+    "short": lambda: synth.watts_strogatz(3000, 8, 0.1, 1),
+    "no_long_lists": lambda: synth.barabasi_albert(3000, 5, 2),
+    "long_lists": lambda: synth.disjoint_union([synth.complete(90), synth.powerlaw_cm(4000, 2.1, 2, 700, 3)]),
+}
+
+
+def _recorded(fn, tmp_path):
+    """Names of the kernels launched by fn (None when no kernel can be recorded here)."""
+    import torch
+    from torch.profiler import ProfilerActivity, profile
+
+    def record(f):
+        with profile(activities=[ProfilerActivity.CUDA]) as p:
+            f()
+            torch.cuda.synchronize()
+        p.export_chrome_trace(str(tmp_path / "trace.json"))
+        return [e["name"] for e in json.load(open(tmp_path / "trace.json"))["traceEvents"] if e.get("cat") == "kernel"]
+
+    x = torch.ones(8, device="cuda")
+    for _ in range(3):   # the first session may record nothing
+        if record(lambda: x.add_(1)):
+            return record(fn)
+    return None
+
+
+@pytest.mark.parametrize("wedge_mode", [0, 1])
+@pytest.mark.parametrize("mode", list(MODES))
+@pytest.mark.parametrize("name", list(GRAPHS))
+def test_kernels_of_a_call(ctx, tmp_path, name, mode, wedge_mode):  # noqa: F811
+    import paper_2306_00606_gb300 as ef
+    g = GRAPHS[name]()
+    rp, ci, res = _dev(g.row_ptr), _dev(g.col_idx), _alloc(g.n)
+
+    def call():
+        ef.ef_compute_ex(ctx.handle, rp, ci, precision="fp32c", profile=True, wedge_mode=wedge_mode, **MODES[mode], **res)
+
+    for layout in (1, 2):
+        before = ef.ef_get_tuning(ctx.handle)
+        ef.ef_set_tuning(ctx.handle, dict(before, layout=layout))
+        try:
+            call()
+            ctx.stats(reset=True)
+            names = _recorded(call, tmp_path)
+            if names is None:
+                pytest.skip("no kernel records on this machine")
+            assert len(names) == ctx.stats(reset=True)["kernels"], sorted(names)
+        finally:
+            ef.ef_set_tuning(ctx.handle, before)

@@ -147,7 +147,9 @@ typedef struct {
                               CSR + out-list hash tables) and omega */
     double wedge_small_ms; /* middle nodes of degree <= 32; where no node has
                               more neighbours also the triangles (one kernel;
-                              orient_ms is then the f table alone) */
+                              orient_ms is then the f table alone, with
+                              trust_input or device_check also the launches
+                              of kernels that return at once) */
     double wedge_big_ms;   /* middle nodes of degree > 32 */
     double tri_hash_ms;    /* always 0: the orientation builds the hash
                               tables of the long out-lists (orient_ms) */

@@ -254,7 +254,7 @@ int part_a(ef_ctx *ctx, const Job &j, const ef::Scratch &s, cudaStream_t st, boo
 }
 
 // Part B; with prof, events 1..4, 6, 7 bracket f table + orientation (with
-// the hash tables), pair tests, small wedges (on the short-row path the fused
+// the hash tables), pair tests, small wedges (with the short-row path's fused
 // kernel), big wedges and finalize.
 int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, PathMode path, bool prof,
            cudaStream_t st) {
@@ -263,14 +263,13 @@ int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, PathMo
     // the f table's capacity covers both paths; behind a gate closed by
     // GATE_SHORT alone it is still built
     LAUNCH(launch_ftab(s.ftab, s.tq, s.counters, fcap, st), "f table");
-    if (path != PATH_GENERAL) {
-        const bool chosen = path == PATH_SHORT;
+    if (path == PATH_SHORT) {
         if (prof)
             for (int e : {2, 3}) CU(cudaEventRecord(ctx->ev[e], st));
-        LAUNCH(launch_short(j.ci, s, j.o.precision, j.n, t, chosen, st), "short rows");
-        if (prof && chosen)
+        LAUNCH(launch_short(j.ci, s, j.o.precision, j.n, t, true, st), "short rows");
+        if (prof)
             for (int e : {4, 6}) CU(cudaEventRecord(ctx->ev[e], st));
-        if (chosen) return EF_OK;
+        return EF_OK;
     }
     const bool gated = path == PATH_DEVICE;
     if (!gated) LAUNCH(launch_clear_triangles(s, j.n, st), "clear");
@@ -280,6 +279,7 @@ int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, PathMo
     // before the wedges, whose hub classes lie over the oriented lists
     LAUNCH(launch_tri_pairs(s, j.n, j.m, t, st, nullptr, gated || ctx->long_lists), "triangle");
     if (prof) CU(cudaEventRecord(ctx->ev[3], st));
+    if (gated) LAUNCH(launch_short(j.ci, s, j.o.precision, j.n, t, false, st), "short rows");
     LAUNCH(launch_wedge_small(j.rp, j.ci, s, j.o.precision, j.n, t, st), "small wedge");
     if (prof) CU(cudaEventRecord(ctx->ev[4], st));
     LAUNCH(launch_wedge_big(j.rp, j.ci, s, j.o.precision, j.o.wedge_mode, j.n, j.m, t, st), "big wedge");

@@ -1,6 +1,7 @@
 """What ef_get_stats says of profiled calls: the kernels that a call launches,
 against the launches that the CUDA profiler records, for every path a call can
-take and every way it is decided."""
+take and every way it is decided; and the pass that the fused kernel of graphs
+without long rows is booked under."""
 import json
 
 import numpy as np
@@ -61,3 +62,16 @@ def test_kernels_of_a_call(ctx, tmp_path, name, mode, wedge_mode):  # noqa: F811
             assert len(names) == ctx.stats(reset=True)["kernels"], sorted(names)
         finally:
             ef.ef_set_tuning(ctx.handle, before)
+
+
+@pytest.mark.parametrize("mode", list(MODES))
+def test_fused_kernel_is_booked_as_small_wedges(ctx, mode):  # noqa: F811
+    """2M nodes: about 0.4 ms of fused kernel beside an f table and launches of 0.1 ms at most."""
+    import paper_2306_00606_gb300 as ef
+    g = synth.watts_strogatz(2_000_000, 8, 0.1, 1)
+    rp, ci, res = _dev(g.row_ptr), _dev(g.col_idx), _alloc(g.n)
+    for _ in range(3):
+        ctx.stats(reset=True)
+        ef.ef_compute_ex(ctx.handle, rp, ci, profile=True, **MODES[mode], **res)
+    st = ctx.stats(reset=True)
+    assert st["wedge_small_ms"] > 2 * (st["orient_ms"] + st["tri_pairs_ms"] + st["wedge_big_ms"]), st

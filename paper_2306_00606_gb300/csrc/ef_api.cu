@@ -8,8 +8,8 @@
 //            check that no entry leaves its graph, in the same row pass
 //   host     one small readback: validation word, symmetry sum and max
 //            degree (skipped with trust_input); part B runs on valid input only
-//            (device_check: no readback here; a one-thread kernel stores the
-//            validation bits where every kernel of part B reads them, so part B
+//            (device_check: no readback here; the f table's kernel stores the
+//            validation bits where every later kernel of part B reads them, so it
 //            does nothing on invalid input, and the host reads the bits once
 //            the call's work is done)
 //   part B   f table (f(d) = d ln d and the triangle corrections, d < 3 maxdeg + 1);
@@ -120,11 +120,11 @@ enum PathMode { PATH_GENERAL, PATH_SHORT, PATH_DEVICE };
 // filled by the row kernel itself), small wedges 4, big wedges (class kernels
 // 2; direct mode: item counts, a scan of 3, direct kernel, reduction), pair
 // tests 1, with long out-lists 3, finalize 1.  Where the device decides: the
-// general ones, whose finalize serves both paths, the fused kernel, the
-// clearing kernel and the gate.
+// general ones, whose finalize serves both paths, the fused kernel and the
+// clearing kernel (the f table's decides).
 int64_t kernels_per_call(PathMode path, bool bins, int wedge_mode, bool long_lists) {
     const int64_t general = (bins ? 5 : 3) + 4 + 4 + (wedge_mode == 1 ? 6 : 2) + (long_lists ? 3 : 1) + 1;
-    return 3 + 1 + (path == PATH_SHORT ? 2 : path == PATH_DEVICE ? general + 3 : general);
+    return 3 + 1 + (path == PATH_SHORT ? 2 : path == PATH_DEVICE ? general + 2 : general);
 }
 
 void set_err(ef_ctx *c, const char *fmt, ...) {
@@ -262,7 +262,10 @@ int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, PathMo
     const Tune &t = ctx->tune;
     // the f table's capacity covers both paths; behind a gate closed by
     // GATE_SHORT alone it is still built
-    LAUNCH(launch_ftab(s.ftab, s.tq, s.counters, fcap, st), "f table");
+    const GateMode decide = path != PATH_DEVICE ? GateMode::host : j.o.trust_input ? GateMode::trusted : GateMode::checked;
+    LAUNCH(launch_ftab(s.ftab, s.tq, s.counters, fcap, st, decide,
+                       decide == GateMode::checked && j.o.async ? ctx->d_sticky : nullptr),
+           "f table");
     if (path == PATH_SHORT) {
         if (prof)
             for (int e : {2, 3}) CU(cudaEventRecord(ctx->ev[e], st));
@@ -345,12 +348,6 @@ int compute_device(ef_ctx *ctx, const Job &j) {
     const bool dev_check = o.device_check != 0 && !o.trust_input;
     // part A in the same stream as part B, with no host decision between them
     const bool a_inline = o.trust_input || dev_check;
-    auto part_a_inline = [&](cudaStream_t cs) -> int {
-        int r = part_a(ctx, j, s, cs, true);
-        if (!r)
-            LAUNCH(launch_gate(s.counters, dev_check && o.async ? ctx->d_sticky : nullptr, dev_check, cs), "gate");
-        return r;
-    };
     PathMode path = PATH_DEVICE;
 
     // f table size: from the validated max degree, else the largest possible
@@ -405,7 +402,7 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         memcpy(ctx->gouts, outs, sizeof outs);
         rc = run_graph(ctx, key, same_outputs, [&](cudaStream_t cs) {
             if (a_inline) {
-                const int r = part_a_inline(cs);
+                const int r = part_a(ctx, j, s, cs, true);
                 if (r) return r;
             }
             return part_b(ctx, j, s, fcap, path, false, cs);
@@ -415,7 +412,7 @@ int compute_device(ef_ctx *ctx, const Job &j) {
     } else {
         if (a_inline) {
             if (prof) CU(cudaEventRecord(ctx->ev[0], st));
-            rc = part_a_inline(st);
+            rc = part_a(ctx, j, s, st, true);
             if (rc) return rc;
         }
         if (prof) CU(cudaEventRecord(ctx->ev[1], st));

@@ -205,9 +205,9 @@ inline int prep_error_bits(const int32_t *h) {
 size_t carve_scratch(char *base, int32_t n, int64_t m, Scratch &s);
 
 // ----------------------------------------------------------------- helpers
-// Device-side validation (ef_options.device_check): k_gate stores the call's
-// validation bits in cnt[CNT_GATE] once the row passes are done, and every
-// kernel after them returns at once when they are set, so nothing indexes by
+// Device-side validation (ef_options.device_check): k_ftab stores the call's
+// validation bits in cnt[CNT_GATE] once the row passes are done, and it and every
+// kernel after it return at once when they are set, so nothing indexes by
 // the column ids (or by anything derived from them) of a graph that failed.
 // The word is 0 in every other mode: the counters start at zero each call,
 // and the host refuses an invalid graph before part B.
@@ -545,12 +545,14 @@ inline bool rows_in_bins_allowed(int64_t m) { return 4 * m <= device_l2_bytes() 
 // cnt: the counters, when the scan is to be skipped behind a closed gate.
 int launch_scan(const int32_t *in, int32_t *out, int32_t n, int32_t *tmp, cudaStream_t st,
                 const int32_t *cnt = nullptr);
-int launch_ftab(float2 *ftab, int64_t *tq, int32_t *cnt, int64_t cap, cudaStream_t st);
-// Device-side decisions after the row passes: with check, the validation
-// bits (error word, symmetry sum, maximum degree above EF_MAX_DEGREE) into
-// cnt[CNT_GATE], and OR-ed into *sticky when it is not null; GATE_SHORT when
-// no row exceeds SMALL_MAX entries.
-int launch_gate(int32_t *cnt, int32_t *sticky, bool check, cudaStream_t st);
+// Who decides what part B does: the host, after its readback, or the f table's
+// kernel, which then stores the gate word in cnt[CNT_GATE]: the validation
+// bits (checked: error word, symmetry sum, maximum degree above EF_MAX_DEGREE;
+// OR-ed into *sticky when it is not null), and GATE_SHORT when no row exceeds
+// SMALL_MAX entries.
+enum class GateMode { host, checked, trusted };
+int launch_ftab(float2 *ftab, int64_t *tq, int32_t *cnt, int64_t cap, cudaStream_t st,
+                GateMode decide = GateMode::host, int32_t *sticky = nullptr);
 // Short-row path (ef_short.cu, ef_final.cu); chosen: by the host (else the
 // kernels look for GATE_SHORT).
 int launch_short(const int32_t *ci, const Scratch &s, int precision, int32_t n, const Tune &t, bool chosen,

@@ -1009,8 +1009,26 @@ __global__ void k_big_chunks(const int32_t *__restrict__ D, const int32_t *__res
 // block 0 publishes it for the finalize pass.
 constexpr int FTAB_BLOCK = 256;
 
-__global__ void k_ftab(float2 *__restrict__ ftab, int64_t *__restrict__ tq, int32_t *__restrict__ cnt, int64_t cap) {
-    if (cnt[CNT_GATE] & ~GATE_SHORT) return;   // both paths read the tables
+// Where the call's path is decided on the device (decide), every block derives
+// the gate word from the row passes' counters and block 0 publishes it (a
+// kernel of one thread for it before cost 1.5 us a call).
+__global__ void k_ftab(float2 *__restrict__ ftab, int64_t *__restrict__ tq, int32_t *__restrict__ cnt, int64_t cap,
+                       GateMode decide, int32_t *__restrict__ sticky) {
+    int gate = 0;   // (unless decided here, 0 whenever part B runs)
+    if (decide != GateMode::host) {
+        unsigned long long sym;
+        memcpy(&sym, cnt + CNT_SYM, sizeof sym);
+        const int bits = decide == GateMode::trusted
+                             ? 0
+                             : cnt[CNT_ERR] | (sym ? ERRB_ASYM : 0) |
+                                   (cnt[CNT_MAXDEG] > EF_MAX_DEGREE ? ERRB_DEGREE : 0);
+        gate = bits | (cnt[BIN_BIG] == 0 ? GATE_SHORT : 0);
+        if (blockIdx.x == 0 && threadIdx.x == 0) {
+            cnt[CNT_GATE] = gate;
+            if (bits && sticky) atomicOr(sticky, bits);
+        }
+    }
+    if (gate & ~GATE_SHORT) return;   // both paths read the tables
     const int64_t maxdeg = cnt[CNT_MAXDEG];
     int64_t L = 3 * maxdeg + 1;
     if (L > cap) L = cap;
@@ -1123,26 +1141,12 @@ int launch_scan(const int32_t *in, int32_t *out, int32_t n, int32_t *tmp, cudaSt
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-__global__ void k_gate(int32_t *__restrict__ cnt, int32_t *__restrict__ sticky, bool check) {
-    unsigned long long sym;
-    memcpy(&sym, cnt + CNT_SYM, sizeof sym);
-    const int bits = !check ? 0
-                            : cnt[CNT_ERR] | (sym ? ERRB_ASYM : 0) |
-                                  (cnt[CNT_MAXDEG] > EF_MAX_DEGREE ? ERRB_DEGREE : 0);
-    cnt[CNT_GATE] = bits | (cnt[BIN_BIG] == 0 ? GATE_SHORT : 0);
-    if (bits && sticky) atomicOr(sticky, bits);
-}
-
-int launch_gate(int32_t *cnt, int32_t *sticky, bool check, cudaStream_t st) {
-    k_gate<<<1, 1, 0, st>>>(cnt, sticky, check);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
-}
-
-int launch_ftab(float2 *ftab, int64_t *tq, int32_t *cnt, int64_t cap, cudaStream_t st) {
+int launch_ftab(float2 *ftab, int64_t *tq, int32_t *cnt, int64_t cap, cudaStream_t st, GateMode decide,
+                int32_t *sticky) {
     int64_t blocks = (cap + FTAB_BLOCK - 1) / FTAB_BLOCK;
     if (blocks > 1024) blocks = 1024;
     if (blocks < 1) blocks = 1;
-    k_ftab<<<(unsigned)blocks, FTAB_BLOCK, 0, st>>>(ftab, tq, cnt, cap);
+    k_ftab<<<(unsigned)blocks, FTAB_BLOCK, 0, st>>>(ftab, tq, cnt, cap, decide, sticky);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 

@@ -103,16 +103,15 @@ typedef struct {
     int32_t graph;         /* 1: run the passes that need no host decision as
                               one CUDA graph, captured on the first call and
                               replayed while the graph's pointers, sizes,
-                              options and tuning stay the same; the output
-                              buffers may change from call to call, the
-                              finalize that writes them is launched after the
-                              graph (ignored with profile) */
+                              options and tuning stay the same; a call with
+                              other output buffers sets them in the captured
+                              graph first (ignored with profile) */
     int32_t device_check;  /* 1: validate on the device with no readback in
                               the middle of the call (ignored with
                               trust_input).  The kernels after the
                               validation do nothing when it failed, so the
                               whole call -- validation included -- is one
-                              CUDA graph and the finalize with graph = 1.  A synchronous call
+                              CUDA graph with graph = 1.  A synchronous call
                               reads the validation result once at its end and
                               returns EF_ERR_GRAPH or EF_ERR_UNSUPPORTED as
                               without device_check; with async the next
@@ -157,8 +156,9 @@ typedef struct {
     double finalize_ms;    /* per-node sums, S, N, EF */
     double total_ms;
     int64_t kernels;       /* kernels launched by profiled calls */
-    int64_t graph_replays; /* calls served by replaying a cached CUDA graph,
-                              with the output buffers of the call before */
+    int64_t graph_replays; /* calls served by replaying a cached CUDA graph as
+                              it was (not those that set other output buffers
+                              in it) */
 } ef_stats;
 
 /* Launch parameters (every choice gives the same results; see ef_autotune). */
@@ -235,7 +235,7 @@ int ef_compute_ex(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m,
  * Validation (unless trust_input) is ef_compute_ex's plus the check that no
  * entry leaves its graph (EF_ERR_GRAPH "edge-between-graphs").  With
  * opt->graph = 1 the passes run as one replayed CUDA graph (with
- * trust_input, the whole call is one graph launch and the finalize).
+ * trust_input, the whole call is one graph launch).
  */
 int ef_compute_batched(ef_ctx *ctx, const ef_csr *g, int64_t m,
                        const int64_t *graph_off, int32_t num_graphs,

@@ -25,10 +25,10 @@
 // than doubles under contention), so they run in sequence.
 //
 // CUDA graphs (ef_options.graph): the part that needs no host decision --
-// part B, or parts A and B together under trust_input or device_check, all
-// but the finalize -- is captured once on a private stream and replayed into
-// the context stream while the input pointers, sizes, options and tuning stay
-// the same (one cached graph per context).
+// part B, or parts A and B together under trust_input or device_check -- is
+// captured once on a private stream and replayed into the context stream while
+// the input pointers, sizes, options and tuning stay the same (one cached graph
+// per context; other output buffers are set in the finalize's node).
 #include "ef_internal.cuh"
 
 #include <algorithm>
@@ -45,10 +45,10 @@ namespace {
 
 // What a captured graph depends on: replayed only when every byte matches
 // (the layout has no padding; keys are zero-filled before use).  The output
-// buffers are not in it: the finalize pass, the only one that writes them, is
-// launched after the graph, so calls whose outputs come from an allocator
-// (another buffer each time) replay too (R-MAT 2^16: 0.15 ms a call for the
-// capture and instantiation, 2 us for the launch).
+// buffers are not in it: a call with others sets them in the node of the
+// finalize pass, the only one that writes them, before its launch, so calls
+// whose outputs come from an allocator (another buffer each time) need no
+// capture and instantiation (R-MAT 2^16: 0.15 ms a call).
 struct GraphKey {
     const void *rp, *ci, *goff_dev, *scratch, *ftab;
     int64_t m, fcap;
@@ -82,8 +82,10 @@ struct ef_ctx {
     ef_stats stats = {};
     ef::Tune tune;
     cudaGraphExec_t gexec = nullptr;
+    cudaGraph_t graph = nullptr;     // what gexec was instantiated from, and its finalize node
+    cudaGraphNode_t gfinal = nullptr;
+    ef_outputs gouts = {};           // the output buffers in that node
     GraphKey gkey;   // zero-filled in ef_ctx_create
-    const void *gouts[6] = {};       // output buffers of the last graph call (only to count replays)
     void *rank = nullptr;            // learned-path buffers (RankScratch)
     size_t rank_bytes = 0;
     double *dtmp = nullptr;          // small device scratch (feature sums)
@@ -158,7 +160,10 @@ inline size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 
 void drop_graph(ef_ctx *ctx) {
     if (ctx->gexec) cudaGraphExecDestroy(ctx->gexec);
+    if (ctx->graph) cudaGraphDestroy(ctx->graph);
     ctx->gexec = nullptr;
+    ctx->graph = nullptr;
+    ctx->gfinal = nullptr;
     memset(&ctx->gkey, 0, sizeof ctx->gkey);
 }
 
@@ -290,40 +295,46 @@ int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, PathMo
     return EF_OK;
 }
 
-// The per-node outputs, after part B.
-int part_c(ef_ctx *ctx, const Job &j, const ef::Scratch &s, PathMode path, cudaStream_t st) {
-    using namespace ef;
-    if (path != PATH_GENERAL)
-        LAUNCH(launch_finalize_short(s, j.o.precision, j.n, j.out, ctx->tune, path == PATH_SHORT, st), "finalize");
-    else LAUNCH(launch_finalize(s, j.o.precision, j.n, j.out, ctx->tune, st), "finalize");
-    return EF_OK;
-}
-
-// Capture fn(capture stream) into the context's graph unless the cached one
-// has the same key; then launch it into the context stream.  A replay is
-// counted when the call's output buffers are also those of the call before.
+// Launch the context's graph into its stream.  Unless the cached one has the
+// same key, fn(capture stream) is captured first, with fin at its end; a cached
+// one with other output buffers gets fin's parameters.  A replay is counted
+// when neither was needed.
 template <typename F>
-int run_graph(ef_ctx *ctx, const GraphKey &key, bool same_outputs, F &&fn) {
+int run_graph(ef_ctx *ctx, const GraphKey &key, const ef::FinalizeCall &fin, F &&fn) {
+    static_assert(sizeof(ef_outputs) == 6 * sizeof(void *), "ef_outputs has padding");
     if (!(ctx->gexec && ctx->gkey == key)) {
         drop_graph(ctx);
         CU(cudaStreamBeginCapture(ctx->capture, cudaStreamCaptureModeThreadLocal));
-        const int rc = fn(ctx->capture);
-        cudaGraph_t g = nullptr;
-        const cudaError_t e = cudaStreamEndCapture(ctx->capture, &g);
-        if (rc) {
-            if (g) cudaGraphDestroy(g);
-            return rc;
+        int rc = fn(ctx->capture);
+        // the finalize launch is then all that the capture stream waits for
+        cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+        const cudaGraphNode_t *last = nullptr;
+        size_t count = 0;
+        cudaError_t e = rc ? cudaSuccess
+                        : fin.launch(ctx->capture)
+                            ? cudaGetLastError()
+                            : cudaStreamGetCaptureInfo(ctx->capture, &status, nullptr, nullptr, &last, nullptr, &count);
+        ctx->gfinal = !rc && e == cudaSuccess && count == 1 ? *last : nullptr;
+        const cudaError_t ee = cudaStreamEndCapture(ctx->capture, &ctx->graph);
+        if (e == cudaSuccess) e = ee;
+        if (!rc && e == cudaSuccess && ctx->gfinal) {
+            e = cudaGraphInstantiate(&ctx->gexec, ctx->graph, 0);
+            if (e != cudaSuccess) ctx->gexec = nullptr;
         }
-        CU(e);
-        const cudaError_t ei = cudaGraphInstantiate(&ctx->gexec, g, 0);
-        cudaGraphDestroy(g);
-        if (ei != cudaSuccess) {
-            ctx->gexec = nullptr;
-            CU(ei);
+        if (!ctx->gexec) {
+            drop_graph(ctx);
+            if (rc) return rc;
+            CU(e);
+            set_err(ctx, "graph capture failed");
+            return EF_ERR_CUDA;
         }
         memcpy(&ctx->gkey, &key, sizeof key);
+        ctx->gouts = fin.f.o;
+    } else if (memcmp(&ctx->gouts, &fin.f.o, sizeof(ef_outputs)) != 0) {
+        CU(cudaGraphExecKernelNodeSetParams(ctx->gexec, ctx->gfinal, &fin.node));
+        ctx->gouts = fin.f.o;
     } else {
-        ctx->stats.graph_replays += same_outputs;
+        ctx->stats.graph_replays += 1;
     }
     CU(cudaGraphLaunch(ctx->gexec, ctx->stream));
     return EF_OK;
@@ -380,6 +391,10 @@ int compute_device(ef_ctx *ctx, const Job &j) {
     s.ftab = reinterpret_cast<float2 *>(ctx->ftab);
     s.tq = reinterpret_cast<int64_t *>(s.ftab + fcap);
 
+    const FinalizeCall fin(s, o.precision, j.n, j.out, ctx->tune,
+                           path == PATH_GENERAL ? FinalPath::general
+                           : path == PATH_SHORT ? FinalPath::short_rows
+                                                : FinalPath::either);
     if (use_graph) {
         GraphKey key;
         memset(&key, 0, sizeof key);
@@ -397,17 +412,13 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         key.trust = o.trust_input | (dev_check ? 2 : 0) | (dev_check && o.async ? 4 : 0);
         key.bins = (int32_t)ctx->bins | (int32_t)path << 1 | (int32_t)ctx->long_lists << 3;
         key.tune = ctx->tune;
-        const void *outs[6] = {j.out.ef, j.out.n_clusters, j.out.s, j.out.t, j.out.triangles, j.out.flag};
-        const bool same_outputs = memcmp(outs, ctx->gouts, sizeof outs) == 0;
-        memcpy(ctx->gouts, outs, sizeof outs);
-        rc = run_graph(ctx, key, same_outputs, [&](cudaStream_t cs) {
+        rc = run_graph(ctx, key, fin, [&](cudaStream_t cs) {
             if (a_inline) {
                 const int r = part_a(ctx, j, s, cs, true);
                 if (r) return r;
             }
             return part_b(ctx, j, s, fcap, path, false, cs);
         });
-        if (!rc) rc = part_c(ctx, j, s, path, st);
         if (rc) return rc;
     } else {
         if (a_inline) {
@@ -417,8 +428,8 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         }
         if (prof) CU(cudaEventRecord(ctx->ev[1], st));
         rc = part_b(ctx, j, s, fcap, path, prof, st);
-        if (!rc) rc = part_c(ctx, j, s, path, st);
         if (rc) return rc;
+        LAUNCH(fin.launch(st), "finalize");
         if (prof) CU(cudaEventRecord(ctx->ev[7], st));
     }
     return EF_OK;

@@ -87,16 +87,6 @@ __device__ __forceinline__ double ef_value(int64_t S, double T, bool wide) {
     return (double)(lnS - __fdiv_rn((float)T, Sf));
 }
 
-struct FinalArgs {
-    const int32_t *D;
-    const int64_t *sig1, *sig2, *omega;
-    const double *Tacc;
-    const void *Ccenter;
-    const int64_t *qacc, *tcnt;
-    int32_t *cnt;
-    ef_outputs o;
-};
-
 template <bool F64>
 __device__ __forceinline__ void finalize_nodes(int32_t n, const FinalArgs &f) {
     const int F = f.cnt[CNT_TRIFRAC];
@@ -128,12 +118,6 @@ __device__ __forceinline__ void finalize_nodes(int32_t n, const FinalArgs &f) {
 // The short-row path's finalize: the fused kernel left a node's integer sums
 // in one word, its triangles in 32 bits and all of T in Tacc, so a node costs
 // 20 bytes read (k_finalize: 60).
-struct ShortFinalArgs {
-    const uint64_t *stat;
-    const int32_t *tri;
-    const double *Tacc;
-};
-
 template <bool F64>
 __device__ __forceinline__ void finalize_short_nodes(int32_t n, const ShortFinalArgs &f, const ef_outputs &o) {
     const uint64_t *__restrict__ stat = f.stat;
@@ -163,14 +147,13 @@ __device__ __forceinline__ void finalize_short_nodes(int32_t n, const ShortFinal
 }
 
 template <bool F64>
-__global__ void __launch_bounds__(256) k_finalize(int32_t n, FinalArgs f) {
+__global__ void __launch_bounds__(256) k_finalize(int32_t n, FinalArgs f, ShortFinalArgs) {
     if (!gate_closed(f.cnt)) finalize_nodes<F64>(n, f);
 }
 
 template <bool F64>
-__global__ void __launch_bounds__(256) k_finalize_short(int32_t n, ShortFinalArgs f, const int32_t *__restrict__ cnt,
-                                                        ef_outputs o) {
-    if (!short_closed(cnt, true)) finalize_short_nodes<F64>(n, f, o);
+__global__ void __launch_bounds__(256) k_finalize_short(int32_t n, FinalArgs f, ShortFinalArgs sf) {
+    if (!short_closed(f.cnt, true)) finalize_short_nodes<F64>(n, sf, f.o);
 }
 
 // The path was chosen on the device: one launch for both instead of one that
@@ -226,35 +209,26 @@ static inline unsigned grid_n(int32_t n, const Tune &t) {
     return (unsigned)(g < 1 ? 1 : (g > cap ? cap : g));
 }
 
-static FinalArgs final_args(const Scratch &s, const ef_outputs &out) {
-    return FinalArgs{s.D, s.sig1, s.sig2, s.omega, s.Tacc, s.Ccenter, s.qacc, s.tcnt, s.counters, out};
+template <bool F64>
+static const void *finalize_kernel(FinalPath path) {
+    return path == FinalPath::general      ? reinterpret_cast<const void *>(k_finalize<F64>)
+           : path == FinalPath::short_rows ? reinterpret_cast<const void *>(k_finalize_short<F64>)
+                                           : reinterpret_cast<const void *>(k_finalize_either<F64>);
 }
 
-static ShortFinalArgs short_final_args(const Scratch &s) {
-    return ShortFinalArgs{reinterpret_cast<const uint64_t *>(s.sig1), s.outdeg, s.Tacc};
+FinalizeCall::FinalizeCall(const Scratch &s, int precision, int32_t n_, const ef_outputs &out, const Tune &t,
+                           FinalPath path)
+    : n(n_), f{s.D, s.sig1, s.sig2, s.omega, s.Tacc, s.Ccenter, s.qacc, s.tcnt, s.counters, out},
+      sf{reinterpret_cast<const uint64_t *>(s.sig1), s.outdeg, s.Tacc}, args{&n, &f, &sf}, node{} {
+    node.func = const_cast<void *>(precision == EF_PREC_FP64 ? finalize_kernel<true>(path)
+                                                             : finalize_kernel<false>(path));
+    node.gridDim = dim3(grid_n(n, t));
+    node.blockDim = dim3(256);
+    node.kernelParams = args;
 }
 
-int launch_finalize(const Scratch &s, int precision, int32_t n, const ef_outputs &out, const Tune &t,
-                    cudaStream_t st) {
-    const FinalArgs f = final_args(s, out);
-    if (precision == EF_PREC_FP64) k_finalize<true><<<grid_n(n, t), 256, 0, st>>>(n, f);
-    else k_finalize<false><<<grid_n(n, t), 256, 0, st>>>(n, f);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
-}
-
-int launch_finalize_short(const Scratch &s, int precision, int32_t n, const ef_outputs &out, const Tune &t,
-                          bool chosen, cudaStream_t st) {
-    const unsigned g = grid_n(n, t);
-    const ShortFinalArgs sf = short_final_args(s);
-    const FinalArgs f = final_args(s, out);
-    if (precision == EF_PREC_FP64) {
-        if (chosen) k_finalize_short<true><<<g, 256, 0, st>>>(n, sf, s.counters, out);
-        else k_finalize_either<true><<<g, 256, 0, st>>>(n, f, sf);
-    } else {
-        if (chosen) k_finalize_short<false><<<g, 256, 0, st>>>(n, sf, s.counters, out);
-        else k_finalize_either<false><<<g, 256, 0, st>>>(n, f, sf);
-    }
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+int FinalizeCall::launch(cudaStream_t st) const {
+    return cudaLaunchKernel(node.func, node.gridDim, node.blockDim, node.kernelParams, 0, st) == cudaSuccess ? 0 : -1;
 }
 
 int launch_finalize_sums(const ef_partials &p, int precision, int32_t n, int32_t frac_bits, const ef_outputs &out,

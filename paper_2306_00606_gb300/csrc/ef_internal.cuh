@@ -557,8 +557,6 @@ int launch_ftab(float2 *ftab, int64_t *tq, int32_t *cnt, int64_t cap, cudaStream
 // kernels look for GATE_SHORT).
 int launch_short(const int32_t *ci, const Scratch &s, int precision, int32_t n, const Tune &t, bool chosen,
                  cudaStream_t st);
-int launch_finalize_short(const Scratch &s, int precision, int32_t n, const ef_outputs &out, const Tune &t,
-                          bool chosen, cudaStream_t st);
 int launch_wedge_small(const int32_t *rp, const int32_t *ci, const Scratch &s, int precision, int32_t n,
                        const Tune &t, cudaStream_t st);
 int launch_wedge_big(const int32_t *rp, const int32_t *ci, const Scratch &s, int precision, int wedge_mode,
@@ -566,8 +564,34 @@ int launch_wedge_big(const int32_t *rp, const int32_t *ci, const Scratch &s, int
 // long_lists: some owner may have more than TRI_LONG out-neighbours.
 int launch_tri_pairs(const Scratch &s, int32_t n, int64_t m, const Tune &t, cudaStream_t st,
                      const int32_t *owner_range = nullptr, bool long_lists = true);
-int launch_finalize(const Scratch &s, int precision, int32_t n, const ef_outputs &out, const Tune &t,
-                    cudaStream_t st);
+// The finalize pass (ef_final.cu): what its kernels take, and one launch of it,
+// into a stream or as the parameters of a captured graph's node.  The path is
+// the host's choice, or both, told apart by the gate word.
+struct FinalArgs {
+    const int32_t *D;
+    const int64_t *sig1, *sig2, *omega;
+    const double *Tacc;
+    const void *Ccenter;
+    const int64_t *qacc, *tcnt;
+    int32_t *cnt;
+    ef_outputs o;
+};
+struct ShortFinalArgs {
+    const uint64_t *stat;
+    const int32_t *tri;
+    const double *Tacc;
+};
+enum class FinalPath { general, short_rows, either };
+struct FinalizeCall {
+    int32_t n;
+    FinalArgs f;
+    ShortFinalArgs sf;
+    void *args[3];
+    cudaKernelNodeParams node;
+    FinalizeCall(const Scratch &s, int precision, int32_t n, const ef_outputs &out, const Tune &t, FinalPath path);
+    FinalizeCall(const FinalizeCall &) = delete;   // args point into the object
+    int launch(cudaStream_t st) const;
+};
 // learned path (ef_mlp.cu, ef_rank.cu)
 int launch_mlp_infer(const ModelDev *M, const float *x, int32_t n, float *out, int num_sms, cudaStream_t st);
 // The same network on rows already standardised and rounded to BF16 (8

@@ -122,7 +122,8 @@ extern "C" int ef_compute_static(const ef_csr *g, int32_t n, int64_t m, int32_t 
         launch_orient(rp, ci, n, m, s, t, st, nullptr, nullptr, bins, false, h_cnt[BIN_BIG] > 0) ||
         launch_tri_pairs(s, n, m, t, st, nullptr, h_cnt[CNT_LONG] != 0) ||
         launch_wedge_small(rp, ci, s, precision, n, t, st) ||
-        launch_wedge_big(rp, ci, s, precision, 0, n, m, t, st) || launch_finalize(s, precision, n, out, t, st))
+        launch_wedge_big(rp, ci, s, precision, 0, n, m, t, st) ||
+        FinalizeCall(s, precision, n, out, t, FinalPath::general).launch(st))
         return fail(EF_ERR_CUDA, "ef_compute_static: launch failed");
     if (cudaStreamSynchronize(st) != cudaSuccess || cudaGetLastError() != cudaSuccess)
         return fail(EF_ERR_CUDA, "ef_compute_static: kernel execution failed");

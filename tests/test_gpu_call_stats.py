@@ -1,7 +1,8 @@
 """What ef_get_stats says of profiled calls: the kernels that a call launches,
 against the launches that the CUDA profiler records, for every path a call can
-take and every way it is decided; and the pass that the fused kernel of graphs
-without long rows is booked under."""
+take and every way it is decided; the pass that the fused kernel of graphs
+without long rows is booked under; and what a replayed graph does with other
+output buffers."""
 import json
 
 import numpy as np
@@ -20,22 +21,22 @@ GRAPHS = {
 }
 
 
-def _recorded(fn, tmp_path):
-    """Names of the kernels launched by fn (None when no kernel can be recorded here)."""
+def _recorded(fn, tmp_path, cat=("kernel",)):
+    """Names of the kernels launched by fn, or of records of other kinds (None when no kernel can be recorded here)."""
     import torch
     from torch.profiler import ProfilerActivity, profile
 
-    def record(f):
+    def record(f, cat=("kernel",)):
         with profile(activities=[ProfilerActivity.CUDA]) as p:
             f()
             torch.cuda.synchronize()
         p.export_chrome_trace(str(tmp_path / "trace.json"))
-        return [e["name"] for e in json.load(open(tmp_path / "trace.json"))["traceEvents"] if e.get("cat") == "kernel"]
+        return [e["name"] for e in json.load(open(tmp_path / "trace.json"))["traceEvents"] if e.get("cat") in cat]
 
     x = torch.ones(8, device="cuda")
     for _ in range(3):   # the first session may record nothing
         if record(lambda: x.add_(1)):
-            return record(fn)
+            return record(fn, cat)
     return None
 
 
@@ -75,3 +76,40 @@ def test_fused_kernel_is_booked_as_small_wedges(ctx, mode):  # noqa: F811
         ef.ef_compute_ex(ctx.handle, rp, ci, profile=True, **MODES[mode], **res)
     st = ctx.stats(reset=True)
     assert st["wedge_small_ms"] > 2 * (st["orient_ms"] + st["tri_pairs_ms"] + st["wedge_big_ms"]), st
+
+
+@pytest.mark.parametrize("mode", list(MODES))
+@pytest.mark.parametrize("name", list(GRAPHS))
+def test_replay_with_other_outputs(ctx, tmp_path, name, mode):  # noqa: F811
+    """Calls with one captured graph and changing output buffers (others, fewer, none, the first again): right
+    results, nothing written to the buffers of another call, and no second instantiation."""
+    import paper_2306_00606_gb300 as ef
+    g = GRAPHS[name]()
+    rp, ci = _dev(g.row_ptr), _dev(g.col_idx)
+    want = {k: v.clone() for k, v in _alloc(g.n).items()}
+    ef.ef_compute_ex(ctx.handle, rp, ci, precision="fp64", **want)
+    sets = [_alloc(g.n), _alloc(g.n), {"ef": _alloc(g.n)["ef"]}, {}, {"triangles": _alloc(g.n)["triangles"]}]
+    ctx.stats(reset=True)
+
+    def call(res):
+        ef.ef_compute_ex(ctx.handle, rp, ci, precision="fp64", graph=True, **MODES[mode], **res)
+
+    call(sets[0])   # captured
+    for i in (1, 2, 3, 4, 0, 1):
+        for res in sets:
+            for v in res.values():
+                v.fill_(7)
+        names = _recorded(lambda: call(sets[i]), tmp_path, ("cuda_runtime", "cuda_driver"))
+        if names is not None:
+            assert any("GraphLaunch" in x for x in names) and not any("Instantiate" in x for x in names), names
+        for j, res in enumerate(sets):
+            for k, v in res.items():
+                if j == i and k in ("ef", "t"):   # sums by atomics: equal up to their order
+                    np.testing.assert_allclose(v.cpu().numpy(), want[k].cpu().numpy(), rtol=1e-12)
+                elif j == i:
+                    assert (v == want[k]).all(), k
+                else:
+                    assert (v == 7).all(), (i, j, k)
+    assert ctx.stats(reset=True)["graph_replays"] == 0
+    call(sets[1])
+    assert ctx.stats(reset=True)["graph_replays"] == 1

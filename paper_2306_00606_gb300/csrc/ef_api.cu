@@ -281,7 +281,8 @@ int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, PathMo
     }
     const bool gated = path == PATH_DEVICE;
     if (!gated) LAUNCH(launch_clear_triangles(s, j.n, st), "clear");
-    LAUNCH(launch_orient(j.rp, j.ci, j.n, j.m, s, t, st, nullptr, nullptr, ctx->bins, gated, true),
+    LAUNCH(launch_orient(j.rp, j.ci, j.n, j.m, s, t, st, nullptr, nullptr, ctx->bins, gated, true,
+                         gated || ctx->long_lists),
            "orientation");
     if (prof) CU(cudaEventRecord(ctx->ev[2], st));
     // before the wedges, whose hub classes lie over the oriented lists
@@ -638,7 +639,9 @@ int features_device(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n
     using namespace ef;
     cudaStream_t st = ctx->stream;
     if (with_orient || mode == 1)
-        LAUNCH(launch_orient(rp, ci, n, m, s, ctx->tune, st, r.nbr_min, r.nbr_max, ctx->bins, false, ctx->big_rows), "orientation");
+        LAUNCH(launch_orient(rp, ci, n, m, s, ctx->tune, st, r.nbr_min, r.nbr_max, ctx->bins, false, ctx->big_rows,
+                             ctx->long_lists),
+               "orientation");
     else
         LAUNCH(launch_omega_mm(rp, ci, n, m, s, r, ctx->tune, st), "omega");
     if (mode == 1) LAUNCH(launch_tri_pairs(s, n, m, ctx->tune, st, nullptr, ctx->long_lists), "triangle");
@@ -661,7 +664,8 @@ int nodes_device(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n, i
     cudaStream_t st = ctx->stream;
     if (global_tri && !tri_done) {
         if (!orient_done)
-            LAUNCH(launch_orient(rp, ci, n, m, s, ctx->tune, st, nullptr, nullptr, ctx->bins, false, ctx->big_rows),
+            LAUNCH(launch_orient(rp, ci, n, m, s, ctx->tune, st, nullptr, nullptr, ctx->bins, false, ctx->big_rows,
+                                 ctx->long_lists),
                    "orientation");
         LAUNCH(launch_tri_pairs(s, n, m, ctx->tune, st, nullptr, ctx->long_lists), "triangle");
     }
@@ -1086,7 +1090,8 @@ int ef_compute_shard(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, int32_t
     cudaStream_t st = ctx->stream;
     int32_t *rng = s.counters + CNT_RANGE;
     LAUNCH(launch_shard_range(rp, n, m, shard, num_shards, rng, st), "shard range");
-    LAUNCH(launch_orient(rp, ci, n, m, s, t, st, nullptr, nullptr, ctx->bins, false, ctx->big_rows), "orientation");
+    LAUNCH(launch_orient(rp, ci, n, m, s, t, st, nullptr, nullptr, ctx->bins, false, ctx->big_rows, ctx->long_lists),
+           "orientation");
     LAUNCH(launch_tri_pairs(s, n, m, t, st, rng, ctx->long_lists), "triangle");
     // the out-degrees are not needed any more: they hold the marks
     LAUNCH(launch_mark_range(rng, n, s.outdeg, t, st), "shard marks");

@@ -273,31 +273,38 @@ __device__ __forceinline__ T group_sum(T v) {
 // lower_bound over a sorted int32 array (generic address space)
 // ----------------------------------------------- out-list membership tables
 // Table of the out-list [ls, le) of one node: buckets of 8 slots (one 32-byte
-// sector) from slot base of out_hash, base = 3 ls rounded up to a multiple of
-// 8 and 3/8 as many buckets as entries, so the tables of consecutive
-// out-lists never overlap.  A bucket is filled from its first slot on, so its
-// last slot says whether it is full; keys that find it full go to the next
-// bucket.  At 2.7 entries per bucket on average a probe in 150 meets a full
-// bucket without its key; the others take one sector.  (Buckets of 4 slots at
-// a mean of 2, home bucket and the next one read together: 1.5 sectors a
-// test, and another round for a few percent of the tests, that is for most
-// warps.  A mean of 2 in 8 slots: 4.9 against 4.8 ms of pair tests and 2.06
-// against 1.99 of orientation on the 87M-entry graph, the larger tables miss
-// L2 more often.)
+// sector) from slot base of out_hash, base = per ls rounded up to a multiple of
+// 8 and per/8 as many buckets as entries (table_per: slots per entry), so the
+// tables of consecutive out-lists never overlap.  A bucket is filled from its
+// first slot on, so its last slot says whether it is full; keys that find it
+// full go to the next bucket.  (Buckets of 4 slots at a mean of 2, home bucket
+// and the next one read together: 1.5 sectors a test, and another round for a
+// few percent of the tests, that is for most warps.)
+// Three slots per entry where some node has more than TRI_LONG out-neighbours:
+// at 2.7 entries per bucket on average a probe in 150 meets a full bucket
+// without its key.  (Four slots per entry: 4.9 against 4.8 ms of pair tests and
+// 2.06 against 1.99 of orientation on the 87M-entry graph, the larger tables
+// miss L2 more often.)  Two elsewhere: the tables of short lists are one or two
+// buckets that hold them either way, and a third less to clear and to write
+// (orientation with its clearing and pair tests, two against three: ER 1M of
+// degree 14 541 and 566 us, BA 1M 328 and 335; with long lists 87M entries 6.60
+// and 6.09 ms, power-law 4M 2.10 and 2.03).
 // Only lists longer than SHORT_MAX have a table, and only when it lies inside
 // the array (always, for a symmetric CSR: the out-lists then hold m/2 entries
 // in all).
 constexpr int BUCKET = 8;
-__host__ __device__ __forceinline__ int64_t hash_slots(int64_t m) { return m + (m + 1) / 2 + 16; }   // slots of out_hash
+__host__ __device__ __forceinline__ int table_per(bool long_lists) { return long_lists ? 3 : 2; }
+// slots of out_hash (cleared; allocated: for three per entry)
+__host__ __device__ __forceinline__ int64_t hash_slots(int64_t m, int per = 3) { return per * ((m + 1) / 2) + 16; }
 
-__host__ __device__ __forceinline__ int64_t table_base(int ls) {
-    return ((int64_t)3 * ls + BUCKET - 1) & ~(int64_t)(BUCKET - 1);
+__host__ __device__ __forceinline__ int64_t table_base(int ls, int per) {
+    return ((int64_t)per * ls + BUCKET - 1) & ~(int64_t)(BUCKET - 1);
 }
 
-__device__ __forceinline__ bool out_table(int ls, int le, int64_t hash_cap, int64_t &base, int &nb) {
+__device__ __forceinline__ bool out_table(int ls, int le, int64_t hash_cap, int per, int64_t &base, int &nb) {
     const int p = le - ls;
-    base = table_base(ls);
-    nb = (3 * p) >> 3;
+    base = table_base(ls, per);
+    nb = (per * p) >> 3;
     return p > SHORT_MAX && base + BUCKET * (int64_t)nb <= hash_cap;
 }
 
@@ -345,10 +352,10 @@ __device__ __forceinline__ unsigned range_bits(int e0, int ls, int le) {
 // The kind sits in bits 30-31 of y (counts and offsets stay below 2^30).
 constexpr int DESC_KIND_SHIFT = 30;
 constexpr int DESC_MASK = (1 << DESC_KIND_SHIFT) - 1;
-__device__ __forceinline__ int2 probe_desc(int ls, int le, int64_t hash_cap) {
+__device__ __forceinline__ int2 probe_desc(int ls, int le, int64_t hash_cap, int per) {
     int64_t hb;
     int nb;
-    if (out_table(ls, le, hash_cap, hb, nb))
+    if (out_table(ls, le, hash_cap, per, hb, nb))
         return make_int2((int)(hb >> 2), (int)((unsigned)nb | 1u << DESC_KIND_SHIFT));
     if (le - ls > SHORT_MAX) return make_int2(ls, (int)((unsigned)le | 2u << DESC_KIND_SHIFT));
     const int q0 = ls >> 2;
@@ -534,10 +541,10 @@ int launch_prep_a(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, co
 // filled as the lists are written).  gated: the call's path is chosen on the
 // device; the triangle accumulators are then cleared here, behind the gate.
 // big_rows: no graph without rows above SMALL_MAX comes here (the short-row
-// path took it).
+// path took it).  long_lists: as launch_tri_pairs.
 int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const Scratch &s, const Tune &t,
                   cudaStream_t st, int32_t *nmin = nullptr, int32_t *nmax = nullptr, bool bins = true,
-                  bool gated = false, bool big_rows = false);
+                  bool gated = false, bool big_rows = false, bool long_lists = true);
 int launch_clear_triangles(const Scratch &s, int32_t n, cudaStream_t st);
 int launch_big_items(const Scratch &s, int32_t n, cudaStream_t st);
 int prepare_kernels();

@@ -659,12 +659,14 @@ __global__ void __launch_bounds__(256) k_node_info(const int32_t *__restrict__ D
     __shared__ int s_items, s_first;
     if (threadIdx.x == 0) s_items = 0;
     __syncthreads();
+    const int per = table_per(cnt[CNT_LONG] != 0);
+    const int64_t slots = hash_slots(m, per);
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
         const int64_t v = base + threadIdx.x;
         int blocks = 0;
         if (v < n) {
             const int ls = out_ptr[v], p = outdeg[v];
-            const int2 pd = probe_desc(ls, ls + p, hash_slots(m));
+            const int2 pd = probe_desc(ls, ls + p, slots, per);
             info[v] = make_int4(D[v], (int)sig1[v], pd.x, pd.y);
             // (the second test holds for every symmetric CSR: room for the sorted records)
             if (p > TRI_LONG && 2 * (int64_t)(ls + p) <= m) blocks = (p + 31) / 32;
@@ -780,7 +782,7 @@ __device__ __forceinline__ void orient_row_warp(const Orient &o, int u, int ua, 
 // match the degree pass's counts returns at once.  (WS batch orientation
 // 4.7 -> 4.3 ms with 8; the power-law graph 0.90 -> 1.02 ms with 8.)
 // Staging area of k_orient<CHUNK>: the entries of one warp step (20 bytes each)
-// and their tables (three slots per entry).  Only the eight-record form (graphs
+// and their tables (up to three slots per entry).  Only the eight-record form (graphs
 // without rows above degree 32) stages: measured on the 4096-graph WS batch,
 // orientation 4.32 -> 2.96 ms; the four-record form (a staging area of 128
 // entries, 5 blocks per SM) was slower on the power-law graph (0.89 -> 0.96
@@ -812,6 +814,7 @@ __global__ void __launch_bounds__(256, CHUNK == 8 ? 3 : 5) k_orient(
     if (threadIdx.x == 0) s_ord.load(cnt, n, bins_ok);
     __syncthreads();
     const RowOrder &ord = s_ord;
+    const int per = table_per(cnt[CNT_LONG] != 0);
     const int total = ord.total();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + w;
@@ -837,8 +840,8 @@ __global__ void __launch_bounds__(256, CHUNK == 8 ? 3 : 5) k_orient(
         }
         const bool stage = CAP > 0 && sum > 0 && sum <= CAP && kend - kmin == sum;
         if (stage) {
-            const int64_t tb0 = table_base(kmin);
-            const int64_t tb1 = table_base(kend);
+            const int64_t tb0 = table_base(kmin, per);
+            const int64_t tb1 = table_base(kend, per);
             const int tlen = (int)(tb1 - tb0);
             for (int t = lane; t < tlen; t += 32) S.tab[w][t] = -1;
             __syncwarp();
@@ -1181,11 +1184,12 @@ int launch_clear_triangles(const Scratch &s, int32_t n, cudaStream_t st) {
 // Where the device chooses the path, what the general path clears (the empty
 // tables, the offsets of the degree-bin layout, the triangle accumulators) is
 // cleared behind the gate; elsewhere memsets do it (2 us less on BA 1M).
-__global__ void __launch_bounds__(256) k_clear_lists(int32_t *__restrict__ hash, int64_t slots,
+__global__ void __launch_bounds__(256) k_clear_lists(int32_t *__restrict__ hash, int64_t m,
                                                      int32_t *__restrict__ out_ptr, int32_t n,
                                                      int64_t *__restrict__ qacc, int64_t *__restrict__ tcnt,
                                                      const int32_t *__restrict__ cnt) {
     if (gate_closed(cnt)) return;
+    const int64_t slots = hash_slots(m, table_per(cnt[CNT_LONG] != 0));
     const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = first; i < slots / 4; i += step) reinterpret_cast<int4 *>(hash)[i] = make_int4(-1, -1, -1, -1);
     if (first < slots % 4) hash[slots / 4 * 4 + first] = -1;
@@ -1208,13 +1212,14 @@ int prepare_orient() {
 
 // Oriented CSR and omega.
 int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const Scratch &s, const Tune &t,
-                  cudaStream_t st, int32_t *nmin, int32_t *nmax, bool bins, bool gated, bool big_rows) {
+                  cudaStream_t st, int32_t *nmin, int32_t *nmax, bool bins, bool gated, bool big_rows,
+                  bool long_lists) {
     const int32_t *gate = gated ? s.counters : nullptr;
     // empty tables and, in layout order, zero offsets (degree-0 nodes keep offset 0 and an empty list)
     if (gated)
         k_clear_lists<<<t.grid(hash_slots(m) / 4, 256), 256, 0, st>>>(
-            s.out_hash, hash_slots(m), bins ? s.out_ptr : nullptr, n, s.qacc, s.tcnt, s.counters);
-    else if (cudaMemsetAsync(s.out_hash, 0xff, (size_t)hash_slots(m) * sizeof(int32_t), st) != cudaSuccess ||
+            s.out_hash, m, bins ? s.out_ptr : nullptr, n, s.qacc, s.tcnt, s.counters);
+    else if (cudaMemsetAsync(s.out_hash, 0xff, (size_t)hash_slots(m, table_per(long_lists)) * sizeof(int32_t), st) != cudaSuccess ||
              (bins && cudaMemsetAsync(s.out_ptr, 0, (size_t)(n + 1) * sizeof(int32_t), st) != cudaSuccess))
         return -1;
     if (bins) {

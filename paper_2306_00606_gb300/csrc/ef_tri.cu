@@ -339,6 +339,12 @@ __device__ __forceinline__ unsigned transpose32(unsigned v) {
 }
 
 constexpr int TL_STEP = 2;   // entries b tested together
+// Small graphs: an item is shared among warps while that leaves each of them at
+// most TL_ROUNDS shares on average, by up to eight chunks of b, then (at most
+// TL_PART_ROUNDS) by up to four parts of a chunk.  A pair of b takes the
+// latency of one L2 load, so the longest list decides there: power-law 100k
+// 31 -> 20 us, 20k 23 -> 10, R-MAT 2^16 100 -> 75; larger graphs have the items.
+constexpr int TL_ROUNDS = 16, TL_PART_ROUNDS = 6;
 
 __global__ void __launch_bounds__(TL_WARPS * 32, 4) k_tri_long(
     const int32_t *__restrict__ out_ptr, const int32_t *__restrict__ out_col, const int32_t *__restrict__ out_hash,
@@ -355,13 +361,21 @@ __global__ void __launch_bounds__(TL_WARPS * 32, 4) k_tri_long(
     // the first item by position, the others from the counter (an atomic by every
     // warp before its first item cost a graph without long owners 3 us a call)
     const int nwarps = gridDim.x * TL_WARPS;
+    // few items: 2^chunks warps share an item's entries b by chunks of 32, then
+    // 2^parts a chunk
+    int chunks = 0, parts = 0;
+    while (chunks < 3 && ((int64_t)total << (chunks + 1)) <= (int64_t)TL_ROUNDS * nwarps) ++chunks;
+    while (chunks == 3 && parts < 2 && ((int64_t)total << (parts + 4)) <= (int64_t)TL_PART_ROUNDS * nwarps) ++parts;
+    const int split = chunks + parts, width = 32 >> parts;
     auto take = [&]() {
         int it = 0;
         if (lane == 0) it = nwarps + atomicAdd(cnt + CNT_TRINEXT, 1);
         return __shfl_sync(FULL, it, 0);
     };
-    for (int it = blockIdx.x * TL_WARPS + w; it < total; it = take()) {
-        const int2 item = items[total - 1 - it];
+    for (int it = blockIdx.x * TL_WARPS + w; it >> split < total; it = take()) {
+        const int2 item = items[total - 1 - (it >> split)];
+        const int first = 32 * (it & ((1 << chunks) - 1)), lo = width * ((it & ((1 << split) - 1)) >> chunks);
+        if (first > item.y * 32) continue;   // (no entries before its candidates there)
         const int a = item.x;
         if (a < a_lo || a >= a_hi) continue;
         const int ls = out_ptr[a], p = outdeg[a], Da = D[a];
@@ -375,14 +389,14 @@ __global__ void __launch_bounds__(TL_WARPS * 32, 4) k_tri_long(
         s_Dc[w][lane] = rc.y;
         int64_t qc = 0;
         int tc = 0;
-        for (int i0 = 0; i0 < last; i0 += 32) {
+        for (int i0 = first; i0 < last; i0 += 32 << chunks) {
             __syncwarp();
             const int4 rb = i0 + lane < last ? rec[ls + i0 + lane] : make_int4(0, 0, 0, 0);
             s_b[w][lane] = rb;
             __syncwarp();
-            const int nb = min(32, last - i0);
+            const int nb = min(lo + width, last - i0);
             unsigned found = 0;   // bit i: {b_i, c} adjacent
-            for (int i = 0; i < nb; i += TL_STEP) {
+            for (int i = lo; i < nb; i += TL_STEP) {
                 int4 x[TL_STEP], y[TL_STEP];
                 const int4 *p0[TL_STEP];
                 unsigned mask[TL_STEP];   // entries of the two quads that count

@@ -51,3 +51,15 @@ def test_long_lists_match_oracle(ctx, name, precision):  # noqa: F811
     np.testing.assert_array_equal(got["triangles"], _host(res)["triangles"])
     np.testing.assert_array_equal(got["s"], ref["S"])
     _close(got["ef"], ref["EF"], precision)
+
+
+@pytest.mark.parametrize("copies", [2, 6, 25, 60, 120, 260])
+def test_items_shared_among_warps(ctx, copies):  # noqa: F811
+    """About 200 items a copy (a clique, a dense random part): 32, 16, 8, 4, 2 warps and one warp per item."""
+    import paper_2306_00606_gb300 as ef
+    one = synth.disjoint_union([synth.complete(98), synth.erdos_renyi(150, 0.5, 2)])
+    ref = {k: np.tile(v, copies) for k, v in alg1_ref(one).items()}
+    g = synth.disjoint_union([one] * copies)
+    res = _alloc(g.n)
+    ef.ef_compute_ex(ctx.handle, _dev(g.row_ptr), _dev(g.col_idx), precision="fp64", **res)
+    assert_parity(_host(res), ref, "fp64")

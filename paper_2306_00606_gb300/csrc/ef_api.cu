@@ -89,7 +89,8 @@ struct ef_ctx {
     void *rank = nullptr;            // learned-path buffers (RankScratch)
     size_t rank_bytes = 0;
     double *dtmp = nullptr;          // small device scratch (feature sums)
-    bool long_lists = true;          // an owner of the current graph has more than TRI_LONG out-neighbours
+    bool long_lists = true;          // an owner of the current graph has more than TRI_LONG out-neighbours,
+    bool wide_lists = true;          // more than TABLE_WIDE
     bool big_rows = false;           // the current graph is known to have rows above SMALL_MAX
     int path = 0;                    // part B kernels of the last exact call (PathMode)
     bool bins = true;                // out-lists of the current graph in degree-bin order (bin_layout)
@@ -282,7 +283,7 @@ int part_b(ef_ctx *ctx, const Job &j, const ef::Scratch &s, int64_t fcap, PathMo
     const bool gated = path == PATH_DEVICE;
     if (!gated) LAUNCH(launch_clear_triangles(s, j.n, st), "clear");
     LAUNCH(launch_orient(j.rp, j.ci, j.n, j.m, s, t, st, nullptr, nullptr, ctx->bins, gated, true,
-                         gated || ctx->long_lists),
+                         gated || ctx->wide_lists),
            "orientation");
     if (prof) CU(cudaEventRecord(ctx->ev[2], st));
     // before the wedges, whose hub classes lie over the oriented lists
@@ -364,7 +365,7 @@ int compute_device(ef_ctx *ctx, const Job &j) {
 
     // f table size: from the validated max degree, else the largest possible
     int64_t fcap;
-    ctx->long_lists = true;
+    ctx->long_lists = ctx->wide_lists = true;
     if (a_inline) {
         int64_t bound = (int64_t)j.n - 1 < j.m ? (int64_t)j.n - 1 : j.m;
         if (bound > EF_MAX_DEGREE) bound = EF_MAX_DEGREE;
@@ -380,6 +381,7 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         if (const int lim = degree_limit(ctx, ctx->h_counters)) return lim;
         path = ctx->h_counters[BIN_BIG] == 0 ? PATH_SHORT : PATH_GENERAL;
         ctx->long_lists = ctx->h_counters[CNT_LONG] != 0;
+        ctx->wide_lists = ctx->h_counters[CNT_WIDE] != 0;
         fcap = 3 * (int64_t)ctx->h_counters[CNT_MAXDEG] + 1;
         ctx->bins = bin_layout(ctx->tune, ctx->h_counters, j.n, j.goff_dev != nullptr);
     }
@@ -411,7 +413,8 @@ int compute_device(ef_ctx *ctx, const Job &j) {
         key.precision = o.precision;
         key.wedge_mode = o.wedge_mode;
         key.trust = o.trust_input | (dev_check ? 2 : 0) | (dev_check && o.async ? 4 : 0);
-        key.bins = (int32_t)ctx->bins | (int32_t)path << 1 | (int32_t)ctx->long_lists << 3;
+        key.bins = (int32_t)ctx->bins | (int32_t)path << 1 | (int32_t)ctx->long_lists << 3 |
+                   (int32_t)ctx->wide_lists << 4;
         key.tune = ctx->tune;
         rc = run_graph(ctx, key, fin, [&](cudaStream_t cs) {
             if (a_inline) {
@@ -594,7 +597,7 @@ int prepare_graph(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n, 
     Job j{rp, ci, n, m, nullptr, 0, o, ef_outputs{}};
     rc = part_a(ctx, j, s, ctx->stream);
     if (rc) return rc;
-    ctx->long_lists = true;
+    ctx->long_lists = ctx->wide_lists = true;
     ctx->big_rows = false;
     if (o.trust_input) {
         const int64_t bound = (int64_t)n - 1 < m ? (int64_t)n - 1 : m;
@@ -609,6 +612,7 @@ int prepare_graph(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n, 
         fcap = 3 * (int64_t)ctx->h_counters[CNT_MAXDEG] + 1;
         ctx->bins = bin_layout(ctx->tune, ctx->h_counters, n, false);
         ctx->long_lists = ctx->h_counters[CNT_LONG] != 0;
+        ctx->wide_lists = ctx->h_counters[CNT_WIDE] != 0;
         ctx->big_rows = ctx->h_counters[BIN_BIG] > 0;
     }
     size_t have = (size_t)ctx->ftab_cap * 2 * sizeof(double);
@@ -640,7 +644,7 @@ int features_device(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n
     cudaStream_t st = ctx->stream;
     if (with_orient || mode == 1)
         LAUNCH(launch_orient(rp, ci, n, m, s, ctx->tune, st, r.nbr_min, r.nbr_max, ctx->bins, false, ctx->big_rows,
-                             ctx->long_lists),
+                             ctx->wide_lists),
                "orientation");
     else
         LAUNCH(launch_omega_mm(rp, ci, n, m, s, r, ctx->tune, st), "omega");
@@ -665,7 +669,7 @@ int nodes_device(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n, i
     if (global_tri && !tri_done) {
         if (!orient_done)
             LAUNCH(launch_orient(rp, ci, n, m, s, ctx->tune, st, nullptr, nullptr, ctx->bins, false, ctx->big_rows,
-                                 ctx->long_lists),
+                                 ctx->wide_lists),
                    "orientation");
         LAUNCH(launch_tri_pairs(s, n, m, ctx->tune, st, nullptr, ctx->long_lists), "triangle");
     }
@@ -1090,7 +1094,7 @@ int ef_compute_shard(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, int32_t
     cudaStream_t st = ctx->stream;
     int32_t *rng = s.counters + CNT_RANGE;
     LAUNCH(launch_shard_range(rp, n, m, shard, num_shards, rng, st), "shard range");
-    LAUNCH(launch_orient(rp, ci, n, m, s, t, st, nullptr, nullptr, ctx->bins, false, ctx->big_rows, ctx->long_lists),
+    LAUNCH(launch_orient(rp, ci, n, m, s, t, st, nullptr, nullptr, ctx->bins, false, ctx->big_rows, ctx->wide_lists),
            "orientation");
     LAUNCH(launch_tri_pairs(s, n, m, t, st, rng, ctx->long_lists), "triangle");
     // the out-degrees are not needed any more: they hold the marks

@@ -84,6 +84,7 @@ constexpr int BIG_ROWS = 256;          // rows per work item of the direct big-n
 constexpr int BIG_TILE = 4096;         // neighbour degrees staged per tile by the direct kernel
 constexpr int ROW_CTA = 512;           // threads of the per-hub-row kernels
 constexpr int TRI_LONG = 32;           // owners of more out-neighbours take a warp per 32 of them in the pair tests
+constexpr int TABLE_WIDE = 24;         // with a longer out-list, the hash tables have three slots per entry, else two
 constexpr int SHORT_MAX = 5;           // out-lists longer than this get a hash table for the triangle pass
 
 // Triangle corrections are integers in units of 2^-F (the pass adds only
@@ -161,6 +162,7 @@ enum : int {
     CNT_TRILONG = 38, // items of the long owners (pair tests), and the next one to take
     CNT_TRINEXT = 39,
     CNT_LONG = 42,    // 1: some node has more than TRI_LONG out-neighbours
+    CNT_WIDE = 43,    // 1: some node has more than TABLE_WIDE out-neighbours
     CNT_RANGE = 40,   // 40, 41: a shard's node range [lo, hi)
     CNT_SYM = 44,     // 44, 45: the symmetry sum (uint64, 8-byte aligned)
     CNT_BIGLO = 46,   // n - 1 - (smallest id of a node of degree > SMALL_MAX), if any
@@ -280,7 +282,7 @@ __device__ __forceinline__ T group_sum(T v) {
 // full go to the next bucket.  (Buckets of 4 slots at a mean of 2, home bucket
 // and the next one read together: 1.5 sectors a test, and another round for a
 // few percent of the tests, that is for most warps.)
-// Three slots per entry where some node has more than TRI_LONG out-neighbours:
+// Three slots per entry where some node has more than TABLE_WIDE out-neighbours:
 // at 2.7 entries per bucket on average a probe in 150 meets a full bucket
 // without its key.  (Four slots per entry: 4.9 against 4.8 ms of pair tests and
 // 2.06 against 1.99 of orientation on the 87M-entry graph, the larger tables
@@ -288,12 +290,13 @@ __device__ __forceinline__ T group_sum(T v) {
 // buckets that hold them either way, and a third less to clear and to write
 // (orientation with its clearing and pair tests, two against three: ER 1M of
 // degree 14 541 and 566 us, BA 1M 328 and 335; with long lists 87M entries 6.60
-// and 6.09 ms, power-law 4M 2.10 and 2.03).
+// and 6.09 ms, power-law 4M 2.10 and 2.03; power-law 50k, lists up to 32 by
+// atomics, 56 and 51 us).
 // Only lists longer than SHORT_MAX have a table, and only when it lies inside
 // the array (always, for a symmetric CSR: the out-lists then hold m/2 entries
 // in all).
 constexpr int BUCKET = 8;
-__host__ __device__ __forceinline__ int table_per(bool long_lists) { return long_lists ? 3 : 2; }
+__host__ __device__ __forceinline__ int table_per(bool wide_lists) { return wide_lists ? 3 : 2; }
 // slots of out_hash (cleared; allocated: for three per entry)
 __host__ __device__ __forceinline__ int64_t hash_slots(int64_t m, int per = 3) { return per * ((m + 1) / 2) + 16; }
 
@@ -541,10 +544,11 @@ int launch_prep_a(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, co
 // filled as the lists are written).  gated: the call's path is chosen on the
 // device; the triangle accumulators are then cleared here, behind the gate.
 // big_rows: no graph without rows above SMALL_MAX comes here (the short-row
-// path took it).  long_lists: as launch_tri_pairs.
+// path took it).  wide_lists: some node may have more than TABLE_WIDE
+// out-neighbours.
 int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const Scratch &s, const Tune &t,
                   cudaStream_t st, int32_t *nmin = nullptr, int32_t *nmax = nullptr, bool bins = true,
-                  bool gated = false, bool big_rows = false, bool long_lists = true);
+                  bool gated = false, bool big_rows = false, bool wide_lists = true);
 int launch_clear_triangles(const Scratch &s, int32_t n, cudaStream_t st);
 int launch_big_items(const Scratch &s, int32_t n, cudaStream_t st);
 int prepare_kernels();

@@ -317,10 +317,11 @@ __device__ __forceinline__ int cross_bits(const RowOut &ro, const int32_t *__res
 // warp cost 40 us on the 1M-node power-law graph).
 __device__ __forceinline__ void add_rows(int32_t *cnt, uint64_t sym, int most) {
     sym = warp_sum(sym);
-    const bool many = __any_sync(FULL, most > TRI_LONG);
+    most = __reduce_max_sync(FULL, most);
     if ((threadIdx.x & 31) == 0) {
         if (sym) atomicAdd(reinterpret_cast<unsigned long long *>(cnt + CNT_SYM), (unsigned long long)sym);
-        if (many) cnt[CNT_LONG] = 1;
+        if (most > TRI_LONG) cnt[CNT_LONG] = 1;
+        if (most > TABLE_WIDE) cnt[CNT_WIDE] = 1;
     }
 }
 
@@ -659,7 +660,7 @@ __global__ void __launch_bounds__(256) k_node_info(const int32_t *__restrict__ D
     __shared__ int s_items, s_first;
     if (threadIdx.x == 0) s_items = 0;
     __syncthreads();
-    const int per = table_per(cnt[CNT_LONG] != 0);
+    const int per = table_per(cnt[CNT_WIDE] != 0);
     const int64_t slots = hash_slots(m, per);
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += (int64_t)gridDim.x * blockDim.x) {
         const int64_t v = base + threadIdx.x;
@@ -814,7 +815,7 @@ __global__ void __launch_bounds__(256, CHUNK == 8 ? 3 : 5) k_orient(
     if (threadIdx.x == 0) s_ord.load(cnt, n, bins_ok);
     __syncthreads();
     const RowOrder &ord = s_ord;
-    const int per = table_per(cnt[CNT_LONG] != 0);
+    const int per = table_per(cnt[CNT_WIDE] != 0);
     const int total = ord.total();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + w;
@@ -1189,7 +1190,7 @@ __global__ void __launch_bounds__(256) k_clear_lists(int32_t *__restrict__ hash,
                                                      int64_t *__restrict__ qacc, int64_t *__restrict__ tcnt,
                                                      const int32_t *__restrict__ cnt) {
     if (gate_closed(cnt)) return;
-    const int64_t slots = hash_slots(m, table_per(cnt[CNT_LONG] != 0));
+    const int64_t slots = hash_slots(m, table_per(cnt[CNT_WIDE] != 0));
     const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = first; i < slots / 4; i += step) reinterpret_cast<int4 *>(hash)[i] = make_int4(-1, -1, -1, -1);
     if (first < slots % 4) hash[slots / 4 * 4 + first] = -1;
@@ -1213,13 +1214,13 @@ int prepare_orient() {
 // Oriented CSR and omega.
 int launch_orient(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, const Scratch &s, const Tune &t,
                   cudaStream_t st, int32_t *nmin, int32_t *nmax, bool bins, bool gated, bool big_rows,
-                  bool long_lists) {
+                  bool wide_lists) {
     const int32_t *gate = gated ? s.counters : nullptr;
     // empty tables and, in layout order, zero offsets (degree-0 nodes keep offset 0 and an empty list)
     if (gated)
         k_clear_lists<<<t.grid(hash_slots(m) / 4, 256), 256, 0, st>>>(
             s.out_hash, m, bins ? s.out_ptr : nullptr, n, s.qacc, s.tcnt, s.counters);
-    else if (cudaMemsetAsync(s.out_hash, 0xff, (size_t)hash_slots(m, table_per(long_lists)) * sizeof(int32_t), st) != cudaSuccess ||
+    else if (cudaMemsetAsync(s.out_hash, 0xff, (size_t)hash_slots(m, table_per(wide_lists)) * sizeof(int32_t), st) != cudaSuccess ||
              (bins && cudaMemsetAsync(s.out_ptr, 0, (size_t)(n + 1) * sizeof(int32_t), st) != cudaSuccess))
         return -1;
     if (bins) {

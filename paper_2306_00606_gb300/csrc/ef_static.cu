@@ -120,7 +120,7 @@ extern "C" int ef_compute_static(const ef_csr *g, int32_t n, int64_t m, int32_t 
     out.ef = out_ef;
     if (launch_ftab(s.ftab, s.tq, s.counters, fcap, st) ||
         launch_orient(rp, ci, n, m, s, t, st, nullptr, nullptr, bins, false, h_cnt[BIN_BIG] > 0,
-                      h_cnt[CNT_LONG] != 0) ||
+                      h_cnt[CNT_WIDE] != 0) ||
         launch_tri_pairs(s, n, m, t, st, nullptr, h_cnt[CNT_LONG] != 0) ||
         launch_wedge_small(rp, ci, s, precision, n, t, st) ||
         launch_wedge_big(rp, ci, s, precision, 0, n, m, t, st) ||

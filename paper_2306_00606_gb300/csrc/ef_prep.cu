@@ -320,8 +320,10 @@ __device__ __forceinline__ void add_rows(int32_t *cnt, uint64_t sym, int most) {
     most = __reduce_max_sync(FULL, most);
     if ((threadIdx.x & 31) == 0) {
         if (sym) atomicAdd(reinterpret_cast<unsigned long long *>(cnt + CNT_SYM), (unsigned long long)sym);
-        if (most > TRI_LONG) cnt[CNT_LONG] = 1;
-        if (most > TABLE_WIDE) cnt[CNT_WIDE] = 1;
+        // (looked at first: stores of thousands of warps to one word cost 6 us)
+        const volatile int32_t *flags = cnt;
+        if (most > TRI_LONG && !flags[CNT_LONG]) cnt[CNT_LONG] = 1;
+        if (most > TABLE_WIDE && !flags[CNT_WIDE]) cnt[CNT_WIDE] = 1;
     }
 }
 

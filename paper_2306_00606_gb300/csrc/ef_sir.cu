@@ -55,19 +55,21 @@ constexpr int SIR_HEAVY = 256;   // frontier nodes of higher degree take a CTA e
 constexpr int SIR_WARPS = 8;     // warps per block of the step kernels
 constexpr int SIR_NODES = 8;     // consecutive nodes per warp step (pull)
 
-// Direction of step t: pull once the frontier's nodes hold a third of all row
-// entries (flen: its length, and those entries).  A pull step reads every
-// node's row and a word row per entry whatever the frontier holds; a push
-// step reads those of the frontier and costs a round trip to memory per
-// successful try.  The entries, not the nodes, say what a push costs: where
-// degrees are uneven, few nodes hold most of them.  Whole calls, gamma = 1/3,
-// R0 = 1.3, in ms, push only / a half / a third / a quarter, and by the number
-// of nodes (one in 8 from 8 words on, else one in 2): BA 500k with 512
-// simulations 82.1 / 36.2 / 35.9 / 36.0 and 36.6, with 20 8.8 / 8.2 / 7.6 / 7.5
-// and 8.9; ER 500k with 250 42.5 / 41.4 / 40.5 / 42.1 and 45.4, with 130 24.9 /
-// 25.1 / 25.1 / 28.4 and 24.8; ER 100k with 250 12.6 / 12.7 / 13.2 / 13.7 and 14.4.
+// Direction of step t: pull once the frontier's nodes hold half of all row
+// entries, a third from eight words of simulations on (flen: its length, and
+// those entries).  A pull step reads every node's row and a word row per entry
+// whatever the frontier holds; a push step reads those of the frontier and
+// costs a round trip to memory per successful try.  The entries, not the
+// nodes, say what a push costs: where degrees are uneven, few nodes hold most of
+// them.  Whole calls, gamma = 1/3, R0 = 1.3, in ms, push only / a half / a third /
+// a quarter, and by the number of nodes (one in 8 from 8 words on, else one in
+// 2): BA 500k with 512 simulations 82.1 / 36.2 / 35.9 / 36.0 and 36.6; ER 500k
+// with 250 42.5 / 41.4 / 40.5 / 42.1 and 45.4, with 130 24.9 / 25.1 / 25.1 / 28.4
+// and 24.8; ER 100k with 250 12.6 / 12.7 / 13.2 / 13.7 and 14.4; a half / a third:
+// ER 300k of degree 10 with 211 26.0 / 26.9 and 25.8, BA 300k with 260 20.3 /
+// 20.2 and 20.5, with 40 7.7 / 7.4 and 8.0.
 __device__ __forceinline__ bool sir_dense(const SirState &st, int t) {
-    return (int64_t)(uint32_t)st.flen[t & 1].y * 3 > st.m;
+    return (int64_t)(uint32_t)st.flen[t & 1].y * (st.WB >= 8 ? 3 : 2) > st.m;
 }
 
 // Room for len nodes with the given row entries in all in the frontier nx, for

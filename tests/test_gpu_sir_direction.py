@@ -1,6 +1,7 @@
 """The direction of SIR steps (push, pull) against the oracle.  The oracle's own
 draws say which nodes are infected at each step, and with them whether a step
-pulls: once the infected nodes' rows hold more than a third of all entries.
+pulls: once the infected nodes' rows hold more than half of all entries, or a
+third from eight words (more than 224 simulations) on.
 Every case is shown to take the directions it is there for.  Sizes at the edges
 of a pull step's share: one group of nodes per warp (small graphs) up to the
 full eight, with a last share that is not full.  Everything is exact."""
@@ -12,13 +13,20 @@ from oracle import sir
 from test_gpu_device_check import _dev, ctx  # noqa: F401
 
 OUTS = ("final_size", "length", "peak_infected", "peak_step", "parent")
-DENSE = 3   # a step pulls when DENSE x the frontier's entries exceed all entries
+
+
+def _dense(sims):
+    """A step pulls when this many times the frontier's entries exceed all entries."""
+    return 3 if sims > 224 else 2
+
 
 # graph, simulations, R0, and whether a push step follows a pull step
 CASES = {
     "ba_1_sim": (lambda: synth.barabasi_albert(1500, 5, 3), 1, 9.0, True),
     "ba_33_sims": (lambda: synth.barabasi_albert(1500, 5, 3), 33, 3.0, True),
     "hubs_70_sims": (lambda: synth.powerlaw_cm(3000, 2.1, 3, 800, 5), 70, 2.0, True),
+    "er_7_words": (lambda: synth.erdos_renyi(4865, 0.002, 6), 224, 2.0, True),
+    "er_8_words": (lambda: synth.erdos_renyi(4865, 0.002, 6), 225, 2.0, True),
     "er_9_words": (lambda: synth.erdos_renyi(4865, 0.002, 6), 260, 1.5, True),
     "share_3_of_1_word": (lambda: synth.barabasi_albert(45001, 4, 7), 20, 3.0, True),
     "share_3_of_5_words": (lambda: synth.barabasi_albert(9999, 5, 8), 130, 2.0, True),
@@ -47,7 +55,7 @@ def _oracle(name):
     finally:
         sir.philox4x32_10 = draw
     deg = np.diff(g.row_ptr).astype(np.int64)
-    return g, idx, args, ref, np.array([DENSE * deg[f].sum() > g.nnz for f in frontiers])
+    return g, idx, args, ref, np.array([_dense(sims) * deg[f].sum() > g.nnz for f in frontiers])
 
 
 @pytest.mark.parametrize("name", list(CASES))

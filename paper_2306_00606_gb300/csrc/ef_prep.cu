@@ -312,20 +312,24 @@ __device__ __forceinline__ int cross_bits(const RowOut &ro, const int32_t *__res
     return ci[a] < ro.goff[lo] || ci[b - 1] >= ro.goff[lo + 1] ? ERRB_CROSS : 0;
 }
 
-// A warp's share of the symmetry sum, and whether one of its rows is a long
-// owner of the pair tests (a plain store of a constant: an atomic maximum per
-// warp cost 40 us on the 1M-node power-law graph).
-__device__ __forceinline__ void add_rows(int32_t *cnt, uint64_t sym, int most) {
+// A warp's share of the symmetry sum, and whether one of its rows is long
+// (CNT_LONG, CNT_WIDE): plain stores of a constant, each by the first warp of a
+// block that has cause (seen: a bit per flag, zero before).  Measured: an atomic
+// maximum per warp 40 us on the 1M-node power-law graph, a store per warp 6 us
+// and a look before it 8 us on 400k nodes of minimum degree 2.
+__device__ __forceinline__ void add_rows(int32_t *cnt, uint64_t sym, int most, int *seen) {
     sym = warp_sum(sym);
     most = __reduce_max_sync(FULL, most);
     if ((threadIdx.x & 31) == 0) {
         if (sym) atomicAdd(reinterpret_cast<unsigned long long *>(cnt + CNT_SYM), (unsigned long long)sym);
-        // (looked at first: stores of thousands of warps to one word cost 6 us)
-        const volatile int32_t *flags = cnt;
-        if (most > TRI_LONG && !flags[CNT_LONG]) cnt[CNT_LONG] = 1;
-        if (most > TABLE_WIDE && !flags[CNT_WIDE]) cnt[CNT_WIDE] = 1;
+        if (most > TABLE_WIDE) {
+            const int bits = most > TRI_LONG ? 3 : 1, mine = bits & ~atomicOr(seen, bits);
+            if (mine & 1) cnt[CNT_WIDE] = 1;
+            if (mine & 2) cnt[CNT_LONG] = 1;
+        }
     }
 }
+static_assert(TABLE_WIDE <= TRI_LONG, "a list of the long ones is a wide one");
 
 // A row of the row pass walked by a whole warp.
 __device__ __forceinline__ void row_stats_warp(const int32_t *__restrict__ ci, const int32_t *__restrict__ D,
@@ -424,7 +428,9 @@ __device__ __forceinline__ void rows_short(const int32_t *__restrict__ rp, const
         }
     }
     if (err) atomicOr(cnt + CNT_ERR, err);
-    add_rows(cnt, sym, 0);
+    sym = warp_sum(sym);
+    if ((threadIdx.x & 31) == 0 && sym)
+        atomicAdd(reinterpret_cast<unsigned long long *>(cnt + CNT_SYM), (unsigned long long)sym);
 }
 
 // Rows of degree < hub_min (RowOrder): a thread per row of degree <= tmax,
@@ -439,7 +445,11 @@ __global__ void __launch_bounds__(256, 6) k_row_stats(const int32_t *__restrict_
         return;
     }
     __shared__ RowOrder s_ord;
-    if (threadIdx.x == 0) s_ord.load(cnt, n, bins_ok);
+    __shared__ int s_seen;
+    if (threadIdx.x == 0) {
+        s_ord.load(cnt, n, bins_ok);
+        s_seen = 0;
+    }
     __syncthreads();
     const RowOrder &ord = s_ord;
     const int total = ord.total();
@@ -493,7 +503,7 @@ __global__ void __launch_bounds__(256, 6) k_row_stats(const int32_t *__restrict_
             }
         }
     }
-    add_rows(cnt, sym, most);
+    add_rows(cnt, sym, most, &s_seen);
 }
 
 __global__ void __launch_bounds__(ROW_CTA) k_row_stats_hub(const int32_t *__restrict__ rp,
@@ -504,6 +514,8 @@ __global__ void __launch_bounds__(ROW_CTA) k_row_stats_hub(const int32_t *__rest
     __shared__ int64_t s_buf[32];
     const int total = hub_total(cnt);
     if ((int)blockIdx.x >= total) return;
+    __shared__ int s_seen;
+    if (threadIdx.x == 0) s_seen = 0;   // (the row sums' barriers lie before its use)
     uint64_t sym = 0;
     int most = 0;
     for (int it = blockIdx.x; it < total; it += gridDim.x) {
@@ -526,7 +538,7 @@ __global__ void __launch_bounds__(ROW_CTA) k_row_stats_hub(const int32_t *__rest
             if (const int e2 = cross_bits(ro, ci, u, a, b)) atomicOr(cnt + CNT_ERR, e2);
         }
     }
-    add_rows(cnt, sym, most);
+    add_rows(cnt, sym, most, &s_seen);
 }
 
 // ------------------------------------------------------------- orientation

@@ -237,6 +237,9 @@ struct RowOrder {
 // Range, self-loop and strict-order checks; sigma1 = sum of neighbour degrees,
 // sigma2 = sum of their squares, and the out-degree in (degree, id) order.
 //
+// Column indices run in 32 unsigned bits here and in the orientation: a step
+// past the last row of a graph with m near 2^31 is above 2^31 - 1.
+//
 // Symmetry check: every entry adds edge_print(v, x) to a per-thread sum,
 // reduced per warp into the global symmetry sum (counters[CNT_SYM]), which
 // is 0 for a symmetric CSR; the host reads it with the validation word.
@@ -262,17 +265,18 @@ struct RowStats {
                                         int v, int Dv, int a, int b) {
         const NodeMix mv = node_mix(v);
         int prev = 0;
-        for (int e0 = a; e0 < b; e0 += 4) {
+        const unsigned end = b;
+        for (unsigned e0 = a; e0 < end; e0 += 4) {
             int x[4], Dx[4];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) x[q] = e0 + q < b ? ci[e0 + q] : 0;
+            for (int q = 0; q < 4; ++q) x[q] = e0 + q < end ? ci[e0 + q] : 0;
 #pragma unroll
-            for (int q = 0; q < 4; ++q) Dx[q] = e0 + q < b && x[q] >= 0 && x[q] < n ? D[x[q]] : 0;
+            for (int q = 0; q < 4; ++q) Dx[q] = e0 + q < end && x[q] >= 0 && x[q] < n ? D[x[q]] : 0;
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
-                if (e0 + q < b) {
+                if (e0 + q < end) {
                     const int xq = x[q];
-                    const bool later = e0 + q > a;
+                    const bool later = e0 + q > (unsigned)a;
                     const int before = prev;
                     prev = xq;
                     if (xq < 0 || xq >= n) {
@@ -337,7 +341,7 @@ __device__ __forceinline__ void row_stats_warp(const int32_t *__restrict__ ci, c
                                                int32_t *__restrict__ cnt, uint64_t &sym, int &most) {
     RowStats r;
     const NodeMix mu = node_mix(u);
-    for (int e = ua + lane; e < ub; e += 32) r.entry(ci, D, n, u, ub - ua, ua, e, mu);
+    for (unsigned e = ua + lane; e < (unsigned)ub; e += 32) r.entry(ci, D, n, u, ub - ua, ua, (int)e, mu);
     const int64_t s1 = warp_sum(r.s1), s2 = warp_sum(r.s2);
     const int od = __reduce_add_sync(FULL, r.od);
     const int err = __reduce_or_sync(FULL, r.err);
@@ -523,7 +527,7 @@ __global__ void __launch_bounds__(ROW_CTA) k_row_stats_hub(const int32_t *__rest
         const int a = rp[u], b = rp[u + 1];
         RowStats r;
         const NodeMix mu = node_mix(u);
-        for (int e = a + threadIdx.x; e < b; e += ROW_CTA) r.entry(ci, D, n, u, b - a, a, e, mu);
+        for (unsigned e = a + threadIdx.x; e < (unsigned)b; e += ROW_CTA) r.entry(ci, D, n, u, b - a, a, (int)e, mu);
         const int64_t s1 = block_sum<int64_t>(r.s1, s_buf);
         const int64_t s2 = block_sum<int64_t>(r.s2, s_buf);
         const int64_t od = block_sum<int64_t>(r.od, s_buf);
@@ -623,11 +627,12 @@ __device__ __forceinline__ int64_t Orient::row(int v, int Dv, int a, int b, int 
         int nb = 0;
         const bool hashed = table(v, hb, nb);
         uint64_t used = 0;   // keys per bucket, 4 bits each
-        for (int e0 = a; e0 < b; e0 += CHUNK) {
+        const unsigned end = b;
+        for (unsigned e0 = a; e0 < end; e0 += CHUNK) {
             int x[CHUNK];
             int4 nf[CHUNK];
 #pragma unroll
-            for (int q = 0; q < CHUNK; ++q) x[q] = e0 + q < b ? ci[e0 + q] : -1;
+            for (int q = 0; q < CHUNK; ++q) x[q] = e0 + q < end ? ci[e0 + q] : -1;
 #pragma unroll
             for (int q = 0; q < CHUNK; ++q) nf[q] = node(x[q]);
 #pragma unroll
@@ -764,12 +769,12 @@ __device__ __forceinline__ void orient_row_warp(const Orient &o, int u, int ua, 
                                                 int64_t *__restrict__ omega) {
     int64_t om = 0;
     int mn = 0x7fffffff, mx = 0;
-    for (int e0 = ua; e0 < ub; e0 += 32) {
-        const int e = e0 + lane;
+    for (unsigned e0 = ua; e0 < (unsigned)ub; e0 += 32) {
+        const unsigned e = e0 + lane;
         int x = 0;
         int4 nf = make_int4(0, 0, 0, 0);
-        const bool isout = e < ub && o.probe(u, ub - ua, e, x, nf, om);
-        if (e < ub && x >= 0 && x < o.n) {
+        const bool in = e < (unsigned)ub, isout = in && o.probe(u, ub - ua, (int)e, x, nf, om);
+        if (in && x >= 0 && x < o.n) {
             mn = min(mn, nf.x);
             mx = max(mx, nf.x);
         }
@@ -922,12 +927,12 @@ __global__ void __launch_bounds__(ROW_CTA) k_orient_hub(const int32_t *__restric
         __syncthreads();
         int64_t om = 0;
         int64_t mn = 0x7fffffff, mx = 0;
-        for (int e0 = a; e0 < b; e0 += ROW_CTA) {
-            const int e = e0 + threadIdx.x;
+        for (unsigned e0 = a; e0 < (unsigned)b; e0 += ROW_CTA) {
+            const unsigned e = e0 + threadIdx.x;
             int x = 0;
             int4 nf = make_int4(0, 0, 0, 0);
-            const bool isout = e < b && o.probe(u, b - a, e, x, nf, om);
-            if (e < b && x >= 0 && x < n) {
+            const bool in = e < (unsigned)b, isout = in && o.probe(u, b - a, (int)e, x, nf, om);
+            if (in && x >= 0 && x < n) {
                 mn = min(mn, (int64_t)nf.x);
                 mx = max(mx, (int64_t)nf.x);
             }

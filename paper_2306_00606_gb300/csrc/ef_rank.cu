@@ -55,10 +55,11 @@ __global__ void k_omega_mm(const int32_t *__restrict__ rp, const int32_t *__rest
         };
         if (in && Dv <= tmax) {
             OmegaRow r;
-            for (int e0 = a; e0 < b; e0 += 4) {
+            const unsigned end = b;   // (unsigned: as in the row pass)
+            for (unsigned e0 = a; e0 < end; e0 += 4) {
                 int x[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) x[q] = e0 + q < b ? ci[e0 + q] : -1;
+                for (int q = 0; q < 4; ++q) x[q] = e0 + q < end ? ci[e0 + q] : -1;
 #pragma unroll
                 for (int q = 0; q < 4; ++q)
                     if (x[q] >= 0 && x[q] < n) r.add(D[x[q]], sig1[x[q]]);
@@ -72,7 +73,7 @@ __global__ void k_omega_mm(const int32_t *__restrict__ rp, const int32_t *__rest
             const int u = (int)(base + j);
             const int ua = __shfl_sync(FULL, a, j), ub = __shfl_sync(FULL, b, j);
             OmegaRow r;
-            for (int e = ua + lane; e < ub; e += 32) {
+            for (unsigned e = ua + lane; e < (unsigned)ub; e += 32) {
                 const int x = ci[e];
                 if (x >= 0 && x < n) r.add(D[x], sig1[x]);
             }
@@ -99,7 +100,7 @@ __global__ void __launch_bounds__(ROW_CTA) k_omega_mm_hub(const int32_t *__restr
         const int u = hub_row(bins, n, cnt, it);
         const int a = rp[u], b = rp[u + 1];
         OmegaRow r;
-        for (int e = a + threadIdx.x; e < b; e += ROW_CTA) {
+        for (unsigned e = a + threadIdx.x; e < (unsigned)b; e += ROW_CTA) {
             const int x = ci[e];
             if (x >= 0 && x < n) r.add(D[x], sig1[x]);
         }

@@ -983,6 +983,13 @@ int ef_autotune(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const ef_opt
     o.graph = 0;
     rc = run_job(ctx, Job{g->row_ptr, g->col_idx, n, m, nullptr, 0, o, none}, &none);
     if (rc) return rc;
+    // Without rows above SMALL_MAX only grid_per_sm reaches a kernel of the path
+    // taken: the other knobs keep their values, which later graphs would get
+    // from the noise of these timings.
+    int32_t big = 0;
+    CU(cudaMemcpyAsync(&big, ctx->scratch_counters + ef::BIN_BIG, sizeof big, cudaMemcpyDeviceToHost,
+                       ctx->stream));
+    CU(cudaStreamSynchronize(ctx->stream));
     o.trust_input = 1;
     const ef::Tune start = ctx->tune;
     o.graph = 1;
@@ -1010,6 +1017,7 @@ int ef_autotune(ef_ctx *ctx, const ef_csr *g, int32_t n, int64_t m, const ef_opt
     if (rc) { ctx->tune = start; return rc; }
     for (int sweep = 0; sweep < 2; ++sweep) {
         for (int knob = 0; knob < 5; ++knob) {
+            if (big == 0 && knob != 3) continue;
             const int *vals = knob == 0 ? rows : knob == 1 ? hubs : knob == 2 ? tris : knob == 3 ? grids : layouts;
             const int nv = knob == 0 ? 3 : knob == 1 ? 3 : knob == 2 ? 2 : knob == 3 ? 4 : 2;
             for (int i = 0; i < nv; ++i) {

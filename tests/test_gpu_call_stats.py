@@ -1,8 +1,8 @@
 """What ef_get_stats says of profiled calls: the kernels that a call launches,
 against the launches that the CUDA profiler records, for every path a call can
 take and every way it is decided; the pass that the fused kernel of graphs
-without long rows is booked under; and what a replayed graph does with other
-output buffers."""
+without long rows is booked under; what a replayed graph does with other output
+buffers; and what the autotuner may learn from such a graph."""
 import json
 
 import numpy as np
@@ -113,3 +113,21 @@ def test_replay_with_other_outputs(ctx, tmp_path, name, mode):  # noqa: F811
     assert ctx.stats(reset=True)["graph_replays"] == 0
     call(sets[1])
     assert ctx.stats(reset=True)["graph_replays"] == 1
+
+
+@pytest.mark.parametrize("kw", [{}, {"trust_input": True}])
+def test_autotune_on_short_rows_keeps_what_it_cannot_measure(ctx, kw):  # noqa: F811
+    """No row above degree 32: row_thread_max, hub_min, tri_variant and layout reach no kernel that such a graph runs."""
+    import torch
+    import paper_2306_00606_gb300 as ef
+    g = synth.watts_strogatz(4000, 8, 0.1, 5)
+    rp, ci = torch.from_numpy(g.row_ptr).cuda(), torch.from_numpy(g.col_idx).cuda()
+    start = dict(row_thread_max=13, hub_min=200, tri_variant=1, grid_per_sm=40, layout=2)
+    ef.ef_set_tuning(ctx.handle, start)
+    try:
+        best = ef.ef_autotune(ctx.handle, rp, ci, precision="fp32c", reps=2, **kw)
+        assert {k: v for k, v in best.items() if k != "grid_per_sm"} == \
+            {k: v for k, v in start.items() if k != "grid_per_sm"}
+        assert ef.ef_get_tuning(ctx.handle) == best
+    finally:
+        ef.ef_set_tuning(ctx.handle, None)

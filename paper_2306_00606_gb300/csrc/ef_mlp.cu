@@ -182,7 +182,7 @@ constexpr int MLP_WARPS = 8;
 constexpr int W2ROW = 40;   // words of a W2 row: 4 k-chunks x 4 lanes x 2 words, padded
 
 struct InferSmem {
-    uint2 w1[MLP_H * 4 + MLP_H / 8 * 4];   // [n][t] of the one k-chunk, 4 words' pad after 8 rows
+    uint2 w1[MLP_H * 4];                   // [n][t] of the one k-chunk
     uint2 w2[MLP_H * W2ROW / 2];           // [n][kc][t]
     float2 b1[MLP_H / 2], b2[MLP_H / 2], w3[MLP_H / 2];
     float mean[MLP_F], istd[MLP_F];
@@ -433,7 +433,8 @@ __global__ void __launch_bounds__(MLP_WARPS * 32, 1) k_mlp_grad(ModelDev *M, con
         uint32_t *h0 = reinterpret_cast<uint32_t *>(S.h1 + (16 * w + g) * HS), *h8 = h0 + 8 * HS / 2;
         uint32_t *d0p = reinterpret_cast<uint32_t *>(S.e2 + (16 * w + g) * HS), *d8p = d0p + 8 * HS / 2;
         uint32_t *f0p = reinterpret_cast<uint32_t *>(S.e1 + (16 * w + g) * HS), *f8p = f0p + 8 * HS / 2;
-        uint32_t h1p[8][2], e2p[8][2];
+        uint32_t e2p[8][2];
+        uint32_t active = 0;   // bit 4 j + i: h1[j][i] > 0 (BF16 rounds the smallest positive values to 0)
         {
             Tile T;
             tile_forward(s, x0, x1, v0, v1, T);
@@ -459,11 +460,10 @@ __global__ void __launch_bounds__(MLP_WARPS * 32, 1) k_mlp_grad(ModelDev *M, con
                 gb2[j][1] += b + d;
                 e2p[j][0] = pack_bf16(a, b);
                 e2p[j][1] = pack_bf16(c, d);
-                // h1 >= 0: a positive value stays positive in BF16 (same exponent range)
-                h1p[j][0] = pack_bf16(T.h1[j][0], T.h1[j][1]);
-                h1p[j][1] = pack_bf16(T.h1[j][2], T.h1[j][3]);
-                h0[4 * j + t] = h1p[j][0];
-                h8[4 * j + t] = h1p[j][1];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) active |= T.h1[j][i] > 0.f ? 1u << (4 * j + i) : 0u;
+                h0[4 * j + t] = pack_bf16(T.h1[j][0], T.h1[j][1]);
+                h8[4 * j + t] = pack_bf16(T.h1[j][2], T.h1[j][3]);
                 d0p[4 * j + t] = e2p[j][0];
                 d8p[4 * j + t] = e2p[j][1];
             }
@@ -479,10 +479,8 @@ __global__ void __launch_bounds__(MLP_WARPS * 32, 1) k_mlp_grad(ModelDev *M, con
                 mma16816(e, a, *reinterpret_cast<const uint32_t *>(&s.w2r[nn * W2S + 16 * kc + 2 * t]),
                          *reinterpret_cast<const uint32_t *>(&s.w2r[nn * W2S + 16 * kc + 2 * t + 8]));
             }
-            e[0] = h1p[j][0] & 0xffffu ? e[0] : 0.f;
-            e[1] = h1p[j][0] >> 16 ? e[1] : 0.f;
-            e[2] = h1p[j][1] & 0xffffu ? e[2] : 0.f;
-            e[3] = h1p[j][1] >> 16 ? e[3] : 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) e[i] = active >> (4 * j + i) & 1u ? e[i] : 0.f;
             gb1[j][0] += e[0] + e[2];
             gb1[j][1] += e[1] + e[3];
             f0p[4 * j + t] = pack_bf16(e[0], e[1]);

@@ -46,3 +46,19 @@ def test_gradient_rows(ctx, rows):  # noqa: F811
         tol = 0.0 if exact else 2.0 ** -6 * np.ravel(sums[k]) + 1e-12
         assert np.all(np.abs(a - b) <= tol), (k, float(np.max(np.abs(a - b))))
         o += size
+
+
+def test_gradient_of_the_smallest_activations(ctx):  # noqa: F811
+    """A hidden unit whose activation is positive in FP32 but rounds to 0 in BF16 is active: its bias has a gradient."""
+    p, X, _ = dyadic_network(13, 32)
+    p["W1"][:] = 0.0
+    p["b1"] = np.resize(np.array([1e-41, 0.0, -1e-41, 0.5, 2e-45]), 64).astype(np.float32).astype(np.float64)
+    y = sg.forward(p, X)[0] - 1.0
+    _, grad = _model(ctx, p).grad(_dev(X.astype(np.float32)), _dev(y.astype(np.float32)))
+    _, ref = sg.loss_and_grads(p, X, y)
+    assert np.count_nonzero(ref["b1"][(p["b1"] > 0) & (p["b1"] < 1e-40)]) > 10
+    o = 0
+    for k in sg.TRAINED:
+        size = int(np.prod(sg.SHAPES[k]))
+        np.testing.assert_allclose(grad[o:o + size].astype(np.float64), np.ravel(ref[k]), rtol=0, atol=1e-37, err_msg=k)
+        o += size

@@ -465,6 +465,30 @@ __device__ __forceinline__ float lg2(float d) {
 // d * log2(d) for integral d >= 1 held in a float.
 __device__ __forceinline__ float dlog2d(float d) { return d * lg2(d); }
 
+// (float)x and (float)sqrt((double)x) for x >= 0 without 64-bit conversions and
+// FP64 operations, which run at a small fraction of the FP32 rate here (they
+// bound the features of a ranking): below 2^32, and 2^46 for the root, by 32-bit
+// ones.  Ranking BA 4M / 8M / 16M: 3.50 -> 3.43, 6.01 -> 5.87, 12.2 -> 12.0 ms.
+__host__ __device__ __forceinline__ float to_float(int64_t x) {
+    return (uint64_t)x >> 32 ? (float)x : (float)(uint32_t)x;
+}
+
+// The root of x = h + l (both exact): an FP32 root r plus a first-order
+// correction c, rounded once.  c is within 2^-20 of itself; where that leaves
+// the rounding open (one value in 300 000) the FP64 root decides, so the
+// result is the FP64 root rounded, for every x.
+__host__ __device__ __forceinline__ float sqrt_exact(int64_t x) {
+    if ((uint64_t)x >> 46) return (float)sqrt((double)x);
+    const uint32_t hi = (uint32_t)(x >> 23), lo = (uint32_t)x & 0x7fffffu;
+    const float a = (float)hi * 8388608.0f, b = (float)lo;   // both exact
+    const float h = a + b, l = b - (h - a);
+    if (h == 0.0f) return 0.0f;
+    const float r = sqrtf(h);
+    const float c = (fmaf(-r, r, h) + l) * (0.5f / r);
+    const float up = fmaf(c, 1.0f + 0x1p-18f, r), down = fmaf(c, 1.0f - 0x1p-18f, r);
+    return up == down ? up : (float)sqrt((double)x);
+}
+
 // Two floats rounded to BF16 (nearest, ties to even), lo in the low half.
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     __nv_bfloat162 h = __floats2bfloat162_rn(lo, hi);

@@ -139,27 +139,6 @@ int launch_omega_mm(const int32_t *rp, const int32_t *ci, int32_t n, int64_t m, 
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-// (float)x and (float)sqrt((double)x) for x >= 0 without 64-bit conversions and
-// FP64 operations, which run at a small fraction of the FP32 rate here (they
-// bound the features of a ranking): below 2^32, and 2^46 for the root, by 32-bit
-// ones.  Ranking BA 4M / 8M / 16M: 3.50 -> 3.43, 6.01 -> 5.87, 12.2 -> 12.0 ms; the
-// features are equal bit for bit on BA 1M, power-law 1M and R-MAT 2^16.
-__device__ __forceinline__ float to_float(int64_t x) {
-    return (uint64_t)x >> 32 ? (float)x : (float)(uint32_t)x;
-}
-
-// The root of x = h + l (both exact) as an FP32 value plus a first-order
-// correction (relative error below 2^-46), rounded once.
-__device__ __forceinline__ float sqrt_exact(int64_t x) {
-    if ((uint64_t)x >> 46) return (float)sqrt((double)x);
-    const uint32_t hi = (uint32_t)(x >> 23), lo = (uint32_t)x & 0x7fffffu;
-    const float a = (float)hi * 8388608.0f, b = (float)lo;   // both exact
-    const float h = a + b, l = b - (h - a);
-    if (h == 0.0f) return 0.0f;
-    const float r = sqrtf(h);
-    return r + (fmaf(-r, r, h) + l) * (0.5f / r);
-}
-
 // The 16 features of every node (in the order of the oracle's FEATURE_NAMES).
 // mode 1 uses the triangle counts tcnt, mode 0 takes t = 0.  BF16: each row
 // standardised with the model's mean and standard deviation, z = (x - mean)

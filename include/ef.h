@@ -57,7 +57,11 @@ enum ef_precision {
     EF_PREC_FP64 = 0,  /* d ln d computed in FP64 (a table held as FP32
                           pairs, within 2^-48); row sums in FP32-pair
                           chunks of at most 32 terms (below 3.6e-12
-                          relative each), everything else in FP64, ln S
+                          relative each); at middle nodes of degree >= 257
+                          such sums at 16 points per octave of neighbour
+                          degree, interpolated in between (which multiplies
+                          their errors by 2.8 at most); everything else
+                          in FP64, ln S
                           and T/S by a table-based logarithm and a refined
                           reciprocal (about 1e-14 relative).  EF within
                           1e-9 relative of the exact value */
@@ -152,7 +156,8 @@ typedef struct {
     double wedge_big_ms;   /* middle nodes of degree > 32 */
     double tri_hash_ms;    /* always 0: the orientation builds the hash
                               tables of the long out-lists (orient_ms) */
-    double tri_pairs_ms;   /* triangle pair tests and corrections (one kernel) */
+    double tri_pairs_ms;   /* triangle pair tests and corrections (with out-
+                              lists of more than 32 entries three kernels) */
     double finalize_ms;    /* per-node sums, S, N, EF */
     double total_ms;
     int64_t kernels;       /* kernels launched by profiled calls */

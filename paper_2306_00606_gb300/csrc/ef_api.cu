@@ -655,8 +655,8 @@ int features_device(ef_ctx *ctx, const int32_t *rp, const int32_t *ci, int32_t n
 }
 
 // Exact EF of list[0..k) (k on the device when kptr is given): the wedge
-// kernels over bins of the listed nodes and their neighbours, then a CTA per
-// listed node.  Triangles: per listed node (few nodes), or (global_tri) the
+// kernels over bins of the listed nodes and their neighbours, then blocks and
+// warps over the listed nodes.  Triangles: per listed node (few nodes), or (global_tri) the
 // full oriented triangle pass, which costs less once the list holds the
 // high-EF nodes next to the hubs; orient_done / tri_done: the features
 // already ran the orientation / the whole triangle pass; listed: about how

@@ -383,7 +383,7 @@ __device__ __forceinline__ int mid_node(const int32_t *bins, int32_t n, const in
     return it < first ? bins[(size_t)BIN_MIDHI * n + it] : bins[(size_t)BIN_MID * n + (it - first)];
 }
 
-// Total number of hub rows (degree > MID_MAX) in the hub buckets.
+// Total number of hub rows (degree >= hub_min) in the hub buckets.
 __device__ __forceinline__ int hub_total(const int32_t *cnt) {
     int t = 0;
 #pragma unroll

@@ -34,13 +34,10 @@
 // 128 entries staged by coalesced loads); loading each test's correction
 // tq[sum] with its probes, to save the second round trip of a hit, was
 // slower too (1.85 against 1.65 ms; the per-unit binary search replaced by
-// a shared-memory unit map changed nothing).  Under ncu (half-size graph)
-// the kernel issues in 46% of cycles, waits on long-scoreboard loads (7.2
-// cycles per issue) with 39% of the warp slots filled (64 registers), and
-// uses 31% of L2 and 8% of DRAM throughput: bound by the latency of its
-// probes at the concurrency its registers allow.  The pass reads about 1.5 GB from DRAM per launch,
-// mostly misses of the long tail of membership probes (10% of the tests spread
-// over about 100 MB of tables and lists).
+// a shared-memory unit map changed nothing).  Short owners of the 2M-node
+// power-law graph: the kernel issues in 48% of its cycles and waits 9.0 cycles
+// per instruction on its loads, with 45% of the warp slots filled (64
+// registers allow half); DRAM 17%, L2 26% of their throughput.
 //
 // The pass is integer-only: g comes from a table in fixed point (units of
 // 2^-F, F chosen per call from the maximum degree), so the sums are exact and
@@ -265,8 +262,8 @@ __global__ void __launch_bounds__(TRI_WARPS * 32, TRI_BLOCKS) k_tri_pairs(
 // sorted by rank (k_sort_long), so that of a pair b before c the lower end is
 // always b.  Then a warp per 32 candidates (k_tri_long): lane l holds c =
 // N+(a)[32 k + l] and the warp walks the earlier entries b, whose table is
-// the same for all lanes: a test is a hash, two 16-byte loads and their
-// compares, with nothing to decide per lane.  The hits of 32 b are kept as a
+// the same for all lanes: a test is a hash, one 32-byte load (of a short list
+// two of 16) and its compares, with nothing to decide per lane.  The hits of 32 b are kept as a
 // bit matrix (a word per lane); its rows give c's credits, its transpose b's,
 // so a correction is looked up only where a triangle is, and the credits go
 // out once per (a, c) and per (a, b, item) instead of once per hit.  (Where
@@ -274,10 +271,10 @@ __global__ void __launch_bounds__(TRI_WARPS * 32, TRI_BLOCKS) k_tri_pairs(
 // large c had bound the pass.)
 //
 // Pair tests of a call, all owners in k_tri_pairs / with the long owners
-// here: R-MAT 2^16 (955k entries) 0.74 / 0.21 ms, R-MAT 2^18 1.9 / 0.62,
-// power-law 4M 1.60 / 1.39, its 87M-entry variant 5.8 / 4.8.  Here the
-// kernel issues in half of the cycles and its loads, one sector per lane, use
-// 63% of the L1 wavefronts; half of the rest is k_tri_pairs.  TRI_LONG = 16:
+// here: R-MAT 2^16 (955k entries) 0.74 / 0.21 ms (0.18 with shared items),
+// R-MAT 2^18 1.9 / 0.62, power-law 4M 1.60 / 1.36, its 87M-entry variant 5.8 /
+// 4.7.  The kernel issues in 54% of its cycles on both (L1 wavefronts 53%,
+// loads waited for 5.4 and 5.8 cycles per instruction).  TRI_LONG = 16:
 // R-MAT 2^16 0.17 but power-law 4M 1.42 and 0.40 against 0.38 at 1M (lanes
 // past the list idle); four entries b together: 1.42.  Without the sort, the
 // lower end of each pair decided per lane and b's credits reduced by warp

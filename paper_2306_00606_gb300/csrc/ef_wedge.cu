@@ -704,11 +704,11 @@ struct HubSmemK {
     static constexpr int value = F64 ? 3072 : HUB_SMEM_K;
 };
 
-// One CTA per hub (degree > MID_MAX; in FP64 also the rows of BIN_MIDHI, from
-// degree MID_SPLIT on), hubs taken largest degree bucket first
-// from an atomic counter.  Global arrays hold the class index of every
-// neighbour (cidx_g, at the hub's own row positions) and, for hubs with more
-// than HUB_SMEM_K classes, the classes themselves (cls_g, q_g).
+// One CTA per hub (degree >= hub_min, by default above MID_MAX; in FP64 also the
+// rows of BIN_MIDHI, from degree MID_SPLIT on), hubs taken largest degree
+// bucket first from an atomic counter.  Global arrays hold the class index of
+// every neighbour (cidx_g, at the hub's own row positions) and, for hubs with
+// more classes than HubSmemK, the classes themselves (cls_g, q_g).
 template <bool F64>
 __global__ void __launch_bounds__(HUB_THREADS) k_wedge_hub(
     const int32_t *__restrict__ rp, const int32_t *__restrict__ ci, const int32_t *__restrict__ D,

@@ -49,12 +49,13 @@ WORKLOADS = {
 BATCHED = {"ws4096"}
 PASSES = ("prep_ms", "orient_ms", "wedge_small_ms", "wedge_big_ms", "tri_pairs_ms", "finalize_ms")
 PASS_KERNEL = {"prep_ms": "k_degrees+k_row_stats+k_row_stats_hub",
-               "orient_ms": "k_ftab+layout+scan+k_node_info+k_orient+k_orient_hub+k_hash_rows",
-               "wedge_small_ms": "k_wedge_small<4,8,16,32>", "wedge_big_ms": "k_wedge_mid+k_wedge_hub",
-               "tri_pairs_ms": "k_tri_pairs", "finalize_ms": "k_finalize"}
+               "orient_ms": "k_ftab+k_clear_lists+layout+scan+k_node_info+k_orient+k_orient_hub+k_hash_rows",
+               "wedge_small_ms": "k_wedge_small<4,8,16,32> or k_short", "wedge_big_ms": "k_wedge_mid+k_wedge_hub",
+               "tri_pairs_ms": "k_tri_pairs+k_sort_long+k_tri_long", "finalize_ms": "k_finalize"}
 PASS_NOTE = {"prep_ms": "bound by random L2 gathers of neighbour degrees",
              "orient_ms": "bound by random L2 gathers of neighbour records; also fills the out-list hash tables",
-             "wedge_small_ms": "bound by MUFU lg2 and FP32 adds (one f evaluation per ordered pair)",
+             "wedge_small_ms": "bound by MUFU lg2 and FP32 adds (one f evaluation per ordered pair); without rows "
+                               "above 32 entries by the instruction issue of the fused kernel, triangles included",
              "wedge_big_ms": "bound by MUFU lg2 and FP32 adds over degree classes, and L2 reductions",
              "tri_pairs_ms": "bound by dependent L2 round trips (1.1e8 membership tests), not HBM bandwidth",
              "finalize_ms": "streaming, HBM-bound"}
@@ -65,15 +66,24 @@ def algorithmic_bytes(g, st):
     written once; gathers that hit L2 are not counted)."""
     n, m = g.n, g.nnz
     d = g.degrees.astype(np.int64)
+    # hash-table slots per oriented entry: three where some out-list has more than 24 entries, else two
+    src = np.repeat(np.arange(n, dtype=np.int32), d)
+    out = (d[src] < d[g.col_idx]) | ((d[src] == d[g.col_idx]) & (src < g.col_idx))
+    slots = 3 if np.bincount(src[out], minlength=1).max() > 24 else 2
     small = d[(d >= 1) & (d <= 32)]
     big = d[d > 32]
     csr = 4 * (n + 1) + 4 * m
+    if not len(big):
+        # the fused path: degrees (4 B) and {row start, word} (8 B) written by the row passes; entries and words
+        # read, packed sums, T and triangles (20 B) written by k_short; those read and EF written
+        return {"prep_ms": csr + 12 * n, "orient_ms": 0, "wedge_small_ms": 4 * m + 28 * n, "wedge_big_ms": 0,
+                "tri_pairs_ms": 0, "finalize_ms": 28 * n}
     return {
         # row_ptr + col_idx read; D, sigma1, sigma2, outdeg written
         "prep_ms": csr + 4 * n + 16 * n + 4 * n,
         # CSR + outdeg read; out_ptr, out_col/out_D/out_src/out_pd (20 B per
-        # oriented entry), hash tables (2 slots per entry), omega written
-        "orient_ms": csr + 4 * n + 4 * (n + 1) + 28 * (m // 2) + 8 * n,
+        # oriented entry), hash tables (4 B per slot), omega written
+        "orient_ms": csr + 4 * n + 4 * (n + 1) + (20 + 4 * slots) * (m // 2) + 8 * n,
         # rows of the middle nodes read; Ccenter written, one 8-byte credit per row entry
         "wedge_small_ms": 4 * len(small) * 2 + 4 * int(small.sum()) + 8 * len(small) + 8 * int(small.sum()),
         "wedge_big_ms": 4 * len(big) * 2 + 4 * int(big.sum()) + 8 * len(big) + 8 * int(big.sum()),
@@ -84,10 +94,11 @@ def algorithmic_bytes(g, st):
     }
 
 
-PASS_PREFIX = {"prep_ms": ("k_degrees", "k_row_stats", "k_gate"),
-               "orient_ms": ("k_ftab", "k_layout", "k_scan", "k_node_info", "k_orient", "k_hash"),
-               "wedge_small_ms": ("k_wedge_small",), "wedge_big_ms": ("k_wedge_mid", "k_wedge_hub", "k_wedge_big", "k_big"),
-               "tri_pairs_ms": ("k_tri_pairs",), "finalize_ms": ("k_finalize",)}
+PASS_PREFIX = {"prep_ms": ("k_degrees", "k_row_stats"),
+               "orient_ms": ("k_ftab", "k_clear_lists", "k_layout", "k_scan", "k_node_info", "k_orient", "k_hash"),
+               "wedge_small_ms": ("k_wedge_small", "k_short"),
+               "wedge_big_ms": ("k_wedge_mid", "k_wedge_hub", "k_wedge_big", "k_big"),
+               "tri_pairs_ms": ("k_tri_pairs", "k_sort_long", "k_tri_long"), "finalize_ms": ("k_finalize",)}
 
 
 def committed_kernels(workload):
@@ -140,12 +151,19 @@ def passes_ncu(workload):
     return res
 
 
-def committed_traffic(kernel, workload):
-    """DRAM bytes per launch of `kernel` (name prefix) from the committed ncu
-    launch list, or None when there is none for this workload or the
-    kernel's source has changed since it was taken."""
-    ks = [r for k, r in committed_kernels(workload).items() if k.startswith(kernel)]
-    return ks[0]["dram_bytes_per_launch"] if len(ks) == 1 else None
+def committed_traffic(pass_name, workload):
+    """DRAM bytes per call of the kernels of a pass, from the committed ncu
+    launch list, or None when there is none for this workload or the source of
+    one of the pass's kernels in it has changed since it was taken."""
+    try:
+        recs = json.load(open(os.path.join(ROOT, "profiles", "traffic.json")))[workload]
+    except (OSError, KeyError, ValueError, TypeError):
+        return None
+    names = [k for k in recs if k.startswith(PASS_PREFIX[pass_name])]
+    fresh = committed_kernels(workload)
+    if not names or any(k not in fresh for k in names):
+        return None
+    return sum(fresh[k]["dram_bytes_per_launch"] for k in names)
 
 
 def parse():
@@ -252,8 +270,9 @@ class ClockSampler:
 
 
 def class_evals(g, hub_min: int = 513) -> int:
-    """f evaluations of the degree-class wedge kernels: K (K + 1) per middle
-    node of degree > 32, K its classes.  Neighbour degrees below 256 (warp
+    """f evaluations of the degree-class wedge kernels in FP32C: K (K + 1) per
+    middle node of degree > 32, K its classes (FP64 takes f from a table, and
+    from degree 257 on sums at 16 points per octave instead of per class).  Neighbour degrees below 256 (warp
     kernel, degree < hub_min) or 2048 (CTA kernel) merge into one class per
     degree; larger ones are a class each, as the kernels build them."""
     d = g.degrees.astype(np.int64)
@@ -905,22 +924,25 @@ def run_ours(args):
         hbm, src = 6800.0, "fallback"
     achieved = alg[dom] / (per[dom] / 1e3) / 1e9
     roofline = {"kernel": PASS_KERNEL[dom], "bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
-                "frac": achieved / hbm, "traffic": committed_traffic(PASS_KERNEL[dom], args.workload),
+                "frac": achieved / hbm, "traffic": committed_traffic(dom, args.workload),
                 "algorithmic_bytes": alg[dom], "launch_ms": per[dom], "peak_source": src,
                 "note": "bytes = each input read once and each output written once (bench.py "
                         "algorithmic_bytes); " + PASS_NOTE[dom]}
-    # the wedge passes against the MUFU issue bound: one lg2 per f evaluation,
-    # 16 special-function results per SM per clock
+    # the wedge passes against the MUFU issue bound (FP32C): one lg2 per f
+    # evaluation, 16 special-function results per SM per clock
     evals = st["small_evals"] + class_evals(g)
     wedge_ms = per["wedge_small_ms"] + per["wedge_big_ms"]
     sms = torch.cuda.get_device_properties(dev).multi_processor_count
     mhz = clocks.get("sm_max_mhz") or 2070.0
     mufu = sms * 16 * mhz * 1e6
-    roofline_alu = {"bound": "alu", "kernels": "wedge passes (k_wedge_small, k_wedge_mid, k_wedge_hub)",
+    roofline_alu = {"bound": "alu", "kernels": "wedge passes (k_wedge_small, k_wedge_mid, k_wedge_hub; k_short, triangles included, "
+                                               "without rows above 32 entries)",
                     "f_evaluations": evals, "achieved": evals / (wedge_ms / 1e3) / 1e9 if wedge_ms > 0 else None,
                     "peak": mufu / 1e9, "unit": "Geval/s",
                     "frac": evals / (wedge_ms / 1e3) / mufu if wedge_ms > 0 else None,
                     "peak_source": f"{sms} SMs x 16 MUFU results per clock x {mhz:.0f} MHz"}
+    if args.precision != "fp32c":
+        roofline_alu = None   # f comes from a table there
     path_bytes = 4 * (n + 1) + 4 * g.nnz + 8 * n
     roofline_path = {"bound": "hbm", "algorithmic_bytes": path_bytes,
                      "achieved": path_bytes / (ms_step / 1e3) / 1e9, "peak": hbm, "unit": "GB/s",

@@ -47,3 +47,32 @@ def test_pair_test_bytes_formula():
     assert alg["tri_pairs_ms"] == 4 * (n + 1) + 10 * m + 16 * n
     assert alg["finalize_ms"] == 68 * n
     assert all(v > 0 for v in alg.values())
+
+
+def test_orientation_bytes_count_the_tables():
+    """Two table slots per oriented entry, three once an out-list has more than 24 entries."""
+    for longest, slots in ((25, 2), (26, 3)):   # K_k: the longest out-list has k - 1 entries
+        g = synth.disjoint_union([synth.complete(longest), synth.star(40)])
+        alg = bench.algorithmic_bytes(g, bench.graph_stats(g))
+        assert alg["orient_ms"] == 8 * (g.n + 1) + 4 * g.nnz + 12 * g.n + (20 + 4 * slots) * (g.nnz // 2)
+
+
+def test_bytes_of_the_fused_path():
+    g = synth.complete(33)   # no row above 32 entries: no oriented copy, no pair tests
+    alg = bench.algorithmic_bytes(g, bench.graph_stats(g))
+    assert alg["orient_ms"] == alg["tri_pairs_ms"] == alg["wedge_big_ms"] == 0
+    assert alg["wedge_small_ms"] == 4 * g.nnz + 28 * g.n
+
+
+def test_every_kernel_of_a_call_belongs_to_a_pass():
+    """The kernels of an exact call in the sources: each is matched by one pass's prefixes."""
+    import os
+    import re
+    names = set()
+    for f in ("ef_prep.cu", "ef_tri.cu", "ef_wedge.cu", "ef_short.cu"):
+        text = open(os.path.join(bench.ROOT, "paper_2306_00606_gb300", "csrc", f)).read()
+        names |= set(re.findall(r"__global__[^;{]*?\b(k_\w+)\s*\(", text))
+    names |= {"k_finalize", "k_finalize_short", "k_finalize_either"}
+    assert {"k_short", "k_tri_long", "k_sort_long", "k_clear_lists", "k_row_stats"} <= names
+    for k in sorted(names):
+        assert len([p for p, pre in bench.PASS_PREFIX.items() if k.startswith(pre)]) == 1, k
